@@ -1542,11 +1542,12 @@ icarus_status icarus_get_padded(icarus_ctx *c, int member, int leaf, double *hos
   CK(cudaMemcpyAsync(raw.data(), static_cast<const char *>(c->U) + slot * stride, raw.size(),
                      cudaMemcpyDeviceToHost, c->stream));
   CK(cudaStreamSynchronize(c->stream));
-  if (c->prec) {
-    const float *f = reinterpret_cast<const float *>(raw.data());
-    for (size_t q = 0; q < n; q++) host[q] = (double)f[q];
-  } else {
-    memcpy(host, raw.data(), raw.size());
+  // [cell][8] to the host's [variable][cell]
+  const size_t pc = (size_t)c->kp.pcells;
+  for (size_t q = 0; q < n; q++) {
+    const size_t at = (q % pc) * NVAR + q / pc;
+    host[q] = c->prec ? (double)reinterpret_cast<const float *>(raw.data())[at]
+                      : reinterpret_cast<const double *>(raw.data())[at];
   }
   return ICARUS_OK;
 }
@@ -2131,6 +2132,33 @@ struct CkFile {
 
 size_t slot_bytes(const icarus_ctx *c) { return (size_t)c->kp.nvs * c->kp.pcells * c->rsize; }
 
+// A checkpoint holds a slot's variables one after the other, the device a
+// cell's side by side (the tracer follows them in both): the slots of `raw`
+// are turned from one form into the other in place.
+template <typename real>
+void turn_slots(const icarus_ctx *c, std::vector<unsigned char> &raw, bool to_file) {
+  const size_t pc = (size_t)c->kp.pcells, per = (size_t)c->kp.nvs * pc;
+  const long long ns = (long long)(raw.size() / (per * sizeof(real)));
+#pragma omp parallel
+  {
+    std::vector<real> tmp(NVAR * pc);
+#pragma omp for schedule(static)
+    for (long long s = 0; s < ns; s++) {
+      real *u = reinterpret_cast<real *>(raw.data()) + (size_t)s * per;
+      for (size_t q = 0; q < pc; q++)
+        for (int v = 0; v < NVAR; v++) {
+          const size_t cell = q * NVAR + v, var = v * pc + q;
+          tmp[to_file ? var : cell] = u[to_file ? cell : var];
+        }
+      memcpy(u, tmp.data(), sizeof(real) * NVAR * pc);
+    }
+  }
+}
+void turn_slots(const icarus_ctx *c, std::vector<unsigned char> &raw, bool to_file) {
+  if (c->prec) turn_slots<float>(c, raw, to_file);
+  else turn_slots<double>(c, raw, to_file);
+}
+
 }  // namespace
 
 extern "C" {
@@ -2182,6 +2210,7 @@ icarus_status icarus_save(icarus_ctx *c, const char *path) {
   F.put(&hits, sizeof(hits));
   const double isl[2] = {c->isl_pe, c->isl_beta};
   F.put(isl, sizeof(isl));
+  turn_slots(c, U, true);
   F.put(U.data(), U.size());
   const int32_t nth = (int32_t)theta.size();
   F.put(&nth, sizeof(nth));
@@ -2250,6 +2279,7 @@ icarus_status icarus_load(icarus_ctx *c, const char *path) {
   std::vector<float> theta(nth);
   F.get(theta.data(), sizeof(float) * nth);
   if (!F.ok) return ICARUS_ERR_ARG;
+  turn_slots(c, U, false);
   // everything read: replace the context's state
   c->mem = std::move(next);
   for (Member &M : c->mem) build_member_map(c, M);

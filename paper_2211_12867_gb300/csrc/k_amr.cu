@@ -12,20 +12,25 @@
 
 namespace {
 
+// variable v of a cell
 template <typename real>
 __device__ __forceinline__ size_t cidx(const KParams &kp, int slot, int v, int p0, int p1, int p2) {
-  return ((((size_t)slot * kp.nvs + v) * kp.P[0] + p0) * kp.P[1] + p1) * kp.P[2] + p2;
+  return v < NVAR ? cell_index(kp, slot, p0, p1, p2) + v : tracer_index(kp, slot, p0, p1, p2);
 }
 
+// the host's [slot][variable][i][j][k] in FP64 from and to the padded cells: a
+// thread takes a cell, so its side of the state is one access and a warp's
+// sides of the host array are eight runs of consecutive values
 template <typename real>
 __global__ void k_pack(const KParams kp, const real *U, int slot0, int nslots, double *out) {
-  const size_t n = (size_t)nslots * NVAR * kp.icells;
+  const size_t n = (size_t)nslots * kp.icells;
   for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
-    const int c = (int)(e % kp.icells);
-    const int v = (int)((e / kp.icells) % NVAR);
-    const int s = (int)(e / ((size_t)kp.icells * NVAR));
+    const int s = (int)(e / kp.icells), c = (int)(e - (size_t)s * kp.icells);
     const int k = c % kp.nb[2], j = (c / kp.nb[2]) % kp.nb[1], i = c / (kp.nb[2] * kp.nb[1]);
-    out[e] = (double)U[cidx<real>(kp, slot0 + s, v, i + NGH, j + NGH, k + NGH)];
+    real u[NVAR];
+    ld_cell(U + cell_index(kp, slot0 + s, i + NGH, j + NGH, k + NGH), u);
+#pragma unroll
+    for (int v = 0; v < NVAR; v++) out[((size_t)s * NVAR + v) * kp.icells + c] = (double)u[v];
   }
 }
 
@@ -44,8 +49,10 @@ __global__ void k_unpack(const KParams kp, real *U, int slot0, int nslots, const
     else
 #pragma unroll
       for (int v = 0; v < NVAR; v++) u[v] = x[v];
+    real o[NVAR];
 #pragma unroll
-    for (int v = 0; v < NVAR; v++) U[cidx<real>(kp, slot0 + s, v, i + NGH, j + NGH, k + NGH)] = (real)u[v];
+    for (int v = 0; v < NVAR; v++) o[v] = (real)u[v];
+    st_cell(U + cell_index(kp, slot0 + s, i + NGH, j + NGH, k + NGH), o);
   }
 }
 
@@ -96,8 +103,9 @@ __global__ void k_estimator(const KParams kp, const real *U, int slot0, double e
     const int p0 = i + NGH, p1 = j + NGH, p2 = k + NGH;
     // the speed gate first: E only matters where it is open, and not at all
     // once this thread has found a refining cell (the flags are unchanged)
-    const double r0 = (double)U[cidx<real>(kp, slot, 0, p0, p1, p2)];
-    const double m0 = (double)U[cidx<real>(kp, slot, 1, p0, p1, p2)];
+    real uc[NVAR];
+    ld_cell(U + cell_index(kp, slot, p0, p1, p2), uc);
+    const double r0 = (double)uc[0], m0 = (double)uc[1];
     {
       const int I = B.ix[0] * kp.nb[0] + i, J = B.ix[1] * kp.nb[1] + j, K = B.ix[2] * kp.nb[2] + k;
       const double vb = vbg[((size_t)(I >> sh) * kp.n_base_cells[1] + (J >> sh)) * kp.n_base_cells[2] + (K >> sh)];
@@ -106,17 +114,20 @@ __global__ void k_estimator(const KParams kp, const real *U, int slot0, double e
     }
     double u0[NVAR];
 #pragma unroll
-    for (int v = 0; v < NVAR; v++) u0[v] = (double)U[cidx<real>(kp, slot, v, p0, p1, p2)];
+    for (int v = 0; v < NVAR; v++) u0[v] = (double)uc[v];
     double rm[3], rp[3], pm[3], pp[3];
     for (int d = 0; d < 3; d++) {
       int m[3] = {p0, p1, p2}, p[3] = {p0, p1, p2};
       m[d]--;
       p[d]++;
       double um[NVAR], up[NVAR];
+      real xm[NVAR], xp[NVAR];
+      ld_cell(U + cell_index(kp, slot, m[0], m[1], m[2]), xm);
+      ld_cell(U + cell_index(kp, slot, p[0], p[1], p[2]), xp);
 #pragma unroll
       for (int v = 0; v < NVAR; v++) {
-        um[v] = (double)U[cidx<real>(kp, slot, v, m[0], m[1], m[2])];
-        up[v] = (double)U[cidx<real>(kp, slot, v, p[0], p[1], p[2])];
+        um[v] = (double)xm[v];
+        up[v] = (double)xp[v];
       }
       rm[d] = um[0];
       rp[d] = up[0];
@@ -228,16 +239,19 @@ __device__ void prolong_child(const KParams &kp, const real *U, int cs, const in
 #pragma unroll
   for (int d = 0; d < 3; d++) pc[d] = Ic[d] - C.ix[d] * kp.nb[d] + NGH;
   real up[NVAR + 1], s[3][NVAR + 1];
+  auto get = [&](int p0, int p1, int p2, real *u) {
+    ld_cell(U + cell_index(kp, cs, p0, p1, p2), u);
+    if (nv > NVAR) u[TRV] = U[tracer_index(kp, cs, p0, p1, p2)];
+  };
+  get(pc[0], pc[1], pc[2], up);
 #pragma unroll
-  for (int v = 0; v < NVAR + 1; v++) {
-    if (v >= nv) break;
-    up[v] = U[cidx<real>(kp, cs, v, pc[0], pc[1], pc[2])];
-    s[0][v] = mc_slope<real>(U[cidx<real>(kp, cs, v, pc[0] - 1, pc[1], pc[2])], up[v],
-                             U[cidx<real>(kp, cs, v, pc[0] + 1, pc[1], pc[2])]);
-    s[1][v] = mc_slope<real>(U[cidx<real>(kp, cs, v, pc[0], pc[1] - 1, pc[2])], up[v],
-                             U[cidx<real>(kp, cs, v, pc[0], pc[1] + 1, pc[2])]);
-    s[2][v] = mc_slope<real>(U[cidx<real>(kp, cs, v, pc[0], pc[1], pc[2] - 1)], up[v],
-                             U[cidx<real>(kp, cs, v, pc[0], pc[1], pc[2] + 1)]);
+  for (int d = 0; d < 3; d++) {
+    real um[NVAR + 1], uq[NVAR + 1];
+    get(pc[0] - (d == 0), pc[1] - (d == 1), pc[2] - (d == 2), um);
+    get(pc[0] + (d == 0), pc[1] + (d == 1), pc[2] + (d == 2), uq);
+#pragma unroll
+    for (int v = 0; v < NVAR + 1; v++)
+      if (v < nv) s[d][v] = mc_slope<real>(um[v], up[v], uq[v]);
   }
   const real *d0 = GeoSel<real>::dlt(kp.geo, Lc, 0), *d1 = GeoSel<real>::dlt(kp.geo, Lc, 1),
              *d2 = GeoSel<real>::dlt(kp.geo, Lc, 2);
@@ -272,9 +286,8 @@ __global__ void k_regrid_move(const KParams kpo, const real *Uold, real *Unew, c
   real val[NVAR + 1];
   const int nv = kpo.nvs;
   if (op.kind == 0) {
-#pragma unroll
-    for (int v = 0; v < NVAR + 1; v++)
-      if (v < nv) val[v] = Uold[cidx<real>(kpo, op.src[0], v, i + NGH, j + NGH, k + NGH)];
+    ld_cell(Uold + cell_index(kpo, op.src[0], i + NGH, j + NGH, k + NGH), val);
+    if (nv > NVAR) val[TRV] = Uold[tracer_index(kpo, op.src[0], i + NGH, j + NGH, k + NGH)];
   } else if (op.kind == 1) {
     const int F[3] = {N.ix[0] * kpo.nb[0] + i, N.ix[1] * kpo.nb[1] + j, N.ix[2] * kpo.nb[2] + k};
     const int Ic[3] = {F[0] >> 1, F[1] >> 1, F[2] >> 1};
@@ -296,17 +309,19 @@ __global__ void k_regrid_move(const KParams kpo, const real *Uold, real *Unew, c
       const int q1 = f[1] - (2 * N.ix[1] + cb[1]) * kpo.nb[1] + NGH;
       const int q2 = f[2] - (2 * N.ix[2] + cb[2]) * kpo.nb[2] + NGH;
       const real V = FG.dr3[f[0] + NGH] * FG.dcos[f[1] + NGH] * FG.dphi;
+      real u[NVAR + 1];
+      ld_cell(Uold + cell_index(kpo, os, q0, q1, q2), u);
+      if (nv > NVAR) u[TRV] = Uold[tracer_index(kpo, os, q0, q1, q2)];
 #pragma unroll
       for (int v = 0; v < NVAR + 1; v++)
-        if (v < nv) sum[v] += V * Uold[cidx<real>(kpo, os, v, q0, q1, q2)];
+        if (v < nv) sum[v] += V * u[v];
       vs += V;
     }
 #pragma unroll
     for (int v = 0; v < NVAR + 1; v++) val[v] = sum[v] / vs;
   }
-#pragma unroll
-  for (int v = 0; v < NVAR + 1; v++)
-    if (v < nv) Unew[cidx<real>(kpo, op.dst, v, i + NGH, j + NGH, k + NGH)] = val[v];
+  st_cell(Unew + cell_index(kpo, op.dst, i + NGH, j + NGH, k + NGH), val);
+  if (nv > NVAR) Unew[tracer_index(kpo, op.dst, i + NGH, j + NGH, k + NGH)] = val[TRV];
 }
 
 // ---- probe ----
@@ -418,7 +433,9 @@ __global__ void k_sums(const KParams kp, const real *U, int slot0, double *parti
     const int k = c % kp.nb[2], j = (c / kp.nb[2]) % kp.nb[1], i = c / (kp.nb[2] * kp.nb[1]);
     const int I = B.ix[0] * kp.nb[0] + i + NGH, J = B.ix[1] * kp.nb[1] + j + NGH;
     const double V = GD.dr3[I] * GD.dcos[J] * GD.dphi;
-    for (int v = 0; v < NVAR; v++) acc[v] += V * (double)U[cidx<real>(kp, slot, v, i + NGH, j + NGH, k + NGH)];
+    real u[NVAR];
+    ld_cell(U + cell_index(kp, slot, i + NGH, j + NGH, k + NGH), u);
+    for (int v = 0; v < NVAR; v++) acc[v] += V * (double)u[v];
   }
   for (int v = 0; v < NVAR; v++) sh[v][threadIdx.x] = acc[v];
   __syncthreads();

@@ -43,32 +43,38 @@ __device__ __forceinline__ int lookup(const KParams &kp, int member, int L, cons
   return kp.lmap[off + ((long long)b0 * n1 + b1) * n2 + b2];
 }
 
-__device__ __forceinline__ size_t cell_index(const KParams &kp, int slot, int v, int p0, int p1, int p2) {
-  return ((((size_t)slot * kp.nvs + v) * kp.P[0] + p0) * kp.P[1] + p1) * kp.P[2] + p2;
-}
-
-// Index of variable 0 at padded index (p0, p1, p2) of leaf `slot` (variable
-// v lies v * P0 P1 P2 further on); with `direct`, a cell of the ghost layer
-// that a same-level leaf holds is located in that leaf's interior (the ghost
-// copy is not filled in the step's fills).
-__device__ __forceinline__ size_t locate(const KParams &kp, int slot, int p0, int p1, int p2, bool direct) {
+// Slot and padded cell that hold padded index (p0, p1, p2) of leaf `slot`:
+// with `direct`, a cell of the ghost layer that a same-level leaf holds is
+// located in that leaf's interior (the ghost copy is not filled in the step's
+// fills).
+struct Place {
+  size_t base;
+  int cell;
+};
+__device__ __forceinline__ Place locate(const KParams &kp, int slot, int p0, int p1, int p2, bool direct) {
   if (direct) {
     const int s0 = p0 < NGH ? -1 : (p0 >= NGH + kp.nb[0] ? 1 : 0);
     const int s1 = p1 < NGH ? -1 : (p1 >= NGH + kp.nb[1] ? 1 : 0);
     const int s2 = p2 < NGH ? -1 : (p2 >= NGH + kp.nb[2] ? 1 : 0);
     if (s0 | s1 | s2) {
       const int o = kp.nb27[(size_t)slot * 27 + (s0 + 1) * 9 + (s1 + 1) * 3 + (s2 + 1)];
-      if (o >= 0) return cell_index(kp, o, 0, p0 - s0 * kp.nb[0], p1 - s1 * kp.nb[1], p2 - s2 * kp.nb[2]);
+      if (o >= 0)
+        return {slot_base(kp, o), pad_cell(kp, p0 - s0 * kp.nb[0], p1 - s1 * kp.nb[1], p2 - s2 * kp.nb[2])};
     }
   }
-  return cell_index(kp, slot, 0, p0, p1, p2);
+  return {slot_base(kp, slot), pad_cell(kp, p0, p1, p2)};
 }
 
-// variable v at padded index (p0, p1, p2) of leaf `slot` (see locate)
+// the variables of a placed cell and, when stored, its tracer (u[TRV])
 template <typename real>
-__device__ __forceinline__ real fetch(const KParams &kp, const real *U, int slot, int v, int p0, int p1, int p2,
-                                      bool direct) {
-  return U[locate(kp, slot, p0, p1, p2, direct) + (size_t)v * kp.P[0] * kp.P[1] * kp.P[2]];
+__device__ __forceinline__ void fetch(const KParams &kp, const real *U, Place c, real *u) {
+  ld_cell(U + c.base + (size_t)NVAR * c.cell, u);
+  if (kp.nvs > NVAR) u[TRV] = U[c.base + (size_t)NVAR * kp.pcells + c.cell];
+}
+template <typename real>
+__device__ __forceinline__ void store(const KParams &kp, real *U, Place c, const real *u) {
+  st_cell(U + c.base + (size_t)NVAR * c.cell, u);
+  if (kp.nvs > NVAR) U[c.base + (size_t)NVAR * kp.pcells + c.cell] = u[TRV];
 }
 
 // Conservative prolongation of coarse cell Ic (global at level Lc, held by
@@ -84,24 +90,23 @@ __device__ __forceinline__ void prolong_into(const KParams &kp, real *U, int cs,
   int pc[3];
 #pragma unroll
   for (int d = 0; d < 3; d++) pc[d] = Ic[d] - C.ix[d] * kp.nb[d] + NGH;
-  const size_t vs = (size_t)kp.P[0] * kp.P[1] * kp.P[2];
-  const size_t i0 = cell_index(kp, cs, 0, pc[0], pc[1], pc[2]);
-  const size_t im0 = locate(kp, cs, pc[0] - 1, pc[1], pc[2], direct), ip0 = locate(kp, cs, pc[0] + 1, pc[1], pc[2], direct);
-  const size_t im1 = locate(kp, cs, pc[0], pc[1] - 1, pc[2], direct), ip1 = locate(kp, cs, pc[0], pc[1] + 1, pc[2], direct);
-  const size_t im2 = locate(kp, cs, pc[0], pc[1], pc[2] - 1, direct), ip2 = locate(kp, cs, pc[0], pc[1], pc[2] + 1, direct);
   // the MHD variables and, when stored, the CME tracer (same slopes and
   // offsets; the positivity decision is the MHD variables')
   const int nv = kp.nvs;
   real up[NVAR + 1], s[3][NVAR + 1];
+  fetch(kp, U, {slot_base(kp, cs), pad_cell(kp, pc[0], pc[1], pc[2])}, up);
+  {
+    real um[3][NVAR + 1], uq[3][NVAR + 1];
 #pragma unroll
-  for (int v = 0; v < NVAR + 1; v++) {
-    if (v < nv) {
-      const size_t o = v * vs;
-      up[v] = U[i0 + o];
-      s[0][v] = mc_slope<real>(U[im0 + o], up[v], U[ip0 + o]);
-      s[1][v] = mc_slope<real>(U[im1 + o], up[v], U[ip1 + o]);
-      s[2][v] = mc_slope<real>(U[im2 + o], up[v], U[ip2 + o]);
+    for (int d = 0; d < 3; d++) {
+      fetch(kp, U, locate(kp, cs, pc[0] - (d == 0), pc[1] - (d == 1), pc[2] - (d == 2), direct), um[d]);
+      fetch(kp, U, locate(kp, cs, pc[0] + (d == 0), pc[1] + (d == 1), pc[2] + (d == 2), direct), uq[d]);
     }
+#pragma unroll
+    for (int d = 0; d < 3; d++)
+#pragma unroll
+      for (int v = 0; v < NVAR + 1; v++)
+        if (v < nv) s[d][v] = mc_slope<real>(um[d][v], up[v], uq[d][v]);
   }
   const real *d0 = GeoSel<real>::dlt(kp.geo, Lc, 0), *d1 = GeoSel<real>::dlt(kp.geo, Lc, 1),
              *d2 = GeoSel<real>::dlt(kp.geo, Lc, 2);
@@ -116,14 +121,16 @@ __device__ __forceinline__ void prolong_into(const KParams &kp, real *U, int cs,
     for (int v = 0; v < NVAR; v++) u[v] = ((up[v] + s[0][v] * a) + s[1][v] * b) + s[2][v] * e;
     if (!(u[0] > real(0)) || !(pressure_of<real>(u, gamma, Isl{(float)kp.isl_pe, (float)kp.isl_beta}) > real(0))) ok = false;
   }
-  const size_t w0 = cell_index(kp, slot, 0, p[0], p[1], p[2]);
+  const size_t wbase = slot_base(kp, slot);
+  const int w0 = pad_cell(kp, p[0], p[1], p[2]);
   const int P1 = kp.P[1], P2 = kp.P[2];
   for (int c = 0; c < 8; c++) {
     const real a = (c & 4) ? a1 : a0, b = (c & 2) ? b1 : b0, e = (c & 1) ? e1 : e0;
-    const size_t wc = w0 + ((size_t)((c >> 2) & 1) * P1 + ((c >> 1) & 1)) * P2 + (c & 1);
+    real u[NVAR + 1];
 #pragma unroll
     for (int v = 0; v < NVAR + 1; v++)
-      if (v < nv) U[wc + v * vs] = ok ? ((up[v] + s[0][v] * a) + s[1][v] * b) + s[2][v] * e : up[v];
+      if (v < nv) u[v] = ok ? ((up[v] + s[0][v] * a) + s[1][v] * b) + s[2][v] * e : up[v];
+    store(kp, U, {wbase, w0 + (((c >> 2) & 1) * P1 + ((c >> 1) & 1)) * P2 + (c & 1)}, u);
   }
 }
 
@@ -153,8 +160,8 @@ __device__ __forceinline__ bool restrict_in_block(const KParams &kp, const real 
   }
   const int fs = lookup_block(kp, member, L + 1, fb);
   if (fs < 0) return false;
-  const size_t vs = (size_t)kp.P[0] * kp.P[1] * kp.P[2];
-  const size_t f0 = cell_index(kp, fs, 0, fq[0], fq[1], fq[2]);
+  const size_t fbase = slot_base(kp, fs);
+  const int f0 = pad_cell(kp, fq[0], fq[1], fq[2]);
   const int P1 = kp.P[1], P2 = kp.P[2];
   real sum[NVAR + 1];
 #pragma unroll
@@ -163,10 +170,11 @@ __device__ __forceinline__ bool restrict_in_block(const KParams &kp, const real 
   for (int c = 0; c < 8; c++) {
     const int c0 = (c >> 2) & 1, c1 = (c >> 1) & 1, c2 = c & 1;
     const real V = F.dr3[2 * G[0] + c0 + NGH] * F.dcos[2 * G[1] + c1 + NGH] * F.dphi;
-    const size_t o = f0 + ((size_t)c0 * P1 + c1) * P2 + c2;
+    real u[NVAR + 1];
+    fetch(kp, U, {fbase, f0 + (c0 * P1 + c1) * P2 + c2}, u);
 #pragma unroll
     for (int v = 0; v < NVAR + 1; v++)
-      if (v < nv) sum[v] += V * U[o + v * vs];
+      if (v < nv) sum[v] += V * u[v];
     vsum += V;
   }
 #pragma unroll
@@ -204,12 +212,9 @@ __global__ void __launch_bounds__(256, sizeof(real) == 4 ? 4 : 2) k_ghost_neighb
     G[d] = bd * nb + q[d] - NGH;      // global cell at level L
   }
   real val[NVAR + 1];
-  const int nv = kp.nvs;
   const int o = lookup_block(kp, member, L, b);
   if (o >= 0) {
-#pragma unroll
-    for (int v = 0; v < NVAR + 1; v++)
-      if (v < nv) val[v] = U[cell_index(kp, o, v, q[0], q[1], q[2])];
+    fetch(kp, U, {slot_base(kp, o), pad_cell(kp, q[0], q[1], q[2])}, val);
   } else if (o == -1) {
     // A coarse cell covers a 2 x 2 x 2 group of ghost cells (blocks start at
     // even global indices and there are two ghost layers): the group's
@@ -234,9 +239,7 @@ __global__ void __launch_bounds__(256, sizeof(real) == 4 ? 4 : 2) k_ghost_neighb
       return;
     }
   }
-#pragma unroll
-  for (int v = 0; v < NVAR + 1; v++)
-    if (v < nv) U[cell_index(kp, slot, v, p[0], p[1], p[2])] = val[v];
+  store(kp, U, {slot_base(kp, slot), pad_cell(kp, p[0], p[1], p[2])}, val);
 }
 
 // Ghost cells of one region of a level-L leaf (one of the 26 around it, r =
@@ -293,10 +296,7 @@ __global__ void __launch_bounds__(256, sizeof(real) == 4 ? 3 : 2) k_ghost_region
       atomicOr(kp.status, ST_TREE);
       return;
     }
-    const int nv = kp.nvs;
-#pragma unroll
-    for (int v = 0; v < NVAR + 1; v++)
-      if (v < nv) U[cell_index(kp, slot, v, p[0], p[1], p[2])] = val[v];
+    store(kp, U, {slot_base(kp, slot), pad_cell(kp, p[0], p[1], p[2])}, val);
   }
 }
 
@@ -372,19 +372,19 @@ __global__ void k_ghost_physical(const KParams kp, real *U, const int2 *sides, i
     const double t = kp.t[B.member] + tfac * kp.dt_used[B.member];
     double u[NVAR + 1];
     inner_state(kp, B.member, L, J, K, t, u);
+    real x[NVAR + 1];
 #pragma unroll
-    for (int v = 0; v < NVAR + 1; v++)
-      if (v < kp.nvs) U[cell_index(kp, slot, v, q[0], q[1], q[2])] = (real)u[v];
+    for (int v = 0; v < NVAR + 1; v++) x[v] = (real)u[v];
+    store(kp, U, {slot_base(kp, slot), pad_cell(kp, q[0], q[1], q[2])}, x);
     return;
   }
   s[dir] = bc == 2 ? pm : pn;
+  real x[NVAR + 1];
+  fetch(kp, U, locate(kp, slot, s[0], s[1], s[2], skip_same != 0), x);
 #pragma unroll
-  for (int v = 0; v < NVAR + 1; v++) {
-    if (v >= kp.nvs) break;
-    real x = fetch(kp, U, slot, v, s[0], s[1], s[2], skip_same != 0);
-    if (bc == 2 && (v == 1 + dir || v == 5 + dir)) x = -x;
-    U[cell_index(kp, slot, v, q[0], q[1], q[2])] = x;
-  }
+  for (int v = 0; v < NVAR; v++)
+    if (bc == 2 && (v == 1 + dir || v == 5 + dir)) x[v] = -x[v];
+  store(kp, U, {slot_base(kp, slot), pad_cell(kp, q[0], q[1], q[2])}, x);
 }
 
 // reflux of coarse blocks with finer face neighbours; one CTA per block
@@ -448,11 +448,12 @@ __global__ void k_reflux(const KParams kp, real *U, const real *flux, const int 
       const real V = G.dr3[I + NGH] * G.dcos[J + NGH] * G.dphi;
       const real *own = flux + (size_t)slot * fstride + foff[f];
       const real sg = hi ? real(-1) : real(1);
+      const size_t ci = cell_index(kp, slot, q[0], q[1], q[2]);
+      real u[NVAR];
+      ld_cell(U + ci, u);
 #pragma unroll
-      for (int v = 0; v < NVAR; v++) {
-        const size_t ci = cell_index(kp, slot, v, q[0], q[1], q[2]);
-        U[ci] += sg * dt / V * (fs[v] - own[(size_t)v * fc[d] + t]);
-      }
+      for (int v = 0; v < NVAR; v++) u[v] += sg * dt / V * (fs[v] - own[(size_t)v * fc[d] + t]);
+      st_cell(U + ci, u);
     }
     __syncthreads();
   }
@@ -471,11 +472,10 @@ __global__ void k_reflux(const KParams kp, real *U, const real *flux, const int 
       q[d1] = NGH + t1;
       q[d2] = NGH + t2;
       real u[NVAR];
-#pragma unroll
-      for (int v = 0; v < NVAR; v++) u[v] = U[cell_index(kp, slot, v, q[0], q[1], q[2])];
+      const size_t ci = cell_index(kp, slot, q[0], q[1], q[2]);
+      ld_cell(U + ci, u);
       hits += apply_floors<real>(u, gamma, pfl, rfl, Isl{(float)kp.isl_pe, (float)kp.isl_beta});
-#pragma unroll
-      for (int v = 0; v < NVAR; v++) U[cell_index(kp, slot, v, q[0], q[1], q[2])] = u[v];
+      st_cell(U + ci, u);
       real w[NVAR];
       cons2prim_speed<real>(u, w, gamma, pfl);
       const int I = B.ix[0] * nb0 + q[0] - NGH + NGH, J = B.ix[1] * nb1 + q[1] - NGH + NGH;
@@ -544,8 +544,7 @@ __global__ void k_dt_full(const KParams kp, const real *U) {
   for (int c = blockIdx.y * blockDim.x + threadIdx.x; c < kp.icells; c += gridDim.y * blockDim.x) {
     const int k = c % kp.nb[2], j = (c / kp.nb[2]) % kp.nb[1], i = c / (kp.nb[2] * kp.nb[1]);
     real u[NVAR], w[NVAR];
-#pragma unroll
-    for (int v = 0; v < NVAR; v++) u[v] = U[cell_index(kp, slot, v, i + NGH, j + NGH, k + NGH)];
+    ld_cell(U + cell_index(kp, slot, i + NGH, j + NGH, k + NGH), u);
     cons2prim_speed<real>(u, w, gamma, pfl);
     const int I = B.ix[0] * kp.nb[0] + i + NGH, J = B.ix[1] * kp.nb[1] + j + NGH;
     real dx0 = G.dr[I], dx1 = G.dth[J], dx2 = G.dphi;

@@ -43,15 +43,13 @@ __global__ void k_features(const KParams kp, const real *U, int slot0, float *ou
   const int n0 = kp.nb[0], n1 = kp.nb[1], n2 = kp.nb[2];
   const int s0 = n0 / 4, s1 = n1 / 4, s2 = n2 / 4, per = s0 * s1 * s2;
   const double gm1 = kp.gamma - 1.0;
-  auto cell = [&](int v, int i, int j, int k) -> double {
-    return (double)U[((((size_t)slot * kp.nvs + v) * kp.P[0] + i) * kp.P[1] + j) * kp.P[2] + k];
-  };
   auto prims = [&](int i, int j, int k, double *w) {  // rho, v_r, p
-    const double r = cell(0, i, j, k), m1 = cell(1, i, j, k), m2 = cell(2, i, j, k), m3 = cell(3, i, j, k);
-    const double b1 = cell(5, i, j, k), b2 = cell(6, i, j, k), b3 = cell(7, i, j, k);
+    real u[NVAR];
+    ld_cell(U + cell_index(kp, slot, i, j, k), u);
+    const double r = u[0], m1 = u[1], m2 = u[2], m3 = u[3], b1 = u[5], b2 = u[6], b3 = u[7];
     w[0] = r;
     w[1] = m1 / r;
-    w[2] = gm1 * (cell(4, i, j, k) - 0.5 * (m1 * m1 + m2 * m2 + m3 * m3) / r - 0.5 * (b1 * b1 + b2 * b2 + b3 * b3));
+    w[2] = gm1 * ((double)u[4] - 0.5 * (m1 * m1 + m2 * m2 + m3 * m3) / r - 0.5 * (b1 * b1 + b2 * b2 + b3 * b3));
   };
   const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
   for (int sc = threadIdx.x >> 5; sc < 64; sc += nw) {

@@ -192,13 +192,13 @@ __global__ void __launch_bounds__(stage_threads(TJ, TK), stage_min_ctas(sizeof(r
     const bool valid = tid < TJ * TK && jl < nvj && kl < nvk;
     const int j = j0 + jl, k = k0 + kl;           // interior indices in the block
 
-    // Planes of U_in are copied asynchronously (cp.async, 4 bytes per copy)
+    // Planes of U_in are copied asynchronously (cp.async, 16 bytes per copy)
     // straight into their ring slot and converted to primitives in place one
     // iteration later, by the thread that copied them (no barrier between
     // copy and conversion).  A unit is two cells half a plane apart, so the
     // threads of a warp write consecutive cells.  Units go to the highest
     // thread indices, which own no second div B position.
-    constexpr int NU = RP / 2;
+    constexpr int NU = RP / 2, CH = Vec16<real>::CH;
     auto slotp = [&](int p) -> real * { return ring + ((p + 5) % 5) * NVAR * RP; };
     auto xslot = [&](int p) -> real * { return xring + ((p + 5) % 5) * RP; };
     // Cells of the plane outside the block that a same-level leaf holds come
@@ -216,20 +216,22 @@ __global__ void __launch_bounds__(stage_threads(TJ, TK), stage_min_ctas(sizeof(r
           const int q = u + h * NU, jj = q / RK, kk = q - (q / RK) * RK;
           const int pj = j0 + jj, pk = k0 + kk;
           if (pj < P1 && pk < P2) {
-            const real *src = Uin + (size_t)(p + NGH) * plane + (size_t)pj * P2 + pk;
+            const real *blk = Uin;
+            size_t cell = (size_t)(p + NGH) * plane + (size_t)pj * P2 + pk;
             if (sl.direct) {
               const int sj = pj < NGH ? -1 : (pj >= NGH + nb1 ? 1 : 0);
               const int sk = pk < NGH ? -1 : (pk >= NGH + nb2 ? 1 : 0);
               if (sr | sj | sk) {
                 const int o = nb27[(sr + 1) * 9 + (sj + 1) * 3 + (sk + 1)];
-                if (o >= 0)
-                  src = Uall + (size_t)o * bstride + (size_t)(p - sr * nb0 + NGH) * plane +
-                        (size_t)(pj - sj * nb1) * P2 + (pk - sk * nb2);
+                if (o >= 0) {
+                  blk = Uall + (size_t)o * bstride;
+                  cell = (size_t)(p - sr * nb0 + NGH) * plane + (size_t)(pj - sj * nb1) * P2 + (pk - sk * nb2);
+                }
               }
             }
 #pragma unroll
-            for (int v = 0; v < NVAR; v++) cp_async<sizeof(real)>(&el<real, RP>(dst, v, q), src + v * vstride);
-            if (trc) cp_async<sizeof(real)>(xslot(p) + q, src + TRV * vstride);
+            for (int v = 0; v < NVAR; v += CH) cp_async<16>(&el<real, RP>(dst, v, q), blk + NVAR * cell + v);
+            if (trc) cp_async<sizeof(real)>(xslot(p) + q, blk + TRV * vstride + cell);
           }
         }
       }
@@ -256,9 +258,9 @@ __global__ void __launch_bounds__(stage_threads(TJ, TK), stage_min_ctas(sizeof(r
     // group so that the group counts stay uniform
     auto issue_u0 = [&](int p) {
       if (valid && p < ie) {
-        const real *src = U0 + (size_t)(p + NGH) * plane + (size_t)(j + NGH) * P2 + (k + NGH);
+        const real *src = U0 + NVAR * ((size_t)(p + NGH) * plane + (size_t)(j + NGH) * P2 + (k + NGH));
 #pragma unroll
-        for (int v = 0; v < NVAR; v++) cp_async<sizeof(real)>(u0s + v * NT + tid, src + v * vstride);
+        for (int v = 0; v < NVAR; v += CH) cp_async<16>(&el<real, NT>(u0s, v, tid), src + v);
       }
       cp_async_commit();
     };
@@ -443,7 +445,6 @@ __global__ void __launch_bounds__(stage_threads(TJ, TK), stage_min_ctas(sizeof(r
         real un[NVAR];
         const size_t cidx = (size_t)(i + NGH) * plane + (size_t)(j + NGH) * P2 + (k + NGH);
         {
-          constexpr int CH = Vec16<real>::CH;
           const int qt = jl * TK + kl, qp = jl * (TK + 1) + kl;
 #pragma unroll
           for (int c = 0; c < NVAR / CH; c++) {
@@ -476,8 +477,7 @@ __global__ void __launch_bounds__(stage_threads(TJ, TK), stage_min_ctas(sizeof(r
         cp_async_wait_group<0>();   // this thread's U^n copy of plane i
         {
           real u0[NVAR];
-#pragma unroll
-          for (int v = 0; v < NVAR; v++) u0[v] = u0s[v * NT + tid];
+          ld8<real, NT>(u0s, tid, u0);
           axpy8<real>(u0, dt, un, un);
         }
         if (S2 && Cd > real(0)) {
@@ -528,8 +528,7 @@ __global__ void __launch_bounds__(stage_threads(TJ, TK), stage_min_ctas(sizeof(r
         }
         hits += apply_floors<real>(un, gamma, pfl, rfl, isl);
         if (!(un[0] == un[0]) || !(un[4] == un[4])) atomicOr(kp.status, ST_NAN);
-#pragma unroll
-        for (int v = 0; v < NVAR; v++) Uout[v * vstride + cidx] = un[v];
+        st_cell(Uout + NVAR * cidx, un);
         if (S2) {
           // CFL contribution of the new state (cells next to a finer face are
           // left to the reflux, which changes them once more)

@@ -33,7 +33,7 @@
 #include <cstdio>
 
 #include "../../include/icarus.h"
-#include "icarus_internal.h"
+#include "mhd_device.cuh"
 
 #define ICARUS_STATIC_SUM_BLOCKS 16384
 #define ICARUS_MAX_DEVICES 64
@@ -57,10 +57,9 @@ __global__ void k_block_sums_static(const KParams kp, const real *U, int slot0, 
     const int k = c % kp.nb[2], j = (c / kp.nb[2]) % kp.nb[1], i = c / (kp.nb[2] * kp.nb[1]);
     const int I = B.ix[0] * kp.nb[0] + i + NGH, J = B.ix[1] * kp.nb[1] + j + NGH;
     const double V = GD.dr3[I] * GD.dcos[J] * GD.dphi;
-    for (int v = 0; v < NVAR; v++) {
-      const size_t idx = ((((size_t)slot * kp.nvs + v) * kp.P[0] + i + NGH) * kp.P[1] + j + NGH) * kp.P[2] + k + NGH;
-      acc[v] += V * (double)U[idx];
-    }
+    real u[NVAR];
+    ld_cell(U + cell_index(kp, slot, i + NGH, j + NGH, k + NGH), u);
+    for (int v = 0; v < NVAR; v++) acc[v] += V * (double)u[v];
   }
   for (int v = 0; v < NVAR; v++) sh[v][threadIdx.x] = acc[v];
   __syncthreads();

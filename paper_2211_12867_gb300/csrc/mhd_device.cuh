@@ -38,6 +38,53 @@ template <> struct RT<float> {
   }
 };
 
+// ---- the padded state ----
+// A slot holds its cells' eight variables side by side, [cell][8] (32 bytes in
+// FP32, one DRAM sector; 64 in FP64), and behind them, when the CME tracer is
+// stored, one value per cell.  A cell is one 256-bit access in FP32 and two in
+// FP64 wherever it lies, so the scattered reads of the ghost fills (7 cells per
+// prolonged group) take one sector each instead of eight, and a stage kernel
+// copies a cell with 16-byte asynchronous copies instead of 4-byte ones.
+__device__ __forceinline__ size_t slot_base(const KParams &kp, int slot) {
+  return (size_t)slot * kp.nvs * kp.pcells;
+}
+__device__ __forceinline__ int pad_cell(const KParams &kp, int p0, int p1, int p2) {
+  return (p0 * kp.P[1] + p1) * kp.P[2] + p2;
+}
+// index of variable 0 of a cell; of its tracer
+__device__ __forceinline__ size_t cell_index(const KParams &kp, int slot, int p0, int p1, int p2) {
+  return slot_base(kp, slot) + (size_t)NVAR * pad_cell(kp, p0, p1, p2);
+}
+__device__ __forceinline__ size_t tracer_index(const KParams &kp, int slot, int p0, int p1, int p2) {
+  return slot_base(kp, slot) + (size_t)NVAR * kp.pcells + pad_cell(kp, p0, p1, p2);
+}
+__device__ __forceinline__ void ld_cell(const float *p, float *u) {
+  asm volatile("ld.global.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=f"(u[0]), "=f"(u[1]), "=f"(u[2]), "=f"(u[3]), "=f"(u[4]), "=f"(u[5]), "=f"(u[6]), "=f"(u[7])
+               : "l"(p)
+               : "memory");
+}
+__device__ __forceinline__ void ld_cell(const double *p, double *u) {
+#pragma unroll
+  for (int h = 0; h < NVAR; h += 4)
+    asm volatile("ld.global.v4.f64 {%0,%1,%2,%3}, [%4];"
+                 : "=d"(u[h]), "=d"(u[h + 1]), "=d"(u[h + 2]), "=d"(u[h + 3])
+                 : "l"(p + h)
+                 : "memory");
+}
+__device__ __forceinline__ void st_cell(float *p, const float *u) {
+  asm volatile("st.global.v8.f32 [%8], {%0,%1,%2,%3,%4,%5,%6,%7};" ::"f"(u[0]), "f"(u[1]), "f"(u[2]), "f"(u[3]),
+               "f"(u[4]), "f"(u[5]), "f"(u[6]), "f"(u[7]), "l"(p)
+               : "memory");
+}
+__device__ __forceinline__ void st_cell(double *p, const double *u) {
+#pragma unroll
+  for (int h = 0; h < NVAR; h += 4)
+    asm volatile("st.global.v4.f64 [%4], {%0,%1,%2,%3};" ::"d"(u[h]), "d"(u[h + 1]), "d"(u[h + 2]), "d"(u[h + 3]),
+                 "l"(p + h)
+                 : "memory");
+}
+
 // Pressure from conserved variables.  In the mixed-precision mode the FP32
 // result is replaced by an FP64 recomputation from the same (FP32-stored)
 // conserved variables where the thermal energy is a small remainder of the
