@@ -30,29 +30,34 @@
 
 namespace {
 
+// plane and row factors staged per work item (see the kernel)
+constexpr int NPF = 8, NRF = 8;
+
 template <typename real>
 struct StageSmem {
-  // tracer: a 5-plane ring of the CME tracer fraction X follows the rest
+  // tracer: a 5-plane ring of the CME tracer fraction X and the sources of the
+  // threads' copies follow the rest
   static constexpr size_t bytes(int tj, int tk, bool tracer = false) {
     return sizeof(real) * (size_t)(5 * NVAR * (tj + 4) * (tk + 4) + 2 * NVAR * (tj + 1) * tk +
                                    2 * NVAR * tj * (tk + 1) + 4 * (tj + 2) * (tk + 2) +
                                    NVAR * ((tj * tk + 31) / 32 * 32) + geo(tj, tk) +
-                                   (tracer ? 5 * (tj + 4) * (tk + 4) : 0));
+                                   (tracer ? 5 * (tj + 4) * (tk + 4) : 0)) +
+           (tracer ? sizeof(void *) * (size_t)((tj + 4) * (tk + 4) + (tj * tk + 31) / 32 * 32) : 0);
   }
-  // geometry of one work item: 6 plane arrays and the faces in r, 6 row
-  // arrays and the faces in theta, 1 column array
+  // factors of the planes (and rc^2), of the tile's rows, three row arrays of
+  // the divergence, one column array; rounded up to 16 bytes
   static constexpr int geo(int tj, int tk) {
-    return 6 * (STAGE_SEG_MAX + 4) + (STAGE_SEG_MAX + 5) + 6 * (tj + 4) + (tj + 5) + (tk + 4);
+    return (NPF * (STAGE_SEG_MAX + 4) + NRF * tj + (STAGE_SEG_MAX + 4) + 3 * (tj + 4) + (tk + 4) + 3) / 4 * 4;
   }
 };
 
 // The inverse time step is accumulated in the working precision (a maximum is
 // exact in any precision) and enters the FP64 reduction once per warp.
 template <typename real>
-__device__ __forceinline__ void flush_acc(const KParams &kp, real &acc, int member, long long &hits) {
+__device__ __forceinline__ void flush_acc(const KParams &kp, real &acc, int member, int &hits) {
   // warp max of the inverse time step, one atomic per warp
   for (int o = 16; o > 0; o >>= 1) acc = RT<real>::max_(acc, __shfl_xor_sync(0xffffffffu, acc, o));
-  long long h = hits;
+  int h = hits;
   for (int o = 16; o > 0; o >>= 1) h += __shfl_xor_sync(0xffffffffu, h, o);
   if ((threadIdx.x & 31) == 0 && member >= 0) {
     if (acc > real(0)) atomic_max_pos(&kp.inv_max[member], (double)acc);
@@ -125,25 +130,29 @@ __global__ void __launch_bounds__(stage_threads(TJ, TK), stage_min_ctas(sizeof(r
   constexpr int NT = stage_threads(TJ, TK), RJ = TJ + 4, RK = TK + 4, RP = RJ * RK;
   constexpr int DJ = TJ + 2, DK = TK + 2, DP = DJ * DK;
   constexpr int NTH = (TJ + 1) * TK, NPH = TJ * (TK + 1);   // theta / phi faces of a plane
+  constexpr int CH = Vec16<real>::CH, NUN = (RP + NT - 1) / NT;
+  constexpr int PL = NVAR * RP;                             // reals of a ring plane
   extern __shared__ __align__(16) unsigned char smem_raw[];
   real *ring = reinterpret_cast<real *>(smem_raw);
-  real *fth = ring + 5 * NVAR * RP;     // two buffers of theta-face fluxes
+  real *fth = ring + 5 * PL;            // two buffers of theta-face fluxes
   real *fph = fth + 2 * NVAR * NTH;     // two buffers of phi-face fluxes
-  real *dring = fph + 2 * NVAR * NPH;
-  real *u0s = dring + 4 * DP;           // U^n of the thread's own cell, next plane
-  // geometry of the work item (plane arrays from plane ib-2, row arrays from
-  // row -2 of the tile, phi centres from column -2)
+  real *u0s = fph + 2 * NVAR * NPH;     // U^n of the thread's own cell, next plane
+  // Factors of the work item's planes (from plane ib-2): areas over volume of
+  // the r faces (halved: the fluxes carry a factor 2), dr2/dr3, Omega^2 r_c,
+  // 1 / two-cell spacing, 1/dr, 1/r_c, divergence factor.  Of the tile's rows:
+  // areas over volume of the theta faces and of the phi faces (halved, to be
+  // multiplied by dr2/dr3), sin, cos, 1 / two-cell spacing, 1/sin, 1/dtheta.
+  // An update so needs neither a face area nor a volume of its own.
   constexpr int NRP = STAGE_SEG_MAX + 4, NJ = TJ + 4;
-  real *s_rc = u0s + NVAR * NT, *s_dr2 = s_rc + NRP, *s_dr3 = s_dr2 + NRP;
-  real *s_r2f = s_dr3 + NRP;                                  // STAGE_SEG_MAX + 5 faces
-  // reciprocal centre spacings over two cells (theta rows, phi columns, r
-  // planes), reciprocal widths and radii: the divergence and the cleaning
-  // gradient take these per row, column or plane
-  real *s_itc2 = s_r2f + NRP + 1, *s_st = s_itc2 + NJ, *s_ct = s_st + NJ, *s_dcos = s_ct + NJ, *s_dth = s_dcos + NJ;
-  real *s_sinf = s_dth + NJ;                                  // TJ + 5 faces
-  real *s_ipc2 = s_sinf + NJ + 1;                             // TK + 4
-  real *s_ird2 = s_ipc2 + TK + 4, *s_idr = s_ird2 + NRP, *s_irc = s_idr + NRP, *s_idth = s_irc + NRP;
-  real *xring = s_idth + NJ;                                  // tracer X, 5 planes (if stored)
+  enum { P_RP, P_RM, P_DR, P_CF, P_ID2, P_IDR, P_IRC, P_FR };
+  enum { R_TP, R_TM, R_PW, R_ST, R_CT, R_ITC2, R_IST, R_IDTH };
+  real *s_pl = u0s + NVAR * NT, *s_row = s_pl + NPF * NRP;
+  real *dring = s_row + NRF * TJ;
+  // for the divergence: r_c^2 per plane; sin, 1 / (sin * two-cell spacing) and
+  // 1/sin per row from row -2; 1 / two-cell spacing per column from column -2
+  real *s_rc2 = dring + 4 * DP, *s_st = s_rc2 + NRP, *s_tt = s_st + NJ, *s_ist = s_tt + NJ, *s_ipc2 = s_ist + NJ;
+  real *xring = u0s + NVAR * NT + StageSmem<real>::geo(TJ, TK) + 4 * DP;   // tracer X, 5 planes (if stored)
+  const real **s_xsrc = reinterpret_cast<const real **>(xring + 5 * RP + (RP & 1));
   const bool trc = kp.nvs > NVAR;
 
   const int tid = threadIdx.x, jl = tid / TK, kl = tid % TK;
@@ -157,6 +166,14 @@ __global__ void __launch_bounds__(stage_threads(TJ, TK), stage_min_ctas(sizeof(r
   const real Om = (real)kp.omega, Cd = (real)kp.cd;
   const Isl isl{(float)kp.isl_pe, (float)kp.isl_beta};
   const real igm1 = real(1) / (gamma - real(1));
+  const int o = (jl + 2) * RK + kl + 2;          // ring cell of the thread's own cell
+  // extra faces of the tile's far edges: the last warps take one more theta
+  // face (row TJ) or phi face (column TK) per thread
+  constexpr int XT = (TK + 31) / 32 * 32;
+  static_assert(XT + TJ <= NT, "one extra face per thread");
+  const int xe = NT - 1 - tid;
+  const bool x_th = xe < TK, x_ph = xe >= XT && xe < XT + TJ;
+  const int xq = x_th ? xe : xe - XT;
 
   // reflux face buffer layout (per slot): faces in order r-lo, r-hi, th-lo,
   // th-hi, ph-lo, ph-hi; each [v][t1][t2]
@@ -164,7 +181,7 @@ __global__ void __launch_bounds__(stage_threads(TJ, TK), stage_min_ctas(sizeof(r
   const size_t fstride = (size_t)NVAR * 2 * (fc0 + fc1 + fc2);
 
   real inv_acc = real(0);
-  long long hits = 0;
+  int hits = 0;
   int cur_member = -1;
 
   for (int w = blockIdx.x; w < nwork; w += gridDim.x) {
@@ -173,12 +190,13 @@ __global__ void __launch_bounds__(stage_threads(TJ, TK), stage_min_ctas(sizeof(r
     rem /= sl.segs;
     const int tk = rem % sl.tiles_k, tj = rem / sl.tiles_k;
     const int slot = sl.list[li];
-    const DevBlock B = kp.blk[slot];
-    const double dtm = kp.dt_used[B.member];
+    const DevBlock &B = kp.blk[slot];
+    const int member = B.member;
+    const double dtm = kp.dt_used[member];
     if (!(dtm > 0.0)) continue;  // member has reached its stop time (uniform)
-    if (S2 && B.member != cur_member) {
+    if (S2 && member != cur_member) {
       flush_acc(kp, inv_acc, cur_member, hits);
-      cur_member = B.member;
+      cur_member = member;
     }
     const real dt = (real)(dtm * sl.dtfac);
     const LevelGeo<real> &G = GeoSel<real>::get(kp.geo, B.level);
@@ -189,187 +207,218 @@ __global__ void __launch_bounds__(stage_threads(TJ, TK), stage_min_ctas(sizeof(r
     const real *Uin = reinterpret_cast<const real *>(sl.Uin) + (size_t)slot * bstride;
     const real *U0 = reinterpret_cast<const real *>(sl.U0) + (size_t)slot * bstride;
     real *Uout = reinterpret_cast<real *>(sl.Uout) + (size_t)slot * bstride;
-    const bool valid = tid < TJ * TK && jl < nvj && kl < nvk;
+    const bool own = tid < TJ * TK, valid = own && jl < nvj && kl < nvk;
     const int j = j0 + jl, k = k0 + kl;           // interior indices in the block
+    // block faces with a finer, and with a coarser or finer, neighbour; those
+    // the thread's column touches
+    unsigned fin = 0, cfb = 0, edge = 0;
+    if (S2) {
+#pragma unroll
+      for (int f = 0; f < 6; f++) {
+        const int q = B.nbr[f];
+        fin |= (unsigned)(q == NB_FINER) << f;
+        cfb |= (unsigned)(q == NB_FINER || q == NB_COARSER) << f;
+      }
+      edge = (unsigned)(j == 0) << 2 | (unsigned)(j == nb1 - 1) << 3 | (unsigned)(k == 0) << 4 |
+             (unsigned)(k == nb2 - 1) << 5;
+    }
 
     // Planes of U_in are copied asynchronously (cp.async, 16 bytes per copy)
     // straight into their ring slot and converted to primitives in place one
     // iteration later, by the thread that copied them (no barrier between
-    // copy and conversion).  A unit is two cells half a plane apart, so the
-    // threads of a warp write consecutive cells.  Units go to the highest
-    // thread indices, which own no second div B position.
-    constexpr int NU = RP / 2, CH = Vec16<real>::CH;
-    auto slotp = [&](int p) -> real * { return ring + ((p + 5) % 5) * NVAR * RP; };
-    auto xslot = [&](int p) -> real * { return xring + ((p + 5) % 5) * RP; };
-    // Cells of the plane outside the block that a same-level leaf holds come
-    // straight from that leaf's interior (sl.direct: the step's ghost fills
-    // leave such ghost copies unfilled); the others from this block's ghost
-    // layer (coarser or finer neighbours, physical boundaries).
-    const int *nb27 = kp.nb27 + (size_t)slot * 27;
-    const real *Uall = reinterpret_cast<const real *>(sl.Uin);
-    auto issue_plane = [&](int p) {
-      real *dst = slotp(p);
-      const int sr = p < 0 ? -1 : (p >= nb0 ? 1 : 0);
-      for (int u = NT - 1 - tid; u < NU; u += NT) {
+    // copy and conversion).  Cells go to the highest thread indices first,
+    // which own no second div B position.  Cells of the plane outside the
+    // block that a same-level leaf holds come straight from that leaf's
+    // interior (sl.direct: the step's ghost fills leave such ghost copies
+    // unfilled); the others from this block's ghost layer (coarser or finer
+    // neighbours, physical boundaries).  A thread's sources change only where
+    // the march enters or leaves the block's r range.
+    const real *src[NUN];
+    int src_side = 2;
+    auto set_src = [&](int sr) {
+      src_side = sr;
 #pragma unroll
-        for (int h = 0; h < 2; h++) {
-          const int q = u + h * NU, jj = q / RK, kk = q - (q / RK) * RK;
-          const int pj = j0 + jj, pk = k0 + kk;
-          if (pj < P1 && pk < P2) {
-            const real *blk = Uin;
-            size_t cell = (size_t)(p + NGH) * plane + (size_t)pj * P2 + pk;
-            if (sl.direct) {
-              const int sj = pj < NGH ? -1 : (pj >= NGH + nb1 ? 1 : 0);
-              const int sk = pk < NGH ? -1 : (pk >= NGH + nb2 ? 1 : 0);
-              if (sr | sj | sk) {
-                const int o = nb27[(sr + 1) * 9 + (sj + 1) * 3 + (sk + 1)];
-                if (o >= 0) {
-                  blk = Uall + (size_t)o * bstride;
-                  cell = (size_t)(p - sr * nb0 + NGH) * plane + (size_t)(pj - sj * nb1) * P2 + (pk - sk * nb2);
-                }
+      for (int u = 0; u < NUN; u++) {
+        const int q = NT - 1 - tid + u * NT, jj = q / RK, kk = q - (q / RK) * RK;
+        const int pj = j0 + jj, pk = k0 + kk;
+        src[u] = nullptr;
+        if (q < RP && pj < P1 && pk < P2) {
+          const real *blk = Uin;
+          long long cell = (long long)NGH * (long long)plane + (long long)pj * P2 + pk;
+          if (sl.direct) {
+            const int sj = pj < NGH ? -1 : (pj >= NGH + nb1 ? 1 : 0);
+            const int sk = pk < NGH ? -1 : (pk >= NGH + nb2 ? 1 : 0);
+            if (sr | sj | sk) {
+              const int n = kp.nb27[(size_t)slot * 27 + (sr + 1) * 9 + (sj + 1) * 3 + (sk + 1)];
+              if (n >= 0) {
+                blk = reinterpret_cast<const real *>(sl.Uin) + (size_t)n * bstride;
+                cell -= (long long)sr * nb0 * (long long)plane + (long long)sj * nb1 * P2 + sk * nb2;
               }
             }
-#pragma unroll
-            for (int v = 0; v < NVAR; v += CH) cp_async<16>(&el<real, RP>(dst, v, q), blk + NVAR * cell + v);
-            if (trc) cp_async<sizeof(real)>(xslot(p) + q, blk + TRV * vstride + cell);
           }
+          src[u] = blk + NVAR * cell;
+          if (trc) s_xsrc[u * NT + tid] = blk + TRV * vstride + cell;
         }
       }
+    };
+    auto issue_plane = [&](int p, int at) {
+      const int sr = p < 0 ? -1 : (p >= nb0 ? 1 : 0);
+      if (sr != src_side) set_src(sr);
+      const long long off = (long long)p * (long long)plane;
+      real *dst = ring + at;
+#pragma unroll
+      for (int u = 0; u < NUN; u++)
+        if (src[u]) {
+          const int q = NT - 1 - tid + u * NT;
+          const real *from = src[u] + NVAR * off;
+#pragma unroll
+          for (int v = 0; v < NVAR; v += CH) cp_async<16>(dst + ((v / CH) * RP + q) * CH, from + v);
+          if (trc) cp_async<sizeof(real)>(xring + at / NVAR + q, s_xsrc[u * NT + tid] + off);
+        }
       cp_async_commit();
     };
-    auto convert_plane = [&](int p) {
-      real *pl = slotp(p);
-      for (int u = NT - 1 - tid; u < NU; u += NT) {
+    auto convert_plane = [&](int at) {
+      real *pl = ring + at;
 #pragma unroll
-        for (int h = 0; h < 2; h++) {
-          const int q = u + h * NU, jj = q / RK, kk = q - (q / RK) * RK;
-          if (j0 + jj < P1 && k0 + kk < P2) {
-            real uu[NVAR], wv[NVAR];
-            ld8<real, RP>(pl, q, uu);
-            cons2prim<real>(uu, wv, gamma, pfl, isl);
-            st8<real, RP>(pl, q, wv);
-            if (trc) xslot(p)[q] *= RT<real>::rcp_(uu[0]);   // rho X -> X
-          }
+      for (int u = 0; u < NUN; u++)
+        if (src[u]) {
+          const int q = NT - 1 - tid + u * NT;
+          real uu[NVAR], wv[NVAR];
+          ld8<real, RP>(pl, q, uu);
+          cons2prim<real>(uu, wv, gamma, pfl, isl);
+          st8<real, RP>(pl, q, wv);
+          if (trc) xring[at / NVAR + q] *= RT<real>::rcp_(uu[0]);   // rho X -> X
         }
-      }
     };
     // U^n of the thread's own cell at plane p, copied asynchronously one
     // plane ahead (only this thread reads it: no barrier); always commits a
     // group so that the group counts stay uniform
+    const real *u0p = U0 + NVAR * ((size_t)(ib + NGH) * plane + (size_t)(j + NGH) * P2 + (k + NGH));
     auto issue_u0 = [&](int p) {
       if (valid && p < ie) {
-        const real *src = U0 + NVAR * ((size_t)(p + NGH) * plane + (size_t)(j + NGH) * P2 + (k + NGH));
 #pragma unroll
-        for (int v = 0; v < NVAR; v += CH) cp_async<16>(&el<real, NT>(u0s, v, tid), src + v);
+        for (int v = 0; v < NVAR; v += CH) cp_async<16>(&el<real, NT>(u0s, v, tid), u0p + v);
+        u0p += NVAR * plane;
       }
       cp_async_commit();
     };
-    auto ringp = [&](int p) -> const real * { return ring + ((p + 5) % 5) * NVAR * RP; };
-    auto gather = [&](const real *pl, int jj, int kk, real *w) { ld8<real, RP>(pl, jj * RK + kk, w); };
-    // half the limited radial slope at plane p of the thread's column
-    auto rslope = [&](int p, real *sl_) {
-      const real *pm = ringp(p - 1), *pc = ringp(p), *pp = ringp(p + 1);
-      const int o = (jl + 2) * RK + kl + 2;
-      real a[NVAR], b[NVAR], c[NVAR];
-      ld8<real, RP>(pm, o, a);
-      ld8<real, RP>(pc, o, b);
-      ld8<real, RP>(pp, o, c);
-      mc_half_slopes8<real>(a, b, c, sl_);
+    // ring offset of the plane after the one at offset a
+    auto next = [](int a) { return a == 4 * PL ? 0 : a + PL; };
+    // half the limited radial slope of the thread's column at the middle of
+    // the planes at offsets m, c, p
+    auto rslope = [&](int m, int c, int p, real *out) {
+      real a[NVAR], b[NVAR], e[NVAR];
+      ld8<real, RP>(ring + m, o, a);
+      ld8<real, RP>(ring + c, o, b);
+      ld8<real, RP>(ring + p, o, e);
+      mc_half_slopes8<real>(a, b, e, out);
     };
-    // radial face between planes p-1 and p from the slopes at both planes
-    auto rflux = [&](int p, const real *sm, const real *sp, real *F) {
-      real b[NVAR], c[NVAR];
-      gather(ringp(p - 1), jl + 2, kl + 2, b);
-      gather(ringp(p), jl + 2, kl + 2, c);
+    // radial face between the planes at offsets m and c from the slopes at both
+    auto rflux = [&](int m, int c, const real *sm, const real *sp, real *F) {
+      real b[NVAR], e[NVAR];
+      ld8<real, RP>(ring + m, o, b);
+      ld8<real, RP>(ring + c, o, e);
       if constexpr (sizeof(real) == 4) {
-        tvdlf_pair<0>(b, c, sm, sp, gamma, igm1, F);
+        tvdlf_pair<0>(b, e, sm, sp, gamma, igm1, F);
       } else {
         real WL[NVAR], WR[NVAR];
         axpy8<real>(b, real(1), sm, WL);
-        axpy8<real>(c, real(-1), sp, WR);
-        tvdlf_states<real, 0>(WL, WR, b, c, gamma, igm1, F);
+        axpy8<real>(e, real(-1), sp, WR);
+        tvdlf_states<real, 0>(WL, WR, b, e, gamma, igm1, F);
       }
     };
-    // div B at plane p on the (TJ+2) x (TK+2) positions around the tile
-    auto divb_plane = [&](int p) {
+    // div B at plane p (offsets of planes p-1, p, p+1) on the (TJ+2) x (TK+2)
+    // positions around the tile
+    auto divb_plane = [&](int p, int m, int c, int e) {
       real *dst = dring + (p & 3) * DP;
-      const real *pm = ringp(p - 1), *pc = ringp(p), *pp = ringp(p + 1);
+      const real *pm = ring + m, *pc = ring + c, *pp = ring + e;
       const int pr = p - ib + 2;   // plane index in the staged arrays
-      const real rcm = s_rc[pr - 1], rcc = s_rc[pr], rcp = s_rc[pr + 1];
-      // plane-uniform radial factors
-      const real wm = spherical ? rcm * rcm : real(1), wp = spherical ? rcp * rcp : real(1);
-      const real fr = RT<real>::rcp_((spherical ? rcc * rcc : real(1)) * (rcp - rcm));
+      const real wm = s_rc2[pr - 1], wp = s_rc2[pr + 1], fr = s_pl[NPF * pr + P_FR], irc = s_pl[NPF * pr + P_IRC];
       for (int q = tid; q < DP; q += NT) {
-        const int dj = q / DK - 1, dk = q - (q / DK) * DK - 1;
-        if (dj > nvj || dk > nvk) continue;
-        const int jj = dj + 2, kk = dk + 2;
-        const int o = jj * RK + kk;
-        const real brm = el<real, RP>(pm, 5, o), brp = el<real, RP>(pp, 5, o);
-        const real btm = el<real, RP>(pc, 6, o - RK), btp = el<real, RP>(pc, 6, o + RK);
-        const real bpm = el<real, RP>(pc, 7, o - 1), bpp = el<real, RP>(pc, 7, o + 1);
-        const real itc2 = s_itc2[dj + 2], ipc2 = s_ipc2[dk + 2];
-        real div;
-        if (spherical) {
-          const real stc = s_st[dj + 2];
-          const real sm = s_st[dj + 1], sp = s_st[dj + 3];
-          const real irs = RT<real>::rcp_(rcc * stc);
-          div = (wp * brp - wm * brm) * fr + (sp * btp - sm * btm) * irs * itc2 + (bpp - bpm) * irs * ipc2;
-        } else {
-          div = (brp - brm) * fr + (btp - btm) * itc2 + (bpp - bpm) * ipc2;
-        }
-        dst[q] = div;
+        const int dj = q / DK, dk = q - (q / DK) * DK;   // row and column + 1
+        if (dj > nvj + 1 || dk > nvk + 1) continue;
+        const int at = (dj + 1) * RK + dk + 1;
+        const real brm = el<real, RP>(pm, 5, at), brp = el<real, RP>(pp, 5, at);
+        const real btm = el<real, RP>(pc, 6, at - RK), btp = el<real, RP>(pc, 6, at + RK);
+        const real bpm = el<real, RP>(pc, 7, at - 1), bpp = el<real, RP>(pc, 7, at + 1);
+        dst[q] = (wp * brp - wm * brm) * fr + ((s_st[dj + 2] * btp - s_st[dj] * btm) * s_tt[dj + 1] +
+                                              (bpp - bpm) * (s_ist[dj + 1] * s_ipc2[dk + 1])) * irc;
       }
     };
 
-    // ---- geometry of the work item into shared memory (read after the
+    // ---- factors of the work item into shared memory (read after the
     // prologue's first barrier); rows / columns past the block's edge are
     // never read and not loaded ----
+    const real dphi = G.dphi, idphi = RT<real>::rcp_(dphi);
     {
       const int npl = ie - ib + 4, ir0 = I0 + ib - 2 + NGH;
       for (int q = tid; q < npl; q += NT) {
-        s_rc[q] = G.rc[ir0 + q];
-        s_dr2[q] = G.dr2[ir0 + q];
-        s_dr3[q] = G.dr3[ir0 + q];
-        s_idr[q] = RT<real>::rcp_(G.dr[ir0 + q]);
-        s_irc[q] = RT<real>::rcp_(G.rc[ir0 + q]);
-        if (q >= 1 && q + 1 < npl) s_ird2[q] = RT<real>::rcp_(G.rc[ir0 + q + 1] - G.rc[ir0 + q - 1]);
+        real *f = s_pl + NPF * q;
+        const real rc = G.rc[ir0 + q], iv3 = RT<real>::rcp_(G.dr3[ir0 + q]);
+        const real irc = spherical ? RT<real>::rcp_(rc) : real(1);
+        f[P_RP] = real(0.5) * G.r2f[ir0 + q + 1] * iv3;
+        f[P_RM] = real(0.5) * G.r2f[ir0 + q] * iv3;
+        f[P_DR] = G.dr2[ir0 + q] * iv3;
+        f[P_CF] = Om * Om * rc;
+        f[P_IDR] = RT<real>::rcp_(G.dr[ir0 + q]);
+        f[P_IRC] = irc;
+        s_rc2[q] = spherical ? rc * rc : real(1);
+        if (q >= 1 && q + 1 < npl) {
+          f[P_ID2] = RT<real>::rcp_(G.rc[ir0 + q + 1] - G.rc[ir0 + q - 1]);
+          f[P_FR] = f[P_ID2] * irc * irc;
+        }
       }
-      for (int q = tid; q <= npl; q += NT) s_r2f[q] = G.r2f[ir0 + q];
       const int jr0 = J0 - 2 + NGH;
       for (int q = tid; q < nvj + 4; q += NT) {
-        if (q >= 1 && q + 1 < nvj + 4) s_itc2[q] = RT<real>::rcp_(G.tc[jr0 + q + 1] - G.tc[jr0 + q - 1]);
-        s_st[q] = G.sintc[jr0 + q];
-        s_ct[q] = G.costc[jr0 + q];
-        s_dcos[q] = G.dcos[jr0 + q];
-        s_dth[q] = G.dth[jr0 + q];
-        s_idth[q] = RT<real>::rcp_(G.dth[jr0 + q]);
+        const real st = G.sintc[jr0 + q], ist = RT<real>::rcp_(st);
+        s_st[q] = st;
+        s_ist[q] = ist;
+        if (q >= 1 && q + 1 < nvj + 4) {
+          const real itc2 = RT<real>::rcp_(G.tc[jr0 + q + 1] - G.tc[jr0 + q - 1]);
+          s_tt[q] = ist * itc2;
+          if (q >= 2 && q < nvj + 2) {
+            real *f = s_row + NRF * (q - 2);
+            const real idc = RT<real>::rcp_(G.dcos[jr0 + q]);
+            f[R_TP] = real(0.5) * G.sinf[jr0 + q + 1] * idc;
+            f[R_TM] = real(0.5) * G.sinf[jr0 + q] * idc;
+            f[R_PW] = real(0.5) * G.dth[jr0 + q] * idc * idphi;
+            f[R_ST] = st;
+            f[R_CT] = G.costc[jr0 + q];
+            f[R_ITC2] = itc2;
+            f[R_IST] = ist;
+            f[R_IDTH] = RT<real>::rcp_(G.dth[jr0 + q]);
+          }
+        }
       }
-      for (int q = tid; q <= nvj + 4; q += NT) s_sinf[q] = G.sinf[jr0 + q];
       const int kr0 = K0 - 2 + NGH;
       for (int q = 1 + tid; q + 1 < nvk + 4; q += NT) s_ipc2[q] = RT<real>::rcp_(G.pc[kr0 + q + 1] - G.pc[kr0 + q - 1]);
     }
-    const real dphi = G.dphi, idphi = RT<real>::rcp_(dphi);
 
     // ---- prologue: planes ib-2 .. ib+2 converted, r flux at face ib ----
-    for (int p = ib - 2; p <= ib + 2; p++) issue_plane(p);
+    // offsets of planes i-1 .. i+3 of the march (plane p sits at p + 2 - ib
+    // planes past the first slot, modulo five)
+    int om = PL, oc = 2 * PL, o1 = 3 * PL, o2 = 4 * PL, o3 = 0;
+    for (int p = 0; p < 5; p++) {
+      issue_plane(ib - 2 + p, p * PL);
+    }
     cp_async_wait_all();
-    for (int p = ib - 2; p <= ib + 2; p++) convert_plane(p);
+    for (int p = 0; p < 5; p++) convert_plane(p * PL);
     __syncthreads();
     if (S2) {
-      divb_plane(ib - 1);
-      divb_plane(ib);
+      divb_plane(ib - 1, 0, om, oc);
+      divb_plane(ib, om, oc, o1);
     }
     real Flo[NVAR], sc[NVAR];
     real xprev = real(0);   // tracer X of this column at the previous plane
     if (valid) {
       real s0[NVAR];
-      rslope(ib - 1, s0);
-      rslope(ib, sc);
-      rflux(ib, s0, sc, Flo);
-      if (trc) xprev = xslot(ib - 1)[(jl + 2) * RK + kl + 2];
+      rslope(0, om, oc, s0);
+      rslope(om, oc, o1, sc);
+      rflux(om, oc, s0, sc, Flo);
+      if (trc) xprev = xring[RP + o];
     }
     __syncthreads();   // plane ib-2 is read no more: its slot takes plane ib+3
-    if (ib + 3 <= ie + 1) issue_plane(ib + 3);
+    if (ib + 3 <= ie + 1) issue_plane(ib + 3, o3);
     else cp_async_commit();
     issue_u0(ib);
 
@@ -384,95 +433,97 @@ __global__ void __launch_bounds__(stage_threads(TJ, TK), stage_min_ctas(sizeof(r
     for (int i = ib; i < ie; i++) {
       real *fthb = fth + (i & 1) * NVAR * NTH, *fphb = fph + (i & 1) * NVAR * NPH;
       {
-        const real *pl = ringp(i);
-        for (int f = tid; f < NTH + NPH; f += NT) {
-          real a[NVAR], b[NVAR], c[NVAR], e[NVAR], F[NVAR];
-          if (f < NTH) {
-            const int row = f / TK, col = f - (f / TK) * TK;
-            if (row <= nvj && col < nvk) {
-              gather(pl, row, col + 2, a);
-              gather(pl, row + 1, col + 2, b);
-              gather(pl, row + 2, col + 2, c);
-              gather(pl, row + 3, col + 2, e);
-              tvdlf_face<real, 1>(a, b, c, e, gamma, igm1, F);
-              st8<real, NTH>(fthb, row * TK + col, F);
-            }
-          } else {
-            // phi faces: the first TJ * TK in rows of TK (a warp's quarters stay
-            // in one row when TK is a multiple of 8), then the last column
-            const int g = f - NTH;
-            const int row = g < TJ * TK ? g / TK : g - TJ * TK;
-            const int col = g < TJ * TK ? g - (g / TK) * TK : TK;
-            if (row < nvj && col <= nvk) {
-              gather(pl, row + 2, col, a);
-              gather(pl, row + 2, col + 1, b);
-              gather(pl, row + 2, col + 2, c);
-              gather(pl, row + 2, col + 3, e);
-              tvdlf_face<real, 2>(a, b, c, e, gamma, igm1, F);
-              st8<real, NPH>(fphb, row * (TK + 1) + col, F);
-            }
+        // the lower theta and phi face of the thread's cell, then an extra one
+        const real *pl = ring + oc;
+        int to = own && jl <= nvj && kl < nvk ? o : -1, po = own && jl < nvj && kl <= nvk ? o : -1;
+        int ts = tid, ps = tid + jl;
+#pragma unroll 1
+        for (int rep = 0;; rep++) {
+          if (to >= 0) {
+            real a[NVAR], b[NVAR], c[NVAR], e[NVAR], F[NVAR];
+            ld8<real, RP>(pl, to - 2 * RK, a);
+            ld8<real, RP>(pl, to - RK, b);
+            ld8<real, RP>(pl, to, c);
+            ld8<real, RP>(pl, to + RK, e);
+            tvdlf_face<real, 1>(a, b, c, e, gamma, igm1, F);
+            st8<real, NTH>(fthb, ts, F);
           }
+          if (po >= 0) {
+            real a[NVAR], b[NVAR], c[NVAR], e[NVAR], F[NVAR];
+            ld8<real, RP>(pl, po - 2, a);
+            ld8<real, RP>(pl, po - 1, b);
+            ld8<real, RP>(pl, po, c);
+            ld8<real, RP>(pl, po + 1, e);
+            tvdlf_face<real, 2>(a, b, c, e, gamma, igm1, F);
+            st8<real, NPH>(fphb, ps, F);
+          }
+          if (rep || !(x_th || x_ph)) break;
+          to = x_th && nvj == TJ && xq < nvk ? (TJ + 2) * RK + xq + 2 : -1;
+          po = x_ph && nvk == TK && xq < nvj ? (xq + 2) * RK + TK + 2 : -1;
+          ts = TJ * TK + xq;
+          ps = xq * (TK + 1) + TK;
         }
       }
-      if (S2) divb_plane(i + 1);
+      if (S2) divb_plane(i + 1, oc, o1, o2);
       if (i + 3 <= ie + 1) {
         cp_async_wait_group<1>();   // plane i+3 landed (U^n of plane i may not have)
-        convert_plane(i + 3);
+        convert_plane(o3);
       }
       __syncthreads();
-      real Fhi[NVAR];
       if (valid) {
-        real sn[NVAR];
-        rslope(i + 1, sn);
-        rflux(i + 1, sc, sn, Fhi);
+        real Fhi[NVAR];
+        {
+          real sn[NVAR];
+          rslope(oc, o1, o2, sn);
+          rflux(oc, o1, sc, sn, Fhi);
 #pragma unroll
-        for (int v = 0; v < NVAR; v++) sc[v] = sn[v];
-      }
-      if (valid) {
-        const int pr = i - ib + 2, jr = jl + 2;   // indices in the staged arrays
-        const real dcos = s_dcos[jr], dr2 = s_dr2[pr];
-        // face areas; the fluxes carry a factor 2 (tvdlf_states), which the
-        // half areas hArm ... hAp take back
-        const real Arm = s_r2f[pr] * dcos * dphi, Arp = s_r2f[pr + 1] * dcos * dphi;
-        const real Atm = s_sinf[jr] * dr2 * dphi, Atp = s_sinf[jr + 1] * dr2 * dphi;
-        const real Ap = dr2 * s_dth[jr];
-        const real hArm = real(0.5) * Arm, hArp = real(0.5) * Arp, hAtm = real(0.5) * Atm, hAtp = real(0.5) * Atp,
-                   hAp = real(0.5) * Ap;
-        const real V = s_dr3[pr] * dcos * dphi;
-        const real iV = RT<real>::rcp_(V);
+          for (int v = 0; v < NVAR; v++) sc[v] = sn[v];
+        }
+        const int pr = i - ib + 2;   // plane index in the staged arrays
+        real pf[NPF], rf[NRF];
+#pragma unroll
+        for (int v = 0; v < NPF; v += CH) Vec16<real>::put(*reinterpret_cast<const typename Vec16<real>::T *>(s_pl + NPF * pr + v), pf + v);
+#pragma unroll
+        for (int v = 0; v < NRF; v += CH) Vec16<real>::put(*reinterpret_cast<const typename Vec16<real>::T *>(s_row + NRF * jl + v), rf + v);
         real w[NVAR];
-        gather(ringp(i), jl + 2, kl + 2, w);
+        ld8<real, RP>(ring + oc, o, w);
         real un[NVAR];
         const size_t cidx = (size_t)(i + NGH) * plane + (size_t)(j + NGH) * P2 + (k + NGH);
+        const real ctp = pf[P_DR] * rf[R_TP], ctm = pf[P_DR] * rf[R_TM], cpw = pf[P_DR] * rf[R_PW];
         {
-          const int qt = jl * TK + kl, qp = jl * (TK + 1) + kl;
+          const int qp = tid + jl;
 #pragma unroll
           for (int c = 0; c < NVAR / CH; c++) {
             real ftl[CH], fth_[CH], fpl[CH], fph_[CH];
             using V = Vec16<real>;
-            V::put(*reinterpret_cast<const typename V::T *>(fthb + (c * NTH + qt) * CH), ftl);
-            V::put(*reinterpret_cast<const typename V::T *>(fthb + (c * NTH + qt + TK) * CH), fth_);
+            V::put(*reinterpret_cast<const typename V::T *>(fthb + (c * NTH + tid) * CH), ftl);
+            V::put(*reinterpret_cast<const typename V::T *>(fthb + (c * NTH + tid + TK) * CH), fth_);
             V::put(*reinterpret_cast<const typename V::T *>(fphb + (c * NPH + qp) * CH), fpl);
             V::put(*reinterpret_cast<const typename V::T *>(fphb + (c * NPH + qp + 1) * CH), fph_);
-            flux_balance<real, CH>(Fhi + c * CH, Flo + c * CH, fth_, ftl, fph_, fpl, hArp, hArm, hAtp, hAtm, hAp,
-                                   iV, un + c * CH);
+            flux_balance<real, CH>(Fhi + c * CH, Flo + c * CH, fth_, ftl, fph_, fpl, pf[P_RP], pf[P_RM], ctp, ctm, cpw,
+                                   un + c * CH);
           }
         }
         if (spherical) {
-          const real gr = (Arp - Arm) * iV, gt = (Atp - Atm) * iV, ir = real(0.5) * gr;
+          // ir = (A_r+ - A_r-) / 2V, gt = (A_th+ - A_th-) / V
+          const real ir = pf[P_RP] - pf[P_RM], gt = real(2) * (ctp - ctm);
           const real rho = w[0], vr = w[1], vt = w[2], vp = w[3], Br = w[5], Bt = w[6], Bp = w[7];
-          const real pt = w[4] + real(0.5) * (Br * Br + Bt * Bt + Bp * Bp);
-          un[1] += (rho * (vt * vt + vp * vp) - (Bt * Bt + Bp * Bp)) * ir + pt * gr;
-          un[2] += (-rho * vr * vt + Br * Bt) * ir + (rho * vp * vp - Bp * Bp) * gt + pt * gt;
-          un[3] += (-rho * vr * vp + Br * Bp) * ir - (rho * vt * vp - Bt * Bp) * gt;
+          const real mt = rho * vt, mp = rho * vp, Bt2 = Bt * Bt, Bp2 = Bp * Bp;
+          const real tpp = mp * vp - Bp2, ttt = mt * vt - Bt2;   // stress without pressure
+          const real pt = w[4] + real(0.5) * (Br * Br + Bt2 + Bp2);
+          un[1] += (tpp + ttt + real(2) * pt) * ir;
+          un[2] += (Br * Bt - mt * vr) * ir + (tpp + pt) * gt;
+          un[3] += (Br * Bp - mp * vr) * ir - (mt * vp - Bt * Bp) * gt;
           un[6] += (vr * Bt - vt * Br) * ir;
           un[7] += (vr * Bp - vp * Br) * ir + (vt * Bp - vp * Bt) * gt;
-          const real rc = s_rc[pr], st = s_st[jr], ct = s_ct[jr];
-          const real vs = vr * st + vt * ct;
-          un[1] += rho * (real(2) * Om * vp * st + Om * Om * rc * st * st);
-          un[2] += rho * (real(2) * Om * vp * ct + Om * Om * rc * st * ct);
-          un[3] += real(-2) * Om * rho * vs;
-          un[4] += rho * Om * Om * rc * st * vs;
+          // Coriolis and centrifugal forces, centrifugal work
+          const real st = rf[R_ST], ct = rf[R_CT], cf = pf[P_CF] * st;
+          const real c2 = real(2) * Om * mp + rho * cf;
+          const real vs = vr * st + vt * ct, mvs = rho * vs;
+          un[1] += c2 * st;
+          un[2] += c2 * ct;
+          un[3] -= real(2) * Om * mvs;
+          un[4] += cf * mvs;
         }
         cp_async_wait_group<0>();   // this thread's U^n copy of plane i
         {
@@ -480,26 +531,17 @@ __global__ void __launch_bounds__(stage_threads(TJ, TK), stage_min_ctas(sizeof(r
           ld8<real, NT>(u0s, tid, u0);
           axpy8<real>(u0, dt, un, un);
         }
+        // reciprocal cell widths (the speeds of the corrector's CFL step, h of
+        // the cleaning)
+        const real irs = pf[P_IRC] * rf[R_IST];
+        const real ix[3] = {pf[P_IDR], spherical ? pf[P_IRC] * rf[R_IDTH] : rf[R_IDTH], spherical ? irs * idphi : idphi};
         if (S2 && Cd > real(0)) {
           const real *dm = dring + ((i - 1) & 3) * DP, *dc = dring + (i & 3) * DP, *dp = dring + ((i + 1) & 3) * DP;
           const int q = (jl + 1) * DK + (kl + 1);
-          const real ird2 = s_ird2[pr], itc2 = s_itc2[jr], ipc2 = s_ipc2[kl + 2];
-          const real idr = s_idr[pr], idth = s_idth[jr];
-          real gr_, gt_, gp_, h2inv;
-          if (spherical) {
-            const real irc = s_irc[pr], irs = RT<real>::rcp_(s_rc[pr] * s_st[jr]);
-            gr_ = (dp[q] - dm[q]) * ird2;
-            gt_ = (dc[q + DK] - dc[q - DK]) * irc * itc2;
-            gp_ = (dc[q + 1] - dc[q - 1]) * irs * ipc2;
-            const real ixt = irc * idth, ixp = irs * idphi;
-            h2inv = idr * idr + ixt * ixt + ixp * ixp;
-          } else {
-            gr_ = (dp[q] - dm[q]) * ird2;
-            gt_ = (dc[q + DK] - dc[q - DK]) * itc2;
-            gp_ = (dc[q + 1] - dc[q - 1]) * ipc2;
-            h2inv = idr * idr + idth * idth + idphi * idphi;
-          }
-          const real f = Cd * RT<real>::rcp_(h2inv);
+          const real gr_ = (dp[q] - dm[q]) * pf[P_ID2];
+          const real gt_ = (dc[q + DK] - dc[q - DK]) * (pf[P_IRC] * rf[R_ITC2]);
+          const real gp_ = (dc[q + 1] - dc[q - 1]) * (irs * s_ipc2[kl + 2]);
+          const real f = Cd * RT<real>::rcp_(ix[0] * ix[0] + ix[1] * ix[1] + ix[2] * ix[2]);
           const real dB0 = f * gr_, dB1 = f * gt_, dB2 = f * gp_;
           un[5] += dB0;
           un[6] += dB1;
@@ -511,85 +553,103 @@ __global__ void __launch_bounds__(stage_threads(TJ, TK), stage_min_ctas(sizeof(r
           // with X from the face's upwind cell
           // X at plane i-1 of this column is carried from the previous plane:
           // that ring slot already receives the copy of plane i+4
-          const int o = (jl + 2) * RK + kl + 2;
-          const real *xc = xslot(i), *xp = xslot(i + 1);
+          const real *xc = xring + oc / NVAR, *xp = xring + o1 / NVAR;
           const real X0 = xc[o];
-          const real ftl0 = el<real, NTH>(fthb, 0, jl * TK + kl), fth0 = el<real, NTH>(fthb, 0, (jl + 1) * TK + kl);
-          const real fpl0 = el<real, NPH>(fphb, 0, jl * (TK + 1) + kl), fph0 = el<real, NPH>(fphb, 0, jl * (TK + 1) + kl + 1);
-          const real arm = hArm * Flo[0] * (Flo[0] > real(0) ? xprev : X0);
-          const real arp = hArp * Fhi[0] * (Fhi[0] > real(0) ? X0 : xp[o]);
-          const real atm = hAtm * ftl0 * (ftl0 > real(0) ? xc[o - RK] : X0);
-          const real atp = hAtp * fth0 * (fth0 > real(0) ? X0 : xc[o + RK]);
-          const real apm = hAp * fpl0 * (fpl0 > real(0) ? xc[o - 1] : X0);
-          const real app = hAp * fph0 * (fph0 > real(0) ? X0 : xc[o + 1]);
-          const real dT = -((arp - arm) + (atp - atm) + (app - apm)) * iV;
+          const real ftl0 = el<real, NTH>(fthb, 0, tid), fth0 = el<real, NTH>(fthb, 0, tid + TK);
+          const real fpl0 = el<real, NPH>(fphb, 0, tid + jl), fph0 = el<real, NPH>(fphb, 0, tid + jl + 1);
+          const real arm = pf[P_RM] * Flo[0] * (Flo[0] > real(0) ? xprev : X0);
+          const real arp = pf[P_RP] * Fhi[0] * (Fhi[0] > real(0) ? X0 : xp[o]);
+          const real atm = ctm * ftl0 * (ftl0 > real(0) ? xc[o - RK] : X0);
+          const real atp = ctp * fth0 * (fth0 > real(0) ? X0 : xc[o + RK]);
+          const real apm = cpw * fpl0 * (fpl0 > real(0) ? xc[o - 1] : X0);
+          const real app = cpw * fph0 * (fph0 > real(0) ? X0 : xc[o + 1]);
+          const real dT = -((arp - arm) + (atp - atm) + (app - apm));
           Uout[TRV * vstride + cidx] = U0[TRV * vstride + cidx] + dt * dT;
           xprev = X0;
         }
-        hits += apply_floors<real>(un, gamma, pfl, rfl, isl);
-        if (!(un[0] == un[0]) || !(un[4] == un[4])) atomicOr(kp.status, ST_NAN);
+        // Floors: the plain pressure of the new state serves the CFL speed and
+        // tells a cell that might be below a floor (see apply_floors), which
+        // takes the precise path
+        real irn = RT<real>::rcp_(un[0]), pn = pressure_for_speed<real>(un, gamma);
+        const real margin = sizeof(real) == 4 ? real(1e-6) : real(0);
+        if (RT<real>::less_(un[0], rfl) || !RT<real>::less_(pfl + margin * RT<real>::abs_(un[4]), pn)) {
+          hits += apply_floors<real>(un, gamma, pfl, rfl, isl);
+          irn = RT<real>::rcp_(un[0]);
+          pn = pressure_for_speed<real>(un, gamma);
+          if (RT<real>::less_(pn, pfl)) pn = pfl;
+        }
+        if (RT<real>::nan_(un[0]) || RT<real>::nan_(un[4])) atomicOr(kp.status, ST_NAN);
         st_cell(Uout + NVAR * cidx, un);
         if (S2) {
+          const unsigned at = edge | (unsigned)(i == 0) | (unsigned)(i == nb0 - 1) << 1;
           // CFL contribution of the new state (cells next to a finer face are
           // left to the reflux, which changes them once more)
-          const bool skip = (i == 0 && B.nbr[0] == NB_FINER) || (i == nb0 - 1 && B.nbr[1] == NB_FINER) ||
-                            (j == 0 && B.nbr[2] == NB_FINER) || (j == nb1 - 1 && B.nbr[3] == NB_FINER) ||
-                            (k == 0 && B.nbr[4] == NB_FINER) || (k == nb2 - 1 && B.nbr[5] == NB_FINER);
-          if (!skip) {
-            real wn[NVAR];
-            cons2prim_speed<real>(un, wn, gamma, pfl);
-            real dx1 = s_dth[jr], dx2 = dphi;
-            if (spherical) {
-              dx1 *= s_rc[pr];
-              dx2 *= s_rc[pr] * s_st[jr];
-            }
-            const real s = (RT<real>::abs_(wn[1]) + fast_speed<real, 0>(wn, gamma)) * s_idr[pr] +
-                           (RT<real>::abs_(wn[2]) + fast_speed<real, 1>(wn, gamma)) * RT<real>::rcp_(dx1) +
-                           (RT<real>::abs_(wn[3]) + fast_speed<real, 2>(wn, gamma)) * RT<real>::rcp_(dx2);
-            inv_acc = RT<real>::max_(inv_acc, s);
+          if (!(at & fin)) {
+            const real vn[3] = {un[1] * irn, un[2] * irn, un[3] * irn};
+            const real s = cfl_rate<real>(irn, vn, pn, un + 5, gamma, ix);
+            inv_acc = RT<real>::less_(inv_acc, s) ? s : inv_acc;
           }
-          if (sl.flux) {
+          if (sl.flux && (at & cfb)) {
+            // area-weighted fluxes of the block's coarse-fine faces
             real *fb = reinterpret_cast<real *>(sl.flux) + (size_t)slot * fstride;
-            // r faces
-            if (i == 0 && (B.nbr[0] == NB_COARSER || B.nbr[0] == NB_FINER))
+            const unsigned hit = at & cfb;
+            const int I = I0 + i + NGH, J = J0 + jl + NGH;
+            const real dcos = G.dcos[J], dr2 = G.dr2[I];
+            const size_t o2_ = (size_t)2 * NVAR * fc0, o4 = o2_ + (size_t)2 * NVAR * fc1;
+            if (hit & 1u) {
+              const real A = real(0.5) * (G.r2f[I] * dcos * dphi);
 #pragma unroll
-              for (int v = 0; v < NVAR; v++) fb[(size_t)v * fc0 + j * nb2 + k] = hArm * Flo[v];
-            if (i == nb0 - 1 && (B.nbr[1] == NB_COARSER || B.nbr[1] == NB_FINER))
+              for (int v = 0; v < NVAR; v++) fb[(size_t)v * fc0 + j * nb2 + k] = A * Flo[v];
+            }
+            if (hit & 2u) {
+              const real A = real(0.5) * (G.r2f[I + 1] * dcos * dphi);
 #pragma unroll
-              for (int v = 0; v < NVAR; v++) fb[(size_t)NVAR * fc0 + (size_t)v * fc0 + j * nb2 + k] = hArp * Fhi[v];
-            const size_t o2 = (size_t)2 * NVAR * fc0, o4 = o2 + (size_t)2 * NVAR * fc1;
-            if (j == 0 && (B.nbr[2] == NB_COARSER || B.nbr[2] == NB_FINER))
-#pragma unroll
-              for (int v = 0; v < NVAR; v++)
-                fb[o2 + (size_t)v * fc1 + i * nb2 + k] = hAtm * el<real, NTH>(fthb, v, jl * TK + kl);
-            if (j == nb1 - 1 && (B.nbr[3] == NB_COARSER || B.nbr[3] == NB_FINER))
-#pragma unroll
-              for (int v = 0; v < NVAR; v++)
-                fb[o2 + (size_t)NVAR * fc1 + (size_t)v * fc1 + i * nb2 + k] = hAtp * el<real, NTH>(fthb, v, (jl + 1) * TK + kl);
-            if (k == 0 && (B.nbr[4] == NB_COARSER || B.nbr[4] == NB_FINER))
-#pragma unroll
-              for (int v = 0; v < NVAR; v++)
-                fb[o4 + (size_t)v * fc2 + i * nb1 + j] = hAp * el<real, NPH>(fphb, v, jl * (TK + 1) + kl);
-            if (k == nb2 - 1 && (B.nbr[5] == NB_COARSER || B.nbr[5] == NB_FINER))
+              for (int v = 0; v < NVAR; v++) fb[(size_t)NVAR * fc0 + (size_t)v * fc0 + j * nb2 + k] = A * Fhi[v];
+            }
+            if (hit & 4u) {
+              const real A = real(0.5) * (G.sinf[J] * dr2 * dphi);
 #pragma unroll
               for (int v = 0; v < NVAR; v++)
-                fb[o4 + (size_t)NVAR * fc2 + (size_t)v * fc2 + i * nb1 + j] = hAp * el<real, NPH>(fphb, v, jl * (TK + 1) + kl + 1);
+                fb[o2_ + (size_t)v * fc1 + i * nb2 + k] = A * el<real, NTH>(fthb, v, tid);
+            }
+            if (hit & 8u) {
+              const real A = real(0.5) * (G.sinf[J + 1] * dr2 * dphi);
+#pragma unroll
+              for (int v = 0; v < NVAR; v++)
+                fb[o2_ + (size_t)NVAR * fc1 + (size_t)v * fc1 + i * nb2 + k] = A * el<real, NTH>(fthb, v, tid + TK);
+            }
+            if (hit & 48u) {
+              const real A = real(0.5) * (dr2 * G.dth[J]);
+              if (hit & 16u)
+#pragma unroll
+                for (int v = 0; v < NVAR; v++)
+                  fb[o4 + (size_t)v * fc2 + i * nb1 + j] = A * el<real, NPH>(fphb, v, tid + jl);
+              if (hit & 32u)
+#pragma unroll
+                for (int v = 0; v < NVAR; v++)
+                  fb[o4 + (size_t)NVAR * fc2 + (size_t)v * fc2 + i * nb1 + j] = A * el<real, NPH>(fphb, v, tid + jl + 1);
+            }
           }
         }
 #pragma unroll
         for (int v = 0; v < NVAR; v++) Flo[v] = Fhi[v];
       }
-      if (i + 4 <= ie + 1) issue_plane(i + 4);
+      if (i + 4 <= ie + 1) issue_plane(i + 4, om);
       else cp_async_commit();
       issue_u0(i + 1);
+      om = oc;
+      oc = o1;
+      o1 = o2;
+      o2 = o3;
+      o3 = next(o3);
     }
     cp_async_wait_all();
     __syncthreads();  // shared memory is reused by the next work item
   }
   if (S2) flush_acc(kp, inv_acc, cur_member, hits);
   else {
-    long long h = hits;
-    for (int o = 16; o > 0; o >>= 1) h += __shfl_xor_sync(0xffffffffu, h, o);
+    int h = hits;
+    for (int q = 16; q > 0; q >>= 1) h += __shfl_xor_sync(0xffffffffu, h, q);
     if ((threadIdx.x & 31) == 0 && h) atomicAdd(kp.floor_hits, (unsigned long long)h);
   }
 }

@@ -11,12 +11,52 @@
 #include "icarus_internal.h"
 
 template <typename real> struct RT;
+// FP64 mode: an FP64-pipe instruction of a warp takes 71 to 83 cycles of its
+// scheduler (measured; 16 to 20 of the SM), an integer one 1 to 2, so the number
+// of FP64-pipe instructions is the time of every FP64 kernel, and comparisons,
+// minima and sign tests (each a DSETP, 80 cycles) go through the bit patterns.
+// Reciprocal and square root: the hardware approximation (20 bits) and one
+// step of third order, 1 + e + e^2 and 1 + e/2 + 3 e^2/8 with e the residual
+// (Householder's iteration; the error e^3 is below 2^-56).  Over 4 M arguments
+// of 2^-900 .. 2^900 both are within 1 ulp of the correctly rounded functions
+// (the reciprocal differs in 0.03 % of them, the root in 12 %), at 3 and 5
+// FP64-pipe instructions instead of 5 and 8.
 template <> struct RT<double> {
-  static __device__ __forceinline__ double sqrt_(double x) { return sqrt(x); }
+  static __device__ __forceinline__ double sqrt_(double x) {
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double g = x * y, e = fma(-g, y, 1.0);
+    const double r = fma(g * e, fma(e, 0.375, 0.5), g);
+    // zero and subnormals, where the approximation is infinite
+    return (__double2hiint(x) & 0x7fffffff) < 0x00100000 ? 0.0 : r;
+  }
   static __device__ __forceinline__ double abs_(double x) { return fabs(x); }
-  static __device__ __forceinline__ double min_(double a, double b) { return fmin(a, b); }
-  static __device__ __forceinline__ double max_(double a, double b) { return fmax(a, b); }
-  static __device__ __forceinline__ double rcp_(double x) { return __drcp_rn(x); }
+  // minimum and maximum of numbers that are not negative
+  static __device__ __forceinline__ double min_(double a, double b) {
+    return __double_as_longlong(a) < __double_as_longlong(b) ? a : b;
+  }
+  static __device__ __forceinline__ double max_(double a, double b) {
+    return __double_as_longlong(a) > __double_as_longlong(b) ? a : b;
+  }
+  static __device__ __forceinline__ double rcp_(double x) {
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double e = fma(-x, y, 1.0);
+    return fma(y, fma(e, e, e), y);
+  }
+  // x > 0; not for NaN
+  static __device__ __forceinline__ bool pos_(double x) {
+    return (unsigned long long)(__double_as_longlong(x) - 1) < 0x7ff0000000000000ull;
+  }
+  static __device__ __forceinline__ bool nan_(double x) {
+    return (unsigned long long)(__double_as_longlong(x) & 0x7fffffffffffffffll) > 0x7ff0000000000000ull;
+  }
+  // a < b; not for NaN (-0 counts as below +0)
+  static __device__ __forceinline__ bool less_(double a, double b) {
+    const long long x = __double_as_longlong(a), y = __double_as_longlong(b);
+    const long long m = 0x7fffffffffffffffll;
+    return (x ^ ((x >> 63) & m)) < (y ^ ((y >> 63) & m)) && !nan_(a) && !nan_(b);
+  }
 };
 // FP32 mode: reciprocal and square root are the hardware approximations
 // (PTX rcp.approx / sqrt.approx, relative error within about 1 ulp); the
@@ -36,6 +76,9 @@ template <> struct RT<float> {
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
   }
+  static __device__ __forceinline__ bool pos_(float x) { return x > 0.f; }
+  static __device__ __forceinline__ bool nan_(float x) { return !(x == x); }
+  static __device__ __forceinline__ bool less_(float a, float b) { return a < b; }
 };
 
 // ---- the padded state ----
@@ -156,7 +199,22 @@ __device__ __forceinline__ void cons2prim(const real *u, real *w, real gamma, re
   w[2] = u[2] * ir;
   w[3] = u[3] * ir;
   real p = pressure_of<real>(u, gamma, isl);
-  w[4] = p < pfloor ? pfloor : p;
+  w[4] = RT<real>::less_(p, pfloor) ? pfloor : p;
+  w[5] = u[5];
+  w[6] = u[6];
+  w[7] = u[7];
+}
+// FP64: the two energies in one chain of products (14 FP64-pipe instructions)
+template <>
+__device__ __forceinline__ void cons2prim<double>(const double *u, double *w, double gamma, double pfloor, Isl) {
+  const double ir = RT<double>::rcp_(u[0]);
+  w[0] = u[0];
+  w[1] = u[1] * ir;
+  w[2] = u[2] * ir;
+  w[3] = u[3] * ir;
+  const double t = u[1] * w[1] + u[2] * w[2] + u[3] * w[3] + u[5] * u[5] + u[6] * u[6] + u[7] * u[7];
+  const double p = (gamma - 1.0) * fma(-0.5, t, u[4]);
+  w[4] = RT<double>::less_(p, pfloor) ? pfloor : p;
   w[5] = u[5];
   w[6] = u[6];
   w[7] = u[7];
@@ -171,7 +229,7 @@ __device__ __forceinline__ void cons2prim_speed(const real *u, real *w, real gam
   w[2] = u[2] * ir;
   w[3] = u[3] * ir;
   real p = pressure_for_speed<real>(u, gamma);
-  w[4] = p < pfloor ? pfloor : p;
+  w[4] = RT<real>::less_(p, pfloor) ? pfloor : p;
   w[5] = u[5];
   w[6] = u[6];
   w[7] = u[7];
@@ -214,6 +272,22 @@ __device__ __forceinline__ real mc_half_slope(real um, real u0, real up) {
   real lim = RT<real>::min_(RT<real>::min_(RT<real>::abs_(dm), RT<real>::abs_(dp)), real(0.25) * RT<real>::abs_(s));
   lim = s > real(0) ? lim : -lim;
   return dm * dp > real(0) ? lim : real(0);
+}
+
+// FP64: the minimum and the signs by bit patterns, the quarter by the exponent
+// (three FP64-pipe instructions, the differences, instead of nine)
+template <>
+__device__ __forceinline__ double mc_half_slope<double>(double um, double u0, double up) {
+  const double dm = u0 - um, dp = up - u0, s = dm + dp;
+  const long long m = 0x7fffffffffffffffll;
+  const long long a = __double_as_longlong(dm), b = __double_as_longlong(dp);
+  long long q = __double_as_longlong(s) & m;
+  q = q < 0x0030000000000000ll ? 0 : q - 0x0020000000000000ll;   // |s| / 4
+  const long long x = a & m, y = b & m;
+  long long lim = x < y ? x : y;
+  lim = q < lim ? q : lim;
+  lim |= a & ~m;
+  return __longlong_as_double((a ^ b) < 0 ? 0 : lim);
 }
 
 template <typename real>
@@ -264,15 +338,16 @@ __device__ __forceinline__ void axpy8<float>(const float *a, float s, const floa
   }
 }
 
-// Half MC slope from the one-sided differences dm, dp and their sum s, by
-// sign arithmetic: with sigma the sign of s, the slope is
-// sigma * max(0, min(sigma dm, sigma dp, |s| / 4)) -- zero unless dm and dp
-// share s's sign, the same value as mc_half_slope (bar the sign of a zero).
-__device__ __forceinline__ float half_mc_signed(float dm, float dp, float s) {
-  const unsigned sg = __float_as_uint(s) & 0x80000000u;
-  const float a = __uint_as_float(__float_as_uint(dm) ^ sg), b = __uint_as_float(__float_as_uint(dp) ^ sg);
-  const float m = fmaxf(fminf(fminf(a, b), 0.25f * fabsf(s)), 0.f);
-  return __uint_as_float(__float_as_uint(m) | sg);
+// Half MC slope from the one-sided differences dm, dp and q = (dm + dp) / 4:
+// min(|dm|, |dp|) carries the product of their signs (min.xorsign.abs), so one
+// maximum with zero clears an extremum; the result takes q's sign.  Four
+// instructions (a scheduler issues this form in 9.4 cycles a slope in a loop
+// of nothing else, sign flips of both differences in 13.7).
+__device__ __forceinline__ float half_mc_signed(float dm, float dp, float q) {
+  float t;
+  asm("min.xorsign.abs.f32 %0, %1, %2;" : "=f"(t) : "f"(dm), "f"(dp));
+  const float m = fmaxf(fminf(t, fabsf(q)), 0.f);
+  return __uint_as_float(__float_as_uint(m) | (__float_as_uint(q) & 0x80000000u));
 }
 
 // Half the monotonised-central slopes of the 8 variables at the middle of
@@ -291,76 +366,84 @@ __device__ __forceinline__ void mc_half_slopes8<float>(const float *um, const fl
     const float2 c = make_float2(u0[v], u0[v + 1]);
     const float2 dm = __fadd2_rn(c, make_float2(-um[v], -um[v + 1]));
     const float2 dp = __fadd2_rn(make_float2(up[v], up[v + 1]), make_float2(-c.x, -c.y));
-    const float2 sm = __fadd2_rn(dm, dp);
+    const float2 sm = __fmul2_rn(make_float2(0.25f, 0.25f), __fadd2_rn(dm, dp));
     out[v] = half_mc_signed(dm.x, dp.x, sm.x);
     out[v + 1] = half_mc_signed(dm.y, dp.y, sm.y);
   }
 }
 
-// Flux balance of CH variables of a cell: out[h] = -((Arp Fhi - Arm Flo) +
-// (Atp Fth - Atm Ftl) + Ap (Fph - Fpl)) * iV, FP32 in packed pairs.
+// Flux balance of CH variables of a cell with the areas over its volume:
+// out[h] = rm Flo - rp Fhi + tm Ftl - tp Fth + pw (Fpl - Fph), FP32 in packed
+// pairs.
 template <typename real, int CH>
 __device__ __forceinline__ void flux_balance(const real *Fhi, const real *Flo, const real *fth, const real *ftl,
-                                             const real *fph, const real *fpl, real Arp, real Arm, real Atp,
-                                             real Atm, real Ap, real iV, real *out) {
+                                             const real *fph, const real *fpl, real rp, real rm, real tp, real tm,
+                                             real pw, real *out) {
 #pragma unroll
-  for (int h = 0; h < CH; h++) {
-    const real div = (Arp * Fhi[h] - Arm * Flo[h]) + (Atp * fth[h] - Atm * ftl[h]) + Ap * (fph[h] - fpl[h]);
-    out[h] = -div * iV;
-  }
+  for (int h = 0; h < CH; h++)
+    out[h] = (rm * Flo[h] - rp * Fhi[h]) + (tm * ftl[h] - tp * fth[h]) + pw * (fpl[h] - fph[h]);
 }
 template <>
 __device__ __forceinline__ void flux_balance<float, 4>(const float *Fhi, const float *Flo, const float *fth,
                                                        const float *ftl, const float *fph, const float *fpl,
-                                                       float Arp, float Arm, float Atp, float Atm, float Ap,
-                                                       float iV, float *out) {
-  const float2 arp = make_float2(Arp, Arp), narm = make_float2(-Arm, -Arm), atp = make_float2(Atp, Atp),
-               natm = make_float2(-Atm, -Atm), ap = make_float2(Ap, Ap), m1 = make_float2(-1.f, -1.f),
-               niv = make_float2(-iV, -iV);
+                                                       float rp, float rm, float tp, float tm, float pw,
+                                                       float *out) {
+  const float2 r1 = make_float2(rm, rm), r2 = make_float2(-rp, -rp), t1 = make_float2(tm, tm),
+               t2 = make_float2(-tp, -tp), p1 = make_float2(pw, pw), m1 = make_float2(-1.f, -1.f);
 #pragma unroll
   for (int h = 0; h < 4; h += 2) {
-    const float2 r = __ffma2_rn(narm, make_float2(Flo[h], Flo[h + 1]),
-                                __fmul2_rn(arp, make_float2(Fhi[h], Fhi[h + 1])));
-    const float2 t = __ffma2_rn(natm, make_float2(ftl[h], ftl[h + 1]),
-                                __fmul2_rn(atp, make_float2(fth[h], fth[h + 1])));
-    const float2 p = __ffma2_rn(m1, make_float2(fpl[h], fpl[h + 1]), make_float2(fph[h], fph[h + 1]));
-    const float2 d = __ffma2_rn(ap, p, __fadd2_rn(r, t));
-    const float2 o = __fmul2_rn(d, niv);
+    const float2 r = __ffma2_rn(r2, make_float2(Fhi[h], Fhi[h + 1]), __fmul2_rn(r1, make_float2(Flo[h], Flo[h + 1])));
+    const float2 t = __ffma2_rn(t2, make_float2(fth[h], fth[h + 1]), __fmul2_rn(t1, make_float2(ftl[h], ftl[h + 1])));
+    const float2 p = __ffma2_rn(m1, make_float2(fph[h], fph[h + 1]), make_float2(fpl[h], fpl[h + 1]));
+    const float2 o = __ffma2_rn(p1, p, __fadd2_rn(r, t));
     out[h] = o.x;
     out[h + 1] = o.y;
   }
 }
 
-// fast magnetosonic speed along D from a face state, its 1/rho and |B|^2
-template <typename real, int D>
-__device__ __forceinline__ real fast_speed_pre(const real *w, real ir, real b2, real gamma) {
-  const real a2 = gamma * w[4] * ir;
-  const real bt2 = b2 * ir;
-  const real bn2 = w[5 + D] * w[5 + D] * ir;
-  const real s = a2 + bt2;
-  real disc = s * s - real(4) * a2 * bn2;
-  disc = disc < real(0) ? real(0) : disc;
-  return RT<real>::sqrt_(real(0.5) * (s + RT<real>::sqrt_(disc)));
+// Fast magnetosonic speed from 1/rho, gamma p, half gamma p, |B|^2 / 2 and the
+// square bt2 of the field across the direction: the discriminant
+// (a^2 + b^2)^2 - 4 a^2 b_n^2 as (a^2 - b^2)^2 + 4 a^2 b_t^2, which has no
+// cancellation and no sign to test; halved, so that the root's sum needs no
+// factor.
+__device__ __forceinline__ double fast_speed_of(double ir, double gp, double hgp, double hb2, double bt2) {
+  const double d = hgp - hb2;
+  return RT<double>::sqrt_((hgp + hb2 + RT<double>::sqrt_(fma(d, d, gp * bt2))) * ir);
+}
+__device__ __forceinline__ float fast_speed_of(float ir, float gp, float hgp, float hb2, float bt2) {
+  // scaled by 1/rho first: the squares stay far from the ends of FP32
+  const float a = hgp * ir, b = hb2 * ir, d = a - b;
+  return RT<float>::sqrt_(a + b + RT<float>::sqrt_(fmaf(d, d, (gp * ir) * (bt2 * ir))));
+}
+
+// Sum over the directions of (|v_d| + c_f,d) / dx_d from 1/rho, the velocity,
+// p and the field (ix: reciprocal widths)
+template <typename real>
+__device__ __forceinline__ real cfl_rate(real ir, const real *v, real p, const real *B, real gamma, const real *ix) {
+  const real gp = gamma * p, hgp = real(0.5) * gp, q0 = B[0] * B[0], q1 = B[1] * B[1], q2 = B[2] * B[2];
+  const real hb2 = real(0.5) * (q0 + q1 + q2);
+  return (RT<real>::abs_(v[0]) + fast_speed_of(ir, gp, hgp, hb2, q1 + q2)) * ix[0] +
+         (RT<real>::abs_(v[1]) + fast_speed_of(ir, gp, hgp, hb2, q0 + q2)) * ix[1] +
+         (RT<real>::abs_(v[2]) + fast_speed_of(ir, gp, hgp, hb2, q0 + q1)) * ix[2];
 }
 
 // One side's part of the TVDLF flux, G = F(W) + sc U(W) with sc = +c_max on
 // the left and -c_max on the right, so that the flux is (G_L + G_R) / 2.
 // Written out per component with w = v_n + sc:
-//   mass rho w;  momentum m_k w - B_n B_k (+ p_T along n);
+//   mass rho w;  momentum (rho w) v_k - B_n B_k (+ p_T along n);
 //   energy e w + p_T v_n - B_n (v.B);  induction B_k w - B_n v_k (k != n).
 template <typename real, int D>
-__device__ __forceinline__ void side_flux(const real *W, real b2, real igm1, real sc, real *G) {
+__device__ __forceinline__ void side_flux(const real *W, real hb2, real igm1, real sc, real *G) {
   const real vn = W[1 + D], Bn = W[5 + D];
   const real w = vn + sc;
-  const real m1 = W[0] * W[1], m2 = W[0] * W[2], m3 = W[0] * W[3];
-  const real rv2 = m1 * W[1] + m2 * W[2] + m3 * W[3];
-  const real pt = W[4] + real(0.5) * b2;
-  const real e = W[4] * igm1 + real(0.5) * (rv2 + b2);
+  const real v2 = W[1] * W[1] + W[2] * W[2] + W[3] * W[3];
+  const real pt = W[4] + hb2;
+  const real e = W[4] * igm1 + (real(0.5) * W[0] * v2 + hb2);
   const real vB = W[1] * W[5] + W[2] * W[6] + W[3] * W[7];
   G[0] = W[0] * w;
-  G[1] = m1 * w - Bn * W[5];
-  G[2] = m2 * w - Bn * W[6];
-  G[3] = m3 * w - Bn * W[7];
+  G[1] = G[0] * W[1] - Bn * W[5];
+  G[2] = G[0] * W[2] - Bn * W[6];
+  G[3] = G[0] * W[3] - Bn * W[7];
   G[1 + D] += pt;
   G[4] = e * w + pt * vn - Bn * vB;
 #pragma unroll
@@ -376,21 +459,23 @@ __device__ __forceinline__ void side_flux(const real *W, real b2, real igm1, rea
 template <typename real, int D>
 __device__ __forceinline__ void tvdlf_states(real *WL, real *WR, const real *b, const real *c, real gamma,
                                              real igm1, real *F2) {
-  if (!(WL[0] > real(0)) || !(WL[4] > real(0)) || !(WR[0] > real(0)) || !(WR[4] > real(0))) {
+  if (!RT<real>::pos_(WL[0]) || !RT<real>::pos_(WL[4]) || !RT<real>::pos_(WR[0]) || !RT<real>::pos_(WR[4])) {
 #pragma unroll
     for (int v = 0; v < NVAR; v++) {
       WL[v] = b[v];
       WR[v] = c[v];
     }
   }
-  const real b2L = WL[5] * WL[5] + WL[6] * WL[6] + WL[7] * WL[7];
-  const real b2R = WR[5] * WR[5] + WR[6] * WR[6] + WR[7] * WR[7];
-  const real cl = RT<real>::abs_(WL[1 + D]) + fast_speed_pre<real, D>(WL, RT<real>::rcp_(WL[0]), b2L, gamma);
-  const real cr = RT<real>::abs_(WR[1 + D]) + fast_speed_pre<real, D>(WR, RT<real>::rcp_(WR[0]), b2R, gamma);
-  const real cm = cl > cr ? cl : cr;
+  constexpr int T1 = 5 + (D + 1) % 3, T2 = 5 + (D + 2) % 3;   // field across the direction
+  const real tL = WL[T1] * WL[T1] + WL[T2] * WL[T2], tR = WR[T1] * WR[T1] + WR[T2] * WR[T2];
+  const real hbL = real(0.5) * (WL[5 + D] * WL[5 + D] + tL), hbR = real(0.5) * (WR[5 + D] * WR[5 + D] + tR);
+  const real hg = real(0.5) * gamma;
+  const real cl = RT<real>::abs_(WL[1 + D]) + fast_speed_of(RT<real>::rcp_(WL[0]), gamma * WL[4], hg * WL[4], hbL, tL);
+  const real cr = RT<real>::abs_(WR[1 + D]) + fast_speed_of(RT<real>::rcp_(WR[0]), gamma * WR[4], hg * WR[4], hbR, tR);
+  const real cm = RT<real>::max_(cl, cr);
   real GL[NVAR], GR[NVAR];
-  side_flux<real, D>(WL, b2L, igm1, cm, GL);
-  side_flux<real, D>(WR, b2R, igm1, -cm, GR);
+  side_flux<real, D>(WL, hbL, igm1, cm, GL);
+  side_flux<real, D>(WR, hbR, igm1, -cm, GR);
   axpy8<real>(GL, real(1), GR, F2);
   F2[5 + D] = real(0);
 }
@@ -412,33 +497,30 @@ __device__ __forceinline__ void tvdlf_pair(const float *b, const float *c, const
 #pragma unroll
     for (int v = 0; v < NVAR; v++) W[v] = make_float2(b[v], c[v]);
   }
-  const float2 half = make_float2(0.5f, 0.5f);
-  const float2 b2 = __ffma2_rn(W[7], W[7], __ffma2_rn(W[6], W[6], __fmul2_rn(W[5], W[5])));
-  // fast magnetosonic speed along D of both states (fast_speed_pre)
+  const float2 half = make_float2(0.5f, 0.5f), m1 = make_float2(-1.f, -1.f);
+  constexpr int T1 = 5 + (D + 1) % 3, T2 = 5 + (D + 2) % 3;   // field across the direction
+  const float2 bt2 = __ffma2_rn(W[T2], W[T2], __fmul2_rn(W[T1], W[T1]));
+  const float2 hb2 = __fmul2_rn(half, __ffma2_rn(W[5 + D], W[5 + D], bt2));
+  // fast magnetosonic speed along D of both states (fast_speed_of)
   const float2 ir = make_float2(RT<float>::rcp_(W[0].x), RT<float>::rcp_(W[0].y));
-  const float2 a2 = __fmul2_rn(__fmul2_rn(make_float2(gamma, gamma), W[4]), ir);
-  const float2 bt2 = __fmul2_rn(b2, ir);
-  const float2 bn2 = __fmul2_rn(__fmul2_rn(W[5 + D], W[5 + D]), ir);
-  const float2 sum = __fadd2_rn(a2, bt2);
-  float2 disc = __ffma2_rn(sum, sum, __fmul2_rn(__fmul2_rn(make_float2(-4.f, -4.f), a2), bn2));
-  disc.x = fmaxf(disc.x, 0.f);
-  disc.y = fmaxf(disc.y, 0.f);
-  const float2 cf2 =
-      __fmul2_rn(half, __fadd2_rn(sum, make_float2(RT<float>::sqrt_(disc.x), RT<float>::sqrt_(disc.y))));
+  const float2 gp = __fmul2_rn(make_float2(gamma, gamma), __fmul2_rn(W[4], ir));
+  const float2 ga = __fmul2_rn(half, gp), gb = __fmul2_rn(hb2, ir), gd = __ffma2_rn(m1, gb, ga);
+  const float2 disc = __ffma2_rn(gd, gd, __fmul2_rn(gp, __fmul2_rn(bt2, ir)));
+  const float2 cf2 = __fadd2_rn(__fadd2_rn(ga, gb),
+                                make_float2(RT<float>::sqrt_(disc.x), RT<float>::sqrt_(disc.y)));
   const float cm = fmaxf(fabsf(W[1 + D].x) + RT<float>::sqrt_(cf2.x), fabsf(W[1 + D].y) + RT<float>::sqrt_(cf2.y));
   // per-side flux with w = v_n + c_max on the left, v_n - c_max on the right
-  const float2 vn = W[1 + D], nBn = __fmul2_rn(W[5 + D], make_float2(-1.f, -1.f));
+  const float2 vn = W[1 + D], nBn = __fmul2_rn(W[5 + D], m1);
   const float2 w = __fadd2_rn(vn, make_float2(cm, -cm));
-  const float2 m1 = __fmul2_rn(W[0], W[1]), m2 = __fmul2_rn(W[0], W[2]), m3 = __fmul2_rn(W[0], W[3]);
-  const float2 rv2 = __ffma2_rn(m3, W[3], __ffma2_rn(m2, W[2], __fmul2_rn(m1, W[1])));
-  const float2 pt = __ffma2_rn(half, b2, W[4]);
-  const float2 en = __ffma2_rn(W[4], make_float2(igm1, igm1), __fmul2_rn(half, __fadd2_rn(rv2, b2)));
+  const float2 v2 = __ffma2_rn(W[3], W[3], __ffma2_rn(W[2], W[2], __fmul2_rn(W[1], W[1])));
+  const float2 pt = __fadd2_rn(hb2, W[4]);
+  const float2 en = __ffma2_rn(W[4], make_float2(igm1, igm1), __ffma2_rn(__fmul2_rn(half, W[0]), v2, hb2));
   const float2 vB = __ffma2_rn(W[3], W[7], __ffma2_rn(W[2], W[6], __fmul2_rn(W[1], W[5])));
   float2 G[NVAR];
   G[0] = __fmul2_rn(W[0], w);
-  G[1] = __ffma2_rn(m1, w, __fmul2_rn(nBn, W[5]));
-  G[2] = __ffma2_rn(m2, w, __fmul2_rn(nBn, W[6]));
-  G[3] = __ffma2_rn(m3, w, __fmul2_rn(nBn, W[7]));
+  G[1] = __ffma2_rn(G[0], W[1], __fmul2_rn(nBn, W[5]));
+  G[2] = __ffma2_rn(G[0], W[2], __fmul2_rn(nBn, W[6]));
+  G[3] = __ffma2_rn(G[0], W[3], __fmul2_rn(nBn, W[7]));
   G[1 + D] = __fadd2_rn(G[1 + D], pt);
   G[4] = __ffma2_rn(en, w, __ffma2_rn(pt, vn, __fmul2_rn(nBn, vB)));
 #pragma unroll
@@ -462,7 +544,8 @@ __device__ __forceinline__ void tvdlf_face(const real *a, const real *b, const r
       const float2 d1 = __fadd2_rn(B, make_float2(-a[v], -a[v + 1]));
       const float2 d2 = __fadd2_rn(C, make_float2(-B.x, -B.y));
       const float2 d3 = __fadd2_rn(make_float2(e[v], e[v + 1]), make_float2(-C.x, -C.y));
-      const float2 s1 = __fadd2_rn(d1, d2), s2 = __fadd2_rn(d2, d3);
+      const float2 quarter = make_float2(0.25f, 0.25f);
+      const float2 s1 = __fmul2_rn(quarter, __fadd2_rn(d1, d2)), s2 = __fmul2_rn(quarter, __fadd2_rn(d2, d3));
       hb[v] = half_mc_signed(d1.x, d2.x, s1.x);
       hb[v + 1] = half_mc_signed(d1.y, d2.y, s1.y);
       hc[v] = half_mc_signed(d2.x, d3.x, s2.x);
@@ -502,7 +585,7 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 template <typename real>
 __device__ __forceinline__ int apply_floors(real *u, real gamma, real pfloor, real rfloor, Isl isl) {
   int hits = 0;
-  if (u[0] < rfloor) {
+  if (RT<real>::less_(u[0], rfloor)) {
     u[0] = rfloor;
     hits++;
   }
@@ -512,7 +595,7 @@ __device__ __forceinline__ int apply_floors(real *u, real gamma, real pfloor, re
   const real margin = sizeof(real) == 4 ? real(1e-6) : real(0);
   if (pq > pfloor + margin * RT<real>::abs_(u[4])) return hits;
   real p = pressure_of<real>(u, gamma, isl);
-  if (p < pfloor) {
+  if (RT<real>::less_(p, pfloor)) {
     real ke = real(0.5) * (u[1] * u[1] + u[2] * u[2] + u[3] * u[3]) / u[0];
     real me = real(0.5) * (u[5] * u[5] + u[6] * u[6] + u[7] * u[7]);
     u[4] = pfloor / (gamma - real(1)) + ke + me;
