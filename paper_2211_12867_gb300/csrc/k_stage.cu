@@ -124,9 +124,23 @@ constexpr int stage_min_ctas(int real_bytes, int tj, int tk) {
                                         (int)(233472 / (StageSmem<float>::bytes(tj, tk) + 1024))));
 }
 
+// The scheme's constants in the working precision.  Converted on the host:
+// conversions from the double parameters in the kernel are FP64-pipe
+// instructions, which the compiler repeats per cell to save registers (13 per
+// cell and 38 % of that pipe's time in the FP32 corrector).
+template <typename real>
+struct StageConst {
+  real gamma, igm1, p_floor, rho_floor, omega, cd;
+  Isl isl;
+  explicit StageConst(const KParams &kp)
+      : gamma((real)kp.gamma), igm1(real(1) / (gamma - real(1))), p_floor((real)kp.p_floor),
+        rho_floor((real)kp.rho_floor), omega((real)kp.omega), cd((real)kp.cd),
+        isl{(float)kp.isl_pe, (float)kp.isl_beta} {}
+};
+
 template <typename real, int TJ, int TK, bool S2>
 __global__ void __launch_bounds__(stage_threads(TJ, TK), stage_min_ctas(sizeof(real), TJ, TK))
-    k_stage(const KParams kp, const StageLaunch sl) {
+    k_stage(const KParams kp, const StageLaunch sl, const StageConst<real> sc_) {
   constexpr int NT = stage_threads(TJ, TK), RJ = TJ + 4, RK = TK + 4, RP = RJ * RK;
   constexpr int DJ = TJ + 2, DK = TK + 2, DP = DJ * DK;
   constexpr int NTH = (TJ + 1) * TK, NPH = TJ * (TK + 1);   // theta / phi faces of a plane
@@ -156,24 +170,32 @@ __global__ void __launch_bounds__(stage_threads(TJ, TK), stage_min_ctas(sizeof(r
   const bool trc = kp.nvs > NVAR;
 
   const int tid = threadIdx.x, jl = tid / TK, kl = tid % TK;
-  const real gamma = (real)kp.gamma, pfl = (real)kp.p_floor, rfl = (real)kp.rho_floor;
+  const real gamma = sc_.gamma, pfl = sc_.p_floor, rfl = sc_.rho_floor;
   const int nb0 = kp.nb[0], nb1 = kp.nb[1], nb2 = kp.nb[2];
   const int P1 = kp.P[1], P2 = kp.P[2];
   const size_t plane = (size_t)P1 * P2, vstride = (size_t)kp.P[0] * plane, bstride = kp.nvs * vstride;
   const int per_block = sl.tiles_j * sl.tiles_k * sl.segs;
   const int nwork = sl.nlist * per_block;
   const bool spherical = kp.geometry == 0;
-  const real Om = (real)kp.omega, Cd = (real)kp.cd;
-  const Isl isl{(float)kp.isl_pe, (float)kp.isl_beta};
-  const real igm1 = real(1) / (gamma - real(1));
-  const int o = (jl + 2) * RK + kl + 2;          // ring cell of the thread's own cell
-  // extra faces of the tile's far edges: the last warps take one more theta
-  // face (row TJ) or phi face (column TK) per thread
-  constexpr int XT = (TK + 31) / 32 * 32;
-  static_assert(XT + TJ <= NT, "one extra face per thread");
-  const int xe = NT - 1 - tid;
-  const bool x_th = xe < TK, x_ph = xe >= XT && xe < XT + TJ;
-  const int xq = x_th ? xe : xe - XT;
+  const real Om = sc_.omega, Cd = sc_.cd, igm1 = sc_.igm1;
+  const Isl isl = sc_.isl;
+  // ring cell of the thread's own cell (a thread without one: cell (2, 2))
+  const int o = tid < TJ * TK ? (jl + 2) * RK + kl + 2 : 2 * RK + 2;
+  // extra faces of the tile's far edges: TK theta faces (row TJ), then TJ phi
+  // faces (column TK), one per thread of the first warps, which convert fewer
+  // cells
+  static_assert(TK + TJ <= NT, "one extra face per thread");
+  const bool x_th = tid < TK;
+  const int xq = x_th ? tid : tid - TK;
+  const int xo = x_th ? (TJ + 2) * RK + xq + 2 : (xq + 2) * RK + TK + 2;
+  // exchanges the theta and phi components
+  auto turn = [](real *x, bool on) {
+    const real v = x[2], b = x[6];
+    x[2] = on ? x[3] : v;
+    x[3] = on ? v : x[3];
+    x[6] = on ? x[7] : b;
+    x[7] = on ? b : x[7];
+  };
 
   // reflux face buffer layout (per slot): faces in order r-lo, r-hi, th-lo,
   // th-hi, ph-lo, ph-hi; each [v][t1][t2]
@@ -209,6 +231,9 @@ __global__ void __launch_bounds__(stage_threads(TJ, TK), stage_min_ctas(sizeof(r
     real *Uout = reinterpret_cast<real *>(sl.Uout) + (size_t)slot * bstride;
     const bool own = tid < TJ * TK, valid = own && jl < nvj && kl < nvk;
     const int j = j0 + jl, k = k0 + kl;           // interior indices in the block
+    const bool has_th = own && jl <= nvj && kl < nvk, has_ph = own && jl < nvj && kl <= nvk;
+    const bool any_face = __any_sync(0xffffffffu, has_th || has_ph);
+    const bool x_face = x_th ? nvj == TJ && xq < nvk : tid < TK + TJ && nvk == TK && xq < nvj;
     // block faces with a finer, and with a coarser or finer, neighbour; those
     // the thread's column touches
     unsigned fin = 0, cfb = 0, edge = 0;
@@ -433,35 +458,41 @@ __global__ void __launch_bounds__(stage_threads(TJ, TK), stage_min_ctas(sizeof(r
     for (int i = ib; i < ie; i++) {
       real *fthb = fth + (i & 1) * NVAR * NTH, *fphb = fph + (i & 1) * NVAR * NPH;
       {
-        // the lower theta and phi face of the thread's cell, then an extra one
+        // The lower theta and phi face of the thread's cell, in one straight
+        // run (a thread without one of the two computes on whatever its ring
+        // cells hold and stores nothing), then the extra face.
         const real *pl = ring + oc;
-        int to = own && jl <= nvj && kl < nvk ? o : -1, po = own && jl < nvj && kl <= nvk ? o : -1;
-        int ts = tid, ps = tid + jl;
-#pragma unroll 1
-        for (int rep = 0;; rep++) {
-          if (to >= 0) {
-            real a[NVAR], b[NVAR], c[NVAR], e[NVAR], F[NVAR];
-            ld8<real, RP>(pl, to - 2 * RK, a);
-            ld8<real, RP>(pl, to - RK, b);
-            ld8<real, RP>(pl, to, c);
-            ld8<real, RP>(pl, to + RK, e);
-            tvdlf_face<real, 1>(a, b, c, e, gamma, igm1, F);
-            st8<real, NTH>(fthb, ts, F);
-          }
-          if (po >= 0) {
-            real a[NVAR], b[NVAR], c[NVAR], e[NVAR], F[NVAR];
-            ld8<real, RP>(pl, po - 2, a);
-            ld8<real, RP>(pl, po - 1, b);
-            ld8<real, RP>(pl, po, c);
-            ld8<real, RP>(pl, po + 1, e);
-            tvdlf_face<real, 2>(a, b, c, e, gamma, igm1, F);
-            st8<real, NPH>(fphb, ps, F);
-          }
-          if (rep || !(x_th || x_ph)) break;
-          to = x_th && nvj == TJ && xq < nvk ? (TJ + 2) * RK + xq + 2 : -1;
-          po = x_ph && nvk == TK && xq < nvj ? (xq + 2) * RK + TK + 2 : -1;
-          ts = TJ * TK + xq;
-          ps = xq * (TK + 1) + TK;
+        if (any_face) {
+          real a[NVAR], b[NVAR], c[NVAR], e[NVAR], F[NVAR];
+          ld8<real, RP>(pl, o - 2 * RK, a);
+          ld8<real, RP>(pl, o - RK, b);
+          ld8<real, RP>(pl, o, c);
+          ld8<real, RP>(pl, o + RK, e);
+          tvdlf_face<real, 1>(a, b, c, e, gamma, igm1, F);
+          if (has_th) st8<real, NTH>(fthb, tid, F);
+          ld8<real, RP>(pl, o - 2, a);
+          ld8<real, RP>(pl, o - 1, b);
+          ld8<real, RP>(pl, o + 1, e);
+          tvdlf_face<real, 2>(a, b, c, e, gamma, igm1, F);
+          if (has_ph) st8<real, NPH>(fphb, tid + jl, F);
+        }
+        if (x_face) {
+          // theta and phi faces in the lanes of one warp: a phi face is a theta
+          // face with the theta and phi components exchanged
+          real a[NVAR], b[NVAR], c[NVAR], e[NVAR], F[NVAR];
+          const int d = x_th ? RK : 1;
+          ld8<real, RP>(pl, xo - 2 * d, a);
+          ld8<real, RP>(pl, xo - d, b);
+          ld8<real, RP>(pl, xo, c);
+          ld8<real, RP>(pl, xo + d, e);
+          turn(a, !x_th);
+          turn(b, !x_th);
+          turn(c, !x_th);
+          turn(e, !x_th);
+          tvdlf_face<real, 1>(a, b, c, e, gamma, igm1, F);
+          turn(F, !x_th);
+          if (x_th) st8<real, NTH>(fthb, TJ * TK + xq, F);
+          else st8<real, NPH>(fphb, xq * (TK + 1) + TK, F);
         }
       }
       if (S2) divb_plane(i + 1, oc, o1, o2);
@@ -671,9 +702,9 @@ int launch_t(const KParams &kp, const StageLaunch &sl, cudaStream_t s) {
   const size_t smem = StageSmem<real>::bytes(TJ, TK, kp.nvs > NVAR);
   ensure_smem<real, TJ, TK>(smem);
   if (sl.stage2)
-    k_stage<real, TJ, TK, true><<<sl.grid, stage_threads(TJ, TK), smem, s>>>(kp, sl);
+    k_stage<real, TJ, TK, true><<<sl.grid, stage_threads(TJ, TK), smem, s>>>(kp, sl, StageConst<real>(kp));
   else
-    k_stage<real, TJ, TK, false><<<sl.grid, stage_threads(TJ, TK), smem, s>>>(kp, sl);
+    k_stage<real, TJ, TK, false><<<sl.grid, stage_threads(TJ, TK), smem, s>>>(kp, sl, StageConst<real>(kp));
   return cudaPeekAtLastError() == cudaSuccess ? 0 : -1;
 }
 

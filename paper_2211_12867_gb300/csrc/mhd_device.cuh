@@ -48,8 +48,11 @@ template <> struct RT<double> {
   static __device__ __forceinline__ bool pos_(double x) {
     return (unsigned long long)(__double_as_longlong(x) - 1) < 0x7ff0000000000000ull;
   }
+  // (magnitudes from the high words: a mask over all 64 bits is compiled to a
+  // floating-point absolute value, which is an FP64-pipe addition)
   static __device__ __forceinline__ bool nan_(double x) {
-    return (unsigned long long)(__double_as_longlong(x) & 0x7fffffffffffffffll) > 0x7ff0000000000000ull;
+    const unsigned h = (unsigned)__double2hiint(x) << 1;
+    return h > 0xffe00000u || (h == 0xffe00000u && __double2loint(x) != 0);
   }
   // a < b; not for NaN (-0 counts as below +0)
   static __device__ __forceinline__ bool less_(double a, double b) {
@@ -274,20 +277,23 @@ __device__ __forceinline__ real mc_half_slope(real um, real u0, real up) {
   return dm * dp > real(0) ? lim : real(0);
 }
 
+__device__ __forceinline__ long long hilo(int hi, int lo) {
+  return (long long)((unsigned long long)(unsigned)hi << 32 | (unsigned)lo);
+}
 // FP64: the minimum and the signs by bit patterns, the quarter by the exponent
 // (three FP64-pipe instructions, the differences, instead of nine)
 template <>
 __device__ __forceinline__ double mc_half_slope<double>(double um, double u0, double up) {
   const double dm = u0 - um, dp = up - u0, s = dm + dp;
-  const long long m = 0x7fffffffffffffffll;
-  const long long a = __double_as_longlong(dm), b = __double_as_longlong(dp);
-  long long q = __double_as_longlong(s) & m;
-  q = q < 0x0030000000000000ll ? 0 : q - 0x0020000000000000ll;   // |s| / 4
-  const long long x = a & m, y = b & m;
+  // magnitudes (see nan_ for the high words)
+  const int ha = __double2hiint(dm), hb = __double2hiint(dp);
+  const int qa = __double2hiint(s) & 0x7fffffff;
+  const long long x = hilo(ha & 0x7fffffff, __double2loint(dm)), y = hilo(hb & 0x7fffffff, __double2loint(dp));
+  const long long q = qa < 0x00300000 ? 0 : hilo(qa - 0x00200000, __double2loint(s));   // |s| / 4
   long long lim = x < y ? x : y;
   lim = q < lim ? q : lim;
-  lim |= a & ~m;
-  return __longlong_as_double((a ^ b) < 0 ? 0 : lim);
+  const int hl = (int)(lim >> 32) | (ha & 0x80000000);
+  return (ha ^ hb) < 0 ? 0.0 : __hiloint2double(hl, (int)lim);
 }
 
 template <typename real>
@@ -491,12 +497,11 @@ template <int D>
 __device__ __forceinline__ void tvdlf_pair(const float *b, const float *c, const float *hb, const float *hc,
                                            float gamma, float igm1, float *F2) {
   float2 W[NVAR];
+  // the fallback multiplies the half slopes by zero: no branch
+  const float m = fminf(fminf(b[0] + hb[0], c[0] - hc[0]), fminf(b[4] + hb[4], c[4] - hc[4]));
+  const float on = m > 0.f ? 1.f : 0.f;
 #pragma unroll
-  for (int v = 0; v < NVAR; v++) W[v] = make_float2(b[v] + hb[v], c[v] - hc[v]);
-  if (!(W[0].x > 0.f) || !(W[4].x > 0.f) || !(W[0].y > 0.f) || !(W[4].y > 0.f)) {
-#pragma unroll
-    for (int v = 0; v < NVAR; v++) W[v] = make_float2(b[v], c[v]);
-  }
+  for (int v = 0; v < NVAR; v++) W[v] = make_float2(fmaf(hb[v], on, b[v]), fmaf(-hc[v], on, c[v]));
   const float2 half = make_float2(0.5f, 0.5f), m1 = make_float2(-1.f, -1.f);
   constexpr int T1 = 5 + (D + 1) % 3, T2 = 5 + (D + 2) % 3;   // field across the direction
   const float2 bt2 = __ffma2_rn(W[T2], W[T2], __fmul2_rn(W[T1], W[T1]));
