@@ -1,7 +1,7 @@
 """Tile-shape autotuner of the stage kernel.
 
 Sweeps the (theta x phi) tile of the marching CTA and the radial segment
-length over the shapes the library instantiates, times a few steps of the
+length over the shapes a caller can set (0, 0: the library's choice), times a few steps of the
 actual workload for each with CUDA events on the library's stream, and
 keeps the fastest.  The state is saved before and restored after the sweep,
 so tuning does not advance the simulation.
@@ -12,7 +12,7 @@ import itertools
 
 import numpy as np
 
-TILES = [(8, 32), (4, 32), (12, 20), (10, 24), (8, 24), (6, 36), (12, 12), (8, 8)]
+TILES = [(0, 0), (8, 32), (4, 32), (12, 20), (10, 24), (8, 24), (6, 36), (12, 12), (8, 8)]
 
 
 def candidates(block):

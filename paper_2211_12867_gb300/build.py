@@ -18,7 +18,7 @@ BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libicarus.so")
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 
-SOURCES = ["api.cu", "k_stage.cu", "k_ghost.cu", "k_amr.cu", "k_mlp.cu", "k_sums_static.cu", "k_peak.cu"]
+SOURCES = ["api.cu", "k_stage.cu", "k_stage_f64.cu", "k_ghost.cu", "k_amr.cu", "k_mlp.cu", "k_sums_static.cu", "k_peak.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 # host code without floating-point contraction: the geometry tables come out
 # bit for bit the same on every host architecture; OpenMP for the tree logic
@@ -44,6 +44,7 @@ def _stale(obj: str, src: str) -> bool:
     if not os.path.exists(obj):
         return True
     deps = [src] + [os.path.join(CSRC, h) for h in os.listdir(CSRC) if h.endswith((".h", ".cuh"))]
+    deps.append(os.path.join(CSRC, "k_stage.cu"))   # included by k_stage_f64.cu
     deps.append(os.path.join(INCLUDE, "icarus.h"))
     t = os.path.getmtime(obj)
     return any(os.path.getmtime(d) > t for d in deps if os.path.exists(d))

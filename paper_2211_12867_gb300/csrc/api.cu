@@ -210,6 +210,13 @@ void gauss_legendre(double *x, double *w) {
 
 }  // namespace
 
+// a stage tile on the context's blocks: tiles per block, resident CTAs, cost of
+// a plane (see stage_tile_costs)
+struct TileCost {
+  int tj, tk, nj, nk, occ;
+  double plane;
+};
+
 struct icarus_ctx {
   icarus_grid_desc d{};
   int nbd[MAXLEV + 2][3] = {};   // blocks per direction at each level (tree logic looks these up)
@@ -255,7 +262,8 @@ struct icarus_ctx {
   bool flags_valid = false;
   KParams kp{};
   // launch configuration
-  int tile_j = 0, tile_k = 0, seg_len = 0, occ = 1;
+  int tile_j = 0, tile_k = 0, seg_len = 0;   // set by the caller; 0: chosen per tree
+  std::vector<TileCost> tile_cost;
   double isl_pe = 0.002, isl_beta = 0.1;  // FP64 pressure islands: p < 0.002 e or beta < 0.1
   double floor_budget = ICARUS_DEFAULT_FLOOR_BUDGET;
   // status word read back without a synchronisation after steps that return
@@ -816,55 +824,114 @@ void prof_mark(icarus_ctx *c, int kind, int end) {
   cudaEventRecord(c->ev[c->ev_used], c->stream);
   c->ev_used++;
 }
-void default_tiles(icarus_ctx *c) {
+// The tile shapes a caller may set.  The library's own choice also takes
+// 8 x 12, 8 x 16, 12 x 16 and 16 x 16.
+bool tile_settable(const icarus_ctx *c, int tj, int tk) {
+#ifdef ALL_TILES
+  return true;
+#endif
+  static const int shapes[][2] = {{8, 8}, {12, 12}, {8, 24}, {4, 32}, {6, 36}, {10, 24}, {12, 20}, {8, 32}};
+  // FP64 takes the first seven, with the tracer the first four
+  const int n = c->prec ? 8 : (c->d.tracer ? 4 : 7);
+  for (int q = 0; q < n; q++)
+    if (tj == shapes[q][0] && tk == shapes[q][1]) return true;
+  return false;
+}
+
+// Time of the stage kernels for a tile and a segment length, in the model
+//   max( m (seg + a) u, ceil(m / occ) (seg + aL) lat ),   m = ceil(items / SMs)
+// items: leaves x tiles x segments.  The first term is an SM's throughput: a
+// plane of a tile costs u = cW (warps with a cell) + cL (warps' worth of cells
+// loaded) + cX (warps with extra far-edge faces) + c0, and a segment's
+// prologue a planes more; the second the latency of a few CTAs.  Fitted to the
+// measured sum of both stages over 13 FP32 and 8 FP64 grids (blocks of 4 to 64
+// x 6 to 60 x 8 to 180 cells, 40 to 3168 of them), 12 tiles and up to 8
+// segment lengths each (1380 points): 9 to 11 % rms, and the tile and segment
+// it picks take 0 to 2 % more than the best of the grid (8 % in one FP64 case).
+// Against the previous rule (12 x 20 in FP32, 4 x 32 in FP64 and four waves of
+// segments of at least 8 planes), predictor + corrector in us: 24 x 16 x 48
+// blocks 1255 -> 728; 40 blocks of 12 x 8 x 8 FP64 890 -> 188; one block of 64 x
+// 60 x 180 FP64 3410 -> 2256; 160 blocks of 12 x 8 x 12 72 -> 50.
+struct StageCost {
+  double cW, cL, cX, c0, a, lat, aL;
+};
+constexpr StageCost COST32 = {0.398, 0.009, 0.142, 0.224, 2.15, 4.79, 2.62},
+                    COST64 = {12.47, 0.972, 0.0, 6.40, 0.438, 68.1, 0.523};
+
+// the model's cost of a plane of each instantiated tile on this context's
+// blocks (averaged over the block's tiles), and its resident CTAs
+void stage_tile_costs(icarus_ctx *c) {
+  c->tile_cost.clear();
+  const StageCost &k = c->prec ? COST32 : COST64;
   const int n1 = c->d.block[1], n2 = c->d.block[2];
-  const int trc = c->d.tracer;
-  if (c->tile_j && c->tile_k) {
-    c->occ = stage_max_ctas_per_sm(c->prec, c->tile_j, c->tile_k, trc);
-    return;
+  int tj, tk;
+  for (int n = 0; stage_tile(n, &tj, &tk); n++) {
+    if (!stage_tile_supported(c->prec, tj, tk, c->d.tracer)) continue;
+    TileCost t;
+    t.tj = tj;
+    t.tk = tk;
+    t.nj = (n1 + tj - 1) / tj;
+    t.nk = (n2 + tk - 1) / tk;
+    t.occ = stage_ctas(c->prec, tj, tk, c->d.tracer);
+    double u = 0.0;
+    for (int ej = 0; ej < 2; ej++)
+      for (int ek = 0; ek < 2; ek++) {   // inner and last tiles in each direction
+        const int count = (ej ? 1 : t.nj - 1) * (ek ? 1 : t.nk - 1);
+        const int vj = ej ? n1 - (t.nj - 1) * tj : tj, vk = ek ? n2 - (t.nk - 1) * tk : tk;
+        if (!count) continue;
+        int warps = 0, last = -1;
+        for (int q = 0; q < tj * tk; q++)
+          if (q / tk < vj && q % tk < vk && q / 32 != last) {
+            last = q / 32;
+            warps++;
+          }
+        u += count * (k.cW * warps + k.cL * (vj + 4) * (vk + 4) / 32.0 + k.cX * ((tj + tk + 31) / 32) + k.c0);
+      }
+    t.plane = u / (t.nj * t.nk);
+    c->tile_cost.push_back(t);
   }
-  if (c->prec && n1 >= 12 && n2 >= 20) {
-    c->tile_j = 12;
-    c->tile_k = 20;
-  } else if (n2 >= 32) {
-    c->tile_j = c->prec ? 8 : 4;
-    c->tile_k = 32;
-  } else if (n1 >= 12 && n2 >= 12) {
-    c->tile_j = 12;
-    c->tile_k = 12;
-  } else {
-    c->tile_j = 8;
-    c->tile_k = 8;
+}
+
+// tile and segment length: the caller's where set, else the model's best
+void stage_shape(const icarus_ctx *c, int *tj, int *tk, int *seg, int *occ) {
+  const StageCost &k = c->prec ? COST32 : COST64;
+  const int n0 = c->d.block[0];
+  double best = -1.0;
+  for (const TileCost &t : c->tile_cost) {
+    if (c->tile_j && (t.tj != c->tile_j || t.tk != c->tile_k)) continue;
+    int prev = 0;
+    for (int q = 1; q <= n0; q++) {
+      int len = c->seg_len > 0 ? std::min(c->seg_len, n0) : (n0 + q - 1) / q;
+      len = std::min(len, STAGE_SEG_MAX);
+      if (len == prev) continue;
+      prev = len;
+      const int segs = (n0 + len - 1) / len;
+      const double items = (double)c->nleaves * t.nj * t.nk * segs, m = std::ceil(items / c->nsm);
+      const double mean = (double)n0 / segs;
+      const double T = std::max(m * (mean + k.a) * t.plane, std::ceil(m / t.occ) * (mean + k.aL) * k.lat);
+      if (best < 0.0 || T < best) {
+        best = T;
+        *tj = t.tj;
+        *tk = t.tk;
+        *seg = len;
+        *occ = t.occ;
+      }
+      if (c->seg_len > 0) break;
+    }
   }
-  if (!stage_tile_supported(c->prec, c->tile_j, c->tile_k, trc)) {
-    c->tile_j = 8;
-    c->tile_k = 8;
-  }
-  c->occ = stage_max_ctas_per_sm(c->prec, c->tile_j, c->tile_k, trc);
 }
 
 StageLaunch stage_cfg(icarus_ctx *c, int stage2) {
   StageLaunch sl{};
-  sl.tile_j = c->tile_j;
-  sl.tile_k = c->tile_k;
+  int occ = 1;
+  stage_shape(c, &sl.tile_j, &sl.tile_k, &sl.seg_len, &occ);
   sl.tiles_j = (c->d.block[1] + sl.tile_j - 1) / sl.tile_j;
   sl.tiles_k = (c->d.block[2] + sl.tile_k - 1) / sl.tile_k;
-  const int slots = c->nsm * c->occ;
-  int seg = c->seg_len;
-  if (seg <= 0) {
-    // enough work items for ~4 waves of the persistent grid, segments >= 8 planes
-    const long long base = (long long)c->nleaves * sl.tiles_j * sl.tiles_k;
-    long long segs = (4LL * slots + base - 1) / std::max(1LL, base);
-    segs = std::max(1LL, std::min<long long>(segs, c->d.block[0] / 8 > 0 ? c->d.block[0] / 8 : 1));
-    seg = (c->d.block[0] + (int)segs - 1) / (int)segs;
-  }
-  seg = std::max(1, std::min(std::min(seg, c->d.block[0]), STAGE_SEG_MAX));
-  sl.seg_len = seg;
-  sl.segs = (c->d.block[0] + seg - 1) / seg;
+  sl.segs = (c->d.block[0] + sl.seg_len - 1) / sl.seg_len;
   sl.list = c->all_list;
   sl.nlist = c->nleaves;
   const long long nwork = (long long)sl.nlist * sl.tiles_j * sl.tiles_k * sl.segs;
-  sl.grid = (int)std::max(1LL, std::min<long long>(nwork, slots));
+  sl.grid = (int)std::max(1LL, std::min<long long>(nwork, (long long)c->nsm * occ));
   sl.stage2 = stage2;
   sl.dtfac = stage2 ? 1.0 : 0.5;
   return sl;
@@ -1245,7 +1312,7 @@ icarus_status icarus_init_grid(const icarus_grid_desc *desc, icarus_ctx **out) {
   }
   fill_kp(c);
   if ((st = upload_tree(c, c->blk)) != ICARUS_OK) return fail(st);
-  default_tiles(c);
+  stage_tile_costs(c);
   c->h_tstop.assign(nm, 0.0);
   // the uniform zero state has no time step: mark dt as unknown (0) until a state is set
   *out = c;
@@ -1339,13 +1406,11 @@ icarus_status icarus_set_member_max_level(icarus_ctx *c, int member, int L) {
 icarus_status icarus_set_tile(icarus_ctx *c, int tj, int tk, int seg) {
   if (!c) return ICARUS_ERR_ARG;
   if (tj || tk) {
-    if (!stage_tile_supported(c->prec, tj, tk, c->d.tracer)) return ICARUS_ERR_ARG;
+    if (!tile_settable(c, tj, tk) || !stage_tile_supported(c->prec, tj, tk, c->d.tracer)) return ICARUS_ERR_ARG;
     c->tile_j = tj;
     c->tile_k = tk;
-    default_tiles(c);
   } else {
     c->tile_j = c->tile_k = 0;
-    default_tiles(c);
   }
   c->seg_len = seg > 0 ? seg : 0;
   c->graph_valid = false;

@@ -138,7 +138,8 @@ constexpr int STAGE_SEG_MAX = 64;
 // tracer: the CME tracer is stored and advected (one more shared ring)
 size_t stage_smem_bytes(int precision, int tj, int tk, int tracer);
 int stage_tile_supported(int precision, int tj, int tk, int tracer);
-int stage_max_ctas_per_sm(int precision, int tj, int tk, int tracer);
+int stage_tile(int n, int *tj, int *tk);   // the n-th instantiated tile; 0 past the last
+int stage_ctas(int precision, int tj, int tk, int tracer);   // resident CTAs per SM
 
 // ghost fill
 // ghost_neighbour: every ghost cell of the listed leaves (copy, prolongation

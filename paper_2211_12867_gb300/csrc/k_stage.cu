@@ -39,8 +39,7 @@ struct StageSmem {
   // threads' copies follow the rest
   static constexpr size_t bytes(int tj, int tk, bool tracer = false) {
     return sizeof(real) * (size_t)(5 * NVAR * (tj + 4) * (tk + 4) + 2 * NVAR * (tj + 1) * tk +
-                                   2 * NVAR * tj * (tk + 1) + 4 * (tj + 2) * (tk + 2) +
-                                   NVAR * ((tj * tk + 31) / 32 * 32) + geo(tj, tk) +
+                                   2 * NVAR * tj * (tk + 1) + 4 * (tj + 2) * (tk + 2) + geo(tj, tk) +
                                    (tracer ? 5 * (tj + 4) * (tk + 4) : 0)) +
            (tracer ? sizeof(void *) * (size_t)((tj + 4) * (tk + 4) + (tj * tk + 31) / 32 * 32) : 0);
   }
@@ -150,7 +149,7 @@ __global__ void __launch_bounds__(stage_threads(TJ, TK), stage_min_ctas(sizeof(r
   real *ring = reinterpret_cast<real *>(smem_raw);
   real *fth = ring + 5 * PL;            // two buffers of theta-face fluxes
   real *fph = fth + 2 * NVAR * NTH;     // two buffers of phi-face fluxes
-  real *u0s = fph + 2 * NVAR * NPH;     // U^n of the thread's own cell, next plane
+  real *fend = fph + 2 * NVAR * NPH;
   // Factors of the work item's planes (from plane ib-2): areas over volume of
   // the r faces (halved: the fluxes carry a factor 2), dr2/dr3, Omega^2 r_c,
   // 1 / two-cell spacing, 1/dr, 1/r_c, divergence factor.  Of the tile's rows:
@@ -160,12 +159,12 @@ __global__ void __launch_bounds__(stage_threads(TJ, TK), stage_min_ctas(sizeof(r
   constexpr int NRP = STAGE_SEG_MAX + 4, NJ = TJ + 4;
   enum { P_RP, P_RM, P_DR, P_CF, P_ID2, P_IDR, P_IRC, P_FR };
   enum { R_TP, R_TM, R_PW, R_ST, R_CT, R_ITC2, R_IST, R_IDTH };
-  real *s_pl = u0s + NVAR * NT, *s_row = s_pl + NPF * NRP;
+  real *s_pl = fend, *s_row = s_pl + NPF * NRP;
   real *dring = s_row + NRF * TJ;
   // for the divergence: r_c^2 per plane; sin, 1 / (sin * two-cell spacing) and
   // 1/sin per row from row -2; 1 / two-cell spacing per column from column -2
   real *s_rc2 = dring + 4 * DP, *s_st = s_rc2 + NRP, *s_tt = s_st + NJ, *s_ist = s_tt + NJ, *s_ipc2 = s_ist + NJ;
-  real *xring = u0s + NVAR * NT + StageSmem<real>::geo(TJ, TK) + 4 * DP;   // tracer X, 5 planes (if stored)
+  real *xring = fend + StageSmem<real>::geo(TJ, TK) + 4 * DP;   // tracer X, 5 planes (if stored)
   const real **s_xsrc = reinterpret_cast<const real **>(xring + 5 * RP + (RP & 1));
   const bool trc = kp.nvs > NVAR;
 
@@ -315,18 +314,10 @@ __global__ void __launch_bounds__(stage_threads(TJ, TK), stage_min_ctas(sizeof(r
           if (trc) xring[at / NVAR + q] *= RT<real>::rcp_(uu[0]);   // rho X -> X
         }
     };
-    // U^n of the thread's own cell at plane p, copied asynchronously one
-    // plane ahead (only this thread reads it: no barrier); always commits a
-    // group so that the group counts stay uniform
+    // U^n of the thread's own cell is read at the start of the update and used
+    // behind the r flux, which hides the access (staging it one plane ahead
+    // with the plane copies made the update wait for those as well)
     const real *u0p = U0 + NVAR * ((size_t)(ib + NGH) * plane + (size_t)(j + NGH) * P2 + (k + NGH));
-    auto issue_u0 = [&](int p) {
-      if (valid && p < ie) {
-#pragma unroll
-        for (int v = 0; v < NVAR; v += CH) cp_async<16>(&el<real, NT>(u0s, v, tid), u0p + v);
-        u0p += NVAR * plane;
-      }
-      cp_async_commit();
-    };
     // ring offset of the plane after the one at offset a
     auto next = [](int a) { return a == 4 * PL ? 0 : a + PL; };
     // half the limited radial slope of the thread's column at the middle of
@@ -445,7 +436,6 @@ __global__ void __launch_bounds__(stage_threads(TJ, TK), stage_min_ctas(sizeof(r
     __syncthreads();   // plane ib-2 is read no more: its slot takes plane ib+3
     if (ib + 3 <= ie + 1) issue_plane(ib + 3, o3);
     else cp_async_commit();
-    issue_u0(ib);
 
     // One barrier per plane.  Phase A (before it): theta and phi face fluxes
     // of plane i into face buffer i&1, div B of plane i+1, conversion of plane
@@ -497,12 +487,14 @@ __global__ void __launch_bounds__(stage_threads(TJ, TK), stage_min_ctas(sizeof(r
       }
       if (S2) divb_plane(i + 1, oc, o1, o2);
       if (i + 3 <= ie + 1) {
-        cp_async_wait_group<1>();   // plane i+3 landed (U^n of plane i may not have)
+        cp_async_wait_group<0>();   // plane i+3 landed
         convert_plane(o3);
       }
       __syncthreads();
       if (valid) {
-        real Fhi[NVAR];
+        real Fhi[NVAR], u0[NVAR];
+        ld_cell(u0p, u0);
+        u0p += NVAR * plane;
         {
           real sn[NVAR];
           rslope(oc, o1, o2, sn);
@@ -556,12 +548,7 @@ __global__ void __launch_bounds__(stage_threads(TJ, TK), stage_min_ctas(sizeof(r
           un[3] -= real(2) * Om * mvs;
           un[4] += cf * mvs;
         }
-        cp_async_wait_group<0>();   // this thread's U^n copy of plane i
-        {
-          real u0[NVAR];
-          ld8<real, NT>(u0s, tid, u0);
-          axpy8<real>(u0, dt, un, un);
-        }
+        axpy8<real>(u0, dt, un, un);
         // reciprocal cell widths (the speeds of the corrector's CFL step, h of
         // the cleaning)
         const real irs = pf[P_IRC] * rf[R_IST];
@@ -667,7 +654,6 @@ __global__ void __launch_bounds__(stage_threads(TJ, TK), stage_min_ctas(sizeof(r
       }
       if (i + 4 <= ie + 1) issue_plane(i + 4, om);
       else cp_async_commit();
-      issue_u0(i + 1);
       om = oc;
       oc = o1;
       o1 = o2;
@@ -708,43 +694,28 @@ int launch_t(const KParams &kp, const StageLaunch &sl, cudaStream_t s) {
   return cudaPeekAtLastError() == cudaSuccess ? 0 : -1;
 }
 
+// the instantiated tiles
+#define STAGE_TILES(X) \
+  X(4, 32) X(6, 36) X(8, 8) X(8, 12) X(8, 16) X(8, 24) X(8, 32) X(10, 24) X(12, 12) X(12, 16) X(12, 20) X(16, 16)
+
 template <typename real>
 int dispatch(const KParams &kp, const StageLaunch &sl, cudaStream_t s) {
-  if (sl.tile_j == 8 && sl.tile_k == 8) return launch_t<real, 8, 8>(kp, sl, s);
-  if (sl.tile_j == 12 && sl.tile_k == 12) return launch_t<real, 12, 12>(kp, sl, s);
-  if (sl.tile_j == 8 && sl.tile_k == 32) return launch_t<real, 8, 32>(kp, sl, s);
-  if (sl.tile_j == 4 && sl.tile_k == 32) return launch_t<real, 4, 32>(kp, sl, s);
-  if (sl.tile_j == 12 && sl.tile_k == 20) return launch_t<real, 12, 20>(kp, sl, s);
-  if (sl.tile_j == 6 && sl.tile_k == 36) return launch_t<real, 6, 36>(kp, sl, s);
-  if (sl.tile_j == 10 && sl.tile_k == 24) return launch_t<real, 10, 24>(kp, sl, s);
-  if (sl.tile_j == 8 && sl.tile_k == 24) return launch_t<real, 8, 24>(kp, sl, s);
+#define X(TJ, TK) \
+  if (sl.tile_j == TJ && sl.tile_k == TK) return launch_t<real, TJ, TK>(kp, sl, s);
+  STAGE_TILES(X)
+#undef X
   return -2;
 }
 
-template <typename real, int TJ, int TK>
-int occupancy_t(bool tracer) {
-  int n = 0;
-  const size_t smem = StageSmem<real>::bytes(TJ, TK, tracer);
-  ensure_smem<real, TJ, TK>(smem);
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_stage<real, TJ, TK, true>, stage_threads(TJ, TK), smem) != cudaSuccess)
-    return 1;
-  return n > 0 ? n : 1;
-}
-
-template <typename real>
-int occupancy(int tj, int tk, bool tracer) {
-  if (tj == 8 && tk == 8) return occupancy_t<real, 8, 8>(tracer);
-  if (tj == 12 && tk == 12) return occupancy_t<real, 12, 12>(tracer);
-  if (tj == 8 && tk == 32) return occupancy_t<real, 8, 32>(tracer);
-  if (tj == 4 && tk == 32) return occupancy_t<real, 4, 32>(tracer);
-  if (tj == 12 && tk == 20) return occupancy_t<real, 12, 20>(tracer);
-  if (tj == 6 && tk == 36) return occupancy_t<real, 6, 36>(tracer);
-  if (tj == 10 && tk == 24) return occupancy_t<real, 10, 24>(tracer);
-  if (tj == 8 && tk == 24) return occupancy_t<real, 8, 24>(tracer);
-  return 1;
-}
-
 }  // namespace
+
+// This file is compiled twice: k_stage_f64.cu defines STAGE_FP64 and holds the
+// FP64 instances only, so that the two sets of kernels compile side by side.
+#ifdef STAGE_FP64
+
+int stage_launch_f64(const KParams &kp, const StageLaunch &sl, cudaStream_t s) { return dispatch<double>(kp, sl, s); }
+
+#else
 
 size_t stage_smem_bytes(int precision, int tj, int tk, int tracer) {
   return precision ? StageSmem<float>::bytes(tj, tk, tracer) : StageSmem<double>::bytes(tj, tk, tracer);
@@ -752,9 +723,10 @@ size_t stage_smem_bytes(int precision, int tj, int tk, int tracer) {
 
 // an instantiated tile whose shared memory fits one CTA on this device
 int stage_tile_supported(int precision, int tj, int tk, int tracer) {
-  const bool known = (tj == 8 && tk == 8) || (tj == 12 && tk == 12) || (tj == 8 && tk == 32) ||
-                     (tj == 4 && tk == 32) || (tj == 12 && tk == 20) || (tj == 6 && tk == 36) ||
-                     (tj == 10 && tk == 24) || (tj == 8 && tk == 24);
+  bool known = false;
+#define X(TJ, TK) known = known || (tj == TJ && tk == TK);
+  STAGE_TILES(X)
+#undef X
   if (!known) return 0;
   int dev = 0, lim = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
@@ -763,11 +735,32 @@ int stage_tile_supported(int precision, int tj, int tk, int tracer) {
   return stage_smem_bytes(precision, tj, tk, tracer) <= (size_t)lim;
 }
 
-int stage_max_ctas_per_sm(int precision, int tj, int tk, int tracer) {
-  return precision ? occupancy<float>(tj, tk, tracer) : occupancy<double>(tj, tk, tracer);
+int stage_tile(int n, int *tj, int *tk) {
+  static const int tiles[][2] = {
+#define X(TJ, TK) {TJ, TK},
+      STAGE_TILES(X)
+#undef X
+  };
+  if (n < 0 || n >= (int)(sizeof(tiles) / sizeof(tiles[0]))) return 0;
+  *tj = tiles[n][0];
+  *tk = tiles[n][1];
+  return 1;
+}
+
+int stage_launch_f64(const KParams &kp, const StageLaunch &sl, cudaStream_t s);
+
+// Resident CTAs of an instance from its shared memory and the registers its
+// launch bounds grant (the kernels use close to all of them)
+int stage_ctas(int precision, int tj, int tk, int tracer) {
+  const int nt = stage_threads(tj, tk);
+  const int by_smem = (int)(233472 / (stage_smem_bytes(precision, tj, tk, tracer) + 1024));
+  const int regs = precision ? cmin(168, 65536 / (nt * stage_min_ctas(4, tj, tk)) / 8 * 8) : 256;
+  return cmax(1, cmin(by_smem, 65536 / (nt * regs)));
 }
 
 int stage_launch(const KParams &kp, const StageLaunch &sl, int precision, cudaStream_t s) {
   if (sl.nlist <= 0) return 0;
-  return precision ? dispatch<float>(kp, sl, s) : dispatch<double>(kp, sl, s);
+  return precision ? dispatch<float>(kp, sl, s) : stage_launch_f64(kp, sl, s);
 }
+
+#endif
