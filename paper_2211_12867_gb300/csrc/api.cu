@@ -41,7 +41,7 @@ struct Region {
 
 struct Layout {
   size_t total = 0;
-  Region geo, tables, blk, blk_alt, nb27, U, Us, Ualt, flux, lmap, lmap_off, bmap, cme, earth, vbg, scal, flags, lists,
+  Region geo, tables, blk, blk_alt, nb27, U, Us, Ualt, flux, lmap, lmap_off, bmap, cme, cone, earth, vbg, scal, flags, lists,
       rent, sides, rlist, ops, shell, rshell, staging, partial, probe_in, probe_out, mlp_par, mlp_feat, mlp_X, mlp_T, mlp_idx,
       mlp_act, mlp_xin;
   size_t staging_doubles = 0, table_doubles = 0;
@@ -73,7 +73,7 @@ size_t table_count(const icarus_grid_desc *d) {
                  N2 = (size_t)d->n_cells[2] << (L - 1);
     n += 2 * (N0 + 2 * NGH + 1) + 4 * (N0 + 2 * NGH);  // rf, r2f | dr3, dr2, rc, dr
     n += 2 * (N1 + 2 * NGH + 1) + 5 * (N1 + 2 * NGH);  // tf, sinf | dcos, tc, sintc, costc, dth
-    n += (N2 + 2 * NGH + 1) + (N2 + 2 * NGH);          // pf | pc
+    n += (N2 + 2 * NGH + 1) + 3 * (N2 + 2 * NGH);      // pf | pc, cosp, sinp
     if (L < d->max_level) n += 2 * (N0 + N1 + N2);     // offsets
   }
   return n;
@@ -147,6 +147,7 @@ Layout make_layout(const icarus_grid_desc *d) {
   L.lmap_off = L.add((size_t)nm * (MAXLEV + 1) * sizeof(long long));
   L.bmap = L.add((size_t)nm * NVAR * d->n_cells[1] * d->n_cells[2] * sizeof(double));
   L.cme = L.add((size_t)nm * sizeof(DevCme));
+  L.cone = L.add((size_t)nm * sizeof(DevCone));
   L.earth = L.add((size_t)nm * sizeof(DevEarth));
   L.vbg = L.add((size_t)nm * d->n_cells[0] * d->n_cells[1] * d->n_cells[2] * sizeof(double));
   L.scal = L.add((size_t)nm * 7 * sizeof(double) + 64);
@@ -237,6 +238,7 @@ struct icarus_ctx {
   double *bmap = nullptr, *vbg = nullptr, *staging = nullptr, *partial = nullptr, *probe_in = nullptr,
          *probe_out = nullptr;
   DevCme *cme = nullptr;
+  DevCone *cone = nullptr;
   DevEarth *earth = nullptr;
   double *t = nullptr, *dt_used = nullptr, *dt_cfl = nullptr, *tstop = nullptr, *updates = nullptr,
          *cells_m = nullptr;
@@ -256,7 +258,7 @@ struct icarus_ctx {
   int lvl_count[MAXLEV + 1] = {0}, lvl_start[MAXLEV + 1] = {0};
   int rent_start[MAXLEV + 1] = {0}, rent_face[MAXLEV + 1] = {0}, rent_count[MAXLEV + 1] = {0};
   int reg_tab[27][3] = {};  // per region: start in the region-ordered shell, group-first cells, cells
-  int side_count[MAXLEV + 1][3] = {{0}}, side_start[MAXLEV + 1][3] = {{0}};
+  int side_count[MAXLEV + 1] = {0}, side_start[MAXLEV + 1] = {0};
   int nrlist = 0, max_level_present = 1;
   std::vector<signed char> hflags;
   bool flags_valid = false;
@@ -472,6 +474,16 @@ bool tree_is_valid(icarus_ctx *c, Member &m) {
   return bad == 0;
 }
 
+// a member's cone CME to the device, with the sines and cosines of its angles
+icarus_status upload_cme(icarus_ctx *c, int m) {
+  const DevCme &q = c->mem[m].cme;
+  const DevCone e{std::sin(q.colat), std::cos(q.colat), std::sin(q.lon), std::cos(q.lon), std::sin(q.half_width)};
+  CK(cudaMemcpyAsync(c->cme + m, &q, sizeof(DevCme), cudaMemcpyHostToDevice, c->stream));
+  CK(cudaMemcpyAsync(c->cone + m, &e, sizeof(DevCone), cudaMemcpyHostToDevice, c->stream));
+  CK(cudaStreamSynchronize(c->stream));
+  return ICARUS_OK;
+}
+
 // device tables that depend on the leaf lists
 icarus_status upload_tree(icarus_ctx *c, DevBlock *blk_dst) {
   const icarus_grid_desc &d = c->d;
@@ -487,8 +499,7 @@ icarus_status upload_tree(icarus_ctx *c, DevBlock *blk_dst) {
   std::vector<int> all(c->nleaves);
   std::vector<std::vector<int>> per_level(MAXLEV + 1);
   std::vector<std::vector<int2>> ent_face(MAXLEV + 1), ent_rest(MAXLEV + 1);
-  std::vector<std::vector<int2>> sd[3];
-  for (int k = 0; k < 3; k++) sd[k].assign(MAXLEV + 1, std::vector<int2>());
+  std::vector<std::vector<int2>> sd(MAXLEV + 1);   // (slot, direction * 2 + side) of the physical faces
   std::vector<int> rl;
   c->max_level_present = 1;
   // the relation of each leaf to the 27 regions around it (0 outside a
@@ -530,7 +541,7 @@ icarus_status upload_tree(icarus_ctx *c, DevBlock *blk_dst) {
         if (rs[r] == 0) {
           B.nbr[f] = NB_PHYS;
           B.phys |= 1 << f;
-          sd[dd][l.level].push_back(make_int2(slot, hi));
+          sd[l.level].push_back(make_int2(slot, f));
           continue;
         }
         B.nbr[f] = rs[r] == 1 ? NB_SAME : (rs[r] == 3 ? NB_FINER : NB_COARSER);
@@ -578,12 +589,11 @@ icarus_status upload_tree(icarus_ctx *c, DevBlock *blk_dst) {
   }
   if (ent.size() > (size_t)items_per_block(&c->d) * c->lay.max_blocks) return ICARUS_ERR_CAPACITY;
   std::vector<int2> sv;
-  for (int L = 1; L <= MAXLEV; L++)
-    for (int k = 0; k < 3; k++) {
-      c->side_start[L][k] = (int)sv.size();
-      c->side_count[L][k] = (int)sd[k][L].size();
-      sv.insert(sv.end(), sd[k][L].begin(), sd[k][L].end());
-    }
+  for (int L = 1; L <= MAXLEV; L++) {
+    c->side_start[L] = (int)sv.size();
+    c->side_count[L] = (int)sd[L].size();
+    sv.insert(sv.end(), sd[L].begin(), sd[L].end());
+  }
   c->nrlist = (int)rl.size();
   {
     std::vector<double> cm(d.n_members);
@@ -639,6 +649,7 @@ void fill_kp(icarus_ctx *c) {
   k.lmap_off = c->lmap_off;
   k.bmap = c->bmap;
   k.cme = c->cme;
+  k.cone = c->cone;
   k.earth = c->earth;
   k.vbg = c->vbg;
   k.t = c->t;
@@ -729,6 +740,13 @@ icarus_status build_geometry(icarus_ctx *c) {
     o.push_back(push(dth));
     o.push_back(push(pf));
     o.push_back(push(pcv));
+    std::vector<double> cosp(pcv.size()), sinp(pcv.size());
+    for (size_t q = 0; q < pcv.size(); q++) {
+      cosp[q] = std::cos(pcv[q]);
+      sinp[q] = std::sin(pcv[q]);
+    }
+    o.push_back(push(cosp));
+    o.push_back(push(sinp));
     hg.d[L].dphi = dphi;
     hg.f[L].dphi = (float)dphi;
     hg.d[L].n[0] = hg.f[L].n[0] = N0;
@@ -797,10 +815,12 @@ icarus_status build_geometry(icarus_ctx *c) {
     G.dth = b + o[12]; F.dth = f + o[12];
     G.pf = b + o[13]; F.pf = f + o[13];
     G.pc = b + o[14]; F.pc = f + o[14];
+    G.cosp = b + o[15]; F.cosp = f + o[15];
+    G.sinp = b + o[16]; F.sinp = f + o[16];
     if (L < d.max_level)
       for (int dd = 0; dd < 3; dd++) {
-        hg.dlt[L][dd] = b + o[15 + dd];
-        hg.dltf[L][dd] = f + o[15 + dd];
+        hg.dlt[L][dd] = b + o[17 + dd];
+        hg.dltf[L][dd] = f + o[17 + dd];
       }
   }
   CK(cudaMemcpyAsync(dbase, hd.data(), sizeof(double) * hd.size(), cudaMemcpyHostToDevice, c->stream));
@@ -974,11 +994,10 @@ int enqueue_ghost(icarus_ctx *c, void *buf, double tfac, bool faces_only = false
                              faces_only ? c->nshell_face : c->lay.nshell, L, c->stream);
       n++;
     }
-    for (int dd = 0; dd < 3; dd++) {
-      if (c->side_count[L][dd] == 0) continue;
+    if (c->side_count[L] > 0) {
       ProfScope p(c, 2);
-      ghost_physical_launch(c->kp, buf, c->prec, c->sides + c->side_start[L][dd], c->side_count[L][dd], dd, L, tfac,
-                            faces_only, skip_same, c->stream);
+      ghost_physical_launch(c->kp, buf, c->prec, c->sides + c->side_start[L], c->side_count[L], L, tfac, faces_only,
+                            skip_same, c->stream);
       n++;
     }
   }
@@ -987,11 +1006,6 @@ int enqueue_ghost(icarus_ctx *c, void *buf, double tfac, bool faces_only = false
 
 int enqueue_step(icarus_ctx *c) {
   int n = 0;
-  {
-    ProfScope p(c, 0);
-    dt_begin_launch(c->kp, c->tstop, c->stream);
-  }
-  n++;
   // the step's fills leave the ghost cells that same-level leaves hold to the
   // stage kernels, which read them from those leaves
   n += enqueue_ghost(c, c->U, 0.0, true, c->direct_halo);
@@ -1025,7 +1039,7 @@ int enqueue_step(icarus_ctx *c) {
   }
   {
     ProfScope p(c, 6);
-    dt_finalize_launch(c->kp, c->d.cfl, c->stream);
+    dt_finalize_launch(c->kp, c->d.cfl, c->tstop, c->stream);
   }
   n++;
   return n;
@@ -1176,6 +1190,7 @@ icarus_status icarus_init_grid(const icarus_grid_desc *desc, icarus_ctx **out) {
   c->lmap_off = at<long long>(c, lay.lmap_off);
   c->bmap = at<double>(c, lay.bmap);
   c->cme = at<DevCme>(c, lay.cme);
+  c->cone = at<DevCone>(c, lay.cone);
   c->earth = at<DevEarth>(c, lay.earth);
   c->vbg = at<double>(c, lay.vbg);
   double *sc = at<double>(c, lay.scal);
@@ -1363,7 +1378,8 @@ icarus_status icarus_inject_cone_cme(icarus_ctx *c, int member, const icarus_con
   dc.active = 1;
   dc.pad = 1;  // background speed recorded below
   M.cme = dc;
-  CK(cudaMemcpyAsync(c->cme + member, &M.cme, sizeof(DevCme), cudaMemcpyHostToDevice, c->stream));
+  const icarus_status up = upload_cme(c, member);
+  if (up != ICARUS_OK) return up;
   const size_t nbc = (size_t)c->d.n_cells[0] * c->d.n_cells[1] * c->d.n_cells[2];
   vbg_launch(c->kp, c->U, c->prec, member, c->mem_off[member], (int)M.leaves.size(), c->vbg + member * nbc,
              c->stream);
@@ -1432,15 +1448,14 @@ icarus_status icarus_use_graph(icarus_ctx *c, int enable) {
 
 icarus_status icarus_kernels_per_step(icarus_ctx *c, int *n) {
   if (!c || !n) return ICARUS_ERR_ARG;
-  int k = 4 + (c->nrlist > 0 ? 1 : 0);  // dt begin, two stages, dt finalize, reflux
+  int k = 3 + (c->nrlist > 0 ? 1 : 0);  // two stages, dt finalize, reflux
   for (int L = 1; L <= c->max_level_present; L++) {
     if (!c->lvl_count[L]) continue;
     // neighbour ghost pass of both fills (with direct halo reads only over
     // the regions held by coarser or finer leaves: faces in the first fill)
     if (c->direct_halo) k += (c->rent_face[L] > 0) + (c->rent_count[L] > 0);
     else k += 2;
-    for (int d = 0; d < 3; d++)
-      if (c->side_count[L][d]) k += 2;   // physical ghost pass, both fills
+    if (c->side_count[L]) k += 2;   // physical ghost pass, both fills
   }
   *n = k;
   return ICARUS_OK;
@@ -1459,6 +1474,11 @@ icarus_status icarus_step(icarus_ctx *c, int n_steps, const double *t_stop, doub
   c->h_tstop.assign(t_stop, t_stop + nm);
   CK(cudaMemcpyAsync(c->tstop, c->h_tstop.data(), sizeof(double) * nm, cudaMemcpyHostToDevice, c->stream));
   if (n_steps > 0) {
+    {
+      // the first step's dt (each step leaves the next one's)
+      ProfScope p(c, 0);
+      dt_begin_launch(c->kp, c->tstop, c->stream);
+    }
     if (c->use_graph && !c->prof_on && c->stream != nullptr) {
       if (!c->graph_valid) {
         if (c->graph) {
@@ -2354,7 +2374,8 @@ icarus_status icarus_load(icarus_ctx *c, const char *path) {
   c->isl_beta = isl[1];
   fill_kp(c);
   cudaStream_t s = c->stream;
-  for (int m = 0; m < nm; m++) CK(cudaMemcpyAsync(c->cme + m, &c->mem[m].cme, sizeof(DevCme), cudaMemcpyHostToDevice, s));
+  for (int m = 0; m < nm; m++)
+    if ((st = upload_cme(c, m)) != ICARUS_OK) return st;
   CK(cudaMemcpyAsync(c->t, t.data(), sizeof(double) * nm, cudaMemcpyHostToDevice, s));
   CK(cudaMemcpyAsync(c->dt_cfl, dtc.data(), sizeof(double) * nm, cudaMemcpyHostToDevice, s));
   CK(cudaMemcpyAsync(c->updates, upd.data(), sizeof(double) * nm, cudaMemcpyHostToDevice, s));

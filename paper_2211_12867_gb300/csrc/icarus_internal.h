@@ -45,6 +45,7 @@ struct LevelGeo {
   const real *dth;   // theta+ - theta-
   const real *pf;    // phi faces
   const real *pc;    // phi centres
+  const real *cosp, *sinp;   // of the phi centres
   real dphi;         // uniform phi width (Cartesian: dz)
   int n[3];
 };
@@ -71,6 +72,12 @@ template <> struct GeoSel<float> {
 struct DevCme {
   double t_start, t_max, colat, lon, half_width, v, rho, p;
   int active, pad;
+};
+
+// sines and cosines of a cone CME's direction and half width (not part of
+// DevCme, which checkpoints hold as it is)
+struct DevCone {
+  double sin_colat, cos_colat, sin_lon, cos_lon, sin_hw;
 };
 
 // Earth's direction for the windows of the shock criterion: colatitude and
@@ -100,6 +107,7 @@ struct KParams {
   const long long *lmap_off;   // [member * (MAXLEV+1) + L]
   const double *bmap;          // [member][8][n1][n2] inner boundary primitives
   const DevCme *cme;           // [member]
+  const DevCone *cone;         // [member]
   const DevEarth *earth;       // [member]
   const double *vbg;           // [member][n0][n1][n2] background v_r
   double *t;                   // [member]
@@ -152,12 +160,14 @@ void ghost_neighbour_launch(const KParams &kp, void *U, int precision, const int
                             const int *shell, int nshell, int level, cudaStream_t s);
 void ghost_regions_launch(const KParams &kp, void *U, int precision, const int2 *items, int nitems,
                           const int *rshell, int level, cudaStream_t s);
-void ghost_physical_launch(const KParams &kp, void *U, int precision, const int2 *sides, int nsides,
-                           int dir, int level, double tshift_fac, bool faces_only, bool skip_same, cudaStream_t s);
+// physical boundaries of a level's leaves in all directions; sides: (slot,
+// direction * 2 + side)
+void ghost_physical_launch(const KParams &kp, void *U, int precision, const int2 *sides, int nsides, int level,
+                           double tshift_fac, bool faces_only, bool skip_same, cudaStream_t s);
 void reflux_launch(const KParams &kp, void *U, const void *flux, int precision, const int *list, int nlist,
                    cudaStream_t s);
 void dt_begin_launch(const KParams &kp, const double *tstop, cudaStream_t s);
-void dt_finalize_launch(const KParams &kp, double cfl, cudaStream_t s);
+void dt_finalize_launch(const KParams &kp, double cfl, const double *tstop, cudaStream_t s);
 void dt_full_launch(const KParams &kp, const void *U, int precision, int nleaves, double cfl, cudaStream_t s);
 
 // state and AMR support

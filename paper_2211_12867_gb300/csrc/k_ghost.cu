@@ -300,9 +300,14 @@ __global__ void __launch_bounds__(256, sizeof(real) == 4 ? 3 : 2) k_ghost_region
   }
 }
 
-// inner boundary state (FP64): map of the containing base cell, cone CME
-// overlay; u[TRV] = rho X with the CME tracer X = 1 in the CME plasma, else 0
-__device__ void inner_state(const KParams &kp, int member, int L, int J, int K, double t, double *u) {
+// Inner boundary state (FP64): map of the containing base cell, cone CME
+// overlay; u[TRV] = rho X with the CME tracer X = 1 in the CME plasma, else 0.
+// A cell is inside the cone where its angle from the axis is at most the
+// opening angle acos(arg) of Eqs. 1-4, that is where the angle's cosine is at
+// least arg: with the tables of the angles' sines and cosines no
+// trigonometric function is left (sin, cos and two acos in FP64 took 19 of the
+// pass's 22 us on the 512 x 60 x 180 wedge).
+__device__ __forceinline__ void inner_state(const KParams &kp, int member, int L, int J, int K, double t, double *u) {
   double X = 0.0;
   const int n1 = kp.n_base_cells[1], n2 = kp.n_base_cells[2];
   const int jb = J >> (L - 1), kb = K >> (L - 1);
@@ -310,29 +315,27 @@ __device__ void inner_state(const KParams &kp, int member, int L, int J, int K, 
   double w[NVAR];
 #pragma unroll
   for (int v = 0; v < NVAR; v++) w[v] = m[((size_t)v * n1 + jb) * n2 + kb];
-  const DevCme c = kp.cme[member];
+  const DevCme &c = kp.cme[member];
   if (c.active) {
-    const LevelGeo<double> &G = kp.geo->d[L];
-    const double th = G.tc[J + NGH], ph = G.pc[K + NGH];
-    const double R = G.rf[NGH];
     const double tau = t - c.t_start;
     if (tau >= 0.0 && tau <= c.t_max) {
-      const double rh = R * sin(c.half_width);
+      const LevelGeo<double> &G = kp.geo->d[L];
+      const DevCone &e = kp.cone[member];
+      const double R = G.rf[NGH];
+      const double rh = R * e.sin_hw;
       const double Rc = tau * c.v + R - rh;
       const double arg = (Rc * Rc + R * R - rh * rh) / (2.0 * Rc * R);
-      if (!(arg > 1.0)) {
-        const double open = acos(arg);
-        double a = sin(th) * sin(c.colat) * cos(ph - c.lon) + cos(th) * cos(c.colat);
-        a = a > 1.0 ? 1.0 : (a < -1.0 ? -1.0 : a);
-        if (acos(a) <= open) {
-          w[0] = c.rho;
-          w[1] = c.v;
-          w[2] = 0.0;
-          w[3] = -kp.omega * R * sin(th);
-          w[4] = c.p;
-          w[5] = w[6] = w[7] = 0.0;
-          X = 1.0;
-        }
+      const double st = G.sintc[J + NGH];
+      const double a = st * e.sin_colat * (G.cosp[K + NGH] * e.cos_lon + G.sinp[K + NGH] * e.sin_lon) +
+                       G.costc[J + NGH] * e.cos_colat;
+      if (arg >= -1.0 && arg <= 1.0 && fmin(a, 1.0) >= arg) {
+        w[0] = c.rho;
+        w[1] = c.v;
+        w[2] = 0.0;
+        w[3] = -kp.omega * R * st;
+        w[4] = c.p;
+        w[5] = w[6] = w[7] = 0.0;
+        X = 1.0;
       }
     }
   }
@@ -340,51 +343,72 @@ __device__ void inner_state(const KParams &kp, int member, int L, int J, int K, 
   u[TRV] = w[0] * X;
 }
 
-// physical boundary of direction `dir`; sides[n] = (slot, side)
-// faces: only the ghost cells inside the block in the two other directions
+// Physical boundaries of all directions of a level's leaves in one launch;
+// sides[n] = (slot, direction * 2 + side).  The boundaries apply in the order
+// r, theta, phi over the whole padded slab, each reading what the earlier ones
+// wrote; here a ghost cell belongs to its highest physical direction and
+// composes the maps of that direction and of the lower ones down to the cell
+// (or inner-boundary state) that its value comes from, so no pass waits for
+// another.  faces: only the ghost cells inside the block in the two other
+// directions.  The two layers of the inner boundary hold one state: a thread
+// writes both.
 template <typename real>
-__global__ void k_ghost_physical(const KParams kp, real *U, const int2 *sides, int dir, int L, double tfac,
-                                 int faces, int skip_same) {
+__global__ void __launch_bounds__(128) k_ghost_physical(const KParams kp, real *U, const int2 *sides, int L, double tfac,
+                                                        int faces, int skip_same) {
   const int2 sd = sides[blockIdx.x];
-  const int slot = sd.x, side = sd.y;
+  const int slot = sd.x, dir = sd.y >> 1, side = sd.y & 1;
   const int da = dir == 0 ? 1 : 0, db = dir == 2 ? 1 : 2;
   const int Pa = faces ? kp.nb[da] : kp.P[da], Pb = faces ? kp.nb[db] : kp.P[db], off = faces ? NGH : 0;
   const int idx = blockIdx.y * blockDim.x + threadIdx.x;
-  if (idx >= NGH * Pa * Pb) return;
-  const int gl = idx / (Pa * Pb), r = idx % (Pa * Pb), a = r / Pb + off, b = r % Pb + off;
-  const int bc = side ? kp.bc_hi[dir] : kp.bc_lo[dir];
-  const int nbd = kp.nb[dir];
-  const int pg = side ? NGH + nbd + gl : NGH - 1 - gl;
-  const int pn = side ? NGH + nbd - 1 : NGH;
-  const int pm = side ? NGH + nbd - 1 - gl : NGH + gl;
-  int q[3], s[3];
-  q[dir] = pg;
+  const bool inner = (side ? kp.bc_hi[dir] : kp.bc_lo[dir]) == 3;
+  if (idx >= (inner ? 1 : NGH) * Pa * Pb) return;
+  const int gl = idx / (Pa * Pb), r = idx - gl * (Pa * Pb), a = r / Pb + off, b = r - (r / Pb) * Pb + off;
+  const DevBlock &B = kp.blk[slot];
+  const int phys = B.phys;
+  int q[3];
+  q[dir] = side ? NGH + kp.nb[dir] + gl : NGH - 1 - gl;
   q[da] = a;
   q[db] = b;
-  s[da] = a;
-  s[db] = b;
-  const DevBlock B = kp.blk[slot];
-  if (bc == 3) {  // inner boundary (r low)
-    bool in1, in2;
-    const int J = wrap_dim(kp, L, 1, B.ix[1] * kp.nb[1] + q[1] - NGH, in1);
-    const int K = wrap_dim(kp, L, 2, B.ix[2] * kp.nb[2] + q[2] - NGH, in2);
-    if (!in1 || !in2) return;
+  int s[3] = {q[0], q[1], q[2]};
+  unsigned flip = 0;
+  bool at_inner = false;
+#pragma unroll
+  for (int d = 2; d >= 0; d--) {
+    const int nb = kp.nb[d];
+    const int lo = s[d] < NGH && (phys >> (2 * d) & 1), hi = s[d] >= NGH + nb && (phys >> (2 * d + 1) & 1);
+    if (!(lo | hi)) continue;
+    if (d > dir) return;   // a higher direction's cell
+    const int bc = hi ? kp.bc_hi[d] : kp.bc_lo[d];
+    if (bc == 3) {
+      at_inner = true;
+    } else if (bc == 2) {
+      s[d] = hi ? 2 * (NGH + nb) - 1 - s[d] : 2 * NGH - 1 - s[d];
+      flip ^= 1u << d;
+    } else {
+      s[d] = hi ? NGH + nb - 1 : NGH;
+    }
+  }
+  real x[NVAR + 1];
+  if (at_inner) {
+    bool in;
+    const int J = wrap_dim(kp, L, 1, B.ix[1] * kp.nb[1] + s[1] - NGH, in);
+    const int K = wrap_dim(kp, L, 2, B.ix[2] * kp.nb[2] + s[2] - NGH, in);
     const double t = kp.t[B.member] + tfac * kp.dt_used[B.member];
     double u[NVAR + 1];
     inner_state(kp, B.member, L, J, K, t, u);
-    real x[NVAR + 1];
 #pragma unroll
     for (int v = 0; v < NVAR + 1; v++) x[v] = (real)u[v];
-    store(kp, U, {slot_base(kp, slot), pad_cell(kp, q[0], q[1], q[2])}, x);
-    return;
+  } else {
+    fetch(kp, U, locate(kp, slot, s[0], s[1], s[2], skip_same != 0), x);
   }
-  s[dir] = bc == 2 ? pm : pn;
-  real x[NVAR + 1];
-  fetch(kp, U, locate(kp, slot, s[0], s[1], s[2], skip_same != 0), x);
 #pragma unroll
-  for (int v = 0; v < NVAR; v++)
-    if (bc == 2 && (v == 1 + dir || v == 5 + dir)) x[v] = -x[v];
+  for (int d = 0; d < 3; d++)
+    if (flip >> d & 1) {
+      x[1 + d] = -x[1 + d];
+      x[5 + d] = -x[5 + d];
+    }
   store(kp, U, {slot_base(kp, slot), pad_cell(kp, q[0], q[1], q[2])}, x);
+  if (inner) store(kp, U, {slot_base(kp, slot), pad_cell(kp, 0, q[1], q[2])}, x);
 }
 
 // reflux of coarse blocks with finer face neighbours; one CTA per block
@@ -501,15 +525,22 @@ __global__ void k_reflux(const KParams kp, real *U, const real *flux, const int 
   }
 }
 
+// the step a member takes next (none once it has reached its stop time)
+__device__ __forceinline__ double next_dt(const KParams &kp, int m, const double *tstop) {
+  const double dt = fmin(kp.dt_cfl[m], tstop[m] - kp.t[m]);
+  return dt > 0.0 ? dt : 0.0;
+}
+
 __global__ void k_dt_begin(const KParams kp, const double *tstop) {
   const int m = blockIdx.x * blockDim.x + threadIdx.x;
   if (m >= kp.n_members) return;
-  double dt = fmin(kp.dt_cfl[m], tstop[m] - kp.t[m]);
-  kp.dt_used[m] = dt > 0.0 ? dt : 0.0;
+  kp.dt_used[m] = next_dt(kp, m, tstop);
 }
 
-__global__ void k_dt_finalize(const KParams kp, double cfl) {
-  const int m = blockIdx.x * blockDim.x + threadIdx.x;
+// End of a step: times, CFL step of the new state, and the next step's dt (so
+// that only the first step of a call has a launch for it)
+__global__ void k_dt_finalize(const KParams kp, double cfl, const double *tstop) {
+  const int m = threadIdx.x;
   if (m == 0) {
     // floor budget: the floors the step applied (both stages) against the
     // leaf cells it advanced
@@ -522,15 +553,18 @@ __global__ void k_dt_finalize(const KParams kp, double cfl) {
       if ((double)d > kp.floor_budget * cells) atomicOr(kp.status, ST_FLOOR);
     }
   }
-  if (m >= kp.n_members) return;
-  const double dt = kp.dt_used[m];
-  if (dt > 0.0) {
-    kp.t[m] += dt;
-    kp.updates[m] += kp.cells_m[m];
-    const double inv = __longlong_as_double((long long)kp.inv_max[m]);
-    if (inv > 0.0) kp.dt_cfl[m] = cfl / inv;
+  __syncthreads();   // the budget has read every member's step
+  for (int q = m; q < kp.n_members; q += blockDim.x) {
+    const double dt = kp.dt_used[q];
+    if (dt > 0.0) {
+      kp.t[q] += dt;
+      kp.updates[q] += kp.cells_m[q];
+      const double inv = __longlong_as_double((long long)kp.inv_max[q]);
+      if (inv > 0.0) kp.dt_cfl[q] = cfl / inv;
+    }
+    kp.inv_max[q] = 0ull;
+    kp.dt_used[q] = next_dt(kp, q, tstop);
   }
-  kp.inv_max[m] = 0ull;
 }
 
 // CFL time step of the whole current state (after set_state / regrid / init)
@@ -591,16 +625,21 @@ void ghost_regions_launch(const KParams &kp, void *U, int precision, const int2 
     k_ghost_regions<double><<<grid, 256, 0, s>>>(kp, (double *)U, items, nitems, rshell, level);
 }
 
-void ghost_physical_launch(const KParams &kp, void *U, int precision, const int2 *sides, int nsides, int dir,
-                           int level, double tfac, bool faces_only, bool skip_same, cudaStream_t s) {
+void ghost_physical_launch(const KParams &kp, void *U, int precision, const int2 *sides, int nsides, int level,
+                           double tfac, bool faces_only, bool skip_same, cudaStream_t s) {
   if (nsides <= 0) return;
-  const int da = dir == 0 ? 1 : 0, db = dir == 2 ? 1 : 2;
-  const int n = faces_only ? NGH * kp.nb[da] * kp.nb[db] : NGH * kp.P[da] * kp.P[db];
+  int n = 0;   // cells of the largest slab that can be physical
+  for (int d = 0; d < 3; d++) {
+    if (kp.bc_lo[d] == 0) continue;
+    const int da = d == 0 ? 1 : 0, db = d == 2 ? 1 : 2;
+    const int c = NGH * (faces_only ? kp.nb[da] * kp.nb[db] : kp.P[da] * kp.P[db]);
+    n = c > n ? c : n;
+  }
   dim3 grid(nsides, (n + 127) / 128);
   if (precision)
-    k_ghost_physical<float><<<grid, 128, 0, s>>>(kp, (float *)U, sides, dir, level, tfac, faces_only, skip_same);
+    k_ghost_physical<float><<<grid, 128, 0, s>>>(kp, (float *)U, sides, level, tfac, faces_only, skip_same);
   else
-    k_ghost_physical<double><<<grid, 128, 0, s>>>(kp, (double *)U, sides, dir, level, tfac, faces_only, skip_same);
+    k_ghost_physical<double><<<grid, 128, 0, s>>>(kp, (double *)U, sides, level, tfac, faces_only, skip_same);
 }
 
 void reflux_launch(const KParams &kp, void *U, const void *flux, int precision, const int *list, int nlist,
@@ -616,8 +655,9 @@ void dt_begin_launch(const KParams &kp, const double *tstop, cudaStream_t s) {
   k_dt_begin<<<(kp.n_members + 127) / 128, 128, 0, s>>>(kp, tstop);
 }
 
-void dt_finalize_launch(const KParams &kp, double cfl, cudaStream_t s) {
-  k_dt_finalize<<<(kp.n_members + 127) / 128, 128, 0, s>>>(kp, cfl);
+void dt_finalize_launch(const KParams &kp, double cfl, const double *tstop, cudaStream_t s) {
+  const int n = kp.n_members < 1024 ? (kp.n_members + 31) / 32 * 32 : 1024;
+  k_dt_finalize<<<1, n, 0, s>>>(kp, cfl, tstop);
 }
 
 void dt_full_launch(const KParams &kp, const void *U, int precision, int nleaves, double cfl, cudaStream_t s) {
