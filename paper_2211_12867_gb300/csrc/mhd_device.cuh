@@ -378,9 +378,8 @@ __device__ __forceinline__ void mc_half_slopes8<float>(const float *um, const fl
   }
 }
 
-// Flux balance of CH variables of a cell with the areas over its volume:
-// out[h] = rm Flo - rp Fhi + tm Ftl - tp Fth + pw (Fpl - Fph), FP32 in packed
-// pairs.
+// Flux balance of CH variables of a cell (FP64) with the areas over its volume:
+// out[h] = rm Flo - rp Fhi + tm Ftl - tp Fth + pw (Fpl - Fph).
 template <typename real, int CH>
 __device__ __forceinline__ void flux_balance(const real *Fhi, const real *Flo, const real *fth, const real *ftl,
                                              const real *fph, const real *fpl, real rp, real rm, real tp, real tm,
@@ -389,19 +388,23 @@ __device__ __forceinline__ void flux_balance(const real *Fhi, const real *Flo, c
   for (int h = 0; h < CH; h++)
     out[h] = (rm * Flo[h] - rp * Fhi[h]) + (tm * ftl[h] - tp * fth[h]) + pw * (fpl[h] - fph[h]);
 }
-template <>
-__device__ __forceinline__ void flux_balance<float, 4>(const float *Fhi, const float *Flo, const float *fth,
-                                                       const float *ftl, const float *fph, const float *fpl,
-                                                       float rp, float rm, float tp, float tm, float pw,
-                                                       float *out) {
-  const float2 r1 = make_float2(rm, rm), r2 = make_float2(-rp, -rp), t1 = make_float2(tm, tm),
-               t2 = make_float2(-tp, -tp), p1 = make_float2(pw, pw), m1 = make_float2(-1.f, -1.f);
+// FP32: out[h] = -((Arp Fhi - Arm Flo) + (Atp Fth - Atm Ftl) + Ap (Fph - Fpl)) iV
+// from the areas, in packed pairs.
+__device__ __forceinline__ void flux_balance32(const float *Fhi, const float *Flo, const float *fth, const float *ftl,
+                                               const float *fph, const float *fpl, float Arp, float Arm, float Atp,
+                                               float Atm, float Ap, float iV, float *out) {
+  const float2 arp = make_float2(Arp, Arp), narm = make_float2(-Arm, -Arm), atp = make_float2(Atp, Atp),
+               natm = make_float2(-Atm, -Atm), ap = make_float2(Ap, Ap), m1 = make_float2(-1.f, -1.f),
+               niv = make_float2(-iV, -iV);
 #pragma unroll
   for (int h = 0; h < 4; h += 2) {
-    const float2 r = __ffma2_rn(r2, make_float2(Fhi[h], Fhi[h + 1]), __fmul2_rn(r1, make_float2(Flo[h], Flo[h + 1])));
-    const float2 t = __ffma2_rn(t2, make_float2(fth[h], fth[h + 1]), __fmul2_rn(t1, make_float2(ftl[h], ftl[h + 1])));
-    const float2 p = __ffma2_rn(m1, make_float2(fph[h], fph[h + 1]), make_float2(fpl[h], fpl[h + 1]));
-    const float2 o = __ffma2_rn(p1, p, __fadd2_rn(r, t));
+    const float2 r = __ffma2_rn(narm, make_float2(Flo[h], Flo[h + 1]),
+                                __fmul2_rn(arp, make_float2(Fhi[h], Fhi[h + 1])));
+    const float2 t = __ffma2_rn(natm, make_float2(ftl[h], ftl[h + 1]),
+                                __fmul2_rn(atp, make_float2(fth[h], fth[h + 1])));
+    const float2 p = __ffma2_rn(m1, make_float2(fpl[h], fpl[h + 1]), make_float2(fph[h], fph[h + 1]));
+    const float2 d = __ffma2_rn(ap, p, __fadd2_rn(r, t));
+    const float2 o = __fmul2_rn(d, niv);
     out[h] = o.x;
     out[h + 1] = o.y;
   }
@@ -416,21 +419,16 @@ __device__ __forceinline__ double fast_speed_of(double ir, double gp, double hgp
   const double d = hgp - hb2;
   return RT<double>::sqrt_((hgp + hb2 + RT<double>::sqrt_(fma(d, d, gp * bt2))) * ir);
 }
-__device__ __forceinline__ float fast_speed_of(float ir, float gp, float hgp, float hb2, float bt2) {
-  // scaled by 1/rho first: the squares stay far from the ends of FP32
-  const float a = hgp * ir, b = hb2 * ir, d = a - b;
-  return RT<float>::sqrt_(a + b + RT<float>::sqrt_(fmaf(d, d, (gp * ir) * (bt2 * ir))));
-}
 
 // Sum over the directions of (|v_d| + c_f,d) / dx_d from 1/rho, the velocity,
 // p and the field (ix: reciprocal widths)
-template <typename real>
-__device__ __forceinline__ real cfl_rate(real ir, const real *v, real p, const real *B, real gamma, const real *ix) {
-  const real gp = gamma * p, hgp = real(0.5) * gp, q0 = B[0] * B[0], q1 = B[1] * B[1], q2 = B[2] * B[2];
-  const real hb2 = real(0.5) * (q0 + q1 + q2);
-  return (RT<real>::abs_(v[0]) + fast_speed_of(ir, gp, hgp, hb2, q1 + q2)) * ix[0] +
-         (RT<real>::abs_(v[1]) + fast_speed_of(ir, gp, hgp, hb2, q0 + q2)) * ix[1] +
-         (RT<real>::abs_(v[2]) + fast_speed_of(ir, gp, hgp, hb2, q0 + q1)) * ix[2];
+__device__ __forceinline__ double cfl_rate(double ir, const double *v, double p, const double *B, double gamma,
+                                           const double *ix) {
+  const double gp = gamma * p, hgp = 0.5 * gp, q0 = B[0] * B[0], q1 = B[1] * B[1], q2 = B[2] * B[2];
+  const double hb2 = 0.5 * (q0 + q1 + q2);
+  return (fabs(v[0]) + fast_speed_of(ir, gp, hgp, hb2, q1 + q2)) * ix[0] +
+         (fabs(v[1]) + fast_speed_of(ir, gp, hgp, hb2, q0 + q2)) * ix[1] +
+         (fabs(v[2]) + fast_speed_of(ir, gp, hgp, hb2, q0 + q1)) * ix[2];
 }
 
 // One side's part of the TVDLF flux, G = F(W) + sc U(W) with sc = +c_max on
@@ -438,14 +436,14 @@ __device__ __forceinline__ real cfl_rate(real ir, const real *v, real p, const r
 // Written out per component with w = v_n + sc:
 //   mass rho w;  momentum (rho w) v_k - B_n B_k (+ p_T along n);
 //   energy e w + p_T v_n - B_n (v.B);  induction B_k w - B_n v_k (k != n).
-template <typename real, int D>
-__device__ __forceinline__ void side_flux(const real *W, real hb2, real igm1, real sc, real *G) {
-  const real vn = W[1 + D], Bn = W[5 + D];
-  const real w = vn + sc;
-  const real v2 = W[1] * W[1] + W[2] * W[2] + W[3] * W[3];
-  const real pt = W[4] + hb2;
-  const real e = W[4] * igm1 + (real(0.5) * W[0] * v2 + hb2);
-  const real vB = W[1] * W[5] + W[2] * W[6] + W[3] * W[7];
+template <int D>
+__device__ __forceinline__ void side_flux(const double *W, double hb2, double igm1, double sc, double *G) {
+  const double vn = W[1 + D], Bn = W[5 + D];
+  const double w = vn + sc;
+  const double v2 = W[1] * W[1] + W[2] * W[2] + W[3] * W[3];
+  const double pt = W[4] + hb2;
+  const double e = W[4] * igm1 + (0.5 * W[0] * v2 + hb2);
+  const double vB = W[1] * W[5] + W[2] * W[6] + W[3] * W[7];
   G[0] = W[0] * w;
   G[1] = G[0] * W[1] - Bn * W[5];
   G[2] = G[0] * W[2] - Bn * W[6];
@@ -453,7 +451,7 @@ __device__ __forceinline__ void side_flux(const real *W, real hb2, real igm1, re
   G[1 + D] += pt;
   G[4] = e * w + pt * vn - Bn * vB;
 #pragma unroll
-  for (int k = 0; k < 3; k++) G[5 + k] = k == D ? real(0) : W[5 + k] * w - Bn * W[1 + k];
+  for (int k = 0; k < 3; k++) G[5 + k] = k == D ? 0.0 : W[5 + k] * w - Bn * W[1 + k];
 }
 
 // TVDLF flux from reconstructed face states WL | WR (primitive variables),
@@ -462,10 +460,10 @@ __device__ __forceinline__ void side_flux(const real *W, real hb2, real igm1, re
 // reconstructed density or pressure is not positive.  F2 receives TWICE the
 // numerical flux (the caller folds the 1/2 into its face areas); the normal
 // magnetic flux is zero.
-template <typename real, int D>
-__device__ __forceinline__ void tvdlf_states(real *WL, real *WR, const real *b, const real *c, real gamma,
-                                             real igm1, real *F2) {
-  if (!RT<real>::pos_(WL[0]) || !RT<real>::pos_(WL[4]) || !RT<real>::pos_(WR[0]) || !RT<real>::pos_(WR[4])) {
+template <int D>
+__device__ __forceinline__ void tvdlf_states(double *WL, double *WR, const double *b, const double *c, double gamma,
+                                             double igm1, double *F2) {
+  if (!RT<double>::pos_(WL[0]) || !RT<double>::pos_(WL[4]) || !RT<double>::pos_(WR[0]) || !RT<double>::pos_(WR[4])) {
 #pragma unroll
     for (int v = 0; v < NVAR; v++) {
       WL[v] = b[v];
@@ -473,17 +471,17 @@ __device__ __forceinline__ void tvdlf_states(real *WL, real *WR, const real *b, 
     }
   }
   constexpr int T1 = 5 + (D + 1) % 3, T2 = 5 + (D + 2) % 3;   // field across the direction
-  const real tL = WL[T1] * WL[T1] + WL[T2] * WL[T2], tR = WR[T1] * WR[T1] + WR[T2] * WR[T2];
-  const real hbL = real(0.5) * (WL[5 + D] * WL[5 + D] + tL), hbR = real(0.5) * (WR[5 + D] * WR[5 + D] + tR);
-  const real hg = real(0.5) * gamma;
-  const real cl = RT<real>::abs_(WL[1 + D]) + fast_speed_of(RT<real>::rcp_(WL[0]), gamma * WL[4], hg * WL[4], hbL, tL);
-  const real cr = RT<real>::abs_(WR[1 + D]) + fast_speed_of(RT<real>::rcp_(WR[0]), gamma * WR[4], hg * WR[4], hbR, tR);
-  const real cm = RT<real>::max_(cl, cr);
-  real GL[NVAR], GR[NVAR];
-  side_flux<real, D>(WL, hbL, igm1, cm, GL);
-  side_flux<real, D>(WR, hbR, igm1, -cm, GR);
-  axpy8<real>(GL, real(1), GR, F2);
-  F2[5 + D] = real(0);
+  const double tL = WL[T1] * WL[T1] + WL[T2] * WL[T2], tR = WR[T1] * WR[T1] + WR[T2] * WR[T2];
+  const double hbL = 0.5 * (WL[5 + D] * WL[5 + D] + tL), hbR = 0.5 * (WR[5 + D] * WR[5 + D] + tR);
+  const double hg = 0.5 * gamma;
+  const double cl = RT<double>::abs_(WL[1 + D]) + fast_speed_of(RT<double>::rcp_(WL[0]), gamma * WL[4], hg * WL[4], hbL, tL);
+  const double cr = RT<double>::abs_(WR[1 + D]) + fast_speed_of(RT<double>::rcp_(WR[0]), gamma * WR[4], hg * WR[4], hbR, tR);
+  const double cm = RT<double>::max_(cl, cr);
+  double GL[NVAR], GR[NVAR];
+  side_flux<D>(WL, hbL, igm1, cm, GL);
+  side_flux<D>(WR, hbR, igm1, -cm, GR);
+  axpy8<double>(GL, 1.0, GR, F2);
+  F2[5 + D] = 0.0;
 }
 
 // FP32 TVDLF flux (twice, see tvdlf_states) with the two face states in
@@ -493,46 +491,67 @@ __device__ __forceinline__ void tvdlf_states(real *WL, real *WR, const real *b, 
 // sides with the f32x2 instructions, each lane rounded as the scalar
 // operation, and the lanes are added at the end.  A face whose reconstructed
 // density or pressure is not positive takes the cell values.
+// D < 0: the direction is theta, or phi where `ph` is set (lanes of a warp may
+// differ); the operations on a face are those of its direction's instance.
 template <int D>
 __device__ __forceinline__ void tvdlf_pair(const float *b, const float *c, const float *hb, const float *hc,
-                                           float gamma, float igm1, float *F2) {
+                                           float gamma, float igm1, float *F2, bool ph = false) {
   float2 W[NVAR];
   // the fallback multiplies the half slopes by zero: no branch
   const float m = fminf(fminf(b[0] + hb[0], c[0] - hc[0]), fminf(b[4] + hb[4], c[4] - hc[4]));
   const float on = m > 0.f ? 1.f : 0.f;
 #pragma unroll
   for (int v = 0; v < NVAR; v++) W[v] = make_float2(fmaf(hb[v], on, b[v]), fmaf(-hc[v], on, c[v]));
-  const float2 half = make_float2(0.5f, 0.5f), m1 = make_float2(-1.f, -1.f);
-  constexpr int T1 = 5 + (D + 1) % 3, T2 = 5 + (D + 2) % 3;   // field across the direction
-  const float2 bt2 = __ffma2_rn(W[T2], W[T2], __fmul2_rn(W[T1], W[T1]));
-  const float2 hb2 = __fmul2_rn(half, __ffma2_rn(W[5 + D], W[5 + D], bt2));
-  // fast magnetosonic speed along D of both states (fast_speed_of)
+  const float2 half = make_float2(0.5f, 0.5f);
+  constexpr int N = D < 0 ? 1 : D;
+  float2 vn = W[1 + N], Bn = W[5 + N];   // normal components
+  if (D < 0) {
+    vn = ph ? W[3] : vn;
+    Bn = ph ? W[7] : Bn;
+  }
+  const float2 b2 = __ffma2_rn(W[7], W[7], __ffma2_rn(W[6], W[6], __fmul2_rn(W[5], W[5])));
+  // fast magnetosonic speed along D of both states (as fast_speed)
   const float2 ir = make_float2(RT<float>::rcp_(W[0].x), RT<float>::rcp_(W[0].y));
-  const float2 gp = __fmul2_rn(make_float2(gamma, gamma), __fmul2_rn(W[4], ir));
-  const float2 ga = __fmul2_rn(half, gp), gb = __fmul2_rn(hb2, ir), gd = __ffma2_rn(m1, gb, ga);
-  const float2 disc = __ffma2_rn(gd, gd, __fmul2_rn(gp, __fmul2_rn(bt2, ir)));
-  const float2 cf2 = __fadd2_rn(__fadd2_rn(ga, gb),
-                                make_float2(RT<float>::sqrt_(disc.x), RT<float>::sqrt_(disc.y)));
-  const float cm = fmaxf(fabsf(W[1 + D].x) + RT<float>::sqrt_(cf2.x), fabsf(W[1 + D].y) + RT<float>::sqrt_(cf2.y));
+  const float2 a2 = __fmul2_rn(__fmul2_rn(make_float2(gamma, gamma), W[4]), ir);
+  const float2 bt2 = __fmul2_rn(b2, ir);
+  const float2 bn2 = __fmul2_rn(__fmul2_rn(Bn, Bn), ir);
+  const float2 sum = __fadd2_rn(a2, bt2);
+  float2 disc = __ffma2_rn(sum, sum, __fmul2_rn(__fmul2_rn(make_float2(-4.f, -4.f), a2), bn2));
+  disc.x = fmaxf(disc.x, 0.f);
+  disc.y = fmaxf(disc.y, 0.f);
+  const float2 cf2 =
+      __fmul2_rn(half, __fadd2_rn(sum, make_float2(RT<float>::sqrt_(disc.x), RT<float>::sqrt_(disc.y))));
+  const float cm = fmaxf(fabsf(vn.x) + RT<float>::sqrt_(cf2.x), fabsf(vn.y) + RT<float>::sqrt_(cf2.y));
   // per-side flux with w = v_n + c_max on the left, v_n - c_max on the right
-  const float2 vn = W[1 + D], nBn = __fmul2_rn(W[5 + D], m1);
+  const float2 nBn = __fmul2_rn(Bn, make_float2(-1.f, -1.f));
   const float2 w = __fadd2_rn(vn, make_float2(cm, -cm));
-  const float2 v2 = __ffma2_rn(W[3], W[3], __ffma2_rn(W[2], W[2], __fmul2_rn(W[1], W[1])));
-  const float2 pt = __fadd2_rn(hb2, W[4]);
-  const float2 en = __ffma2_rn(W[4], make_float2(igm1, igm1), __ffma2_rn(__fmul2_rn(half, W[0]), v2, hb2));
+  const float2 m1 = __fmul2_rn(W[0], W[1]), m2 = __fmul2_rn(W[0], W[2]), m3 = __fmul2_rn(W[0], W[3]);
+  const float2 rv2 = __ffma2_rn(m3, W[3], __ffma2_rn(m2, W[2], __fmul2_rn(m1, W[1])));
+  const float2 pt = __ffma2_rn(half, b2, W[4]);
+  const float2 en = __ffma2_rn(W[4], make_float2(igm1, igm1), __fmul2_rn(half, __fadd2_rn(rv2, b2)));
   const float2 vB = __ffma2_rn(W[3], W[7], __ffma2_rn(W[2], W[6], __fmul2_rn(W[1], W[5])));
   float2 G[NVAR];
   G[0] = __fmul2_rn(W[0], w);
-  G[1] = __ffma2_rn(G[0], W[1], __fmul2_rn(nBn, W[5]));
-  G[2] = __ffma2_rn(G[0], W[2], __fmul2_rn(nBn, W[6]));
-  G[3] = __ffma2_rn(G[0], W[3], __fmul2_rn(nBn, W[7]));
-  G[1 + D] = __fadd2_rn(G[1 + D], pt);
+  G[1] = __ffma2_rn(m1, w, __fmul2_rn(nBn, W[5]));
+  G[2] = __ffma2_rn(m2, w, __fmul2_rn(nBn, W[6]));
+  G[3] = __ffma2_rn(m3, w, __fmul2_rn(nBn, W[7]));
+  if (D < 0) {
+    const float2 gt = __fadd2_rn(G[2], pt), gp = __fadd2_rn(G[3], pt);
+    G[2] = ph ? G[2] : gt;
+    G[3] = ph ? gp : G[3];
+  } else {
+    G[1 + N] = __fadd2_rn(G[1 + N], pt);
+  }
   G[4] = __ffma2_rn(en, w, __ffma2_rn(pt, vn, __fmul2_rn(nBn, vB)));
 #pragma unroll
   for (int k = 0; k < 3; k++)
     if (k != D) G[5 + k] = __ffma2_rn(W[5 + k], w, __fmul2_rn(nBn, W[1 + k]));
 #pragma unroll
-  for (int v = 0; v < NVAR; v++) F2[v] = v == 5 + D ? 0.f : G[v].x + G[v].y;
+  for (int v = 0; v < NVAR; v++) F2[v] = D >= 0 && v == 5 + D ? 0.f : G[v].x + G[v].y;
+  if (D < 0) {
+    F2[6] = ph ? F2[6] : 0.f;
+    F2[7] = ph ? 0.f : F2[7];
+  }
 }
 
 // TVDLF face flux (twice, see tvdlf_states) from the four cells a, b | c, e
@@ -540,7 +559,7 @@ __device__ __forceinline__ void tvdlf_pair(const float *b, const float *c, const
 // both half slopes, then tvdlf_pair.
 template <typename real, int D>
 __device__ __forceinline__ void tvdlf_face(const real *a, const real *b, const real *c, const real *e,
-                                           real gamma, real igm1, real *F2) {
+                                           real gamma, real igm1, real *F2, bool ph = false) {
   if constexpr (sizeof(real) == 4) {
     float hb[NVAR], hc[NVAR];
 #pragma unroll
@@ -556,15 +575,18 @@ __device__ __forceinline__ void tvdlf_face(const real *a, const real *b, const r
       hc[v] = half_mc_signed(d2.x, d3.x, s2.x);
       hc[v + 1] = half_mc_signed(d2.y, d3.y, s2.y);
     }
-    tvdlf_pair<D>(b, c, hb, hc, gamma, igm1, F2);
+    tvdlf_pair<D>(b, c, hb, hc, gamma, igm1, F2, ph);
     return;
   }
-  real sb[NVAR], sc[NVAR], WL[NVAR], WR[NVAR];
-  mc_half_slopes8<real>(a, b, c, sb);
-  mc_half_slopes8<real>(b, c, e, sc);
-  axpy8<real>(b, real(1), sb, WL);
-  axpy8<real>(c, real(-1), sc, WR);
-  tvdlf_states<real, D>(WL, WR, b, c, gamma, igm1, F2);
+  if constexpr (sizeof(real) == 8) {
+    static_assert(D >= 0);
+    real sb[NVAR], sc[NVAR], WL[NVAR], WR[NVAR];
+    mc_half_slopes8<real>(a, b, c, sb);
+    mc_half_slopes8<real>(b, c, e, sc);
+    axpy8<real>(b, real(1), sb, WL);
+    axpy8<real>(c, real(-1), sc, WR);
+    tvdlf_states<D>(WL, WR, b, c, gamma, igm1, F2);
+  }
 }
 
 // asynchronous global -> shared copies of 8 or 16 bytes (cp.async)
