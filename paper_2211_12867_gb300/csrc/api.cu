@@ -169,13 +169,13 @@ Layout make_layout(const icarus_grid_desc *d) {
   L.probe_in = L.add(4096 * 3 * sizeof(double));
   L.probe_out = L.add(4096 * NVAR * sizeof(double));
   // learned pre-flagger: parameters, gradient and Adam moments (4 x n), leaf
-  // features and probabilities, training set, batch activations
+  // features and probabilities, training set, partial gradients of a batch
   L.mlp_par = L.add((size_t)4 * mlp_n_params() * sizeof(float) + 64);
   L.mlp_feat = L.add(mb * (64 + 1) * sizeof(float));
   L.mlp_X = L.add((size_t)MLP_CAP * 64 * sizeof(float));
   L.mlp_T = L.add((size_t)MLP_CAP * sizeof(float));
   L.mlp_idx = L.add((size_t)MLP_CAP * sizeof(int));
-  L.mlp_act = L.add((size_t)MLP_BMAX * (4 * 128 + 2) * sizeof(float));
+  L.mlp_act = L.add((MLP_BMAX + mlp_partial_floats()) * sizeof(float));   // outputs, partial gradients
   L.mlp_xin = L.add((size_t)MLP_BMAX * 65 * sizeof(float));
   return L;
 }
@@ -284,9 +284,8 @@ struct icarus_ctx {
   int kernels_per_step = 0;
   // learned pre-flagger
   float *mlp_theta = nullptr, *mlp_grad = nullptr, *mlp_m = nullptr, *mlp_v = nullptr, *mlp_loss = nullptr;
-  float *mlp_feat = nullptr, *mlp_prob = nullptr, *mlp_X = nullptr, *mlp_T = nullptr, *mlp_h1 = nullptr,
-        *mlp_h2 = nullptr, *mlp_dh2 = nullptr, *mlp_dh1 = nullptr, *mlp_y = nullptr, *mlp_dz = nullptr,
-        *mlp_xin = nullptr, *mlp_tin = nullptr;
+  float *mlp_feat = nullptr, *mlp_prob = nullptr, *mlp_X = nullptr, *mlp_T = nullptr, *mlp_y = nullptr,
+        *mlp_part = nullptr, *mlp_xin = nullptr, *mlp_tin = nullptr;
   int *mlp_idx = nullptr;
   int mlp_n = 0, mlp_step = 0;
   bool mlp_ready = false;
@@ -875,7 +874,7 @@ bool tile_settable(const icarus_ctx *c, int tj, int tk) {
 struct StageCost {
   double cW, cL, cX, c0, a, lat, aL;
 };
-constexpr StageCost COST32 = {0.398, 0.009, 0.142, 0.224, 2.15, 4.79, 2.62},
+constexpr StageCost COST32 = {0.4485, 0.0, 0.158, 0.1985, 2.105, 5.07, 2.66},
                     COST64 = {12.47, 0.972, 0.0, 6.40, 0.438, 68.1, 0.523};
 
 // the model's cost of a plane of each instantiated tile on this context's
@@ -1051,8 +1050,7 @@ void mlp_leaf_probabilities(icarus_ctx *c) {
   mlp_features_launch(c->kp, c->U, c->prec, 0, c->nleaves, c->mlp_feat, c->stream);
   for (int b0 = 0; b0 < c->nleaves; b0 += MLP_BMAX) {
     const int B = std::min(MLP_BMAX, c->nleaves - b0);
-    mlp_forward_launch(c->mlp_theta, c->mlp_feat + (size_t)b0 * 64, nullptr, B, c->mlp_h1, c->mlp_h2,
-                       c->mlp_prob + b0, c->stream);
+    mlp_forward_launch(c->mlp_theta, c->mlp_feat + (size_t)b0 * 64, nullptr, B, c->mlp_prob + b0, c->stream);
   }
 }
 
@@ -1231,13 +1229,8 @@ icarus_status icarus_init_grid(const icarus_grid_desc *desc, icarus_ctx **out) {
     c->mlp_X = at<float>(c, lay.mlp_X);
     c->mlp_T = at<float>(c, lay.mlp_T);
     c->mlp_idx = at<int>(c, lay.mlp_idx);
-    float *act = at<float>(c, lay.mlp_act);
-    c->mlp_h1 = act;
-    c->mlp_h2 = act + (size_t)MLP_BMAX * 128;
-    c->mlp_dh2 = act + (size_t)2 * MLP_BMAX * 128;
-    c->mlp_dh1 = act + (size_t)3 * MLP_BMAX * 128;
-    c->mlp_y = act + (size_t)4 * MLP_BMAX * 128;
-    c->mlp_dz = c->mlp_y + MLP_BMAX;
+    c->mlp_y = at<float>(c, lay.mlp_act);
+    c->mlp_part = c->mlp_y + MLP_BMAX;
     c->mlp_xin = at<float>(c, lay.mlp_xin);
     c->mlp_tin = c->mlp_xin + (size_t)MLP_BMAX * 64;
   }
@@ -2088,7 +2081,7 @@ icarus_status icarus_mlp_predict(icarus_ctx *c, const float *x_host, int n, floa
   if (!c || !x_host || !y_host || n < 0 || n > MLP_BMAX) return ICARUS_ERR_ARG;
   if (!c->mlp_ready) return ICARUS_ERR_STATE;
   CK(cudaMemcpyAsync(c->mlp_xin, x_host, sizeof(float) * 64 * n, cudaMemcpyHostToDevice, c->stream));
-  mlp_forward_launch(c->mlp_theta, c->mlp_xin, nullptr, n, c->mlp_h1, c->mlp_h2, c->mlp_y, c->stream);
+  mlp_forward_launch(c->mlp_theta, c->mlp_xin, nullptr, n, c->mlp_y, c->stream);
   CK(cudaPeekAtLastError());
   CK(cudaMemcpyAsync(y_host, c->mlp_y, sizeof(float) * n, cudaMemcpyDeviceToHost, c->stream));
   CK(cudaStreamSynchronize(c->stream));
@@ -2102,9 +2095,7 @@ icarus_status icarus_mlp_grad(icarus_ctx *c, const float *x_host, const float *t
   CK(cudaMemcpyAsync(c->mlp_xin, x_host, sizeof(float) * 64 * n, cudaMemcpyHostToDevice, c->stream));
   CK(cudaMemcpyAsync(c->mlp_tin, t_host, sizeof(float) * n, cudaMemcpyHostToDevice, c->stream));
   CK(cudaMemsetAsync(c->mlp_loss, 0, sizeof(float), c->stream));
-  mlp_forward_launch(c->mlp_theta, c->mlp_xin, nullptr, n, c->mlp_h1, c->mlp_h2, c->mlp_y, c->stream);
-  mlp_backward_launch(c->mlp_theta, c->mlp_xin, c->mlp_tin, nullptr, n, c->mlp_h1, c->mlp_h2, c->mlp_y, c->mlp_dz,
-                      c->mlp_dh2, c->mlp_dh1, c->mlp_grad, c->mlp_loss, c->stream);
+  mlp_grad_launch(c->mlp_theta, c->mlp_xin, c->mlp_tin, nullptr, n, c->mlp_part, c->mlp_grad, c->mlp_loss, c->stream);
   CK(cudaPeekAtLastError());
   CK(cudaMemcpyAsync(grad_host, c->mlp_grad, sizeof(float) * mlp_n_params(), cudaMemcpyDeviceToHost, c->stream));
   float l = 0.f;
@@ -2148,10 +2139,8 @@ icarus_status icarus_mlp_train(icarus_ctx *c, int n_train, int epochs, int batch
     for (int b0 = 0; b0 < n_train; b0 += batch) {
       const int B = std::min(batch, n_train - b0);
       const int *idx = c->mlp_idx + b0;
-      mlp_forward_launch(c->mlp_theta, c->mlp_X, idx, B, c->mlp_h1, c->mlp_h2, c->mlp_y, c->stream);
-      mlp_backward_launch(c->mlp_theta, c->mlp_X, c->mlp_T, idx, B, c->mlp_h1, c->mlp_h2, c->mlp_y, c->mlp_dz,
-                          c->mlp_dh2, c->mlp_dh1, c->mlp_grad, c->mlp_loss, c->stream);
-      mlp_adam_launch(c->mlp_theta, c->mlp_grad, c->mlp_m, c->mlp_v, (float)lr, ++c->mlp_step, c->stream);
+      mlp_step_launch(c->mlp_theta, c->mlp_m, c->mlp_v, c->mlp_X, c->mlp_T, idx, B, c->mlp_part, c->mlp_loss, (float)lr,
+                      ++c->mlp_step, c->stream);
     }
     CK(cudaPeekAtLastError());
     float l = 0.f;

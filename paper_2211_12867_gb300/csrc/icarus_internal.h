@@ -199,12 +199,16 @@ void vbg_launch(const KParams &kp, const void *U, int precision, int member, int
 int mlp_n_params();
 void mlp_features_launch(const KParams &kp, const void *U, int precision, int slot0, int nslots, float *out,
                          cudaStream_t s);
-void mlp_forward_launch(const float *theta, const float *X, const int *idx, int B, float *h1, float *h2, float *y,
-                        cudaStream_t s);
-void mlp_backward_launch(const float *theta, const float *X, const float *T, const int *idx, int B,
-                         const float *h1, const float *h2, const float *y, float *dz, float *dh2, float *dh1,
-                         float *grad, float *loss, cudaStream_t s);
-void mlp_adam_launch(float *theta, const float *g, float *m, float *v, float lr, int step, cudaStream_t s);
+void mlp_forward_launch(const float *theta, const float *X, const int *idx, int B, float *y, cudaStream_t s);
+// partial gradients of at most MLP_MAX_CTAS CTAs
+constexpr int MLP_MAX_CTAS = 152;
+size_t mlp_partial_floats();
+// gradient of the mean cross-entropy; the summed cross-entropy adds to *loss
+void mlp_grad_launch(const float *theta, const float *X, const float *T, const int *idx, int B, float *part, float *grad,
+                     float *loss, cudaStream_t s);
+// the same and the Adam step with it
+void mlp_step_launch(float *theta, float *m, float *v, const float *X, const float *T, const int *idx, int B, float *part,
+                     float *loss, float lr, int step, cudaStream_t s);
 void mlp_combine_launch(const float *prob, const DevBlock *blk, signed char *flags, int n, cudaStream_t s);
 
 struct icarus_ctx;

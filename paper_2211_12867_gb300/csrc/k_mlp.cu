@@ -5,11 +5,16 @@
 // index-space gradient magnitude of density, radial speed and pressure, each
 // divided by the cell's magnitude, averaged over the three variables and over
 // 4 x 4 x 4 sub-cubes -> 64 inputs; MLP 64 -> 128 (ReLU) -> 128 (ReLU) -> 1
-// (sigmoid); binary cross-entropy; Adam.  FP32 storage and accumulation.  The
-// layers are tiny (batch x 128 x 128), so they are plain FMA loops: one thread
-// per hidden unit in the forward and backward vectors, one thread per
-// parameter for the weight gradients (a fixed-order sum over the batch, so the
-// gradient is deterministic).
+// (sigmoid); binary cross-entropy; Adam.  FP32 storage and accumulation.
+//
+// A training batch is two launches.  k_mlp holds both weight matrices in shared
+// memory and takes groups of 8 samples through the forward pass, the backward
+// pass and the outer products of the weight gradients, which stay in registers
+// (96 per thread) until the CTA has done its groups; k_reduce adds the CTAs'
+// partial gradients in a fixed order (the gradient is the same bits on every
+// call) and takes the Adam step.  Four launches with the activations in global
+// memory and one thread per parameter summing over the batch took 120 us for
+// a batch of 1024, latency all of it (50 MFLOP).
 #include "mhd_device.cuh"
 
 #define MLP_IN 64
@@ -32,179 +37,325 @@ __host__ __device__ inline MlpView mlp_view(const float *th) {
   return m;
 }
 
-// One warp per sub-cube (4 x 4 x 4 sub-cubes of s0 x s1 x s2 cells with
-// s = n / 4; cells past 4 s in a direction belong to none): the lanes take
-// the sub-cube's cells in a fixed stride, add in FP64 and reduce in a fixed
-// shuffle tree, so the features are the same bits on every run and for
-// every member.
+// rho, v_r and p of a cell in FP64
 template <typename real>
-__global__ void k_features(const KParams kp, const real *U, int slot0, float *out) {
+__device__ __forceinline__ void feature_prims(const KParams &kp, const real *U, int slot, int i, int j, int k, double *w) {
+  real u[NVAR];
+  ld_cell(U + cell_index(kp, slot, i, j, k), u);
+  const double r = widen(u[0]), m1 = widen(u[1]), m2 = widen(u[2]), m3 = widen(u[3]);
+  const double b1 = widen(u[5]), b2 = widen(u[6]), b3 = widen(u[7]);
+  const double ir = RT<double>::rcp_(r);
+  w[0] = r;
+  w[1] = m1 * ir;
+  w[2] = (kp.gamma - 1.0) * fma(-0.5, (m1 * m1 + m2 * m2 + m3 * m3) * ir + (b1 * b1 + b2 * b2 + b3 * b3), widen(u[4]));
+}
+
+// Sum over the three primitives of the index-space gradient magnitude over the
+// cell's magnitude: w0 the cell, d the differences of its neighbours per
+// direction and primitive
+__device__ __forceinline__ double feature_of(const double *w0, const double (*d)[3]) {
+  double g = 0.0;
+#pragma unroll
+  for (int q = 0; q < 3; q++) {
+    const double s = d[0][q] * d[0][q] + d[1][q] * d[1][q] + d[2][q] * d[2][q];
+    g += RT<double>::sqrt_(s) * RT<double>::rcp_(fabs(w0[q]) + 1e-30);
+  }
+  return g;   // of doubled differences: the caller divides by 2 and by 3
+}
+
+// Features of 4 x 4 x 4 sub-cubes of s0 x s1 x s2 cells with s = n / 4.  One
+// CTA per leaf marches along r with the primitives of three planes (and one
+// halo cell around them) in shared memory, so a cell is converted 1.6 times
+// (12^3 block) instead of 7: the FP64 pipe bounds this kernel (one instruction
+// of a warp per 19 cycles of an SM, conversions from FP32 included), with 72
+// such instructions a cell instead of 400.  12^3 blocks, 808 leaves, ghost fill
+// included: 1283 ->
+// 389 us.  Each column sums its cells along r, then one warp per sub-cube its
+// columns in a fixed lane stride and shuffle tree, all in FP64: the features
+// are the same bits on every run and for every member.
+template <typename real>
+__global__ void __launch_bounds__(256) k_features(const KParams kp, const real *U, int slot0, float *out) {
+  extern __shared__ double smd[];
   const int slot = slot0 + blockIdx.x;
-  const int n0 = kp.nb[0], n1 = kp.nb[1], n2 = kp.nb[2];
-  const int s0 = n0 / 4, s1 = n1 / 4, s2 = n2 / 4, per = s0 * s1 * s2;
-  const double gm1 = kp.gamma - 1.0;
-  auto prims = [&](int i, int j, int k, double *w) {  // rho, v_r, p
-    real u[NVAR];
-    ld_cell(U + cell_index(kp, slot, i, j, k), u);
-    const double r = u[0], m1 = u[1], m2 = u[2], m3 = u[3], b1 = u[5], b2 = u[6], b3 = u[7];
-    w[0] = r;
-    w[1] = m1 / r;
-    w[2] = gm1 * ((double)u[4] - 0.5 * (m1 * m1 + m2 * m2 + m3 * m3) / r - 0.5 * (b1 * b1 + b2 * b2 + b3 * b3));
+  const int n1 = kp.nb[1], n2 = kp.nb[2], h2 = n2 + 2, H = (n1 + 2) * h2;
+  const int s0 = kp.nb[0] / 4, s1 = n1 / 4, s2 = n2 / 4, per = s0 * s1 * s2;
+  double *acc = smd + 9 * H;   // [ring plane][primitive][cell], then per column
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  auto plane = [&](int i) {   // primitives of padded plane i
+    double *P = smd + (i % 3) * 3 * H;
+    for (int c = threadIdx.x; c < H; c += blockDim.x) {
+      double w[3];
+      feature_prims(kp, U, slot, i, NGH - 1 + c / h2, NGH - 1 + c % h2, w);
+      P[c] = w[0];
+      P[H + c] = w[1];
+      P[2 * H + c] = w[2];
+    }
   };
+  plane(NGH - 1);
+  plane(NGH);
+  for (int a = 0; a < 4; a++) {
+    for (int t = threadIdx.x; t < n1 * n2; t += blockDim.x) acc[t] = 0.0;
+    for (int i = NGH + a * s0; i < NGH + (a + 1) * s0; i++) {
+      plane(i + 1);
+      __syncthreads();
+      const double *Pm = smd + ((i - 1) % 3) * 3 * H, *P = smd + (i % 3) * 3 * H, *Pp = smd + ((i + 1) % 3) * 3 * H;
+      for (int t = threadIdx.x; t < n1 * n2; t += blockDim.x) {
+        const int c = (t / n2 + 1) * h2 + t % n2 + 1;
+        double w0[3], d[3][3];
+#pragma unroll
+        for (int q = 0; q < 3; q++) {
+          w0[q] = P[q * H + c];
+          d[0][q] = Pp[q * H + c] - Pm[q * H + c];
+          d[1][q] = P[q * H + c + h2] - P[q * H + c - h2];
+          d[2][q] = P[q * H + c + 1] - P[q * H + c - 1];
+        }
+        acc[t] += feature_of(w0, d);
+      }
+      __syncthreads();   // plane i - 1 is read no more
+    }
+    for (int sc = warp; sc < 16; sc += (int)blockDim.x >> 5) {
+      const int b = sc / 4, cc = sc % 4;
+      double s = 0.0;
+      for (int t = lane; t < s1 * s2; t += 32) s += acc[(b * s1 + t / s2) * n2 + cc * s2 + t % s2];
+      for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+      if (lane == 0) out[(size_t)blockIdx.x * 64 + a * 16 + sc] = (float)(s / (6.0 * per));
+    }
+    __syncthreads();
+  }
+}
+
+// The same features where three planes do not fit in shared memory: one warp
+// per sub-cube, every cell converting its six neighbours.
+template <typename real>
+__global__ void __launch_bounds__(256) k_features_large(const KParams kp, const real *U, int slot0, float *out) {
+  const int slot = slot0 + blockIdx.x;
+  const int s0 = kp.nb[0] / 4, s1 = kp.nb[1] / 4, s2 = kp.nb[2] / 4, per = s0 * s1 * s2;
   const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
   for (int sc = threadIdx.x >> 5; sc < 64; sc += nw) {
     const int a = sc / 16, b = (sc / 4) % 4, cc = sc % 4;
     double acc = 0.0;
     for (int t = lane; t < per; t += 32) {
-      const int i = a * s0 + t / (s1 * s2), j = b * s1 + (t / s2) % s1, k = cc * s2 + t % s2;
-      const int p0 = i + NGH, p1 = j + NGH, p2 = k + NGH;
-      double w0[3], wm[3][3], wp[3][3];
-      prims(p0, p1, p2, w0);
-      prims(p0 - 1, p1, p2, wm[0]);
-      prims(p0 + 1, p1, p2, wp[0]);
-      prims(p0, p1 - 1, p2, wm[1]);
-      prims(p0, p1 + 1, p2, wp[1]);
-      prims(p0, p1, p2 - 1, wm[2]);
-      prims(p0, p1, p2 + 1, wp[2]);
-      double g = 0.0;
-      for (int q = 0; q < 3; q++) {
-        double s = 0.0;
-        for (int d = 0; d < 3; d++) {
-          const double cd = 0.5 * (wp[d][q] - wm[d][q]);
-          s += cd * cd;
-        }
-        g += sqrt(s) / (fabs(w0[q]) + 1e-30);
+      const int p0 = NGH + a * s0 + t / (s1 * s2), p1 = NGH + b * s1 + (t / s2) % s1, p2 = NGH + cc * s2 + t % s2;
+      double w0[3], d[3][3];
+      feature_prims(kp, U, slot, p0, p1, p2, w0);
+#pragma unroll
+      for (int e = 0; e < 3; e++) {
+        double wm[3], wp[3];
+        feature_prims(kp, U, slot, p0 - (e == 0), p1 - (e == 1), p2 - (e == 2), wm);
+        feature_prims(kp, U, slot, p0 + (e == 0), p1 + (e == 1), p2 + (e == 2), wp);
+#pragma unroll
+        for (int q = 0; q < 3; q++) d[e][q] = wp[q] - wm[q];
       }
-      acc += g / 3.0;
+      acc += feature_of(w0, d);
     }
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (lane == 0) out[(size_t)blockIdx.x * 64 + sc] = (float)(acc / per);
+    if (lane == 0) out[(size_t)blockIdx.x * 64 + sc] = (float)(acc / (6.0 * per));
   }
 }
 
-// forward over rows of X (row index list `idx` or identity), 4 samples per CTA
-constexpr int SPC = 4;
-__global__ void k_forward(const float *theta, const float *X, const int *idx, int B, float *h1g, float *h2g,
-                          float *y) {
-  __shared__ float xs[SPC][MLP_IN];
-  __shared__ float hs[SPC][MLP_H];
-  __shared__ float red[SPC][MLP_H / 32];
-  const MlpView m = mlp_view(theta);
-  const int s0 = blockIdx.x * SPC, j = threadIdx.x;
-  for (int e = j; e < SPC * MLP_IN; e += MLP_H) {
-    const int s = e / MLP_IN, i = e % MLP_IN;
-    const int row = s0 + s < B ? (idx ? idx[s0 + s] : s0 + s) : -1;
-    xs[s][i] = row >= 0 ? X[(size_t)row * MLP_IN + i] : 0.f;
-  }
-  __syncthreads();
-  float a[SPC];
-  for (int s = 0; s < SPC; s++) a[s] = m.b1[j];
-  for (int i = 0; i < MLP_IN; i++) {
-    const float wv = m.W1[j * MLP_IN + i];
-    for (int s = 0; s < SPC; s++) a[s] = fmaf(wv, xs[s][i], a[s]);
-  }
-  for (int s = 0; s < SPC; s++) {
-    const float h = fmaxf(a[s], 0.f);
-    hs[s][j] = h;
-    if (s0 + s < B) h1g[(size_t)(s0 + s) * MLP_H + j] = h;
-  }
-  __syncthreads();
-  for (int s = 0; s < SPC; s++) a[s] = m.b2[j];
-  for (int k = 0; k < MLP_H; k++) {
-    const float wv = m.W2[j * MLP_H + k];
-    for (int s = 0; s < SPC; s++) a[s] = fmaf(wv, hs[s][k], a[s]);
-  }
-  float z[SPC];
-  for (int s = 0; s < SPC; s++) {
-    const float h = fmaxf(a[s], 0.f);
-    if (s0 + s < B) h2g[(size_t)(s0 + s) * MLP_H + j] = h;
-    z[s] = m.w3[j] * h;
-  }
-  for (int s = 0; s < SPC; s++) {
-    float v = z[s];
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if ((j & 31) == 0) red[s][j / 32] = v;
-  }
-  __syncthreads();
-  if (j < SPC && s0 + j < B) {
-    float zz = m.b3[0];
-    for (int w = 0; w < MLP_H / 32; w++) zz += red[j][w];
-    y[s0 + j] = 1.f / (1.f + expf(-zz));
-  }
-}
+constexpr int NT = 256;          // threads of k_mlp
+constexpr int GS = 8;            // samples of a group: two quads
+constexpr int S1 = MLP_IN + 1, S2 = MLP_H + 1;   // row strides in shared memory (no bank conflicts by row or column)
+constexpr int NPAR = MLP_H * MLP_IN + MLP_H + MLP_H * MLP_H + MLP_H + MLP_H + 1;
+constexpr int PART = NPAR + 1;   // a CTA's partial gradient and loss
+constexpr int MLP_SMEM = (MLP_H * S1 + MLP_H * S2 + GS * (MLP_IN + 3 * MLP_H) + GS * (NT / 32) + 2 * GS) * 4;
 
-// per-sample backward vectors; loss accumulates the summed cross-entropy
-__global__ void k_backvec(const float *theta, const float *T, const int *idx, int B, const float *h1g,
-                          const float *h2g, const float *y, float *dz, float *dh2g, float *dh1g, float *loss) {
-  __shared__ float d2[SPC][MLP_H];
+// Forward pass of the rows of X (row index list `idx` or identity), and with
+// GRAD the gradient of the mean cross-entropy over the batch: every CTA's share
+// of it, and of the summed cross-entropy, to part[CTA].  Per group a thread
+// has one hidden unit and one quad of samples; vectors over units lie in
+// shared memory as [quad][unit][4], so a weight meets four samples per load.
+// The weight gradients are 8 x 8 and 8 x 4 tiles of outer products per thread.
+template <bool GRAD>
+__global__ void __launch_bounds__(NT) k_mlp(const float *theta, const float *X, const float *T, const int *idx, int B,
+                                            float *y, float *part) {
+  extern __shared__ __align__(16) float sm[];
+  float *xs = sm, *h1s = xs + GS * MLP_IN, *d2s = h1s + GS * MLP_H, *d1s = d2s + GS * MLP_H;
+  float *red = d1s + GS * MLP_H, *dzs = red + GS * (NT / 32), *W1s = dzs + 2 * GS, *W2s = W1s + MLP_H * S1;
   const MlpView m = mlp_view(theta);
-  const int s0 = blockIdx.x * SPC, k = threadIdx.x;
-  for (int s = 0; s < SPC; s++) {
-    const int b = s0 + s;
-    float dzz = 0.f;
-    if (b < B) {
-      const float t = T[idx ? idx[b] : b];
-      dzz = (y[b] - t) / (float)B;
-      if (k == 0) {
-        dz[b] = dzz;
-        const float yc = fminf(fmaxf(y[b], 1e-7f), 1.f - 1e-7f);
-        atomicAdd(loss, -(t * logf(yc) + (1.f - t) * logf(1.f - yc)));
-      }
-      const float v = h2g[(size_t)b * MLP_H + k] > 0.f ? dzz * m.w3[k] : 0.f;
-      d2[s][k] = v;
-      dh2g[(size_t)b * MLP_H + k] = v;
-    } else {
-      d2[s][k] = 0.f;
+  const int tid = threadIdx.x, j = tid & (MLP_H - 1), q = tid >> 7, warp = tid >> 5;
+  for (int e = tid; e < MLP_H * MLP_IN; e += NT) W1s[(e / MLP_IN) * S1 + e % MLP_IN] = m.W1[e];
+  for (int e = tid; e < MLP_H * MLP_H; e += NT) W2s[(e / MLP_H) * S2 + e % MLP_H] = m.W2[e];
+  const float b1 = m.b1[j], b2 = m.b2[j], w3 = m.w3[j], b3 = m.b3[0];
+  const int tj = tid >> 4, tk = tid & 15;   // gradient tile: rows tj + 16 a, columns tk + 16 b
+  float g2[8][8], g1[8][4], gb1 = 0.f, gb2 = 0.f, gw3 = 0.f, gb3 = 0.f, loss = 0.f;
+  if (GRAD) {
+#pragma unroll
+    for (int a = 0; a < 8; a++) {
+#pragma unroll
+      for (int b = 0; b < 8; b++) g2[a][b] = 0.f;
+#pragma unroll
+      for (int b = 0; b < 4; b++) g1[a][b] = 0.f;
     }
   }
-  __syncthreads();
-  float acc[SPC];
-  for (int s = 0; s < SPC; s++) acc[s] = 0.f;
-  for (int j = 0; j < MLP_H; j++) {
-    const float wv = m.W2[j * MLP_H + k];
-    for (int s = 0; s < SPC; s++) acc[s] = fmaf(wv, d2[s][j], acc[s]);
+  auto quad = [](const float *v, int n, int unit, int qd) -> float4 {
+    return *reinterpret_cast<const float4 *>(v + (qd * n + unit) * 4);
+  };
+  for (int s0 = blockIdx.x * GS; s0 < B; s0 += gridDim.x * GS) {
+    __syncthreads();   // the previous group's vectors (and, first, the weights)
+    for (int e = tid; e < GS * MLP_IN; e += NT) {
+      const int s = e / MLP_IN, i = e % MLP_IN;
+      const int row = s0 + s < B ? (idx ? idx[s0 + s] : s0 + s) : -1;
+      xs[((s >> 2) * MLP_IN + i) * 4 + (s & 3)] = row >= 0 ? X[(size_t)row * MLP_IN + i] : 0.f;
+    }
+    __syncthreads();
+    float a0 = b1, a1 = b1, a2 = b1, a3 = b1;
+#pragma unroll 8
+    for (int i = 0; i < MLP_IN; i++) {
+      const float w = W1s[j * S1 + i];
+      const float4 x = quad(xs, MLP_IN, i, q);
+      a0 = fmaf(w, x.x, a0);
+      a1 = fmaf(w, x.y, a1);
+      a2 = fmaf(w, x.z, a2);
+      a3 = fmaf(w, x.w, a3);
+    }
+    const float4 h1 = make_float4(fmaxf(a0, 0.f), fmaxf(a1, 0.f), fmaxf(a2, 0.f), fmaxf(a3, 0.f));
+    *reinterpret_cast<float4 *>(h1s + (q * MLP_H + j) * 4) = h1;
+    __syncthreads();
+    a0 = a1 = a2 = a3 = b2;
+#pragma unroll 8
+    for (int k = 0; k < MLP_H; k++) {
+      const float w = W2s[j * S2 + k];
+      const float4 x = quad(h1s, MLP_H, k, q);
+      a0 = fmaf(w, x.x, a0);
+      a1 = fmaf(w, x.y, a1);
+      a2 = fmaf(w, x.z, a2);
+      a3 = fmaf(w, x.w, a3);
+    }
+    const float4 h2 = make_float4(fmaxf(a0, 0.f), fmaxf(a1, 0.f), fmaxf(a2, 0.f), fmaxf(a3, 0.f));
+    float z[4] = {w3 * h2.x, w3 * h2.y, w3 * h2.z, w3 * h2.w};
+#pragma unroll
+    for (int s = 0; s < 4; s++) {
+      for (int o = 16; o > 0; o >>= 1) z[s] += __shfl_xor_sync(0xffffffffu, z[s], o);
+      if ((tid & 31) == 0) red[s * (NT / 32) + warp] = z[s];
+    }
+    __syncthreads();
+    if (tid < GS) {
+      float zz = b3, dz = 0.f;
+      for (int w = 0; w < MLP_H / 32; w++) zz += red[(tid & 3) * (NT / 32) + (tid >> 2) * (MLP_H / 32) + w];
+      if (s0 + tid < B) {
+        const float yy = 1.f / (1.f + expf(-zz));
+        if (y) y[s0 + tid] = yy;
+        if (GRAD) {
+          const float t = T[idx ? idx[s0 + tid] : s0 + tid];
+          dz = (yy - t) / (float)B;
+          const float yc = fminf(fmaxf(yy, 1e-7f), 1.f - 1e-7f);
+          loss += -(t * logf(yc) + (1.f - t) * logf(1.f - yc));
+          gb3 += dz;
+        }
+      }
+      dzs[tid] = dz;
+    }
+    if (!GRAD) continue;
+    __syncthreads();
+    const float4 dz = *reinterpret_cast<const float4 *>(dzs + 4 * q);
+    const float4 d2 = make_float4(h2.x > 0.f ? dz.x * w3 : 0.f, h2.y > 0.f ? dz.y * w3 : 0.f,
+                                  h2.z > 0.f ? dz.z * w3 : 0.f, h2.w > 0.f ? dz.w * w3 : 0.f);
+    *reinterpret_cast<float4 *>(d2s + (q * MLP_H + j) * 4) = d2;
+    gb2 += (d2.x + d2.y) + (d2.z + d2.w);
+    gw3 = fmaf(dz.x, h2.x, fmaf(dz.y, h2.y, fmaf(dz.z, h2.z, fmaf(dz.w, h2.w, gw3))));
+    __syncthreads();
+    a0 = a1 = a2 = a3 = 0.f;
+#pragma unroll 8
+    for (int i = 0; i < MLP_H; i++) {
+      const float w = W2s[i * S2 + j];
+      const float4 x = quad(d2s, MLP_H, i, q);
+      a0 = fmaf(w, x.x, a0);
+      a1 = fmaf(w, x.y, a1);
+      a2 = fmaf(w, x.z, a2);
+      a3 = fmaf(w, x.w, a3);
+    }
+    const float4 d1 = make_float4(h1.x > 0.f ? a0 : 0.f, h1.y > 0.f ? a1 : 0.f, h1.z > 0.f ? a2 : 0.f,
+                                  h1.w > 0.f ? a3 : 0.f);
+    *reinterpret_cast<float4 *>(d1s + (q * MLP_H + j) * 4) = d1;
+    gb1 += (d1.x + d1.y) + (d1.z + d1.w);
+    __syncthreads();
+    for (int qd = 0; qd < GS / 4; qd++) {
+      float4 c[8];
+#pragma unroll
+      for (int b = 0; b < 8; b++) c[b] = quad(h1s, MLP_H, tk + 16 * b, qd);
+#pragma unroll
+      for (int a = 0; a < 8; a++) {
+        const float4 r = quad(d2s, MLP_H, tj + 16 * a, qd);
+#pragma unroll
+        for (int b = 0; b < 8; b++)
+          g2[a][b] = fmaf(r.x, c[b].x, fmaf(r.y, c[b].y, fmaf(r.z, c[b].z, fmaf(r.w, c[b].w, g2[a][b]))));
+      }
+#pragma unroll
+      for (int b = 0; b < 4; b++) c[b] = quad(xs, MLP_IN, tk + 16 * b, qd);
+#pragma unroll
+      for (int a = 0; a < 8; a++) {
+        const float4 r = quad(d1s, MLP_H, tj + 16 * a, qd);
+#pragma unroll
+        for (int b = 0; b < 4; b++)
+          g1[a][b] = fmaf(r.x, c[b].x, fmaf(r.y, c[b].y, fmaf(r.z, c[b].z, fmaf(r.w, c[b].w, g1[a][b]))));
+      }
+    }
   }
-  for (int s = 0; s < SPC; s++) {
-    const int b = s0 + s;
-    if (b < B) dh1g[(size_t)b * MLP_H + k] = h1g[(size_t)b * MLP_H + k] > 0.f ? acc[s] : 0.f;
+  if (GRAD) {
+    float *p = part + (size_t)blockIdx.x * PART;
+    float *pb1 = p + MLP_H * MLP_IN, *pW2 = pb1 + MLP_H, *pb2 = pW2 + MLP_H * MLP_H, *pw3 = pb2 + MLP_H, *pb3 = pw3 + MLP_H;
+#pragma unroll
+    for (int a = 0; a < 8; a++) {
+#pragma unroll
+      for (int b = 0; b < 8; b++) pW2[(tj + 16 * a) * MLP_H + tk + 16 * b] = g2[a][b];
+#pragma unroll
+      for (int b = 0; b < 4; b++) p[(tj + 16 * a) * MLP_IN + tk + 16 * b] = g1[a][b];
+    }
+    // the two quads of a unit, and the samples of b3 and the loss
+    __syncthreads();
+    float *v = xs;
+    if (q == 1) {
+      v[j] = gb1;
+      v[MLP_H + j] = gb2;
+      v[2 * MLP_H + j] = gw3;
+    }
+    if (tid < GS) {
+      dzs[tid] = gb3;
+      dzs[GS + tid] = loss;
+    }
+    __syncthreads();
+    if (q == 0) {
+      pb1[j] = gb1 + v[j];
+      pb2[j] = gb2 + v[MLP_H + j];
+      pw3[j] = gw3 + v[2 * MLP_H + j];
+    }
+    if (tid < 2) {
+      float t = 0.f;
+      for (int i = 0; i < GS; i++) t += dzs[tid * GS + i];
+      pb3[tid] = t;
+    }
   }
 }
 
-// parameter gradients: one thread per parameter, fixed-order sum over the batch
-__global__ void k_wgrad(const float *X, const int *idx, int B, const float *h1g, const float *h2g,
-                        const float *dz, const float *dh2g, const float *dh1g, float *grad) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  const int n1 = MLP_H * MLP_IN, n2 = n1 + MLP_H, n3 = n2 + MLP_H * MLP_H, n4 = n3 + MLP_H, n5 = n4 + MLP_H;
-  if (p > n5) return;
+// Sum of the CTAs' partial gradients (4 threads per parameter, each a fixed
+// part of the CTAs), then the Adam step if theta is given, else the gradient
+// to grad; the loss adds to *loss.
+__global__ void __launch_bounds__(256) k_reduce(const float *part, int nparts, float *grad, float *loss, float *theta,
+                                                float *m, float *v, float lr, float b1, float b2, float eps, float bc1,
+                                                float bc2) {
+  __shared__ float sh[4][64];
+  const int c = threadIdx.x & 63, sl = threadIdx.x >> 6, p = blockIdx.x * 64 + c;
   float s = 0.f;
-  if (p < n1) {
-    const int j = p / MLP_IN, i = p % MLP_IN;
-    for (int b = 0; b < B; b++) s = fmaf(dh1g[(size_t)b * MLP_H + j], X[(size_t)(idx ? idx[b] : b) * MLP_IN + i], s);
-  } else if (p < n2) {
-    const int j = p - n1;
-    for (int b = 0; b < B; b++) s += dh1g[(size_t)b * MLP_H + j];
-  } else if (p < n3) {
-    const int q = p - n2, j = q / MLP_H, k = q % MLP_H;
-    for (int b = 0; b < B; b++) s = fmaf(dh2g[(size_t)b * MLP_H + j], h1g[(size_t)b * MLP_H + k], s);
-  } else if (p < n4) {
-    const int j = p - n3;
-    for (int b = 0; b < B; b++) s += dh2g[(size_t)b * MLP_H + j];
-  } else if (p < n5) {
-    const int j = p - n4;
-    for (int b = 0; b < B; b++) s = fmaf(dz[b], h2g[(size_t)b * MLP_H + j], s);
-  } else {
-    for (int b = 0; b < B; b++) s += dz[b];
+  if (p < PART) {
+    const int per = (nparts + 3) / 4, e = min(nparts, (sl + 1) * per);
+#pragma unroll 8
+    for (int n = sl * per; n < e; n++) s += part[(size_t)n * PART + p];
   }
-  grad[p] = s;
-}
-
-__global__ void k_adam(float *theta, const float *g, float *m, float *v, int n, float lr, float b1, float b2,
-                       float eps, float bc1, float bc2) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= n) return;
-  const float gg = g[p];
-  const float mm = b1 * m[p] + (1.f - b1) * gg;
-  const float vv = b2 * v[p] + (1.f - b2) * gg * gg;
+  sh[sl][c] = s;
+  __syncthreads();
+  if (sl || p >= PART) return;
+  const float g = (sh[0][c] + sh[1][c]) + (sh[2][c] + sh[3][c]);
+  if (p == NPAR) {
+    *loss += g;
+    return;
+  }
+  if (!theta) {
+    grad[p] = g;
+    return;
+  }
+  const float mm = b1 * m[p] + (1.f - b1) * g;
+  const float vv = b2 * v[p] + (1.f - b2) * g * g;
   m[p] = mm;
   v[p] = vv;
   theta[p] -= lr * (mm / bc1) / (sqrtf(vv / bc2) + eps);
@@ -219,37 +370,63 @@ __global__ void k_combine(const float *prob, const DevBlock *blk, signed char *f
 
 }  // namespace
 
-int mlp_n_params() { return MLP_H * MLP_IN + MLP_H + MLP_H * MLP_H + MLP_H + MLP_H + 1; }
+int mlp_n_params() { return NPAR; }
+size_t mlp_partial_floats() { return (size_t)MLP_MAX_CTAS * PART; }
+
+namespace {
+template <typename real>
+void features(const KParams &kp, const real *U, int slot0, int nslots, float *out, cudaStream_t s) {
+  // three planes in at most 100 KB (two CTAs per SM): blocks of up to 36 x 36
+  // columns; above, the kernel without shared planes
+  const size_t smem = sizeof(double) * (9 * (size_t)(kp.nb[1] + 2) * (kp.nb[2] + 2) + (size_t)kp.nb[1] * kp.nb[2]);
+  if (smem > 100 * 1024) {
+    k_features_large<real><<<nslots, 256, 0, s>>>(kp, U, slot0, out);
+    return;
+  }
+  cudaFuncSetAttribute(k_features<real>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  k_features<real><<<nslots, 256, smem, s>>>(kp, U, slot0, out);
+}
+}  // namespace
 
 void mlp_features_launch(const KParams &kp, const void *U, int precision, int slot0, int nslots, float *out,
                          cudaStream_t s) {
   if (nslots <= 0) return;
   if (precision)
-    k_features<float><<<nslots, 256, 0, s>>>(kp, (const float *)U, slot0, out);
+    features(kp, (const float *)U, slot0, nslots, out, s);
   else
-    k_features<double><<<nslots, 256, 0, s>>>(kp, (const double *)U, slot0, out);
+    features(kp, (const double *)U, slot0, nslots, out, s);
 }
 
-void mlp_forward_launch(const float *theta, const float *X, const int *idx, int B, float *h1, float *h2, float *y,
-                        cudaStream_t s) {
+namespace {
+// one CTA per SM at most (the weights take 99 KB of shared memory each)
+template <bool GRAD>
+int mlp_launch(const float *theta, const float *X, const float *T, const int *idx, int B, float *y, float *part,
+               cudaStream_t s) {
+  cudaFuncSetAttribute(k_mlp<GRAD>, cudaFuncAttributeMaxDynamicSharedMemorySize, MLP_SMEM);
+  const int groups = (B + GS - 1) / GS, n = groups < MLP_MAX_CTAS ? groups : MLP_MAX_CTAS;
+  k_mlp<GRAD><<<n, NT, MLP_SMEM, s>>>(theta, X, T, idx, B, y, part);
+  return n;
+}
+}  // namespace
+
+void mlp_forward_launch(const float *theta, const float *X, const int *idx, int B, float *y, cudaStream_t s) {
+  if (B > 0) mlp_launch<false>(theta, X, nullptr, idx, B, y, nullptr, s);
+}
+
+void mlp_grad_launch(const float *theta, const float *X, const float *T, const int *idx, int B, float *part, float *grad,
+                     float *loss, cudaStream_t s) {
   if (B <= 0) return;
-  k_forward<<<(B + SPC - 1) / SPC, MLP_H, 0, s>>>(theta, X, idx, B, h1, h2, y);
+  const int n = mlp_launch<true>(theta, X, T, idx, B, nullptr, part, s);
+  k_reduce<<<(PART + 63) / 64, 256, 0, s>>>(part, n, grad, loss, nullptr, nullptr, nullptr, 0.f, 0.f, 0.f, 0.f, 1.f, 1.f);
 }
 
-void mlp_backward_launch(const float *theta, const float *X, const float *T, const int *idx, int B,
-                         const float *h1, const float *h2, const float *y, float *dz, float *dh2, float *dh1,
-                         float *grad, float *loss, cudaStream_t s) {
+void mlp_step_launch(float *theta, float *m, float *v, const float *X, const float *T, const int *idx, int B, float *part,
+                     float *loss, float lr, int step, cudaStream_t s) {
   if (B <= 0) return;
-  k_backvec<<<(B + SPC - 1) / SPC, MLP_H, 0, s>>>(theta, T, idx, B, h1, h2, y, dz, dh2, dh1, loss);
-  const int np = mlp_n_params();
-  k_wgrad<<<(np + 255) / 256, 256, 0, s>>>(X, idx, B, h1, h2, dz, dh2, dh1, grad);
-}
-
-void mlp_adam_launch(float *theta, const float *g, float *m, float *v, float lr, int step, cudaStream_t s) {
   const float b1 = 0.9f, b2 = 0.999f;
   const float bc1 = 1.f - powf(b1, (float)step), bc2 = 1.f - powf(b2, (float)step);
-  const int np = mlp_n_params();
-  k_adam<<<(np + 255) / 256, 256, 0, s>>>(theta, g, m, v, np, lr, b1, b2, 1e-8f, bc1, bc2);
+  const int n = mlp_launch<true>(theta, X, T, idx, B, nullptr, part, s);
+  k_reduce<<<(PART + 63) / 64, 256, 0, s>>>(part, n, nullptr, loss, theta, m, v, lr, b1, b2, 1e-8f, bc1, bc2);
 }
 
 void mlp_combine_launch(const float *prob, const DevBlock *blk, signed char *flags, int n, cudaStream_t s) {
