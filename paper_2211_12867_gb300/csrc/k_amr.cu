@@ -105,16 +105,21 @@ __global__ void k_estimator(const KParams kp, const real *U, int slot0, double e
     // once this thread has found a refining cell (the flags are unchanged)
     real uc[NVAR];
     ld_cell(U + cell_index(kp, slot, p0, p1, p2), uc);
-    const double r0 = (double)uc[0], m0 = (double)uc[1];
+    const double r0 = widen(uc[0]), m0 = widen(uc[1]);
     {
       const int I = B.ix[0] * kp.nb[0] + i, J = B.ix[1] * kp.nb[1] + j, K = B.ix[2] * kp.nb[2] + k;
       const double vb = vbg[((size_t)(I >> sh) * kp.n_base_cells[1] + (J >> sh)) * kp.n_base_cells[2] + (K >> sh)];
+      // The gate compares the rounded quotient m / rho.  The sign of m - g rho is
+      // exact after its one rounding, and where it is not positive the rounded
+      // quotient cannot exceed g either: most cells need no division.
+      const double gate = __dadd_rn(vb, dv);
+      if (r0 > 0.0 && !(__fma_rn(-gate, r0, m0) > 0.0)) continue;
       const double vr = __ddiv_rn(m0, r0);
-      if (!(vr > __dadd_rn(vb, dv)) || refine) continue;
+      if (!(vr > gate) || refine) continue;
     }
     double u0[NVAR];
 #pragma unroll
-    for (int v = 0; v < NVAR; v++) u0[v] = (double)uc[v];
+    for (int v = 0; v < NVAR; v++) u0[v] = widen(uc[v]);
     double rm[3], rp[3], pm[3], pp[3];
     for (int d = 0; d < 3; d++) {
       int m[3] = {p0, p1, p2}, p[3] = {p0, p1, p2};
@@ -126,8 +131,8 @@ __global__ void k_estimator(const KParams kp, const real *U, int slot0, double e
       ld_cell(U + cell_index(kp, slot, p[0], p[1], p[2]), xp);
 #pragma unroll
       for (int v = 0; v < NVAR; v++) {
-        um[v] = (double)xm[v];
-        up[v] = (double)xp[v];
+        um[v] = widen(xm[v]);
+        up[v] = widen(xp[v]);
       }
       rm[d] = um[0];
       rp[d] = up[0];
