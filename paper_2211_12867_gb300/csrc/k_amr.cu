@@ -8,7 +8,11 @@
 // background.  It is evaluated in FP64 with explicitly rounded operations in a
 // fixed order (no contraction), so the block flags agree bit for bit with any
 // IEEE FP64 evaluation of the same formula on the same stored state.
+#include <cooperative_groups.h>
+
 #include "mhd_device.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace {
 
@@ -80,6 +84,32 @@ __device__ __forceinline__ double loehner(const double *um, double u0, const dou
   return __dsqrt_rn(__ddiv_rn(num, den));
 }
 
+// E of a cell, every operation rounded on its own
+template <typename real>
+__device__ __forceinline__ double exact_E(const KParams &kp, const real *U, int slot, int p0, int p1, int p2, double eps) {
+  auto get = [&](int a, int b, int c, double *u) {
+    real x[NVAR];
+    ld_cell(U + cell_index(kp, slot, a, b, c), x);
+#pragma unroll
+    for (int v = 0; v < NVAR; v++) u[v] = widen(x[v]);
+  };
+  double u0[NVAR], rm[3], rp[3], pm[3], pp[3];
+  get(p0, p1, p2, u0);
+#pragma unroll
+  for (int d = 0; d < 3; d++) {
+    double um[NVAR], up[NVAR];
+    get(p0 - (d == 0), p1 - (d == 1), p2 - (d == 2), um);
+    get(p0 + (d == 0), p1 + (d == 1), p2 + (d == 2), up);
+    rm[d] = um[0];
+    rp[d] = up[0];
+    pm[d] = est_pressure(um, kp.gamma);
+    pp[d] = est_pressure(up, kp.gamma);
+  }
+  const double er = loehner(rm, u0[0], rp, eps);
+  const double ep = loehner(pm, est_pressure(u0, kp.gamma), pp, eps);
+  return er > ep ? er : ep;
+}
+
 template <typename real>
 __global__ void k_estimator(const KParams kp, const real *U, int slot0, double e_ref, double e_crs, double eps,
                             double dv, signed char *flags) {
@@ -117,31 +147,7 @@ __global__ void k_estimator(const KParams kp, const real *U, int slot0, double e
       const double vr = __ddiv_rn(m0, r0);
       if (!(vr > gate) || refine) continue;
     }
-    double u0[NVAR];
-#pragma unroll
-    for (int v = 0; v < NVAR; v++) u0[v] = widen(uc[v]);
-    double rm[3], rp[3], pm[3], pp[3];
-    for (int d = 0; d < 3; d++) {
-      int m[3] = {p0, p1, p2}, p[3] = {p0, p1, p2};
-      m[d]--;
-      p[d]++;
-      double um[NVAR], up[NVAR];
-      real xm[NVAR], xp[NVAR];
-      ld_cell(U + cell_index(kp, slot, m[0], m[1], m[2]), xm);
-      ld_cell(U + cell_index(kp, slot, p[0], p[1], p[2]), xp);
-#pragma unroll
-      for (int v = 0; v < NVAR; v++) {
-        um[v] = widen(xm[v]);
-        up[v] = widen(xp[v]);
-      }
-      rm[d] = um[0];
-      rp[d] = up[0];
-      pm[d] = est_pressure(um, kp.gamma);
-      pp[d] = est_pressure(up, kp.gamma);
-    }
-    const double er = loehner(rm, u0[0], rp, eps);
-    const double ep = loehner(pm, est_pressure(u0, kp.gamma), pp, eps);
-    const double E = er > ep ? er : ep;
+    const double E = exact_E(kp, U, slot, p0, p1, p2, eps);
     if (E > e_ref) {
       refine = 1;
       s_refine = 1;
@@ -151,6 +157,167 @@ __global__ void k_estimator(const KParams kp, const real *U, int slot0, double e
   refine = __syncthreads_or(refine);
   keep = __syncthreads_or(keep);
   if (threadIdx.x == 0) flags[blockIdx.x] = refine ? 1 : (keep ? 0 : -1);
+}
+
+// The same flags with the leaf's planes split over the four CTAs of a cluster
+// and FP32 comparisons where they decide.  The FP64 pipe bounds the estimator
+// (19 cycles of an SM per instruction of a warp; 280 instructions a cell with the
+// speed gate open, seven pressures with a division each among them), and one
+// CTA per leaf left the leaves inside the CME to few SMs.  Here a CTA rounds
+// the density and pressure of its slab and one halo cell around it to FP32 in
+// shared memory (from FP32 state without the FP64 pipe) and evaluates
+// E = |second differences| / |s| there with a bound on the FP32 error; a cell
+// whose comparison the bound leaves open takes the exact operations.  A slab
+// without an open gate is done after its gate test.  Five CTAs per SM (48
+// registers, spills on the exact path only): a slab is a chain of short phases,
+// and two CTAs per SM at 108 registers took 201 us for 1914 leaves of 12^3 FP32
+// cells on three levels; now 119 us, one CTA per leaf 367.  808 leaves: 53 us,
+// before 220.
+constexpr int EST_CTAS = 4;
+
+// Pressure to within one FP32 rounding.  FP64 state: FP64 operations.  FP32
+// state: in pairs of FP32 numbers (exact products and sums by fused
+// multiply-adds, Dekker's and Knuth's error-free transformations), whose error
+// is below 2^-42 e; NaN, which is not decided, where the pressure is below
+// 2^-16 e.
+__device__ __forceinline__ float rounded_pressure(const double *u, double gamma, float) {
+  const double ke2 = (u[1] * u[1] + u[2] * u[2] + u[3] * u[3]) * RT<double>::rcp_(u[0]);
+  return (float)((gamma - 1.0) * fma(-0.5, ke2 + (u[5] * u[5] + u[6] * u[6] + u[7] * u[7]), u[4]));
+}
+__device__ __forceinline__ void pair_add(float a, float &h, float &l) {   // (h, l) += a
+  const float s = __fadd_rn(h, a), t = __fsub_rn(s, h);
+  l = __fadd_rn(l, __fadd_rn(__fsub_rn(h, __fsub_rn(s, t)), __fsub_rn(a, t)));
+  h = s;
+}
+__device__ __forceinline__ void pair_add_square(float x, float &h, float &l) {
+  const float p = __fmul_rn(x, x);
+  l = __fadd_rn(l, __fmaf_rn(x, x, -p));
+  pair_add(p, h, l);
+}
+__device__ __forceinline__ float rounded_pressure(const float *u, double, float gm1) {
+  float h = 0.f, l = 0.f;
+  pair_add_square(u[1], h, l);
+  pair_add_square(u[2], h, l);
+  pair_add_square(u[3], h, l);
+  const float r = RT<float>::rcp_(u[0]), q = __fmul_rn(h, r);   // (h, l) / rho
+  l = __fmul_rn(__fadd_rn(__fmaf_rn(-q, u[0], h), l), r);
+  h = q;
+  pair_add_square(u[5], h, l);
+  pair_add_square(u[6], h, l);
+  pair_add_square(u[7], h, l);
+  h *= -0.5f;
+  l *= -0.5f;
+  pair_add(u[4], h, l);
+  const float p = __fmul_rn(gm1, __fadd_rn(h, l));
+  return p > 1.52587890625e-5f * fabsf(u[4]) ? p : nanf("");
+}
+
+// E > e from FP32 values: 1 yes, 0 no, -1 not decided.  Inputs carry a relative
+// error of 2^-22 (see rounded_pressure), each difference and sum one more per
+// operation: |N_f - N| and |S_f - S| stay below 2^-20 (1 + eps) of the sum of the
+// w, for N the norm of the second differences and S that of s.  NaN and
+// infinities are not decided.
+__device__ __forceinline__ void loehner32(const float *um, float u0, const float *up, float eps, float *N, float *S,
+                                          float *W) {
+  float n = 0.f, d = 0.f, t = 0.f;
+#pragma unroll
+  for (int e = 0; e < 3; e++) {
+    const float t1 = up[e] - u0, t2 = u0 - um[e], d2 = t1 - t2;
+    const float w = fabsf(up[e]) + 2.f * fabsf(u0) + fabsf(um[e]);
+    const float s = fabsf(t1) + fabsf(t2) + eps * w;
+    n = fmaf(d2, d2, n);
+    d = fmaf(s, s, d);
+    t += w;
+  }
+  *N = sqrtf(n);
+  *S = sqrtf(d);
+  *W = t * (1.f + eps);
+}
+__device__ __forceinline__ int decide(float N, float S, float W, float e) {
+  const float x = N - e * S, tol = (1.f + e) * 9.5367431640625e-7f * W;
+  return x > tol ? 1 : (x < -tol ? 0 : -1);
+}
+
+template <typename real>
+__global__ void __cluster_dims__(EST_CTAS, 1, 1) __launch_bounds__(256, 5)
+    k_estimator_slabs(const KParams kp, const real *U, int slot0, double e_ref, double e_crs, double eps, double dv,
+                      signed char *flags) {
+  extern __shared__ float est_sm[];
+  __shared__ int s_any, s_code[EST_CTAS];   // s_code: of the cluster's CTAs, in its first one
+  __shared__ volatile int s_refine;
+  const int part = blockIdx.x % EST_CTAS, leaf = blockIdx.x / EST_CTAS, slot = slot0 + leaf;
+  const DevBlock &B = kp.blk[slot];
+  const int sh = B.level - 1, tid = threadIdx.x;
+  const int n1 = kp.nb[1], n2 = kp.nb[2], rows = n1 * n2, h2 = n2 + 2, H = (n1 + 2) * h2;
+  const int ns = (kp.nb[0] + EST_CTAS - 1) / EST_CTAS, i0 = part * ns, i1 = min(kp.nb[0], i0 + ns);
+  const size_t nbc = (size_t)kp.n_base_cells[0] * kp.n_base_cells[1] * kp.n_base_cells[2];
+  const double *vbg = kp.vbg + (size_t)B.member * nbc;
+  float *rho = est_sm, *pr = est_sm + (size_t)(ns + 2) * H;
+  unsigned char *open = reinterpret_cast<unsigned char *>(pr + (size_t)(ns + 2) * H);
+  // without a recorded background the gate is closed everywhere
+  const int cells = kp.cme[B.member].pad != 0 ? max(0, i1 - i0) * rows : 0;
+  int code = 0, any = 0;   // code: 1 a cell keeps the leaf, 2 one refines it
+  if (tid == 0) s_any = s_refine = 0;
+  __syncthreads();
+  for (int c = tid; c < cells; c += blockDim.x) {
+    const int i = i0 + c / rows, r = c % rows, j = r / n2, k = r - (r / n2) * n2;
+    const real *u = U + cell_index(kp, slot, i + NGH, j + NGH, k + NGH);
+    const double r0 = widen(u[0]), m0 = widen(u[1]);
+    const int I = B.ix[0] * kp.nb[0] + i, J = B.ix[1] * n1 + j, K = B.ix[2] * n2 + k;
+    const double gate = __dadd_rn(vbg[((size_t)(I >> sh) * kp.n_base_cells[1] + (J >> sh)) * kp.n_base_cells[2] + (K >> sh)], dv);
+    // see k_estimator; an excess of 4 ulp of the gate leaves no doubt either
+    const double x = __fma_rn(-gate, r0, m0);
+    bool on = !(r0 > 0.0) || x > 0.0;
+    if (on && !(r0 > 0.0 && x > 1e-15 * fabs(gate) * r0)) on = __ddiv_rn(m0, r0) > gate;
+    open[c] = on;
+    any |= on;
+  }
+  if (any) s_any = 1;
+  __syncthreads();
+  if (s_any) {
+    const float gm1 = (float)(kp.gamma - 1.0);
+    for (int c = tid; c < (i1 - i0 + 2) * H; c += blockDim.x) {
+      const int a = c / H, r = c - a * H, b = r / h2, e = r - b * h2;
+      // edges and corners of the halo are not read
+      if ((a == 0 || a == i1 - i0 + 1) + (b == 0 || b == n1 + 1) + (e == 0 || e == n2 + 1) > 1) continue;
+      real x[NVAR];
+      ld_cell(U + cell_index(kp, slot, i0 + a - 1 + NGH, b - 1 + NGH, e - 1 + NGH), x);
+      rho[c] = (float)x[0];
+      pr[c] = rounded_pressure(x, kp.gamma, gm1);
+    }
+    __syncthreads();
+    // one refining cell settles the leaf's flag: the CTA stops at it
+    const float epsf = (float)eps, refl = (float)e_ref, crsl = (float)e_crs;
+    const bool fast = eps >= 0.0 && e_ref >= 0.0 && e_crs >= 0.0;
+    for (int c = tid; c < cells && !s_refine; c += blockDim.x) {
+      if (!open[c]) continue;
+      const int a = c / rows, r = c - a * rows, j = r / n2, k = r - j * n2;
+      const int at = (a + 1) * H + (j + 1) * h2 + k + 1;
+      const float rm[3] = {rho[at - H], rho[at - h2], rho[at - 1]}, rp[3] = {rho[at + H], rho[at + h2], rho[at + 1]};
+      const float pm[3] = {pr[at - H], pr[at - h2], pr[at - 1]}, pp[3] = {pr[at + H], pr[at + h2], pr[at + 1]};
+      float Nr, Sr, Wr, Np, Sp, Wp;
+      loehner32(rm, rho[at], rp, epsf, &Nr, &Sr, &Wr);
+      loehner32(pm, pr[at], pp, epsf, &Np, &Sp, &Wp);
+      const int r1 = decide(Nr, Sr, Wr, refl), p1 = decide(Np, Sp, Wp, refl);
+      const int r2 = decide(Nr, Sr, Wr, crsl), p2 = decide(Np, Sp, Wp, crsl);
+      if (!(fast && (r1 | p1 | r2 | p2) >= 0)) {
+        const double E = exact_E(kp, U, slot, i0 + a + NGH, j + NGH, k + NGH, eps);
+        code |= (E > e_ref ? 2 : 0) | (E > e_crs ? 1 : 0);
+      } else {
+        code |= (r1 | p1) << 1 | (r2 | p2);
+      }
+      if (code & 2) s_refine = 1;
+    }
+  }
+  code = (__syncthreads_or(code & 2) ? 2 : 0) | (__syncthreads_or(code & 1) ? 1 : 0);
+  cg::cluster_group cl = cg::this_cluster();
+  if (tid == 0) *cl.map_shared_rank(&s_code[part], 0) = code;
+  cl.sync();
+  if (part == 0 && tid == 0) {
+    int all = 0;
+    for (int q = 0; q < EST_CTAS; q++) all |= s_code[q];
+    flags[leaf] = all & 2 ? 1 : (all & 1 ? 0 : -1);
+  }
 }
 
 // ---- shock criterion (Sect. 3.2) ----
@@ -486,13 +653,30 @@ void unpack_state_launch(const KParams &kp, void *U, int precision, int slot0, i
     k_unpack<double><<<1024, 256, 0, s>>>(kp, (double *)U, slot0, nslots, in, is_prim);
 }
 
+namespace {
+template <typename real>
+void estimator(const KParams &kp, const real *U, int slot0, int nslots, double e_ref, double e_crs, double eps, double dv,
+               signed char *flags, cudaStream_t s) {
+  // four slabs of a leaf in at most 100 KB each (two CTAs per SM): 12^3 blocks
+  // take 8 KB; above, one CTA per leaf without shared planes
+  const size_t ns = (kp.nb[0] + EST_CTAS - 1) / EST_CTAS, H = (size_t)(kp.nb[1] + 2) * (kp.nb[2] + 2);
+  const size_t smem = 2 * sizeof(float) * (ns + 2) * H + ns * kp.nb[1] * kp.nb[2];
+  if (smem > 100 * 1024) {
+    k_estimator<real><<<nslots, 256, 0, s>>>(kp, U, slot0, e_ref, e_crs, eps, dv, flags);
+    return;
+  }
+  cudaFuncSetAttribute(k_estimator_slabs<real>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  k_estimator_slabs<real><<<nslots * EST_CTAS, 256, smem, s>>>(kp, U, slot0, e_ref, e_crs, eps, dv, flags);
+}
+}  // namespace
+
 void estimator_launch(const KParams &kp, const void *U, int precision, int slot0, int nslots, double e_ref,
                       double e_crs, double eps, double dv, signed char *flags, cudaStream_t s) {
   if (nslots <= 0) return;
   if (precision)
-    k_estimator<float><<<nslots, 256, 0, s>>>(kp, (const float *)U, slot0, e_ref, e_crs, eps, dv, flags);
+    estimator<float>(kp, (const float *)U, slot0, nslots, e_ref, e_crs, eps, dv, flags, s);
   else
-    k_estimator<double><<<nslots, 256, 0, s>>>(kp, (const double *)U, slot0, e_ref, e_crs, eps, dv, flags);
+    estimator<double>(kp, (const double *)U, slot0, nslots, e_ref, e_crs, eps, dv, flags, s);
 }
 
 void shock_estimator_launch(const KParams &kp, const void *U, int precision, int slot0, int nslots,
