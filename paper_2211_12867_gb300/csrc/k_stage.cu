@@ -323,8 +323,9 @@ __global__ void __launch_bounds__(stage_threads(TJ, TK), stage_min_ctas(sizeof(r
         }
     };
     // U^n of the thread's own cell is read at the start of the update and used
-    // behind the r flux, which hides the access (staging it one plane ahead
-    // with the plane copies made the update wait for those as well)
+    // behind the r flux, which hides an access to L2 (staging it one plane
+    // ahead with the plane copies made the update wait for those as well); the
+    // corrector, whose input is another array, brings it there one plane ahead
     const real *u0p = U0 + NVAR * ((size_t)(ib + NGH) * plane + (size_t)(j + NGH) * P2 + (k + NGH));
     // ring offset of the plane after the one at offset a
     auto next = [](int a) { return a == 4 * PL ? 0 : a + PL; };
@@ -385,6 +386,14 @@ __global__ void __launch_bounds__(stage_threads(TJ, TK), stage_min_ctas(sizeof(r
       }
     };
 
+    // ---- prologue: planes ib-2 .. ib+2 converted, r flux at face ib ----
+    // offsets of planes i-1 .. i+3 of the march (plane p sits at p + 2 - ib
+    // planes past the first slot, modulo five)
+    int om = PL, oc = 2 * PL, o1 = 3 * PL, o2 = 4 * PL, o3 = 0;
+    for (int p = 0; p < 5; p++) {
+      issue_plane(ib - 2 + p, p * PL);
+    }
+    if (S2 && valid) prefetch_cell(u0p);
     // ---- factors of the work item into shared memory (read after the
     // prologue's first barrier); rows / columns past the block's edge are
     // never read and not loaded ----
@@ -448,13 +457,6 @@ __global__ void __launch_bounds__(stage_threads(TJ, TK), stage_min_ctas(sizeof(r
       for (int q = 1 + tid; q + 1 < nvk + 4; q += NT) s_ipc2[q] = RT<real>::rcp_(G.pc[kr0 + q + 1] - G.pc[kr0 + q - 1]);
     }
 
-    // ---- prologue: planes ib-2 .. ib+2 converted, r flux at face ib ----
-    // offsets of planes i-1 .. i+3 of the march (plane p sits at p + 2 - ib
-    // planes past the first slot, modulo five)
-    int om = PL, oc = 2 * PL, o1 = 3 * PL, o2 = 4 * PL, o3 = 0;
-    for (int p = 0; p < 5; p++) {
-      issue_plane(ib - 2 + p, p * PL);
-    }
     cp_async_wait_all();
     for (int p = 0; p < 5; p++) convert_plane(p * PL);
     __syncthreads();
@@ -539,6 +541,7 @@ __global__ void __launch_bounds__(stage_threads(TJ, TK), stage_min_ctas(sizeof(r
         real Fhi[NVAR], u0[NVAR];
         ld_cell(u0p, u0);
         u0p += NVAR * plane;
+        if (S2 && i + 1 < ie) prefetch_cell(u0p);
         {
           real sn[NVAR];
           rslope(oc, o1, o2, sn);

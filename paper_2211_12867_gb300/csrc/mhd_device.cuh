@@ -142,6 +142,13 @@ __device__ __forceinline__ void st_cell(double *p, const double *u) {
                  : "memory");
 }
 
+// a cell's sector(s) into L2
+__device__ __forceinline__ void prefetch_cell(const float *p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+__device__ __forceinline__ void prefetch_cell(const double *p) {
+  asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
+  asm volatile("prefetch.global.L2 [%0];" ::"l"(p + 4));
+}
+
 // Pressure from conserved variables.  In the mixed-precision mode the FP32
 // result is replaced by an FP64 recomputation from the same (FP32-stored)
 // conserved variables where the thermal energy is a small remainder of the
