@@ -331,12 +331,32 @@ __global__ void __launch_bounds__(stage_threads(TJ, TK), stage_min_ctas(sizeof(r
     auto next = [](int a) { return a == 4 * PL ? 0 : a + PL; };
     // half the limited radial slope of the thread's column at the middle of
     // the planes at offsets m, c, p
-    auto rslope = [&](int m, int c, int p, real *out) {
-      real a[NVAR], b[NVAR], e[NVAR];
-      ld8<real, RP>(ring + m, o, a);
-      ld8<real, RP>(ring + c, o, b);
-      ld8<real, RP>(ring + p, o, e);
-      mc_half_slopes8<real>(a, b, e, out);
+    // (FP64: the difference across the later face is kept for the next plane)
+    real rdiff[F32 ? 1 : NVAR];
+    auto rslope = [&](int m, int c, int p, real *out, bool carried) {
+      if constexpr (F32) {
+        real a[NVAR], b[NVAR], e[NVAR];
+        ld8<real, RP>(ring + m, o, a);
+        ld8<real, RP>(ring + c, o, b);
+        ld8<real, RP>(ring + p, o, e);
+        mc_half_slopes8<real>(a, b, e, out);
+      } else {
+        real b[NVAR], e[NVAR];
+        ld8<real, RP>(ring + c, o, b);
+        ld8<real, RP>(ring + p, o, e);
+        if (!carried) {
+          real a[NVAR];
+          ld8<real, RP>(ring + m, o, a);
+#pragma unroll
+          for (int v = 0; v < NVAR; v++) rdiff[v] = b[v] - a[v];
+        }
+#pragma unroll
+        for (int v = 0; v < NVAR; v++) {
+          const real dp = e[v] - b[v];
+          out[v] = mc_half_of(rdiff[v], dp);
+          rdiff[v] = dp;
+        }
+      }
     };
     // radial face between the planes at offsets m and c from the slopes at both
     auto rflux = [&](int m, int c, const real *sm, const real *sp, real *F) {
@@ -468,8 +488,8 @@ __global__ void __launch_bounds__(stage_threads(TJ, TK), stage_min_ctas(sizeof(r
     real xprev = real(0);   // tracer X of this column at the previous plane
     if (valid) {
       real s0[NVAR];
-      rslope(0, om, oc, s0);
-      rslope(om, oc, o1, sc);
+      rslope(0, om, oc, s0, false);
+      rslope(om, oc, o1, sc, true);
       rflux(om, oc, s0, sc, Flo);
       if (trc) xprev = xring[RP + o];
     }
@@ -544,7 +564,7 @@ __global__ void __launch_bounds__(stage_threads(TJ, TK), stage_min_ctas(sizeof(r
         if (S2 && i + 1 < ie) prefetch_cell(u0p);
         {
           real sn[NVAR];
-          rslope(oc, o1, o2, sn);
+          rslope(oc, o1, o2, sn, true);
           rflux(oc, o1, sc, sn, Fhi);
 #pragma unroll
           for (int v = 0; v < NVAR; v++) sc[v] = sn[v];

@@ -300,9 +300,8 @@ __device__ __forceinline__ long long hilo(int hi, int lo) {
 }
 // FP64: the minimum and the signs by bit patterns, the quarter by the exponent
 // (three FP64-pipe instructions, the differences, instead of nine)
-template <>
-__device__ __forceinline__ double mc_half_slope<double>(double um, double u0, double up) {
-  const double dm = u0 - um, dp = up - u0, s = dm + dp;
+__device__ __forceinline__ double mc_half_of(double dm, double dp) {
+  const double s = dm + dp;
   // magnitudes (see nan_ for the high words)
   const int ha = __double2hiint(dm), hb = __double2hiint(dp);
   const int qa = __double2hiint(s) & 0x7fffffff;
@@ -312,6 +311,10 @@ __device__ __forceinline__ double mc_half_slope<double>(double um, double u0, do
   lim = q < lim ? q : lim;
   const int hl = (int)(lim >> 32) | (ha & 0x80000000);
   return (ha ^ hb) < 0 ? 0.0 : __hiloint2double(hl, (int)lim);
+}
+template <>
+__device__ __forceinline__ double mc_half_slope<double>(double um, double u0, double up) {
+  return mc_half_of(u0 - um, up - u0);
 }
 
 template <typename real>
@@ -404,7 +407,7 @@ __device__ __forceinline__ void flux_balance(const real *Fhi, const real *Flo, c
                                              real pw, real *out) {
 #pragma unroll
   for (int h = 0; h < CH; h++)
-    out[h] = (rm * Flo[h] - rp * Fhi[h]) + (tm * ftl[h] - tp * fth[h]) + pw * (fpl[h] - fph[h]);
+    out[h] = fma(pw, fpl[h] - fph[h], fma(-tp, fth[h], fma(tm, ftl[h], fma(-rp, Fhi[h], rm * Flo[h]))));
 }
 // FP32: out[h] = -((Arp Fhi - Arm Flo) + (Atp Fth - Atm Ftl) + Ap (Fph - Fpl)) iV
 // from the areas, in packed pairs.
@@ -438,6 +441,20 @@ __device__ __forceinline__ double fast_speed_of(double ir, double gp, double hgp
   return RT<double>::sqrt_((hgp + hb2 + RT<double>::sqrt_(fma(d, d, gp * bt2))) * ir);
 }
 
+// The same from rho: sqrt(X / rho) = X / sqrt(X rho), one step of third order from
+// the approximate reciprocal root (seven FP64-pipe instructions; reciprocal,
+// product and root are nine).  Products below the normal range take the other
+// form.
+__device__ __forceinline__ double face_speed(double rho, double gp, double hgp, double hb2, double bt2) {
+  const double d = hgp - hb2;
+  const double X = hgp + hb2 + RT<double>::sqrt_(fma(d, d, gp * bt2)), m = X * rho;
+  if (__double2hiint(m) < 0x00100000) return RT<double>::sqrt_(X * RT<double>::rcp_(rho));
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(m));
+  const double e = fma(-(m * y), y, 1.0), g = X * y;
+  return fma(g * e, fma(e, 0.375, 0.5), g);
+}
+
 // Sum over the directions of (|v_d| + c_f,d) / dx_d from 1/rho, the velocity,
 // p and the field (ix: reciprocal widths)
 __device__ __forceinline__ double cfl_rate(double ir, const double *v, double p, const double *B, double gamma,
@@ -450,26 +467,35 @@ __device__ __forceinline__ double cfl_rate(double ir, const double *v, double p,
 }
 
 // One side's part of the TVDLF flux, G = F(W) + sc U(W) with sc = +c_max on
-// the left and -c_max on the right, so that the flux is (G_L + G_R) / 2.
+// the left and -c_max on the right (the flux is (G_L + G_R) / 2), added to the
+// other side's G by the same multiply-adds that form it (LAST) or started.
 // Written out per component with w = v_n + sc:
 //   mass rho w;  momentum (rho w) v_k - B_n B_k (+ p_T along n);
 //   energy e w + p_T v_n - B_n (v.B);  induction B_k w - B_n v_k (k != n).
-template <int D>
+template <int D, bool LAST>
 __device__ __forceinline__ void side_flux(const double *W, double hb2, double igm1, double sc, double *G) {
   const double vn = W[1 + D], Bn = W[5 + D];
   const double w = vn + sc;
   const double v2 = W[1] * W[1] + W[2] * W[2] + W[3] * W[3];
   const double pt = W[4] + hb2;
-  const double e = W[4] * igm1 + (0.5 * W[0] * v2 + hb2);
+  const double e = fma(W[4], igm1, fma(0.5 * W[0], v2, hb2));
   const double vB = W[1] * W[5] + W[2] * W[6] + W[3] * W[7];
-  G[0] = W[0] * w;
-  G[1] = G[0] * W[1] - Bn * W[5];
-  G[2] = G[0] * W[2] - Bn * W[6];
-  G[3] = G[0] * W[3] - Bn * W[7];
-  G[1 + D] += pt;
-  G[4] = e * w + pt * vn - Bn * vB;
+  const double m = W[0] * w;
+  auto add = [&](double a, double b, double &g) { g = LAST ? fma(a, b, g) : a * b; };
+  if (LAST) G[0] += m;
+  else G[0] = m;
 #pragma unroll
-  for (int k = 0; k < 3; k++) G[5 + k] = k == D ? 0.0 : W[5 + k] * w - Bn * W[1 + k];
+  for (int k = 0; k < 3; k++) {
+    add(m, W[1 + k], G[1 + k]);
+    G[1 + k] = fma(-Bn, W[5 + k], G[1 + k]);
+    if (k != D) {
+      add(W[5 + k], w, G[5 + k]);
+      G[5 + k] = fma(-Bn, W[1 + k], G[5 + k]);
+    }
+  }
+  G[1 + D] += pt;
+  add(e, w, G[4]);
+  G[4] = fma(-Bn, vB, fma(pt, vn, G[4]));
 }
 
 // TVDLF flux from reconstructed face states WL | WR (primitive variables),
@@ -492,13 +518,11 @@ __device__ __forceinline__ void tvdlf_states(double *WL, double *WR, const doubl
   const double tL = WL[T1] * WL[T1] + WL[T2] * WL[T2], tR = WR[T1] * WR[T1] + WR[T2] * WR[T2];
   const double hbL = 0.5 * (WL[5 + D] * WL[5 + D] + tL), hbR = 0.5 * (WR[5 + D] * WR[5 + D] + tR);
   const double hg = 0.5 * gamma;
-  const double cl = RT<double>::abs_(WL[1 + D]) + fast_speed_of(RT<double>::rcp_(WL[0]), gamma * WL[4], hg * WL[4], hbL, tL);
-  const double cr = RT<double>::abs_(WR[1 + D]) + fast_speed_of(RT<double>::rcp_(WR[0]), gamma * WR[4], hg * WR[4], hbR, tR);
+  const double cl = RT<double>::abs_(WL[1 + D]) + face_speed(WL[0], gamma * WL[4], hg * WL[4], hbL, tL);
+  const double cr = RT<double>::abs_(WR[1 + D]) + face_speed(WR[0], gamma * WR[4], hg * WR[4], hbR, tR);
   const double cm = RT<double>::max_(cl, cr);
-  double GL[NVAR], GR[NVAR];
-  side_flux<D>(WL, hbL, igm1, cm, GL);
-  side_flux<D>(WR, hbR, igm1, -cm, GR);
-  axpy8<double>(GL, 1.0, GR, F2);
+  side_flux<D, false>(WL, hbL, igm1, cm, F2);
+  side_flux<D, true>(WR, hbR, igm1, -cm, F2);
   F2[5 + D] = 0.0;
 }
 
