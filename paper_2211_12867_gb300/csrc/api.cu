@@ -1108,6 +1108,19 @@ icarus_status recompute_dt(icarus_ctx *c) {
   return ICARUS_OK;
 }
 
+// Device address of n doubles of pinned host memory, or nullptr (pageable
+// memory, or a range that does not lie in one piece).
+double *mapped_host(double *host, size_t n) {
+  cudaPointerAttributes a{}, b{};
+  if (cudaPointerGetAttributes(&a, host) != cudaSuccess || cudaPointerGetAttributes(&b, host + n - 1) != cudaSuccess) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  if (a.type != cudaMemoryTypeHost || b.type != cudaMemoryTypeHost || !a.devicePointer || !b.devicePointer) return nullptr;
+  double *d = static_cast<double *>(a.devicePointer);
+  return d + (n - 1) == b.devicePointer ? d : nullptr;
+}
+
 bool member_ok(icarus_ctx *c, int m) { return c && m >= 0 && m < c->d.n_members; }
 
 }  // namespace
@@ -1598,6 +1611,15 @@ icarus_status icarus_get_state(icarus_ctx *c, int member, double *host, size_t n
   const size_t per = (size_t)NVAR * c->kp.icells;
   const int nl = (int)c->mem[member].leaves.size();
   if (n != per * nl) return ICARUS_ERR_ARG;
+  // Into pinned memory the packing kernel writes over the link itself (the link's
+  // 193 GB/s; packing 64 MB pieces to a buffer, copying and synchronising each
+  // reached 107 to 170); pageable memory goes through the buffer.
+  if (double *direct = n ? mapped_host(host, n) : nullptr) {
+    pack_state_launch(c->kp, c->U, c->prec, c->mem_off[member], nl, direct, c->stream);
+    CK(cudaPeekAtLastError());
+    CK(cudaStreamSynchronize(c->stream));
+    return ICARUS_OK;
+  }
   const int chunk = (int)(c->lay.staging_doubles / per);
   for (int s0 = 0; s0 < nl; s0 += chunk) {
     const int ns = std::min(chunk, nl - s0);
@@ -1630,72 +1652,42 @@ icarus_status icarus_get_padded(icarus_ctx *c, int member, int leaf, double *hos
   return ICARUS_OK;
 }
 
-}  // extern "C"
-
-namespace {
-
-// the tracer plane (padded) of every leaf of a member into / out of host
-// memory: one strided copy
-icarus_status tracer_planes(icarus_ctx *c, int member, std::vector<unsigned char> &raw, bool to_host) {
-  const size_t nl = c->mem[member].leaves.size();
-  const size_t plane = (size_t)c->kp.pcells * c->rsize, stride = (size_t)c->kp.nvs * plane;
-  char *base = static_cast<char *>(c->U) + (size_t)c->mem_off[member] * stride + (size_t)TRV * plane;
-  if (to_host) {
-    raw.resize(nl * plane);
-    CK(cudaMemcpy2DAsync(raw.data(), plane, base, stride, plane, nl, cudaMemcpyDeviceToHost, c->stream));
-  } else {
-    CK(cudaMemcpy2DAsync(base, stride, raw.data(), plane, plane, nl, cudaMemcpyHostToDevice, c->stream));
+// the tracer of a member's leaves through the staging buffer, packed on the
+// device
+static icarus_status tracer_copy(icarus_ctx *c, int member, double *out, const double *in) {
+  const int nl = (int)c->mem[member].leaves.size();
+  const size_t ic = (size_t)c->kp.icells;
+  const int chunk = (int)(c->lay.staging_doubles / ic);
+  for (int s0 = 0; s0 < nl; s0 += chunk) {
+    const int ns = std::min(chunk, nl - s0), slot = c->mem_off[member] + s0;
+    if (out) {
+      pack_tracer_launch(c->kp, c->U, c->prec, slot, ns, c->staging, c->stream);
+      CK(cudaPeekAtLastError());
+      CK(cudaMemcpyAsync(out + (size_t)s0 * ic, c->staging, sizeof(double) * ic * ns, cudaMemcpyDeviceToHost, c->stream));
+    } else {
+      CK(cudaMemcpyAsync(c->staging, in + (size_t)s0 * ic, sizeof(double) * ic * ns, cudaMemcpyHostToDevice, c->stream));
+      unpack_tracer_launch(c->kp, c->U, c->prec, slot, ns, c->staging, c->stream);
+      CK(cudaPeekAtLastError());
+    }
+    CK(cudaStreamSynchronize(c->stream));
   }
-  CK(cudaStreamSynchronize(c->stream));
   return ICARUS_OK;
 }
-
-template <typename F>
-void for_interior(const icarus_ctx *c, F f) {
-  const int *nb = c->d.block;
-  const int P1 = nb[1] + 2 * NGH, P2 = nb[2] + 2 * NGH;
-  size_t q = 0;
-  for (int i = 0; i < nb[0]; i++)
-    for (int j = 0; j < nb[1]; j++)
-      for (int k = 0; k < nb[2]; k++, q++) f(q, ((size_t)(i + NGH) * P1 + j + NGH) * P2 + k + NGH);
-}
-
-}  // namespace
-
-extern "C" {
 
 icarus_status icarus_get_tracer(icarus_ctx *c, int member, double *host, size_t n) {
   if (!member_ok(c, member) || !host) return ICARUS_ERR_ARG;
   if (!c->d.tracer) return ICARUS_ERR_STATE;
-  const size_t nl = c->mem[member].leaves.size(), ic = (size_t)c->kp.icells, pc = (size_t)c->kp.pcells;
-  if (n != nl * ic) return ICARUS_ERR_ARG;
-  std::vector<unsigned char> raw;
-  icarus_status st = tracer_planes(c, member, raw, true);
-  if (st != ICARUS_OK) return st;
-  for (size_t b = 0; b < nl; b++)
-    for_interior(c, [&](size_t q, size_t pidx) {
-      host[b * ic + q] = c->prec ? (double)reinterpret_cast<const float *>(raw.data())[b * pc + pidx]
-                                 : reinterpret_cast<const double *>(raw.data())[b * pc + pidx];
-    });
-  return ICARUS_OK;
+  if (n != c->mem[member].leaves.size() * (size_t)c->kp.icells) return ICARUS_ERR_ARG;
+  return tracer_copy(c, member, host, nullptr);
 }
 
 icarus_status icarus_set_tracer(icarus_ctx *c, int member, const double *host, size_t n) {
   if (!member_ok(c, member) || !host) return ICARUS_ERR_ARG;
   if (!c->d.tracer) return ICARUS_ERR_STATE;
   if (c->poisoned) return ICARUS_ERR_STATE;
-  const size_t nl = c->mem[member].leaves.size(), ic = (size_t)c->kp.icells, pc = (size_t)c->kp.pcells;
-  if (n != nl * ic) return ICARUS_ERR_ARG;
+  if (n != c->mem[member].leaves.size() * (size_t)c->kp.icells) return ICARUS_ERR_ARG;
   c->ghosts_fresh = false;
-  std::vector<unsigned char> raw;
-  icarus_status st = tracer_planes(c, member, raw, true);   // keep the ghost layers
-  if (st != ICARUS_OK) return st;
-  for (size_t b = 0; b < nl; b++)
-    for_interior(c, [&](size_t q, size_t pidx) {
-      if (c->prec) reinterpret_cast<float *>(raw.data())[b * pc + pidx] = (float)host[b * ic + q];
-      else reinterpret_cast<double *>(raw.data())[b * pc + pidx] = host[b * ic + q];
-    });
-  return tracer_planes(c, member, raw, false);
+  return tracer_copy(c, member, nullptr, host);
 }
 
 icarus_status icarus_get_dt(icarus_ctx *c, double *dt) {

@@ -173,6 +173,10 @@ void dt_full_launch(const KParams &kp, const void *U, int precision, int nleaves
 // state and AMR support
 void pack_state_launch(const KParams &kp, const void *U, int precision, int slot0, int nslots, double *out,
                        cudaStream_t s);
+void pack_tracer_launch(const KParams &kp, const void *U, int precision, int slot0, int nslots, double *out,
+                        cudaStream_t s);
+void unpack_tracer_launch(const KParams &kp, void *U, int precision, int slot0, int nslots, const double *in,
+                          cudaStream_t s);
 void unpack_state_launch(const KParams &kp, void *U, int precision, int slot0, int nslots, const double *in,
                          int is_prim, cudaStream_t s);
 void estimator_launch(const KParams &kp, const void *U, int precision, int slot0, int nslots, double e_ref,

@@ -60,6 +60,26 @@ __global__ void k_unpack(const KParams kp, real *U, int slot0, int nslots, const
   }
 }
 
+// the tracer between the host's [slot][i][j][k] in FP64 and the padded planes
+template <typename real>
+__global__ void k_pack_tracer(const KParams kp, const real *U, int slot0, int nslots, double *out) {
+  const size_t n = (size_t)nslots * kp.icells;
+  for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
+    const int s = (int)(e / kp.icells), c = (int)(e - (size_t)s * kp.icells);
+    const int k = c % kp.nb[2], j = (c / kp.nb[2]) % kp.nb[1], i = c / (kp.nb[2] * kp.nb[1]);
+    out[e] = (double)U[tracer_index(kp, slot0 + s, i + NGH, j + NGH, k + NGH)];
+  }
+}
+template <typename real>
+__global__ void k_unpack_tracer(const KParams kp, real *U, int slot0, int nslots, const double *in) {
+  const size_t n = (size_t)nslots * kp.icells;
+  for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
+    const int s = (int)(e / kp.icells), c = (int)(e - (size_t)s * kp.icells);
+    const int k = c % kp.nb[2], j = (c / kp.nb[2]) % kp.nb[1], i = c / (kp.nb[2] * kp.nb[1]);
+    U[tracer_index(kp, slot0 + s, i + NGH, j + NGH, k + NGH)] = (real)in[e];
+  }
+}
+
 // ---- estimator ----
 __device__ __forceinline__ double est_pressure(const double *u, double gamma) {
   double msq = __dadd_rn(__dadd_rn(__dmul_rn(u[1], u[1]), __dmul_rn(u[2], u[2])), __dmul_rn(u[3], u[3]));
@@ -642,6 +662,24 @@ void pack_state_launch(const KParams &kp, const void *U, int precision, int slot
     k_pack<float><<<1024, 256, 0, s>>>(kp, (const float *)U, slot0, nslots, out);
   else
     k_pack<double><<<1024, 256, 0, s>>>(kp, (const double *)U, slot0, nslots, out);
+}
+
+void pack_tracer_launch(const KParams &kp, const void *U, int precision, int slot0, int nslots, double *out,
+                        cudaStream_t s) {
+  if (nslots <= 0) return;
+  if (precision)
+    k_pack_tracer<float><<<1024, 256, 0, s>>>(kp, (const float *)U, slot0, nslots, out);
+  else
+    k_pack_tracer<double><<<1024, 256, 0, s>>>(kp, (const double *)U, slot0, nslots, out);
+}
+
+void unpack_tracer_launch(const KParams &kp, void *U, int precision, int slot0, int nslots, const double *in,
+                          cudaStream_t s) {
+  if (nslots <= 0) return;
+  if (precision)
+    k_unpack_tracer<float><<<1024, 256, 0, s>>>(kp, (float *)U, slot0, nslots, in);
+  else
+    k_unpack_tracer<double><<<1024, 256, 0, s>>>(kp, (double *)U, slot0, nslots, in);
 }
 
 void unpack_state_launch(const KParams &kp, void *U, int precision, int slot0, int nslots, const double *in,
