@@ -1,0 +1,158 @@
+"""The size-dependent paths of the kernels at the sizes where they change:
+stage tiles, estimator slabs, features, training groups, physical corners and
+the read-back of the state."""
+import math
+
+import numpy as np
+import pytest
+
+from gpu_common import make_pair, rel_linf, wind_setup
+from oracle import mlp as M
+from paper_2211_12867_gb300 import inputs as I
+from paper_2211_12867_gb300.icarus import BC_OUTFLOW, BC_PERIODIC, BC_REFLECT, FP32_MIXED, FP64
+
+from test_gpu_mlp import _grad_magnitudes
+
+pytestmark = pytest.mark.gpu
+STR = dict(x_min=(0.1, math.pi / 6, 0.0), x_max=(2.0, 5 * math.pi / 6, 2 * math.pi), stretch=True)
+
+
+# blocks at and around the edges of the tiles (theta x phi): smaller than every
+# tile, exact, one row or column more, several ragged tiles; 4 to 66 planes
+@pytest.mark.parametrize("nb", [(4, 4, 4), (6, 8, 12), (12, 8, 16), (10, 12, 18), (4, 16, 16), (8, 18, 34),
+                                (66, 10, 22)])
+def test_chosen_tile_and_segment(nb):
+    """FP64 against the oracle (first-step bar of the parity tests: 1e-12);
+    FP32 the same bits whatever the tile."""
+    n = (2 * nb[0], nb[1], 2 * nb[2])
+    g, o = make_pair(n=n, nb=nb, **STR)
+    wind_setup(g, o)
+    g.step(2)
+    o.advance(2)
+    assert rel_linf(g.get_state(0), o.get_state()).max() < 1e-12
+    states = []
+    for tile in ((0, 0, 0), (8, 8, 0), (12, 20, 5)):
+        f, p = make_pair(n=n, nb=nb, precision=FP32_MIXED, tracer=True, **STR)
+        wind_setup(f, p)
+        f.set_tracer(0, 0.25 * f.get_state(0)[:, 0])
+        f.set_tile(*tile)
+        f.step(3)
+        states.append((f.get_state(0), f.get_tracer(0), f.dt()))
+    for s in states[1:]:
+        assert all(np.array_equal(x, y) for x, y in zip(s, states[0]))
+
+
+# four slabs of 1 to 4 planes, some of them empty; (8, 40, 96) has no room for
+# its planes in shared memory
+@pytest.mark.parametrize("precision", [FP64, FP32_MIXED])
+@pytest.mark.parametrize("nb", [(4, 6, 8), (6, 12, 12), (10, 4, 14), (14, 8, 6), (8, 40, 96)])
+def test_estimator_flags(nb, precision):
+    """bit for bit the oracle's flags on the blocks the device filled, at
+    thresholds between and on the values E takes"""
+    g, o = make_pair(n=(2 * nb[0], nb[1], 2 * nb[2]), nb=nb, precision=precision, **STR)
+    wind_setup(g, o)
+    g.inject_cone_cme(0, t_start=100.0, **I.cme_config2(seed=0))
+    o.snapshot_vbg()
+    U = g.get_state(0)
+    rng = np.random.default_rng(3)
+    # faster plasma in half of the cells, rougher from leaf to leaf, some near-vacuum
+    for leaf in range(len(U)):
+        f = 1.0 + (0.3 if leaf % 2 else 0.003) * rng.random(U.shape[2:])
+        U[leaf, :, ...] *= f
+        U[leaf, 1] *= np.where(rng.random(U.shape[2:]) < 0.5, 1.4, 1.0)
+        U[leaf, 4] += np.where(rng.random(U.shape[2:]) < 0.02, 1e-7, 1.0) * U[leaf, 1] ** 2 / U[leaf, 0]
+    g.set_state(0, U)
+    o.set_state(g.get_state(0))
+    for crit in (dict(e_refine=0.1, e_coarsen=0.0125), dict(e_refine=0.01, e_coarsen=0.001, eps=0.0),
+                 dict(e_refine=0.5, e_coarsen=0.2, dv=0.0), dict(e_refine=0.0, e_coarsen=0.0, dv=1e9)):
+        crit = dict(dict(eps=0.01, dv=0.5), **crit)
+        fg = g.flag_refine(**crit)
+        for n in range(o.nleaves):
+            o.set_padded(n, g.get_padded(0, n))
+        assert np.array_equal(fg, o.flag(**crit)), crit
+
+
+# sub-cubes of one cell to 100; the last two blocks have no room for three
+# planes in shared memory
+@pytest.mark.parametrize("precision", [FP64, FP32_MIXED])
+@pytest.mark.parametrize("nb", [(4, 4, 4), (8, 4, 12), (12, 20, 8), (8, 40, 40), (4, 8, 180)])
+def test_features(nb, precision):
+    """features of the padded blocks the device read: FP64 operations on both
+    sides, rounded to FP32 at the end (2^-24, doubled for a tie either way)"""
+    g, o = make_pair(n=(2 * nb[0], nb[1], nb[2]), nb=nb, precision=precision, **STR)
+    wind_setup(g, o)
+    g.step(3)
+    F = g.mlp_features()
+    for n in range(o.nleaves):
+        ref = M.features_from_padded(g.get_padded(0, n), 1.5)
+        assert np.allclose(F[n], ref, rtol=2.0 ** -22, atol=1e-12), n
+
+
+# groups of 8 samples: a part of one, one, one more, a last group of 1; more
+# groups than CTAs
+@pytest.mark.parametrize("batch", [1, 7, 8, 9, 1217, 4096])
+def test_gradient_of_a_batch(batch):
+    g, _ = make_pair(n=(24, 12, 12), nb=(12, 12, 12), **STR)
+    rng = np.random.default_rng(batch)
+    theta = I.mlp_init(1).astype(np.float32)
+    g.mlp_set_params(theta)
+    X = rng.uniform(0, 0.3, (batch, 64)).astype(np.float32)
+    T = (rng.random(batch) < 0.3).astype(np.float32)
+    gg, loss = g.mlp_grad(X, T)
+    again, loss2 = g.mlp_grad(X, T)
+    assert np.array_equal(gg, again) and loss == loss2
+    th, X64, T64 = theta.astype(np.float64), X.astype(np.float64), T.astype(np.float64)
+    go = M.grad(th, X64, T64)
+    # 1e-5 of the value plus 16 FP32 ulps of the running-error magnitude
+    assert np.all(np.abs(gg - go) <= 1e-5 * np.abs(go) + 1e-6 * _grad_magnitudes(th, X64, T64))
+    assert abs(loss - M.loss(th, X64, T64)) < 1e-5
+    assert np.allclose(g.mlp_predict(X), M.forward(th, X64)[0], rtol=1e-5, atol=1e-6)
+
+
+@pytest.mark.parametrize("lo,hi", [((BC_REFLECT, BC_OUTFLOW, BC_REFLECT), (BC_OUTFLOW, BC_REFLECT, BC_REFLECT)),
+                                   ((BC_OUTFLOW, BC_REFLECT, BC_PERIODIC), (BC_REFLECT, BC_REFLECT, BC_PERIODIC)),
+                                   ((BC_PERIODIC, BC_OUTFLOW, BC_OUTFLOW), (BC_PERIODIC, BC_OUTFLOW, BC_REFLECT))])
+def test_physical_corners(lo, hi):
+    """every ghost cell of a box, corners between boundaries of different
+    kinds among them: copies, the same bits"""
+    g, o = make_pair(n=(8, 6, 16), nb=(4, 6, 8), geometry=1, x_min=(0.0, 0.0, 0.0), x_max=(1.0, 1.0, 1.0), omega=0.0,
+                     bc_lo=lo, bc_hi=hi)
+    rng = np.random.default_rng(0)
+    W = rng.uniform(0.5, 2.0, (g.n_leaves(0), 8) + g.block)
+    g.set_state(0, W, prim=True)
+    o.set_state(g.get_state(0))
+    g.ghost_fill()
+    o.ghost_fill()
+    for n in range(o.nleaves):
+        assert np.array_equal(g.get_padded(0, n), o.get_padded(n, 0)), n
+
+
+@pytest.mark.parametrize("hours", [0.0, 0.7, 2.5, 4.1, 30.0])
+def test_inner_boundary_with_the_cone(hours):
+    """inner ghost cells while the cone opens, is open, closes and is gone:
+    the oracle's mask (arc cosines) cell by cell, values to 1e-14"""
+    g, o = make_pair(n=(24, 48, 96), nb=(12, 12, 12), **STR)
+    wind_setup(g, o)
+    cme = dict(I.cme_config2(seed=0), t_start=0.0)
+    g.inject_cone_cme(0, **cme)
+    o.set_cme(**cme)
+    g.set_time(0, I.hours(hours))
+    o.t = I.hours(hours)
+    g.ghost_fill()
+    o.ghost_fill()
+    for n, row in enumerate(o.tree()):
+        if row[1] == 0:
+            a, b = g.get_padded(0, n), o.get_padded(n, 0)
+            scale = np.abs(b).max(axis=(1, 2, 3), keepdims=True) + 1e-300
+            assert (np.abs(a - b) / scale).max() < 1e-14, n
+
+
+@pytest.mark.parametrize("precision", [FP64, FP32_MIXED])
+def test_state_into_pinned_memory(precision):
+    import torch
+    g, o = make_pair(n=(24, 8, 20), nb=(12, 8, 10), precision=precision, **STR)
+    wind_setup(g, o)
+    plain = g.get_state(0)
+    pinned = torch.zeros(plain.size + 8, dtype=torch.float64).pin_memory()
+    got = g.get_state(0, out=pinned[:plain.size].view(plain.shape).numpy())
+    assert np.array_equal(got, plain) and not pinned[plain.size:].any()
