@@ -153,8 +153,8 @@ Layout make_layout(const icarus_grid_desc *d) {
   L.scal = L.add((size_t)nm * 7 * sizeof(double) + 64);
   L.flags = L.add(mb);
   L.lists = L.add(2 * mb * sizeof(int));        // all-leaf list + per-level lists
-  L.rent = L.add((size_t)items_per_block(d) * mb * sizeof(int2));   // per level: ghost-fill work items
-  L.sides = L.add(6 * mb * sizeof(int2));       // (slot, side) per level, per direction
+  L.rent = L.add((size_t)items_per_block(d) * mb * sizeof(int2));   // ghost-fill work items
+  L.sides = L.add((amr ? 12 : 6) * mb * sizeof(int2));   // (slot, direction * 2 + side) per level; those next to another level
   L.rlist = L.add(mb * sizeof(int));
   L.ops = L.add(amr ? mb * sizeof(MoveOp) : 0);
   L.nshell = shell_count(d);
@@ -254,7 +254,7 @@ struct icarus_ctx {
   unsigned int *status = nullptr;
   signed char *flags = nullptr;
   int *all_list = nullptr, *lvl_list = nullptr, *rlist = nullptr, *shell = nullptr;
-  int2 *rent = nullptr;     // per level: (slot, region | finer << 8 | chunk << 9), up to 32 ghost tasks of a region held by coarser / finer leaves
+  int2 *rent = nullptr;     // (slot, region | finer << 8 | chunk << 9), up to 32 ghost tasks of a region held by coarser / finer leaves
   int *rshell = nullptr;    // per region (start, group-first cells, cells), then the shell cells ordered by region
   int2 *sides = nullptr;
   MoveOp *ops = nullptr;
@@ -265,9 +265,10 @@ struct icarus_ctx {
   std::vector<DevBlock> hblk;
   UploadBuffers upload;
   int lvl_count[MAXLEV + 1] = {0}, lvl_start[MAXLEV + 1] = {0};
-  int rent_start[MAXLEV + 1] = {0}, rent_face[MAXLEV + 1] = {0}, rent_count[MAXLEV + 1] = {0};
+  int res_face = 0, res_count = 0, pro_face = 0, pro_count = 0;   // items (faces first): restriction, then prolongation
   int reg_tab[27][3] = {};  // per region: start in the region-ordered shell, group-first cells, cells
   int side_count[MAXLEV + 1] = {0}, side_start[MAXLEV + 1] = {0};
+  int nsides = 0, nsides_mixed = 0;   // all of them; again those of leaves next to another level
   int nrlist = 0, max_level_present = 1;
   std::vector<signed char> hflags;
   bool flags_valid = false;
@@ -512,7 +513,8 @@ icarus_status upload_tree(icarus_ctx *c, DevBlock *blk_dst) {
   ent.clear();
   sv.clear();
   std::vector<std::vector<int>> per_level(MAXLEV + 1);
-  std::vector<std::vector<int2>> ent_face(MAXLEV + 1), ent_rest(MAXLEV + 1);
+  std::vector<int2> items[2][2];                   // [coarser, finer][face, rest]
+  std::vector<int2> sd2;                           // physical faces of leaves next to another level
   std::vector<std::vector<int2>> sd(MAXLEV + 1);   // (slot, direction * 2 + side) of the physical faces
   c->max_level_present = 1;
   // the relation of each leaf to the 27 regions around it (0 outside a
@@ -547,7 +549,7 @@ icarus_status upload_tree(icarus_ctx *c, DevBlock *blk_dst) {
       B.lmax = M.max_level;
       for (int k = 0; k < 3; k++) B.ix[k] = l.ix[k];
       B.phys = 0;
-      bool finer = false;
+      bool finer = false, mixed = false;
       for (int f = 0; f < 6; f++) {
         const int dd = f / 2, hi = f % 2;
         const int r = 13 + (hi ? 1 : -1) * (dd == 0 ? 9 : (dd == 1 ? 3 : 1));
@@ -570,8 +572,11 @@ icarus_status upload_tree(icarus_ctx *c, DevBlock *blk_dst) {
         const bool face = (dx != 0) + (dy != 0) + (dz != 0) == 1, fin = rs[r] == 3;
         const int tasks = fin ? c->reg_tab[r][2] : c->reg_tab[r][1];
         for (int ch = 0; 32 * ch < tasks; ch++)
-          (face ? ent_face : ent_rest)[l.level].push_back(make_int2(slot, r | (fin ? 256 : 0) | ch << 9));
+          items[fin][!face].push_back(make_int2(slot, r | (fin ? 256 : 0) | ch << 9));
+        mixed = true;
       }
+      for (int f = 0; f < 6 && mixed; f++)
+        if (B.nbr[f] == NB_PHYS) sd2.push_back(make_int2(slot, f));
       all[slot] = slot;
       per_level[l.level].push_back(slot);
       c->max_level_present = std::max(c->max_level_present, l.level);
@@ -593,18 +598,22 @@ icarus_status upload_tree(icarus_ctx *c, DevBlock *blk_dst) {
     c->lvl_start[L] = (int)lv.size();
     c->lvl_count[L] = (int)per_level[L].size();
     lv.insert(lv.end(), per_level[L].begin(), per_level[L].end());
-    c->rent_start[L] = (int)ent.size();
-    c->rent_face[L] = (int)ent_face[L].size();
-    c->rent_count[L] = (int)(ent_face[L].size() + ent_rest[L].size());
-    ent.insert(ent.end(), ent_face[L].begin(), ent_face[L].end());
-    ent.insert(ent.end(), ent_rest[L].begin(), ent_rest[L].end());
   }
+  for (const auto &part : {&items[1][0], &items[1][1], &items[0][0], &items[0][1]})
+    ent.insert(ent.end(), part->begin(), part->end());
+  c->res_face = (int)items[1][0].size();
+  c->res_count = c->res_face + (int)items[1][1].size();
+  c->pro_face = (int)items[0][0].size();
+  c->pro_count = c->pro_face + (int)items[0][1].size();
   if (ent.size() > (size_t)items_per_block(&c->d) * c->lay.max_blocks) return ICARUS_ERR_CAPACITY;
   for (int L = 1; L <= MAXLEV; L++) {
     c->side_start[L] = (int)sv.size();
     c->side_count[L] = (int)sd[L].size();
     sv.insert(sv.end(), sd[L].begin(), sd[L].end());
   }
+  c->nsides = (int)sv.size();
+  c->nsides_mixed = (int)sd2.size();
+  sv.insert(sv.end(), sd2.begin(), sd2.end());
   c->nrlist = (int)rl.size();
   {
     std::vector<double> &cm = u.cm;
@@ -986,20 +995,11 @@ struct ProfScope {
 // transverse halo; the corrector's cleaning takes div B on the ring around
 // the tile, which reaches edge ghosts, and the probe, the estimators and the
 // regrid get every ghost cell too.
-int enqueue_ghost(icarus_ctx *c, void *buf, double tfac, bool faces_only = false, bool skip_same = false) {
+int enqueue_ghost(icarus_ctx *c, void *buf, double tfac, bool faces_only = false) {
   int n = 0;
   for (int L = 1; L <= c->max_level_present; L++) {
     if (c->lvl_count[L] == 0) continue;
-    if (skip_same) {
-      // the ghost cells same-level leaves hold are read by the stage kernels
-      // from those leaves: only the regions held by coarser or finer leaves
-      const int ne = faces_only ? c->rent_face[L] : c->rent_count[L];
-      if (ne > 0) {
-        ProfScope p(c, 1);
-        ghost_regions_launch(c->kp, buf, c->prec, c->rent + c->rent_start[L], ne, c->rshell, L, c->stream);
-        n++;
-      }
-    } else {
+    {
       ProfScope p(c, 1);
       ghost_neighbour_launch(c->kp, buf, c->prec, c->lvl_list + c->lvl_start[L], c->lvl_count[L], c->shell,
                              faces_only ? c->nshell_face : c->lay.nshell, L, c->stream);
@@ -1007,19 +1007,57 @@ int enqueue_ghost(icarus_ctx *c, void *buf, double tfac, bool faces_only = false
     }
     if (c->side_count[L] > 0) {
       ProfScope p(c, 2);
-      ghost_physical_launch(c->kp, buf, c->prec, c->sides + c->side_start[L], c->side_count[L], L, tfac, faces_only,
-                            skip_same, c->stream);
+      ghost_physical_launch(c->kp, buf, c->prec, c->sides + c->side_start[L], c->side_count[L], tfac, faces_only,
+                            false, false, c->stream);
       n++;
     }
   }
   return n;
 }
 
+// launches of a fill that leaves the ghost cells of same-level leaves out
+struct DirectFill {
+  bool first, prolong, rest;
+};
+DirectFill direct_fill(const icarus_ctx *c, bool faces_only) {
+  return {(faces_only ? c->res_face : c->res_count) > 0 || c->nsides > 0,
+          (faces_only ? c->pro_face : c->pro_count) > 0, !faces_only && c->nsides_mixed > 0};
+}
+
+// The same without the ghost cells that same-level leaves hold (the stage
+// kernels read them from those leaves), all levels at once: at most three
+// launches whatever the number of levels (one launch for each level's regions
+// and one for its physical faces cost 80 of a 298 us step of a three-level
+// grid of 808 leaves of 8^3).
+int enqueue_ghost_direct(icarus_ctx *c, void *buf, double tfac, bool faces_only) {
+  const DirectFill f = direct_fill(c, faces_only);
+  if (f.first) {
+    ProfScope p(c, 2);
+    ghost_first_launch(c->kp, buf, c->prec, c->rent, faces_only ? c->res_face : c->res_count, c->rshell, c->sides,
+                       c->nsides, tfac, faces_only, c->stream);
+  }
+  if (f.prolong) {
+    ProfScope p(c, 1);
+    ghost_prolong_launch(c->kp, buf, c->prec, c->rent + c->res_count, faces_only ? c->pro_face : c->pro_count,
+                         c->rshell, c->stream);
+  }
+  if (f.rest) {
+    ProfScope p(c, 2);
+    ghost_physical_launch(c->kp, buf, c->prec, c->sides + c->nsides, c->nsides_mixed, tfac, false, true, true,
+                          c->stream);
+  }
+  return f.first + f.prolong + f.rest;
+}
+
+int enqueue_step_ghost(icarus_ctx *c, void *buf, double tfac, bool faces_only) {
+  return c->direct_halo ? enqueue_ghost_direct(c, buf, tfac, faces_only) : enqueue_ghost(c, buf, tfac, faces_only);
+}
+
 int enqueue_step(icarus_ctx *c) {
   int n = 0;
   // the step's fills leave the ghost cells that same-level leaves hold to the
   // stage kernels, which read them from those leaves
-  n += enqueue_ghost(c, c->U, 0.0, true, c->direct_halo);
+  n += enqueue_step_ghost(c, c->U, 0.0, true);
   StageLaunch s1 = stage_cfg(c, 0);
   s1.direct = c->direct_halo;
   s1.Uin = c->U;
@@ -1031,7 +1069,7 @@ int enqueue_step(icarus_ctx *c) {
     stage_launch(c->kp, s1, c->prec, c->stream);
   }
   n++;
-  n += enqueue_ghost(c, c->Us, 0.5, false, c->direct_halo);
+  n += enqueue_step_ghost(c, c->Us, 0.5, false);
   StageLaunch s2 = stage_cfg(c, 1);
   s2.direct = c->direct_halo;
   s2.Uin = c->Us;
@@ -1468,13 +1506,14 @@ icarus_status icarus_use_graph(icarus_ctx *c, int enable) {
 icarus_status icarus_kernels_per_step(icarus_ctx *c, int *n) {
   if (!c || !n) return ICARUS_ERR_ARG;
   int k = 3 + (c->nrlist > 0 ? 1 : 0);  // two stages, dt finalize, reflux
-  for (int L = 1; L <= c->max_level_present; L++) {
-    if (!c->lvl_count[L]) continue;
-    // neighbour ghost pass of both fills (with direct halo reads only over
-    // the regions held by coarser or finer leaves: faces in the first fill)
-    if (c->direct_halo) k += (c->rent_face[L] > 0) + (c->rent_count[L] > 0);
-    else k += 2;
-    if (c->side_count[L]) k += 2;   // physical ghost pass, both fills
+  // the two ghost fills
+  for (const bool faces : {true, false}) {
+    if (c->direct_halo) {
+      const DirectFill f = direct_fill(c, faces);
+      k += f.first + f.prolong + f.rest;
+    } else {
+      for (int L = 1; L <= c->max_level_present; L++) k += (c->lvl_count[L] > 0) + (c->side_count[L] > 0);
+    }
   }
   *n = k;
   return ICARUS_OK;

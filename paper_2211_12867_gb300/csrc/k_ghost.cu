@@ -82,11 +82,14 @@ __device__ __forceinline__ void store(const KParams &kp, real *U, Place c, const
 // padded index p: child (i, j, k) = parent + MC slopes x offsets; if any
 // child's density or pressure is not positive all eight take the parent
 // value.  The seven stencil cells are located once (all their loads are
-// independent); a first pass checks the eight children, a second writes them.
+// independent); a first pass checks the eight children, a second writes them
+// (one pass that wrote them and undid a failure, and two to eight lanes a
+// group, were slower: 267 to 270-274 us the step of 808 leaves of three levels
+// that takes two such launches).
 template <typename real>
 __device__ __forceinline__ void prolong_into(const KParams &kp, real *U, int cs, int Lc, const int *Ic, int slot, const int *p,
                              bool direct) {
-  const DevBlock C = kp.blk[cs];
+  const DevBlock &C = kp.blk[cs];
   int pc[3];
 #pragma unroll
   for (int d = 0; d < 3; d++) pc[d] = Ic[d] - C.ix[d] * kp.nb[d] + NGH;
@@ -242,62 +245,76 @@ __global__ void __launch_bounds__(256, sizeof(real) == 4 ? 4 : 2) k_ghost_neighb
   store(kp, U, {slot_base(kp, slot), pad_cell(kp, p[0], p[1], p[2])}, val);
 }
 
-// Ghost cells of one region of a level-L leaf (one of the 26 around it, r =
-// 9 (sx + 1) + 3 (sy + 1) + sz + 1) that a coarser leaf holds (one lane per
-// 2 x 2 x 2 group, prolongation) or finer leaves hold (one lane per cell,
-// restriction).  A work item is up to 32 such tasks of one region, taken
-// by one warp: item = (slot, r | finer << 8 | chunk << 9), tasks 32 chunk
-// .. 32 chunk + 31 of the region-ordered shell list (group-first cells
-// first) behind its table of (start, group-first cells, cells) per region.
+// The ghost fill of a step covers the regions around a leaf (one of the 26,
+// r = 9 (sx + 1) + 3 (sy + 1) + sz + 1) that a coarser leaf holds (one lane
+// per 2 x 2 x 2 group, prolongation) or finer leaves hold (one lane per cell,
+// restriction).  A work item is up to 32 such tasks of one region, taken by
+// one warp: item = (slot, r | finer << 8 | chunk << 9), tasks 32 chunk ..
+// 32 chunk + 31 of the region-ordered shell list (group-first cells first)
+// behind its table of (start, group-first cells, cells) per region.
 // Same-level halo cells the prolongation's stencil reaches are read from
 // the neighbouring leaf (the step's fills leave those ghost copies unfilled).
-template <typename real>
-__global__ void __launch_bounds__(256, sizeof(real) == 4 ? 3 : 2) k_ghost_regions(const KParams kp, real *U, const int2 *items, int nitems, const int *rshell, int L) {
-  const int w = blockIdx.x * 8 + (threadIdx.x >> 5);
-  if (w >= nitems) return;
-  const int2 e = items[w];
-  const int slot = e.x, r = e.y & 255;
-  const bool finer = ((e.y >> 8) & 1) != 0;
-  const int t = ((e.y >> 9) << 5) + (threadIdx.x & 31);
-  if (t >= (finer ? rshell[3 * r + 2] : rshell[3 * r + 1])) return;
-  const int code = rshell[81 + rshell[3 * r] + t];
-  const int p[3] = {code >> 20, (code >> 10) & 1023, code & 1023};
-  const DevBlock B = kp.blk[slot];
+struct Task {
+  int member, L, slot;
+  int p[3];   // padded index in the leaf
+  int b[3];   // block across, at the leaf's level
+  int q[3];   // padded index in that block
+  int G[3];   // global cell
+};
+__device__ __forceinline__ bool region_task(const KParams &kp, const int2 e, const int *rshell, Task &t) {
+  const int r = e.y & 255, n = ((e.y >> 9) << 5) + (threadIdx.x & 31);
+  if (n >= rshell[3 * r + 1 + ((e.y >> 8) & 1)]) return false;
+  const int code = rshell[81 + rshell[3 * r] + n];
+  const DevBlock &B = kp.blk[e.x];
   const int side[3] = {r / 9 - 1, (r / 3) % 3 - 1, r % 3 - 1};
-  int b[3], q[3], G[3];
+  t.member = B.member;
+  t.L = B.level;
+  t.slot = e.x;
+  t.p[0] = code >> 20;
+  t.p[1] = (code >> 10) & 1023;
+  t.p[2] = code & 1023;
 #pragma unroll
   for (int d = 0; d < 3; d++) {
     // items exist only for neighbours inside the domain or across a
     // periodic direction
-    const int nbl = kp.nbase[d] << (L - 1);
+    const int nbl = kp.nbase[d] << (t.L - 1);
     int bd = B.ix[d] + side[d];
     if (bd < 0) bd += nbl;
     else if (bd >= nbl) bd -= nbl;
-    b[d] = bd;
-    q[d] = p[d] - side[d] * kp.nb[d];   // padded index inside block b
-    G[d] = bd * kp.nb[d] + q[d] - NGH;
+    t.b[d] = bd;
+    t.q[d] = t.p[d] - side[d] * kp.nb[d];
+    t.G[d] = bd * kp.nb[d] + t.q[d] - NGH;
   }
-  if (!finer) {
-    int cb[3], Ic[3];
+  return true;
+}
+
+// Prolongation items of all levels: latency bound (a chain of five dependent
+// loads ahead of the stencil's), so one launch of all levels instead of one a
+// level.  A stencil reaches interiors, restricted
+// ghost cells and physical ghost cells straight across a face of the coarse
+// leaf, all of which the launch before has filled, and never a prolonged one:
+// with 2:1 balance over faces, edges and corners a cell within two coarse
+// cells of the fine leaf along an axis either touches it, so that its leaf is
+// at most one level coarser than the fine one, or lies in the coarse leaf
+// itself (blocks are four cells or more).
+template <typename real>
+__global__ void __launch_bounds__(128, sizeof(real) == 4 ? 5 : 3) k_ghost_prolong(const KParams kp, real *U, const int2 *items, int nitems, const int *rshell) {
+  const int w = blockIdx.x * 4 + (threadIdx.x >> 5);
+  if (w >= nitems) return;
+  Task t;
+  if (!region_task(kp, items[w], rshell, t)) return;
+  int cb[3], Ic[3];
 #pragma unroll
-    for (int d = 0; d < 3; d++) {
-      cb[d] = b[d] >> 1;
-      Ic[d] = G[d] >> 1;
-    }
-    const int cs = lookup_block(kp, B.member, L - 1, cb);
-    if (cs < 0) {
-      atomicOr(kp.status, ST_TREE);
-      return;
-    }
-    prolong_into<real>(kp, U, cs, L - 1, Ic, slot, p, true);
-  } else {
-    real val[NVAR + 1];
-    if (!restrict_in_block<real>(kp, U, B.member, L, b, q, G, val)) {
-      atomicOr(kp.status, ST_TREE);
-      return;
-    }
-    store(kp, U, {slot_base(kp, slot), pad_cell(kp, p[0], p[1], p[2])}, val);
+  for (int d = 0; d < 3; d++) {
+    cb[d] = t.b[d] >> 1;
+    Ic[d] = t.G[d] >> 1;
   }
+  const int cs = lookup_block(kp, t.member, t.L - 1, cb);
+  if (cs < 0) {
+    atomicOr(kp.status, ST_TREE);
+    return;
+  }
+  prolong_into<real>(kp, U, cs, t.L - 1, Ic, t.slot, t.p, true);
 }
 
 // Inner boundary state (FP64): map of the containing base cell, cone CME
@@ -343,28 +360,29 @@ __device__ __forceinline__ void inner_state(const KParams &kp, int member, int L
   u[TRV] = w[0] * X;
 }
 
-// Physical boundaries of all directions of a level's leaves in one launch;
-// sides[n] = (slot, direction * 2 + side).  The boundaries apply in the order
-// r, theta, phi over the whole padded slab, each reading what the earlier ones
-// wrote; here a ghost cell belongs to its highest physical direction and
-// composes the maps of that direction and of the lower ones down to the cell
-// (or inner-boundary state) that its value comes from, so no pass waits for
-// another.  faces: only the ghost cells inside the block in the two other
-// directions.  The two layers of the inner boundary hold one state: a thread
-// writes both.
+// Physical boundaries of all directions; side = (slot, direction * 2 + side),
+// idx a cell of its slab.  The boundaries apply in the order r, theta, phi
+// over the whole padded slab, each reading what the earlier ones wrote; here a
+// ghost cell belongs to its highest physical direction and composes the maps
+// of that direction and of the lower ones down to the cell (or inner-boundary
+// state) that its value comes from, so no pass waits for another.  faces: only
+// the ghost cells inside the block in the two other directions.  The two
+// layers of the inner boundary hold one state: a thread writes both.
+// part: the cells whose value comes from an interior, a same-level leaf or the
+// inner boundary (PHYS_READY), from a ghost cell under a coarser or finer leaf
+// (PHYS_REST), or both.
+enum { PHYS_READY = 1, PHYS_REST = 2 };
 template <typename real>
-__global__ void __launch_bounds__(128) k_ghost_physical(const KParams kp, real *U, const int2 *sides, int L, double tfac,
-                                                        int faces, int skip_same) {
-  const int2 sd = sides[blockIdx.x];
+__device__ __forceinline__ void physical_cell(const KParams &kp, real *U, const int2 sd, int idx, double tfac,
+                                              int faces, int skip_same, int part) {
   const int slot = sd.x, dir = sd.y >> 1, side = sd.y & 1;
   const int da = dir == 0 ? 1 : 0, db = dir == 2 ? 1 : 2;
   const int Pa = faces ? kp.nb[da] : kp.P[da], Pb = faces ? kp.nb[db] : kp.P[db], off = faces ? NGH : 0;
-  const int idx = blockIdx.y * blockDim.x + threadIdx.x;
   const bool inner = (side ? kp.bc_hi[dir] : kp.bc_lo[dir]) == 3;
   if (idx >= (inner ? 1 : NGH) * Pa * Pb) return;
   const int gl = idx / (Pa * Pb), r = idx - gl * (Pa * Pb), a = r / Pb + off, b = r - (r / Pb) * Pb + off;
   const DevBlock &B = kp.blk[slot];
-  const int phys = B.phys;
+  const int phys = B.phys, L = B.level;
   int q[3];
   q[dir] = side ? NGH + kp.nb[dir] + gl : NGH - 1 - gl;
   q[da] = a;
@@ -388,6 +406,16 @@ __global__ void __launch_bounds__(128) k_ghost_physical(const KParams kp, real *
       s[d] = hi ? NGH + nb - 1 : NGH;
     }
   }
+  if (part != (PHYS_READY | PHYS_REST)) {
+    bool ready = at_inner;
+    if (!ready) {
+      int r = 0;
+#pragma unroll
+      for (int d = 0; d < 3; d++) r = 3 * r + (s[d] < NGH ? 0 : (s[d] >= NGH + kp.nb[d] ? 2 : 1));
+      ready = r == 13 || kp.nb27[(size_t)slot * 27 + r] >= 0;
+    }
+    if (ready != (part == PHYS_READY)) return;
+  }
   real x[NVAR + 1];
   if (at_inner) {
     bool in;
@@ -409,6 +437,36 @@ __global__ void __launch_bounds__(128) k_ghost_physical(const KParams kp, real *
     }
   store(kp, U, {slot_base(kp, slot), pad_cell(kp, q[0], q[1], q[2])}, x);
   if (inner) store(kp, U, {slot_base(kp, slot), pad_cell(kp, 0, q[1], q[2])}, x);
+}
+
+template <typename real>
+__global__ void __launch_bounds__(128) k_ghost_physical(const KParams kp, real *U, const int2 *sides, double tfac,
+                                                        int faces, int skip_same, int part) {
+  physical_cell(kp, U, sides[blockIdx.x], blockIdx.y * 128 + threadIdx.x, tfac, faces, skip_same, part);
+}
+
+// First launch of a step's ghost fill, all levels: restriction items (the
+// first rblocks CTAs), then the physical ghost cells that come from interiors
+// (nchunk CTAs a side).  Neither reads what the other writes.
+template <typename real>
+__global__ void __launch_bounds__(128) k_ghost_first(const KParams kp, real *U, const int2 *items, int nitems,
+                                                     const int *rshell, int rblocks, const int2 *sides, int nchunk,
+                                                     double tfac, int faces) {
+  if ((int)blockIdx.x >= rblocks) {
+    const int n = blockIdx.x - rblocks, s = n / nchunk;
+    physical_cell(kp, U, sides[s], (n - s * nchunk) * 128 + threadIdx.x, tfac, faces, 1, (int)PHYS_READY);
+    return;
+  }
+  const int w = blockIdx.x * 4 + (threadIdx.x >> 5);
+  if (w >= nitems) return;
+  Task t;
+  if (!region_task(kp, items[w], rshell, t)) return;
+  real val[NVAR + 1];
+  if (!restrict_in_block<real>(kp, U, t.member, t.L, t.b, t.q, t.G, val)) {
+    atomicOr(kp.status, ST_TREE);
+    return;
+  }
+  store(kp, U, {slot_base(kp, t.slot), pad_cell(kp, t.p[0], t.p[1], t.p[2])}, val);
 }
 
 // reflux of coarse blocks with finer face neighbours; one CTA per block
@@ -615,31 +673,52 @@ void ghost_neighbour_launch(const KParams &kp, void *U, int precision, const int
     k_ghost_neighbour<double><<<grid, 256, 0, s>>>(kp, (double *)U, list, shell, nshell, level);
 }
 
-void ghost_regions_launch(const KParams &kp, void *U, int precision, const int2 *items, int nitems,
-                          const int *rshell, int level, cudaStream_t s) {
-  if (nitems <= 0) return;
-  const int grid = (nitems + 7) / 8;   // one warp per item
-  if (precision)
-    k_ghost_regions<float><<<grid, 256, 0, s>>>(kp, (float *)U, items, nitems, rshell, level);
-  else
-    k_ghost_regions<double><<<grid, 256, 0, s>>>(kp, (double *)U, items, nitems, rshell, level);
-}
-
-void ghost_physical_launch(const KParams &kp, void *U, int precision, const int2 *sides, int nsides, int level,
-                           double tfac, bool faces_only, bool skip_same, cudaStream_t s) {
-  if (nsides <= 0) return;
-  int n = 0;   // cells of the largest slab that can be physical
+namespace {
+// chunks of 128 cells of the largest slab that can be physical
+int physical_chunks(const KParams &kp, bool faces_only) {
+  int n = 0;
   for (int d = 0; d < 3; d++) {
     if (kp.bc_lo[d] == 0) continue;
     const int da = d == 0 ? 1 : 0, db = d == 2 ? 1 : 2;
     const int c = NGH * (faces_only ? kp.nb[da] * kp.nb[db] : kp.P[da] * kp.P[db]);
     n = c > n ? c : n;
   }
-  dim3 grid(nsides, (n + 127) / 128);
+  return (n + 127) / 128;
+}
+}  // namespace
+
+void ghost_first_launch(const KParams &kp, void *U, int precision, const int2 *items, int nitems, const int *rshell,
+                        const int2 *sides, int nsides, double tfac, bool faces_only, cudaStream_t s) {
+  const int nchunk = physical_chunks(kp, faces_only), rblocks = (nitems + 3) / 4;   // one warp per item
+  const int grid = rblocks + nsides * nchunk;
+  if (grid <= 0) return;
   if (precision)
-    k_ghost_physical<float><<<grid, 128, 0, s>>>(kp, (float *)U, sides, level, tfac, faces_only, skip_same);
+    k_ghost_first<float><<<grid, 128, 0, s>>>(kp, (float *)U, items, nitems, rshell, rblocks, sides, nchunk, tfac,
+                                              faces_only);
   else
-    k_ghost_physical<double><<<grid, 128, 0, s>>>(kp, (double *)U, sides, level, tfac, faces_only, skip_same);
+    k_ghost_first<double><<<grid, 128, 0, s>>>(kp, (double *)U, items, nitems, rshell, rblocks, sides, nchunk, tfac,
+                                               faces_only);
+}
+
+void ghost_prolong_launch(const KParams &kp, void *U, int precision, const int2 *items, int nitems, const int *rshell,
+                          cudaStream_t s) {
+  if (nitems <= 0) return;
+  const int grid = (nitems + 3) / 4;
+  if (precision)
+    k_ghost_prolong<float><<<grid, 128, 0, s>>>(kp, (float *)U, items, nitems, rshell);
+  else
+    k_ghost_prolong<double><<<grid, 128, 0, s>>>(kp, (double *)U, items, nitems, rshell);
+}
+
+void ghost_physical_launch(const KParams &kp, void *U, int precision, const int2 *sides, int nsides, double tfac,
+                           bool faces_only, bool skip_same, bool rest_only, cudaStream_t s) {
+  if (nsides <= 0) return;
+  dim3 grid(nsides, physical_chunks(kp, faces_only));
+  const int part = rest_only ? PHYS_REST : PHYS_READY | PHYS_REST;
+  if (precision)
+    k_ghost_physical<float><<<grid, 128, 0, s>>>(kp, (float *)U, sides, tfac, faces_only, skip_same, part);
+  else
+    k_ghost_physical<double><<<grid, 128, 0, s>>>(kp, (double *)U, sides, tfac, faces_only, skip_same, part);
 }
 
 void reflux_launch(const KParams &kp, void *U, const void *flux, int precision, const int *list, int nlist,

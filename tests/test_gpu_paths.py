@@ -156,3 +156,45 @@ def test_state_into_pinned_memory(precision):
     pinned = torch.zeros(plain.size + 8, dtype=torch.float64).pin_memory()
     got = g.get_state(0, out=pinned[:plain.size].view(plain.shape).numpy())
     assert np.array_equal(got, plain) and not pinned[plain.size:].any()
+
+
+WALLS = dict(geometry=1, x_min=(0.0, 0.0, 0.0), x_max=(1.0, 1.0, 1.0), omega=0.0)
+
+
+# the smallest blocks and ragged ones; all kinds of boundaries and a periodic
+# direction two blocks wide
+@pytest.mark.parametrize("precision", [FP64, FP32_MIXED])
+@pytest.mark.parametrize("nb,kw", [
+    ((4, 4, 4), STR), ((6, 4, 10), STR),
+    ((4, 4, 4), dict(WALLS, bc_lo=(BC_REFLECT, BC_OUTFLOW, BC_REFLECT), bc_hi=(BC_OUTFLOW, BC_REFLECT, BC_REFLECT))),
+    ((4, 6, 8), dict(WALLS, bc_lo=(BC_OUTFLOW, BC_REFLECT, BC_PERIODIC), bc_hi=(BC_REFLECT, BC_REFLECT, BC_PERIODIC))),
+    ((8, 4, 6), dict(WALLS, bc_lo=(BC_PERIODIC,) * 3, bc_hi=(BC_PERIODIC,) * 3))])
+def test_step_fill_of_all_levels_at_once(nb, kw, precision):
+    """random trees of three levels: the bits of steps whose fills go level by
+    level over every ghost cell"""
+    runs = []
+    for direct in (True, False):
+        g, o = make_pair(n=tuple(2 * b for b in nb), nb=nb, max_level=3, max_blocks=600, precision=precision,
+                         tracer=True, **kw)
+        rng = np.random.default_rng(7)
+        if "geometry" in kw:
+            W = 1.0 + 0.2 * rng.random((g.n_leaves(0), 8) + g.block)
+            g.set_state(0, W, prim=True)
+        else:
+            wind_setup(g, o)
+        for _ in range(2):
+            f = rng.random(g.n_leaves(0)) < 0.3
+            f[np.argmax(g.tree(0)[:, 0])] = True   # the first leaf of the finest level
+            g.set_flags(f.astype(np.int8))
+            g.regrid()
+        U = g.get_state(0)
+        U[:, :5] *= 1.0 + 0.02 * rng.random(U[:, :1].shape)
+        g.set_state(0, U)
+        g.set_tracer(0, U[:, 0] * rng.random(U[:, 0].shape))
+        g.set_direct_halo(direct)
+        g.step(4)
+        assert g.status()[0] & ~2 == 0   # floors may apply (bit 1)
+        runs.append((g.tree(0), g.get_state(0), g.get_tracer(0), g.dt()))
+    assert runs[0][0][:, 0].max() == 3
+    for a, b in zip(*runs):
+        assert np.array_equal(a, b)
