@@ -66,15 +66,12 @@ __device__ __forceinline__ double feature_of(const double *w0, const double (*d)
 // Features of 4 x 4 x 4 sub-cubes of s0 x s1 x s2 cells with s = n / 4.  One
 // CTA per leaf marches along r with the primitives of three planes (and one
 // halo cell around them) in shared memory, so a cell is converted 1.6 times
-// (12^3 block) instead of 7: the FP64 pipe bounds this kernel (one instruction
-// of a warp per 19 cycles of an SM, conversions from FP32 included), with 72
-// such instructions a cell instead of 400.  12^3 blocks, 808 leaves, ghost fill
-// included: 1283 ->
-// 389 us.  Each column sums its cells along r, then one warp per sub-cube its
-// columns in a fixed lane stride and shuffle tree, all in FP64: the features
-// are the same bits on every run and for every member.
-template <typename real>
-__global__ void __launch_bounds__(256) k_features(const KParams kp, const real *U, int slot0, float *out) {
+// (12^3 block) instead of 7.  Each column sums its cells along r, then one warp
+// per sub-cube its columns in a fixed lane stride and shuffle tree: the
+// features are the same bits on every run and for every member.
+// FP64 states: the FP64 pipe bounds this kernel (one instruction of a warp per
+// 19 cycles of an SM), with 72 such instructions a cell.
+__global__ void __launch_bounds__(256) k_features(const KParams kp, const double *U, int slot0, float *out) {
   extern __shared__ double smd[];
   const int slot = slot0 + blockIdx.x;
   const int n1 = kp.nb[1], n2 = kp.nb[2], h2 = n2 + 2, H = (n1 + 2) * h2;
@@ -124,32 +121,243 @@ __global__ void __launch_bounds__(256) k_features(const KParams kp, const real *
   }
 }
 
+// Sum over a sub-cube in FP64 by one warp, every cell converting its six
+// neighbours.
+template <typename real>
+__device__ __forceinline__ double subcube_sum(const KParams &kp, const real *U, int slot, int sc, int lane) {
+  const int s0 = kp.nb[0] / 4, s1 = kp.nb[1] / 4, s2 = kp.nb[2] / 4, per = s0 * s1 * s2;
+  const int a = sc / 16, b = (sc / 4) % 4, cc = sc % 4;
+  double acc = 0.0;
+  for (int t = lane; t < per; t += 32) {
+    const int p0 = NGH + a * s0 + t / (s1 * s2), p1 = NGH + b * s1 + (t / s2) % s1, p2 = NGH + cc * s2 + t % s2;
+    double w0[3], d[3][3];
+    feature_prims(kp, U, slot, p0, p1, p2, w0);
+#pragma unroll
+    for (int e = 0; e < 3; e++) {
+      double wm[3], wp[3];
+      feature_prims(kp, U, slot, p0 - (e == 0), p1 - (e == 1), p2 - (e == 2), wm);
+      feature_prims(kp, U, slot, p0 + (e == 0), p1 + (e == 1), p2 + (e == 2), wp);
+#pragma unroll
+      for (int q = 0; q < 3; q++) d[e][q] = wp[q] - wm[q];
+    }
+    acc += feature_of(w0, d);
+  }
+  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+  return acc;
+}
+
 // The same features where three planes do not fit in shared memory: one warp
-// per sub-cube, every cell converting its six neighbours.
+// per sub-cube.
 template <typename real>
 __global__ void __launch_bounds__(256) k_features_large(const KParams kp, const real *U, int slot0, float *out) {
-  const int slot = slot0 + blockIdx.x;
-  const int s0 = kp.nb[0] / 4, s1 = kp.nb[1] / 4, s2 = kp.nb[2] / 4, per = s0 * s1 * s2;
-  const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  const int slot = slot0 + blockIdx.x, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  const int per = (kp.nb[0] / 4) * (kp.nb[1] / 4) * (kp.nb[2] / 4);
   for (int sc = threadIdx.x >> 5; sc < 64; sc += nw) {
-    const int a = sc / 16, b = (sc / 4) % 4, cc = sc % 4;
-    double acc = 0.0;
-    for (int t = lane; t < per; t += 32) {
-      const int p0 = NGH + a * s0 + t / (s1 * s2), p1 = NGH + b * s1 + (t / s2) % s1, p2 = NGH + cc * s2 + t % s2;
-      double w0[3], d[3][3];
-      feature_prims(kp, U, slot, p0, p1, p2, w0);
-#pragma unroll
-      for (int e = 0; e < 3; e++) {
-        double wm[3], wp[3];
-        feature_prims(kp, U, slot, p0 - (e == 0), p1 - (e == 1), p2 - (e == 2), wm);
-        feature_prims(kp, U, slot, p0 + (e == 0), p1 + (e == 1), p2 + (e == 2), wp);
-#pragma unroll
-        for (int q = 0; q < 3; q++) d[e][q] = wp[q] - wm[q];
-      }
-      acc += feature_of(w0, d);
-    }
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    const double acc = subcube_sum(kp, U, slot, sc, lane);
     if (lane == 0) out[(size_t)blockIdx.x * 64 + sc] = (float)(acc / (6.0 * per));
+  }
+}
+
+// ---- FP32 states: the same sums in pairs of floats ----
+//
+// A number is h + l with |l| about half an ulp of h: 48 bits, by the
+// error-free sums and products of Dekker (1971) and Knuth.  A cell takes 430
+// instructions of the FP32 pipe instead of 72 of the FP64 pipe, of which each
+// costs 61 times as much.  Results are rounded to FP32 (2^-24), and the pairs'
+// errors stay below that (see FEAT_REL): against 80-bit arithmetic the largest
+// and mean errors on winds with and without CMEs are the FP64 kernel's to ten
+// digits (5.84e-8, 2.28e-8).  808 leaves of 12^3 on three levels: FP64 290 us
+// (the FP64 pipe 86 % busy), pairs 67 us; features with the ghost fill and
+// the copy to the host 390 -> 169 us.
+__device__ __forceinline__ float2 two_sum(float a, float b) {
+  const float s = __fadd_rn(a, b), t = __fsub_rn(s, a);
+  return make_float2(s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t)));
+}
+__device__ __forceinline__ float2 renorm(float h, float l) {   // |h| >= |l|
+  const float s = __fadd_rn(h, l);
+  return make_float2(s, __fsub_rn(l, __fsub_rn(s, h)));
+}
+__device__ __forceinline__ float2 pair_add(float2 a, float2 b) {
+  const float2 s = two_sum(a.x, b.x);
+  return renorm(s.x, __fadd_rn(s.y, __fadd_rn(a.y, b.y)));
+}
+__device__ __forceinline__ float2 pair_mul(float2 a, float2 b) {   // not renormalised
+  const float p = __fmul_rn(a.x, b.x);
+  return make_float2(p, __fmaf_rn(a.y, b.x, __fmaf_rn(a.x, b.y, __fmaf_rn(a.x, b.x, -p))));
+}
+__device__ __forceinline__ float2 pair_rcp(float2 a) {
+  float y;
+  asm("rcp.approx.f32 %0, %1;" : "=f"(y) : "f"(a.x));
+  const float e = __fmaf_rn(-a.y, y, __fmaf_rn(-a.x, y, 1.f));
+  return make_float2(y, __fmul_rn(y, __fmaf_rn(e, e, e)));
+}
+// a^2 + b^2 + c^2 of pairs
+__device__ __forceinline__ float2 pair_norm2(float2 a, float2 b, float2 c) {
+  const float p = __fmul_rn(a.x, a.x), q = __fmul_rn(b.x, b.x), r = __fmul_rn(c.x, c.x);
+  const float ep = __fmaf_rn(a.x + a.x, a.y, __fmaf_rn(a.x, a.x, -p));
+  const float eq = __fmaf_rn(b.x + b.x, b.y, __fmaf_rn(b.x, b.x, -q));
+  const float er = __fmaf_rn(c.x + c.x, c.y, __fmaf_rn(c.x, c.x, -r));
+  const float2 s = two_sum(p, q), t = two_sum(s.x, r);
+  return renorm(t.x, __fadd_rn(t.y, __fadd_rn(s.y, __fadd_rn(ep, __fadd_rn(eq, er)))));
+}
+
+// A cell's primitives carry relative errors of about 2^-46, the pressure
+// 2^-46 E / p from the difference that it is.  Cells with p < 2^-12 E, or out
+// of the range in which no product of theirs overflows or loses its low part,
+// are converted in FP64.  ratio: at least E / p of the others.
+__device__ __forceinline__ void pair_prims(const KParams &kp, const float *U, int slot, int i, int j, int k, float2 gm1,
+                                           float2 *w, float &ratio) {
+  float u[NVAR];
+  ld_cell(U + cell_index(kp, slot, i, j, k), u);
+  const float r = u[0], E = u[4];
+  const float2 z = make_float2(0.f, 0.f);
+  const float2 ir = pair_rcp(make_float2(r, 0.f));
+  const float2 M = pair_norm2(make_float2(u[1], 0.f), make_float2(u[2], 0.f), make_float2(u[3], 0.f));
+  const float2 B = pair_norm2(make_float2(u[5], 0.f), make_float2(u[6], 0.f), make_float2(u[7], 0.f));
+  const float2 K = pair_add(pair_mul(M, ir), B);
+  const float2 P = pair_add(make_float2(E, 0.f), make_float2(-0.5f * K.x, -0.5f * K.y));
+  if (P.x >= 0x1p-12f * E && E > 1e-20f && E < 1e15f && r > 1e-24f && r < 1e15f && r * E > 1e-31f) {
+    const float2 v = pair_mul(make_float2(u[1], 0.f), ir), p = pair_mul(P, gm1);
+    w[0] = make_float2(r, 0.f);
+    w[1] = renorm(v.x, v.y);
+    w[2] = renorm(p.x, p.y);
+    ratio = fmaxf(ratio, __fdividef(E, P.x));
+  } else {
+    double x[3];
+    feature_prims(kp, U, slot, i, j, k, x);
+#pragma unroll
+    for (int q = 0; q < 3; q++) {
+      w[q] = z;
+      w[q].x = (float)x[q];
+      w[q].y = (float)(x[q] - (double)w[q].x);
+    }
+  }
+}
+
+// feature_of in pairs, of the cell at P[q stride] (planes before, of and behind
+// it; rows of h2); the differences are taken relative to the cell first, so
+// that their squares stay in range whatever the units
+__device__ __forceinline__ float2 pair_feature(const float2 *Pm, const float2 *P, const float2 *Pp, int stride, int h2) {
+  float2 g = make_float2(0.f, 0.f);
+#pragma unroll
+  for (int q = 0; q < 3; q++) {
+    const float2 *C = P + q * stride;
+    auto diff = [](float2 a, float2 b) { return pair_add(a, make_float2(-b.x, -b.y)); };
+    const float2 d0 = diff(Pp[q * stride], Pm[q * stride]), d1 = diff(C[h2], C[-h2]), d2 = diff(C[1], C[-1]);
+    const float sg = C->x < 0.f ? -1.f : 1.f;
+    float2 w = make_float2(sg * C->x, sg * C->y);
+    if (w.x < 1e-15f) {   // where the 1e-30 that the magnitude is raised by counts
+      w = pair_add(w, make_float2(1e-30f, 0.f));
+      // too small for a pair: nothing if the neighbours are equal, else FP64
+      if (w.x < 1e-22f) {
+        if (!(d0.x == 0.f && d1.x == 0.f && d2.x == 0.f)) g.x = INFINITY;
+        continue;
+      }
+    }
+    const float2 y = pair_rcp(w);
+    const float2 s = pair_norm2(pair_mul(d0, y), pair_mul(d1, y), pair_mul(d2, y));
+    if (s.x != 0.f) {
+      float t;
+      asm("rsqrt.approx.f32 %0, %1;" : "=f"(t) : "f"(s.x));
+      const float f = __fmul_rn(s.x, t), e = __fadd_rn(__fmaf_rn(-f, f, s.x), s.y);
+      g = pair_add(g, make_float2(f, __fmul_rn(0.5f * t, e)));
+    }
+  }
+  return g;
+}
+
+// A sub-cube whose feature is below FEAT_REL E / p (its differences are within
+// the pairs' last 26 bits) is done again in FP64: the feature's relative
+// error is 2^-46 (E / p) / f at most, 2^-26 where the pairs are kept, a
+// quarter of the final rounding.  Smooth wind has features of 1e-3 and more
+// and E / p of 100 to 300.
+constexpr float FEAT_REL = 0x1p-20f;
+
+// k_features for FP32 states.  The halo cells at a plane's corners are not
+// read: a 12 x 12 plane takes the 192 threads once.  A sub-cube's sum and its
+// shuffles stay in pairs; the 64 divisions come at the end.
+constexpr int FEAT_NT = 192;
+__global__ void __launch_bounds__(FEAT_NT, 6) k_features_pairs(const KParams kp, const float *U, int slot0,
+                                                               float *out) {
+  extern __shared__ double smd[];
+  __shared__ unsigned worst;   // bits of the leaf's largest E / p
+  __shared__ float2 sums[64];
+  __shared__ float feat[64];
+  const int slot = slot0 + blockIdx.x;
+  const int n1 = kp.nb[1], n2 = kp.nb[2], h2 = n2 + 2, H = (n1 + 2) * h2;
+  const int s0 = kp.nb[0] / 4, s1 = n1 / 4, s2 = n2 / 4;
+  float2 *sm = reinterpret_cast<float2 *>(smd), *acc = sm + 9 * H;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const double gd = kp.gamma - 1.0;
+  const float2 gm1 = make_float2((float)gd, (float)(gd - (double)(float)gd));
+  float ratio = 1.f;
+  // the c-th cell of a plane and its halo: the rows of the block, then those
+  // before and behind it; the halo index of column t
+  const int mid = n1 * h2, cells = mid + 2 * n2;
+  auto halo = [&](int c) { return c < mid ? c + h2 : (c < mid + n2 ? c - mid + 1 : c - n2 + h2 + 1); };
+  auto column = [&](int t) { return (t / n2 + 1) * h2 + t % n2 + 1; };
+  const int hc = halo(tid), tc = column(tid), h_row = hc / h2, h_col = hc - h_row * h2;
+  auto plane = [&](int i) {   // primitives of padded plane i
+    float2 *P = sm + (i % 3) * 3 * H;
+    for (int c = tid; c < cells; c += FEAT_NT) {
+      int h = hc, row = h_row, col = h_col;
+      if (c != tid) {
+        h = halo(c);
+        row = h / h2;
+        col = h - row * h2;
+      }
+      float2 w[3];
+      pair_prims(kp, U, slot, i, NGH - 1 + row, NGH - 1 + col, gm1, w, ratio);
+      P[h] = w[0];
+      P[H + h] = w[1];
+      P[2 * H + h] = w[2];
+    }
+  };
+  if (tid == 0) worst = 0;
+  plane(NGH - 1);
+  plane(NGH);
+  for (int a = 0; a < 4; a++) {
+    for (int t = tid; t < n1 * n2; t += FEAT_NT) acc[t] = make_float2(0.f, 0.f);
+    for (int i = NGH + a * s0; i < NGH + (a + 1) * s0; i++) {
+      plane(i + 1);
+      __syncthreads();
+      const float2 *Pm = sm + ((i - 1) % 3) * 3 * H, *P = sm + (i % 3) * 3 * H, *Pp = sm + ((i + 1) % 3) * 3 * H;
+      for (int t = tid; t < n1 * n2; t += FEAT_NT) {
+        const int c = t == tid ? tc : column(t);
+        acc[t] = pair_add(acc[t], pair_feature(Pm + c, P + c, Pp + c, H, h2));
+      }
+      __syncthreads();   // plane i - 1 is read no more
+    }
+    for (int sc = warp; sc < 16; sc += FEAT_NT / 32) {
+      const int b = sc / 4, cc = sc % 4;
+      float2 s = make_float2(0.f, 0.f);
+      for (int t = lane; t < s1 * s2; t += 32) s = pair_add(s, acc[(b * s1 + t / s2) * n2 + cc * s2 + t % s2]);
+      for (int o = 16; o > 0; o >>= 1)
+        s = pair_add(s, make_float2(__shfl_xor_sync(0xffffffffu, s.x, o), __shfl_xor_sync(0xffffffffu, s.y, o)));
+      if (lane == 0) sums[a * 16 + sc] = s;
+    }
+    if (a < 3) __syncthreads();
+  }
+  {
+    const unsigned m = __reduce_max_sync(0xffffffffu, __float_as_uint(ratio));
+    if (lane == 0) atomicMax(&worst, m);
+  }
+  __syncthreads();
+  const double n6 = 6.0 * (s0 * s1 * s2);
+  if (tid < 64) {
+    const float2 s = sums[tid];
+    const float f = (float)(((double)s.x + (double)s.y) / n6);
+    feat[tid] = f;
+    out[(size_t)blockIdx.x * 64 + tid] = f;
+  }
+  __syncthreads();
+  const float least = FEAT_REL * __uint_as_float(worst);
+  for (int sc = warp; sc < 64; sc += FEAT_NT / 32) {
+    const float f = feat[sc];
+    if (f != 0.f && !(f >= least && f < 1e15f)) {   // NaN and overflow among them
+      const float x = (float)(subcube_sum(kp, U, slot, sc, lane) / n6);
+      if (lane == 0) out[(size_t)blockIdx.x * 64 + sc] = x;
+    }
   }
 }
 
@@ -383,8 +591,13 @@ void features(const KParams &kp, const real *U, int slot0, int nslots, float *ou
     k_features_large<real><<<nslots, 256, 0, s>>>(kp, U, slot0, out);
     return;
   }
-  cudaFuncSetAttribute(k_features<real>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  k_features<real><<<nslots, 256, smem, s>>>(kp, U, slot0, out);
+  if constexpr (sizeof(real) == 4) {
+    cudaFuncSetAttribute(k_features_pairs, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    k_features_pairs<<<nslots, FEAT_NT, smem, s>>>(kp, U, slot0, out);
+  } else {
+    cudaFuncSetAttribute(k_features, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    k_features<<<nslots, 256, smem, s>>>(kp, U, slot0, out);
+  }
 }
 }  // namespace
 

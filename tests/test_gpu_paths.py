@@ -88,6 +88,34 @@ def test_features(nb, precision):
         assert np.allclose(F[n], ref, rtol=2.0 ** -22, atol=1e-12), n
 
 
+# the FP32 mode's sums in float pairs and where they give way to FP64: units in
+# which densities are 1e-21, pressures 1e-5 of the energy, speeds of 0 and near
+# it, near-uniform and uniform leaves
+@pytest.mark.parametrize("kind", ["wind", "si", "cold", "still", "noise", "uniform"])
+def test_features_of_fp32_states(kind):
+    g, o = make_pair(n=(8, 24, 24), nb=(8, 12, 12), precision=FP32_MIXED, **dict(
+        geometry=1, x_min=(0.0, 0.0, 0.0), x_max=(1.0, 1.0, 1.0), omega=0.0, bc_lo=(BC_OUTFLOW,) * 3,
+        bc_hi=(BC_OUTFLOW,) * 3))
+    rng = np.random.default_rng(4)
+    a = {"noise": 2e-7, "uniform": 0.0}.get(kind, 0.1)
+    W = 1.0 + a * rng.random((g.n_leaves(0), 8) + g.block)
+    W[:, 1] *= 3.0
+    W[:, 4] *= 0.2
+    if kind == "si":
+        W *= np.array([1e-21, 4e5, 4e5, 4e5, 1e-11, 5e-6, 5e-6, 5e-6])[:, None, None, None]
+    if kind == "cold":
+        W[:, 4] *= np.where(rng.random(W[:, 4].shape) < 0.3, 1e-4, 1.0)
+    if kind == "still":
+        W[:, 1] *= np.where(rng.random(W[:, 1].shape) < 0.3, 0.0, 1e-12)
+        W[0, 1] = 0.0
+    g.set_state(0, W, prim=True)
+    F = g.mlp_features()
+    for n in range(o.nleaves):
+        ref = M.features_from_padded(g.get_padded(0, n), g.desc.gamma)
+        # the final rounding (2^-24) and both sides' own errors, at most as much
+        assert np.allclose(F[n], ref, rtol=2.0 ** -23, atol=0.0), (n, np.abs(F[n] / ref - 1).max())
+
+
 # groups of 8 samples: a part of one, one, one more, a last group of 1; more
 # groups than CTAs
 @pytest.mark.parametrize("batch", [1, 7, 8, 9, 1217, 4096])
