@@ -152,9 +152,9 @@ Layout make_layout(const icarus_grid_desc *d) {
   L.vbg = L.add((size_t)nm * d->n_cells[0] * d->n_cells[1] * d->n_cells[2] * sizeof(double));
   L.scal = L.add((size_t)nm * 7 * sizeof(double) + 64);
   L.flags = L.add(mb);
-  L.lists = L.add(2 * mb * sizeof(int));        // all-leaf list + per-level lists
+  L.lists = L.add(mb * sizeof(int));            // all-leaf list
   L.rent = L.add((size_t)items_per_block(d) * mb * sizeof(int2));   // ghost-fill work items
-  L.sides = L.add((amr ? 12 : 6) * mb * sizeof(int2));   // (slot, direction * 2 + side) per level; those next to another level
+  L.sides = L.add((amr ? 12 : 6) * mb * sizeof(int2));   // (slot, direction * 2 + side); those next to another level
   L.rlist = L.add(mb * sizeof(int));
   L.ops = L.add(amr ? mb * sizeof(MoveOp) : 0);
   L.nshell = shell_count(d);
@@ -220,7 +220,7 @@ struct TileCost {
 
 // host side of the tree's device tables, alive until their copies have landed
 struct UploadBuffers {
-  std::vector<int> nb27, all, rl, lm, lv;
+  std::vector<int> nb27, all, rl, lm;
   std::vector<long long> off;
   std::vector<int2> ent, sv;
   std::vector<double> cm;
@@ -253,7 +253,7 @@ struct icarus_ctx {
   unsigned long long *inv_max = nullptr, *floor_hits = nullptr, *floor_prev = nullptr;
   unsigned int *status = nullptr;
   signed char *flags = nullptr;
-  int *all_list = nullptr, *lvl_list = nullptr, *rlist = nullptr, *shell = nullptr;
+  int *all_list = nullptr, *rlist = nullptr, *shell = nullptr;
   int2 *rent = nullptr;     // (slot, region | finer << 8 | chunk << 9), up to 32 ghost tasks of a region held by coarser / finer leaves
   int *rshell = nullptr;    // per region (start, group-first cells, cells), then the shell cells ordered by region
   int2 *sides = nullptr;
@@ -264,10 +264,8 @@ struct icarus_ctx {
   std::vector<int> mem_off;                 // first slot of each member
   std::vector<DevBlock> hblk;
   UploadBuffers upload;
-  int lvl_count[MAXLEV + 1] = {0}, lvl_start[MAXLEV + 1] = {0};
   int res_face = 0, res_count = 0, pro_face = 0, pro_count = 0;   // items (faces first): restriction, then prolongation
   int reg_tab[27][3] = {};  // per region: start in the region-ordered shell, group-first cells, cells
-  int side_count[MAXLEV + 1] = {0}, side_start[MAXLEV + 1] = {0};
   int nsides = 0, nsides_mixed = 0;   // all of them; again those of leaves next to another level
   int nrlist = 0, max_level_present = 1;
   std::vector<signed char> hflags;
@@ -504,18 +502,15 @@ icarus_status upload_tree(icarus_ctx *c, DevBlock *blk_dst) {
   if (c->nleaves > c->lay.max_blocks) return ICARUS_ERR_CAPACITY;
   c->hblk.assign(c->nleaves, DevBlock{});
   UploadBuffers &u = c->upload;
-  std::vector<int> &nb27 = u.nb27, &all = u.all, &rl = u.rl, &lm = u.lm, &lv = u.lv;
+  std::vector<int> &nb27 = u.nb27, &all = u.all, &rl = u.rl, &lm = u.lm;
   std::vector<int2> &ent = u.ent, &sv = u.sv;
   nb27.assign((size_t)c->nleaves * 27, -1);
   all.resize(c->nleaves);
   rl.clear();
-  lv.clear();
   ent.clear();
   sv.clear();
-  std::vector<std::vector<int>> per_level(MAXLEV + 1);
   std::vector<int2> items[2][2];                   // [coarser, finer][face, rest]
-  std::vector<int2> sd2;                           // physical faces of leaves next to another level
-  std::vector<std::vector<int2>> sd(MAXLEV + 1);   // (slot, direction * 2 + side) of the physical faces
+  std::vector<int2> sd2;                           // physical faces (slot, direction * 2 + side) of leaves next to another level
   c->max_level_present = 1;
   // the relation of each leaf to the 27 regions around it (0 outside a
   // non-periodic direction, 1 same-level leaf, 2 coarser, 3 finer) and the
@@ -556,7 +551,7 @@ icarus_status upload_tree(icarus_ctx *c, DevBlock *blk_dst) {
         if (rs[r] == 0) {
           B.nbr[f] = NB_PHYS;
           B.phys |= 1 << f;
-          sd[l.level].push_back(make_int2(slot, f));
+          sv.push_back(make_int2(slot, f));
           continue;
         }
         B.nbr[f] = rs[r] == 1 ? NB_SAME : (rs[r] == 3 ? NB_FINER : NB_COARSER);
@@ -578,7 +573,6 @@ icarus_status upload_tree(icarus_ctx *c, DevBlock *blk_dst) {
       for (int f = 0; f < 6 && mixed; f++)
         if (B.nbr[f] == NB_PHYS) sd2.push_back(make_int2(slot, f));
       all[slot] = slot;
-      per_level[l.level].push_back(slot);
       c->max_level_present = std::max(c->max_level_present, l.level);
     }
   }
@@ -594,11 +588,6 @@ icarus_status upload_tree(icarus_ctx *c, DevBlock *blk_dst) {
       for (size_t q = 0; q < mp.size(); q++) lm[o + q] = mp[q] >= 0 ? mp[q] + c->mem_off[m] : mp[q];
       o += (long long)mp.size();
     }
-  for (int L = 1; L <= MAXLEV; L++) {
-    c->lvl_start[L] = (int)lv.size();
-    c->lvl_count[L] = (int)per_level[L].size();
-    lv.insert(lv.end(), per_level[L].begin(), per_level[L].end());
-  }
   for (const auto &part : {&items[1][0], &items[1][1], &items[0][0], &items[0][1]})
     ent.insert(ent.end(), part->begin(), part->end());
   c->res_face = (int)items[1][0].size();
@@ -606,11 +595,6 @@ icarus_status upload_tree(icarus_ctx *c, DevBlock *blk_dst) {
   c->pro_face = (int)items[0][0].size();
   c->pro_count = c->pro_face + (int)items[0][1].size();
   if (ent.size() > (size_t)items_per_block(&c->d) * c->lay.max_blocks) return ICARUS_ERR_CAPACITY;
-  for (int L = 1; L <= MAXLEV; L++) {
-    c->side_start[L] = (int)sv.size();
-    c->side_count[L] = (int)sd[L].size();
-    sv.insert(sv.end(), sd[L].begin(), sd[L].end());
-  }
   c->nsides = (int)sv.size();
   c->nsides_mixed = (int)sd2.size();
   sv.insert(sv.end(), sd2.begin(), sd2.end());
@@ -628,7 +612,6 @@ icarus_status upload_tree(icarus_ctx *c, DevBlock *blk_dst) {
   CK(cudaMemcpyAsync(c->lmap, lm.data(), sizeof(int) * lm.size(), cudaMemcpyHostToDevice, s));
   CK(cudaMemcpyAsync(c->lmap_off, off.data(), sizeof(long long) * off.size(), cudaMemcpyHostToDevice, s));
   CK(cudaMemcpyAsync(c->all_list, all.data(), sizeof(int) * all.size(), cudaMemcpyHostToDevice, s));
-  CK(cudaMemcpyAsync(c->lvl_list, lv.data(), sizeof(int) * lv.size(), cudaMemcpyHostToDevice, s));
   if (!ent.empty()) CK(cudaMemcpyAsync(c->rent, ent.data(), sizeof(int2) * ent.size(), cudaMemcpyHostToDevice, s));
   if (!sv.empty()) CK(cudaMemcpyAsync(c->sides, sv.data(), sizeof(int2) * sv.size(), cudaMemcpyHostToDevice, s));
   if (!rl.empty()) CK(cudaMemcpyAsync(c->rlist, rl.data(), sizeof(int) * rl.size(), cudaMemcpyHostToDevice, s));
@@ -995,46 +978,27 @@ struct ProfScope {
 // transverse halo; the corrector's cleaning takes div B on the ring around
 // the tile, which reaches edge ghosts, and the probe, the estimators and the
 // regrid get every ghost cell too.
-int enqueue_ghost(icarus_ctx *c, void *buf, double tfac, bool faces_only = false) {
-  int n = 0;
-  for (int L = 1; L <= c->max_level_present; L++) {
-    if (c->lvl_count[L] == 0) continue;
-    {
-      ProfScope p(c, 1);
-      ghost_neighbour_launch(c->kp, buf, c->prec, c->lvl_list + c->lvl_start[L], c->lvl_count[L], c->shell,
-                             faces_only ? c->nshell_face : c->lay.nshell, L, c->stream);
-      n++;
-    }
-    if (c->side_count[L] > 0) {
-      ProfScope p(c, 2);
-      ghost_physical_launch(c->kp, buf, c->prec, c->sides + c->side_start[L], c->side_count[L], tfac, faces_only,
-                            false, false, c->stream);
-      n++;
-    }
-  }
-  return n;
-}
-
-// launches of a fill that leaves the ghost cells of same-level leaves out
-struct DirectFill {
+// direct: without the ghost cells that same-level leaves hold (the stage
+// kernels read them from those leaves).  All levels at once, in at most three
+// launches whatever the number of levels (a launch for each level's regions and
+// one for its physical faces cost 80 of a 298 us step of 808 leaves of 12^3 on
+// three levels, now 48, and 75 us a full fill of them, now 51).
+struct Fill {
+  int nshell;
   bool first, prolong, rest;
+  int launches() const { return first + prolong + rest; }
 };
-DirectFill direct_fill(const icarus_ctx *c, bool faces_only) {
-  return {(faces_only ? c->res_face : c->res_count) > 0 || c->nsides > 0,
+Fill ghost_fill_of(const icarus_ctx *c, bool faces_only, bool direct) {
+  const int nshell = direct ? 0 : (faces_only ? c->nshell_face : c->lay.nshell);
+  return {nshell, nshell > 0 || (faces_only ? c->res_face : c->res_count) > 0 || c->nsides > 0,
           (faces_only ? c->pro_face : c->pro_count) > 0, !faces_only && c->nsides_mixed > 0};
 }
-
-// The same without the ghost cells that same-level leaves hold (the stage
-// kernels read them from those leaves), all levels at once: at most three
-// launches whatever the number of levels (one launch for each level's regions
-// and one for its physical faces cost 80 of a 298 us step of a three-level
-// grid of 808 leaves of 8^3).
-int enqueue_ghost_direct(icarus_ctx *c, void *buf, double tfac, bool faces_only) {
-  const DirectFill f = direct_fill(c, faces_only);
+int enqueue_ghost(icarus_ctx *c, void *buf, double tfac, bool faces_only = false, bool direct = false) {
+  const Fill f = ghost_fill_of(c, faces_only, direct);
   if (f.first) {
     ProfScope p(c, 2);
     ghost_first_launch(c->kp, buf, c->prec, c->rent, faces_only ? c->res_face : c->res_count, c->rshell, c->sides,
-                       c->nsides, tfac, faces_only, c->stream);
+                       c->nsides, tfac, faces_only, c->shell, f.nshell, c->nleaves, c->stream);
   }
   if (f.prolong) {
     ProfScope p(c, 1);
@@ -1043,21 +1007,16 @@ int enqueue_ghost_direct(icarus_ctx *c, void *buf, double tfac, bool faces_only)
   }
   if (f.rest) {
     ProfScope p(c, 2);
-    ghost_physical_launch(c->kp, buf, c->prec, c->sides + c->nsides, c->nsides_mixed, tfac, false, true, true,
-                          c->stream);
+    ghost_physical_launch(c->kp, buf, c->prec, c->sides + c->nsides, c->nsides_mixed, tfac, false, c->stream);
   }
-  return f.first + f.prolong + f.rest;
-}
-
-int enqueue_step_ghost(icarus_ctx *c, void *buf, double tfac, bool faces_only) {
-  return c->direct_halo ? enqueue_ghost_direct(c, buf, tfac, faces_only) : enqueue_ghost(c, buf, tfac, faces_only);
+  return f.launches();
 }
 
 int enqueue_step(icarus_ctx *c) {
   int n = 0;
   // the step's fills leave the ghost cells that same-level leaves hold to the
   // stage kernels, which read them from those leaves
-  n += enqueue_step_ghost(c, c->U, 0.0, true);
+  n += enqueue_ghost(c, c->U, 0.0, true, c->direct_halo);
   StageLaunch s1 = stage_cfg(c, 0);
   s1.direct = c->direct_halo;
   s1.Uin = c->U;
@@ -1069,7 +1028,7 @@ int enqueue_step(icarus_ctx *c) {
     stage_launch(c->kp, s1, c->prec, c->stream);
   }
   n++;
-  n += enqueue_step_ghost(c, c->Us, 0.5, false);
+  n += enqueue_ghost(c, c->Us, 0.5, false, c->direct_halo);
   StageLaunch s2 = stage_cfg(c, 1);
   s2.direct = c->direct_halo;
   s2.Uin = c->Us;
@@ -1268,7 +1227,6 @@ icarus_status icarus_init_grid(const icarus_grid_desc *desc, icarus_ctx **out) {
   c->floor_prev = reinterpret_cast<unsigned long long *>(sc + 7 * nm + 2);
   c->flags = at<signed char>(c, lay.flags);
   c->all_list = at<int>(c, lay.lists);
-  c->lvl_list = c->all_list + lay.max_blocks;
   c->rent = at<int2>(c, lay.rent);
   c->sides = at<int2>(c, lay.sides);
   c->rlist = at<int>(c, lay.rlist);
@@ -1506,15 +1464,7 @@ icarus_status icarus_use_graph(icarus_ctx *c, int enable) {
 icarus_status icarus_kernels_per_step(icarus_ctx *c, int *n) {
   if (!c || !n) return ICARUS_ERR_ARG;
   int k = 3 + (c->nrlist > 0 ? 1 : 0);  // two stages, dt finalize, reflux
-  // the two ghost fills
-  for (const bool faces : {true, false}) {
-    if (c->direct_halo) {
-      const DirectFill f = direct_fill(c, faces);
-      k += f.first + f.prolong + f.rest;
-    } else {
-      for (int L = 1; L <= c->max_level_present; L++) k += (c->lvl_count[L] > 0) + (c->side_count[L] > 0);
-    }
-  }
+  for (const bool faces : {true, false}) k += ghost_fill_of(c, faces, c->direct_halo).launches();
   *n = k;
   return ICARUS_OK;
 }

@@ -150,23 +150,21 @@ int stage_tile(int n, int *tj, int *tk);   // the n-th instantiated tile; 0 past
 int stage_ctas(int precision, int tj, int tk, int tracer);   // resident CTAs per SM
 
 // ghost fill
-// ghost_neighbour, then ghost_physical, level by level from the coarsest:
-// every ghost cell of the listed leaves (copy, prolongation or restriction;
-// sides: (slot, direction * 2 + side) of the physical faces).
-// The step's fills leave the ghost cells that same-level leaves hold to their
-// readers and take all levels at once: ghost_first (restriction items, and
-// the physical ghost cells that come from interiors), ghost_prolong, and
-// ghost_physical with rest_only (the physical edges that come from a ghost
-// cell under a coarser or finer leaf; none with faces_only).  Items: up to 32
-// cells (or 2x2x2 groups) of the regions around a leaf.
-void ghost_neighbour_launch(const KParams &kp, void *U, int precision, const int *list, int nlist,
-                            const int *shell, int nshell, int level, cudaStream_t s);
+// Three launches fill the ghost cells of all levels: ghost_first (restriction
+// items, the physical ghost cells that come from interiors, and copies of the
+// shell's cells from same-level leaves), ghost_prolong, and ghost_physical
+// (the physical edges that come from a ghost cell under a coarser or finer
+// leaf; none with faces_only).  The step's fills leave the ghost cells that
+// same-level leaves hold to their readers (nshell 0).  Items: up to 32 cells
+// (or 2x2x2 groups) of the regions around a leaf; sides: (slot, direction * 2
+// + side) of the physical faces.
 void ghost_first_launch(const KParams &kp, void *U, int precision, const int2 *items, int nitems, const int *rshell,
-                        const int2 *sides, int nsides, double tshift_fac, bool faces_only, cudaStream_t s);
+                        const int2 *sides, int nsides, double tshift_fac, bool faces_only, const int *shell, int nshell,
+                        int nleaves, cudaStream_t s);
 void ghost_prolong_launch(const KParams &kp, void *U, int precision, const int2 *items, int nitems, const int *rshell,
                           cudaStream_t s);
 void ghost_physical_launch(const KParams &kp, void *U, int precision, const int2 *sides, int nsides,
-                           double tshift_fac, bool faces_only, bool skip_same, bool rest_only, cudaStream_t s);
+                           double tshift_fac, bool faces_only, cudaStream_t s);
 void reflux_launch(const KParams &kp, void *U, const void *flux, int precision, const int *list, int nlist,
                    cudaStream_t s);
 void dt_begin_launch(const KParams &kp, const double *tstop, cudaStream_t s);

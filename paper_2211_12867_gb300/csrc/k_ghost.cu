@@ -1,8 +1,10 @@
 // Ghost-cell fill, reflux and time-step kernels.
 //
-// Two ghost layers per block (arXiv 2211.12867, Sect. 2.1).  Ghosts are
-// filled level by level, coarse to fine, so that a prolongation always reads
-// a coarse block whose own ghosts are complete:
+// Two ghost layers per block (arXiv 2211.12867, Sect. 2.1).  All levels are
+// filled at once, in an order in which no cell is read before it is written
+// (first launch: copies, restrictions and physical cells; second:
+// prolongations; third: the physical cells that come from ghost cells under
+// another level).  By what holds a ghost cell:
 //   * same-level leaf      -> copy of its interior cell
 //   * coarser leaf          -> conservative prolongation: parent value plus
 //                             monotonised-central slopes of the conserved
@@ -43,24 +45,21 @@ __device__ __forceinline__ int lookup(const KParams &kp, int member, int L, cons
   return kp.lmap[off + ((long long)b0 * n1 + b1) * n2 + b2];
 }
 
-// Slot and padded cell that hold padded index (p0, p1, p2) of leaf `slot`:
-// with `direct`, a cell of the ghost layer that a same-level leaf holds is
-// located in that leaf's interior (the ghost copy is not filled in the step's
-// fills).
+// Slot and padded cell that hold padded index (p0, p1, p2) of leaf `slot`: a
+// cell of the ghost layer that a same-level leaf holds is located in that
+// leaf's interior.
 struct Place {
   size_t base;
   int cell;
 };
-__device__ __forceinline__ Place locate(const KParams &kp, int slot, int p0, int p1, int p2, bool direct) {
-  if (direct) {
-    const int s0 = p0 < NGH ? -1 : (p0 >= NGH + kp.nb[0] ? 1 : 0);
-    const int s1 = p1 < NGH ? -1 : (p1 >= NGH + kp.nb[1] ? 1 : 0);
-    const int s2 = p2 < NGH ? -1 : (p2 >= NGH + kp.nb[2] ? 1 : 0);
-    if (s0 | s1 | s2) {
-      const int o = kp.nb27[(size_t)slot * 27 + (s0 + 1) * 9 + (s1 + 1) * 3 + (s2 + 1)];
-      if (o >= 0)
-        return {slot_base(kp, o), pad_cell(kp, p0 - s0 * kp.nb[0], p1 - s1 * kp.nb[1], p2 - s2 * kp.nb[2])};
-    }
+__device__ __forceinline__ Place locate(const KParams &kp, int slot, int p0, int p1, int p2) {
+  const int s0 = p0 < NGH ? -1 : (p0 >= NGH + kp.nb[0] ? 1 : 0);
+  const int s1 = p1 < NGH ? -1 : (p1 >= NGH + kp.nb[1] ? 1 : 0);
+  const int s2 = p2 < NGH ? -1 : (p2 >= NGH + kp.nb[2] ? 1 : 0);
+  if (s0 | s1 | s2) {
+    const int o = kp.nb27[(size_t)slot * 27 + (s0 + 1) * 9 + (s1 + 1) * 3 + (s2 + 1)];
+    if (o >= 0)
+      return {slot_base(kp, o), pad_cell(kp, p0 - s0 * kp.nb[0], p1 - s1 * kp.nb[1], p2 - s2 * kp.nb[2])};
   }
   return {slot_base(kp, slot), pad_cell(kp, p0, p1, p2)};
 }
@@ -87,8 +86,7 @@ __device__ __forceinline__ void store(const KParams &kp, real *U, Place c, const
 // group, were slower: 267 to 270-274 us the step of 808 leaves of three levels
 // that takes two such launches).
 template <typename real>
-__device__ __forceinline__ void prolong_into(const KParams &kp, real *U, int cs, int Lc, const int *Ic, int slot, const int *p,
-                             bool direct) {
+__device__ __forceinline__ void prolong_into(const KParams &kp, real *U, int cs, int Lc, const int *Ic, int slot, const int *p) {
   const DevBlock &C = kp.blk[cs];
   int pc[3];
 #pragma unroll
@@ -102,8 +100,8 @@ __device__ __forceinline__ void prolong_into(const KParams &kp, real *U, int cs,
     real um[3][NVAR + 1], uq[3][NVAR + 1];
 #pragma unroll
     for (int d = 0; d < 3; d++) {
-      fetch(kp, U, locate(kp, cs, pc[0] - (d == 0), pc[1] - (d == 1), pc[2] - (d == 2), direct), um[d]);
-      fetch(kp, U, locate(kp, cs, pc[0] + (d == 0), pc[1] + (d == 1), pc[2] + (d == 2), direct), uq[d]);
+      fetch(kp, U, locate(kp, cs, pc[0] - (d == 0), pc[1] - (d == 1), pc[2] - (d == 2)), um[d]);
+      fetch(kp, U, locate(kp, cs, pc[0] + (d == 0), pc[1] + (d == 1), pc[2] + (d == 2)), uq[d]);
     }
 #pragma unroll
     for (int d = 0; d < 3; d++)
@@ -185,67 +183,7 @@ __device__ __forceinline__ bool restrict_in_block(const KParams &kp, const real 
   return true;
 }
 
-// Same-level copy, prolongation or restriction into the ghost cells of the
-// level-L leaves.  The shell list holds the padded (p0, p1, p2) of a block's
-// ghost cells packed as p0 << 20 | p1 << 10 | p2; the neighbouring block and
-// the cell's index inside it follow from which side of the interior the
-// ghost lies on (no divisions).
-template <typename real>
-__global__ void __launch_bounds__(256, sizeof(real) == 4 ? 4 : 2) k_ghost_neighbour(const KParams kp, real *U, const int *list, const int *shell, int nshell,
-                                  int L) {
-  const int s = blockIdx.y * blockDim.x + threadIdx.x;
-  if (s >= nshell) return;
-  const int slot = list[blockIdx.x];
-  const int member = kp.blk[slot].member;
-  const int code = shell[s];
-  const int p[3] = {code >> 20, (code >> 10) & 1023, code & 1023};
-  int b[3], q[3], G[3];
-#pragma unroll
-  for (int d = 0; d < 3; d++) {
-    const int nb = kp.nb[d];
-    const int side = p[d] < NGH ? -1 : (p[d] >= NGH + nb ? 1 : 0);
-    const int nbl = kp.nbase[d] << (L - 1);
-    int bd = kp.blk[slot].ix[d] + side;
-    if (bd < 0 || bd >= nbl) {
-      if (kp.bc_lo[d] != 0) return;  // physical boundary pass fills it
-      bd += bd < 0 ? nbl : -nbl;     // periodic
-    }
-    b[d] = bd;
-    q[d] = p[d] - side * nb;          // padded index inside block b
-    G[d] = bd * nb + q[d] - NGH;      // global cell at level L
-  }
-  real val[NVAR + 1];
-  const int o = lookup_block(kp, member, L, b);
-  if (o >= 0) {
-    fetch(kp, U, {slot_base(kp, o), pad_cell(kp, q[0], q[1], q[2])}, val);
-  } else if (o == -1) {
-    // A coarse cell covers a 2 x 2 x 2 group of ghost cells (blocks start at
-    // even global indices and there are two ghost layers): the group's
-    // first cell computes the eight children once and writes all of them.
-    if ((p[0] | p[1] | p[2]) & 1) return;
-    int cb[3], Ic[3];
-#pragma unroll
-    for (int d = 0; d < 3; d++) {
-      cb[d] = b[d] >> 1;
-      Ic[d] = G[d] >> 1;
-    }
-    const int cs = lookup_block(kp, member, L - 1, cb);
-    if (cs < 0) {
-      atomicOr(kp.status, ST_TREE);
-      return;
-    }
-    prolong_into<real>(kp, U, cs, L - 1, Ic, slot, p, false);
-    return;
-  } else {
-    if (!restrict_in_block<real>(kp, U, member, L, b, q, G, val)) {
-      atomicOr(kp.status, ST_TREE);
-      return;
-    }
-  }
-  store(kp, U, {slot_base(kp, slot), pad_cell(kp, p[0], p[1], p[2])}, val);
-}
-
-// The ghost fill of a step covers the regions around a leaf (one of the 26,
+// The ghost fill's work items cover the regions around a leaf (one of the 26,
 // r = 9 (sx + 1) + 3 (sy + 1) + sz + 1) that a coarser leaf holds (one lane
 // per 2 x 2 x 2 group, prolongation) or finer leaves hold (one lane per cell,
 // restriction).  A work item is up to 32 such tasks of one region, taken by
@@ -253,7 +191,8 @@ __global__ void __launch_bounds__(256, sizeof(real) == 4 ? 4 : 2) k_ghost_neighb
 // 32 chunk + 31 of the region-ordered shell list (group-first cells first)
 // behind its table of (start, group-first cells, cells) per region.
 // Same-level halo cells the prolongation's stencil reaches are read from
-// the neighbouring leaf (the step's fills leave those ghost copies unfilled).
+// the neighbouring leaf (the step's fills leave those ghost copies unfilled,
+// and the others fill them in the same launch).
 struct Task {
   int member, L, slot;
   int p[3];   // padded index in the leaf
@@ -314,7 +253,7 @@ __global__ void __launch_bounds__(128, sizeof(real) == 4 ? 5 : 3) k_ghost_prolon
     atomicOr(kp.status, ST_TREE);
     return;
   }
-  prolong_into<real>(kp, U, cs, t.L - 1, Ic, t.slot, t.p, true);
+  prolong_into<real>(kp, U, cs, t.L - 1, Ic, t.slot, t.p);
 }
 
 // Inner boundary state (FP64): map of the containing base cell, cone CME
@@ -369,12 +308,12 @@ __device__ __forceinline__ void inner_state(const KParams &kp, int member, int L
 // the ghost cells inside the block in the two other directions.  The two
 // layers of the inner boundary hold one state: a thread writes both.
 // part: the cells whose value comes from an interior, a same-level leaf or the
-// inner boundary (PHYS_READY), from a ghost cell under a coarser or finer leaf
-// (PHYS_REST), or both.
+// inner boundary (PHYS_READY) or from a ghost cell under a coarser or finer
+// leaf (PHYS_REST).
 enum { PHYS_READY = 1, PHYS_REST = 2 };
 template <typename real>
 __device__ __forceinline__ void physical_cell(const KParams &kp, real *U, const int2 sd, int idx, double tfac,
-                                              int faces, int skip_same, int part) {
+                                              int faces, int part) {
   const int slot = sd.x, dir = sd.y >> 1, side = sd.y & 1;
   const int da = dir == 0 ? 1 : 0, db = dir == 2 ? 1 : 2;
   const int Pa = faces ? kp.nb[da] : kp.P[da], Pb = faces ? kp.nb[db] : kp.P[db], off = faces ? NGH : 0;
@@ -406,7 +345,7 @@ __device__ __forceinline__ void physical_cell(const KParams &kp, real *U, const 
       s[d] = hi ? NGH + nb - 1 : NGH;
     }
   }
-  if (part != (PHYS_READY | PHYS_REST)) {
+  {
     bool ready = at_inner;
     if (!ready) {
       int r = 0;
@@ -427,7 +366,7 @@ __device__ __forceinline__ void physical_cell(const KParams &kp, real *U, const 
 #pragma unroll
     for (int v = 0; v < NVAR + 1; v++) x[v] = (real)u[v];
   } else {
-    fetch(kp, U, locate(kp, slot, s[0], s[1], s[2], skip_same != 0), x);
+    fetch(kp, U, locate(kp, slot, s[0], s[1], s[2]), x);
   }
 #pragma unroll
   for (int d = 0; d < 3; d++)
@@ -439,34 +378,52 @@ __device__ __forceinline__ void physical_cell(const KParams &kp, real *U, const 
   if (inner) store(kp, U, {slot_base(kp, slot), pad_cell(kp, 0, q[1], q[2])}, x);
 }
 
+// the physical cells left by k_ghost_first, after the prolongation
 template <typename real>
 __global__ void __launch_bounds__(128) k_ghost_physical(const KParams kp, real *U, const int2 *sides, double tfac,
-                                                        int faces, int skip_same, int part) {
-  physical_cell(kp, U, sides[blockIdx.x], blockIdx.y * 128 + threadIdx.x, tfac, faces, skip_same, part);
+                                                        int faces) {
+  physical_cell(kp, U, sides[blockIdx.x], blockIdx.y * 128 + threadIdx.x, tfac, faces, PHYS_REST);
 }
 
-// First launch of a step's ghost fill, all levels: restriction items (the
-// first rblocks CTAs), then the physical ghost cells that come from interiors
-// (nchunk CTAs a side).  Neither reads what the other writes.
+// First launch of a ghost fill, all levels: restriction items (the first
+// rblocks CTAs), the physical ghost cells that come from interiors (nchunk
+// CTAs a side), and, in the fills that cover them, copies from same-level
+// leaves (ccopy CTAs a leaf; shell: the padded (p0, p1, p2) of a block's ghost
+// cells packed as p0 << 20 | p1 << 10 | p2).  None reads what another writes.
 template <typename real>
 __global__ void __launch_bounds__(128) k_ghost_first(const KParams kp, real *U, const int2 *items, int nitems,
-                                                     const int *rshell, int rblocks, const int2 *sides, int nchunk,
-                                                     double tfac, int faces) {
-  if ((int)blockIdx.x >= rblocks) {
-    const int n = blockIdx.x - rblocks, s = n / nchunk;
-    physical_cell(kp, U, sides[s], (n - s * nchunk) * 128 + threadIdx.x, tfac, faces, 1, (int)PHYS_READY);
+                                                     const int *rshell, int rblocks, const int2 *sides, int nsides,
+                                                     int nchunk, double tfac, int faces, const int *shell, int nshell,
+                                                     int ccopy) {
+  int n = blockIdx.x;
+  if (n < rblocks) {
+    const int w = n * 4 + (threadIdx.x >> 5);
+    if (w >= nitems) return;
+    Task t;
+    if (!region_task(kp, items[w], rshell, t)) return;
+    real val[NVAR + 1];
+    if (!restrict_in_block<real>(kp, U, t.member, t.L, t.b, t.q, t.G, val)) {
+      atomicOr(kp.status, ST_TREE);
+      return;
+    }
+    store(kp, U, {slot_base(kp, t.slot), pad_cell(kp, t.p[0], t.p[1], t.p[2])}, val);
     return;
   }
-  const int w = blockIdx.x * 4 + (threadIdx.x >> 5);
-  if (w >= nitems) return;
-  Task t;
-  if (!region_task(kp, items[w], rshell, t)) return;
+  n -= rblocks;
+  if (n < nsides * nchunk) {
+    const int s = n / nchunk;
+    physical_cell(kp, U, sides[s], (n - s * nchunk) * 128 + threadIdx.x, tfac, faces, PHYS_READY);
+    return;
+  }
+  n -= nsides * nchunk;
+  const int slot = n / ccopy, c = (n - slot * ccopy) * 128 + threadIdx.x;
+  if (c >= nshell) return;
+  const int code = shell[c], p0 = code >> 20, p1 = (code >> 10) & 1023, p2 = code & 1023;
+  const Place from = locate(kp, slot, p0, p1, p2), to = {slot_base(kp, slot), pad_cell(kp, p0, p1, p2)};
+  if (from.base == to.base && from.cell == to.cell) return;   // not a same-level leaf's
   real val[NVAR + 1];
-  if (!restrict_in_block<real>(kp, U, t.member, t.L, t.b, t.q, t.G, val)) {
-    atomicOr(kp.status, ST_TREE);
-    return;
-  }
-  store(kp, U, {slot_base(kp, t.slot), pad_cell(kp, t.p[0], t.p[1], t.p[2])}, val);
+  fetch(kp, U, from, val);
+  store(kp, U, to, val);
 }
 
 // reflux of coarse blocks with finer face neighbours; one CTA per block
@@ -663,16 +620,6 @@ __global__ void k_dt_from_max(const KParams kp, double cfl) {
 
 }  // namespace
 
-void ghost_neighbour_launch(const KParams &kp, void *U, int precision, const int *list, int nlist, const int *shell,
-                            int nshell, int level, cudaStream_t s) {
-  if (nlist <= 0) return;
-  dim3 grid(nlist, (nshell + 255) / 256);
-  if (precision)
-    k_ghost_neighbour<float><<<grid, 256, 0, s>>>(kp, (float *)U, list, shell, nshell, level);
-  else
-    k_ghost_neighbour<double><<<grid, 256, 0, s>>>(kp, (double *)U, list, shell, nshell, level);
-}
-
 namespace {
 // chunks of 128 cells of the largest slab that can be physical
 int physical_chunks(const KParams &kp, bool faces_only) {
@@ -688,16 +635,17 @@ int physical_chunks(const KParams &kp, bool faces_only) {
 }  // namespace
 
 void ghost_first_launch(const KParams &kp, void *U, int precision, const int2 *items, int nitems, const int *rshell,
-                        const int2 *sides, int nsides, double tfac, bool faces_only, cudaStream_t s) {
+                        const int2 *sides, int nsides, double tfac, bool faces_only, const int *shell, int nshell,
+                        int nleaves, cudaStream_t s) {
   const int nchunk = physical_chunks(kp, faces_only), rblocks = (nitems + 3) / 4;   // one warp per item
-  const int grid = rblocks + nsides * nchunk;
+  const int ccopy = (nshell + 127) / 128, grid = rblocks + nsides * nchunk + nleaves * ccopy;
   if (grid <= 0) return;
   if (precision)
-    k_ghost_first<float><<<grid, 128, 0, s>>>(kp, (float *)U, items, nitems, rshell, rblocks, sides, nchunk, tfac,
-                                              faces_only);
+    k_ghost_first<float><<<grid, 128, 0, s>>>(kp, (float *)U, items, nitems, rshell, rblocks, sides, nsides, nchunk, tfac,
+        faces_only, shell, nshell, ccopy);
   else
-    k_ghost_first<double><<<grid, 128, 0, s>>>(kp, (double *)U, items, nitems, rshell, rblocks, sides, nchunk, tfac,
-                                               faces_only);
+    k_ghost_first<double><<<grid, 128, 0, s>>>(kp, (double *)U, items, nitems, rshell, rblocks, sides, nsides, nchunk, tfac,
+        faces_only, shell, nshell, ccopy);
 }
 
 void ghost_prolong_launch(const KParams &kp, void *U, int precision, const int2 *items, int nitems, const int *rshell,
@@ -711,14 +659,13 @@ void ghost_prolong_launch(const KParams &kp, void *U, int precision, const int2 
 }
 
 void ghost_physical_launch(const KParams &kp, void *U, int precision, const int2 *sides, int nsides, double tfac,
-                           bool faces_only, bool skip_same, bool rest_only, cudaStream_t s) {
+                           bool faces_only, cudaStream_t s) {
   if (nsides <= 0) return;
   dim3 grid(nsides, physical_chunks(kp, faces_only));
-  const int part = rest_only ? PHYS_REST : PHYS_READY | PHYS_REST;
   if (precision)
-    k_ghost_physical<float><<<grid, 128, 0, s>>>(kp, (float *)U, sides, tfac, faces_only, skip_same, part);
+    k_ghost_physical<float><<<grid, 128, 0, s>>>(kp, (float *)U, sides, tfac, faces_only);
   else
-    k_ghost_physical<double><<<grid, 128, 0, s>>>(kp, (double *)U, sides, tfac, faces_only, skip_same, part);
+    k_ghost_physical<double><<<grid, 128, 0, s>>>(kp, (double *)U, sides, tfac, faces_only);
 }
 
 void reflux_launch(const KParams &kp, void *U, const void *flux, int precision, const int *list, int nlist,

@@ -226,3 +226,37 @@ def test_step_fill_of_all_levels_at_once(nb, kw, precision):
     assert runs[0][0][:, 0].max() == 3
     for a, b in zip(*runs):
         assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("nb,kw", [
+    ((4, 4, 4), STR), ((6, 4, 10), dict(STR, bc_lo=(3, 1, 0), bc_hi=(1, 2, 0))),
+    ((4, 6, 8), dict(WALLS, bc_lo=(BC_OUTFLOW, BC_REFLECT, BC_PERIODIC), bc_hi=(BC_REFLECT, BC_REFLECT, BC_PERIODIC))),
+    ((8, 4, 6), dict(WALLS, bc_lo=(BC_PERIODIC,) * 3, bc_hi=(BC_PERIODIC,) * 3))])
+def test_full_fill_of_a_tree(nb, kw):
+    """every ghost cell of a random tree of three levels against the oracle,
+    which fills level by level; 1e-13 of a variable's largest value (the bar of
+    the prolonged data of the regrid tests)"""
+    g, o = make_pair(n=(2 * nb[0], 2 * nb[1], nb[2]), nb=nb, max_level=3, max_blocks=600, **kw)
+    rng = np.random.default_rng(11)
+    if "geometry" in kw:
+        g.set_state(0, 1.0 + 0.2 * rng.random((g.n_leaves(0), 8) + g.block), prim=True)
+        o.set_state(g.get_state(0))
+    else:
+        wind_setup(g, o)
+    for _ in range(2):
+        f = rng.random(g.n_leaves(0)) < 0.3
+        f[np.argmax(g.tree(0)[:, 0])] = True
+        f = f.astype(np.int8)
+        g.set_flags(f)
+        g.regrid()
+        o.regrid(f)
+    assert np.array_equal(g.tree(0), o.tree()) and g.tree(0)[:, 0].max() == 3
+    U = g.get_state(0)
+    U[:, :5] *= 1.0 + 0.02 * rng.random(U[:, :1].shape)
+    g.set_state(0, U)
+    o.set_state(g.get_state(0))
+    g.ghost_fill()
+    o.ghost_fill()
+    scale = np.abs(U).max(axis=(0, 2, 3, 4))[:, None, None, None] + 1e-300
+    for n in range(o.nleaves):
+        assert (np.abs(g.get_padded(0, n) - o.get_padded(n, 0)) / scale).max() < 1e-13, n
