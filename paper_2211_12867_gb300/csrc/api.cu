@@ -2140,7 +2140,7 @@ icarus_status icarus_mlp_train(icarus_ctx *c, int n_train, int epochs, int batch
       const int B = std::min(batch, n_train - b0);
       const int *idx = c->mlp_idx + b0;
       mlp_step_launch(c->mlp_theta, c->mlp_m, c->mlp_v, c->mlp_X, c->mlp_T, idx, B, c->mlp_part, c->mlp_loss, (float)lr,
-                      ++c->mlp_step, c->stream);
+                      ++c->mlp_step, b0 > 0, c->stream);
     }
     CK(cudaPeekAtLastError());
     float l = 0.f;

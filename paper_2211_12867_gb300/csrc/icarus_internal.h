@@ -211,9 +211,10 @@ size_t mlp_partial_floats();
 // gradient of the mean cross-entropy; the summed cross-entropy adds to *loss
 void mlp_grad_launch(const float *theta, const float *X, const float *T, const int *idx, int B, float *part, float *grad,
                      float *loss, cudaStream_t s);
-// the same and the Adam step with it
+// the same and the Adam step with it; more: the launch before in the stream is
+// such a step's, on the same X, T and index list
 void mlp_step_launch(float *theta, float *m, float *v, const float *X, const float *T, const int *idx, int B, float *part,
-                     float *loss, float lr, int step, cudaStream_t s);
+                     float *loss, float lr, int step, bool more, cudaStream_t s);
 void mlp_combine_launch(const float *prob, const DevBlock *blk, signed char *flags, int n, cudaStream_t s);
 
 struct icarus_ctx;

@@ -12,9 +12,11 @@
 // pass and the outer products of the weight gradients, which stay in registers
 // (96 per thread) until the CTA has done its groups; k_reduce adds the CTAs'
 // partial gradients in a fixed order (the gradient is the same bits on every
-// call) and takes the Adam step.  Four launches with the activations in global
-// memory and one thread per parameter summing over the batch took 120 us for
-// a batch of 1024, latency all of it (50 MFLOP).
+// call) and takes the Adam step.  Latency bounds both (50 MFLOP and 13 MB of
+// partial gradients for a batch of 1024): 15 and 7 us, beginnings and ends
+// overlapping (four launches with the activations in global memory and one
+// thread per parameter summing over the batch took 120 us; weights copied and
+// partial gradients written word by word 25 and 8 us).
 #include "mhd_device.cuh"
 
 #define MLP_IN 64
@@ -363,9 +365,15 @@ __global__ void __launch_bounds__(FEAT_NT, 6) k_features_pairs(const KParams kp,
 
 constexpr int NT = 256;          // threads of k_mlp
 constexpr int GS = 8;            // samples of a group: two quads
-constexpr int S1 = MLP_IN + 1, S2 = MLP_H + 1;   // row strides in shared memory (no bank conflicts by row or column)
-constexpr int NPAR = MLP_H * MLP_IN + MLP_H + MLP_H * MLP_H + MLP_H + MLP_H + 1;
-constexpr int PART = NPAR + 1;   // a CTA's partial gradient and loss
+// row strides in shared memory: 16-byte rows, and an odd number of 16-byte
+// units, so neither four columns of 32 rows nor one row of 32 columns conflict
+constexpr int S1 = MLP_IN + 4, S2 = MLP_H + 4;
+constexpr int NW = MLP_H * (MLP_IN + MLP_H);   // weights
+constexpr int NPAR = NW + MLP_H + MLP_H + MLP_H + 1;
+// A CTA's partial gradient in the order its threads hold it: the weights as
+// [4 columns of a tile's row][thread][4], W2 first, then b1, b2, w3, b3, the
+// loss, rounded up to 16 bytes
+constexpr int PART = (NPAR + 1 + 3) / 4 * 4;
 constexpr int MLP_SMEM = (MLP_H * S1 + MLP_H * S2 + GS * (MLP_IN + 3 * MLP_H) + GS * (NT / 32) + 2 * GS) * 4;
 
 // Forward pass of the rows of X (row index list `idx` or identity), and with
@@ -374,6 +382,12 @@ constexpr int MLP_SMEM = (MLP_H * S1 + MLP_H * S2 + GS * (MLP_IN + 3 * MLP_H) + 
 // has one hidden unit and one quad of samples; vectors over units lie in
 // shared memory as [quad][unit][4], so a weight meets four samples per load.
 // The weight gradients are 8 x 8 and 8 x 4 tiles of outer products per thread.
+// Programmatic dependent launch: waits until the kernel before in the stream
+// has completed, and lets the next one be launched (both without effect in a
+// plain launch)
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_launch_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 template <bool GRAD>
 __global__ void __launch_bounds__(NT) k_mlp(const float *theta, const float *X, const float *T, const int *idx, int B,
                                             float *y, float *part) {
@@ -382,8 +396,20 @@ __global__ void __launch_bounds__(NT) k_mlp(const float *theta, const float *X, 
   float *red = d1s + GS * MLP_H, *dzs = red + GS * (NT / 32), *W1s = dzs + 2 * GS, *W2s = W1s + MLP_H * S1;
   const MlpView m = mlp_view(theta);
   const int tid = threadIdx.x, j = tid & (MLP_H - 1), q = tid >> 7, warp = tid >> 5;
-  for (int e = tid; e < MLP_H * MLP_IN; e += NT) W1s[(e / MLP_IN) * S1 + e % MLP_IN] = m.W1[e];
-  for (int e = tid; e < MLP_H * MLP_H; e += NT) W2s[(e / MLP_H) * S2 + e % MLP_H] = m.W2[e];
+  auto gather = [&](int s0) {
+    for (int e = tid; e < GS * MLP_IN; e += NT) {
+      const int s = e / MLP_IN, i = e % MLP_IN;
+      const int row = s0 + s < B ? (idx ? idx[s0 + s] : s0 + s) : -1;
+      xs[((s >> 2) * MLP_IN + i) * 4 + (s & 3)] = row >= 0 ? X[(size_t)row * MLP_IN + i] : 0.f;
+    }
+  };
+  // the first group's samples while the step of the batch before may still run
+  // (see mlp_step_launch), then the weights that it leaves
+  gather(blockIdx.x * GS);
+  grid_wait();
+  for (int e = 4 * tid; e < MLP_H * MLP_IN; e += 4 * NT) cp_async<16>(W1s + (e / MLP_IN) * S1 + e % MLP_IN, m.W1 + e);
+  for (int e = 4 * tid; e < MLP_H * MLP_H; e += 4 * NT) cp_async<16>(W2s + (e / MLP_H) * S2 + e % MLP_H, m.W2 + e);
+  cp_async_commit();
   const float b1 = m.b1[j], b2 = m.b2[j], w3 = m.w3[j], b3 = m.b3[0];
   const int tj = tid >> 4, tk = tid & 15;   // gradient tile: rows tj + 16 a, columns tk + 16 b
   float g2[8][8], g1[8][4], gb1 = 0.f, gb2 = 0.f, gw3 = 0.f, gb3 = 0.f, loss = 0.f;
@@ -400,36 +426,34 @@ __global__ void __launch_bounds__(NT) k_mlp(const float *theta, const float *X, 
     return *reinterpret_cast<const float4 *>(v + (qd * n + unit) * 4);
   };
   for (int s0 = blockIdx.x * GS; s0 < B; s0 += gridDim.x * GS) {
-    __syncthreads();   // the previous group's vectors (and, first, the weights)
-    for (int e = tid; e < GS * MLP_IN; e += NT) {
-      const int s = e / MLP_IN, i = e % MLP_IN;
-      const int row = s0 + s < B ? (idx ? idx[s0 + s] : s0 + s) : -1;
-      xs[((s >> 2) * MLP_IN + i) * 4 + (s & 3)] = row >= 0 ? X[(size_t)row * MLP_IN + i] : 0.f;
+    if (s0 != (int)blockIdx.x * GS) {
+      __syncthreads();   // the previous group's vectors
+      gather(s0);
     }
+    cp_async_wait_all();
     __syncthreads();
     float a0 = b1, a1 = b1, a2 = b1, a3 = b1;
-#pragma unroll 8
-    for (int i = 0; i < MLP_IN; i++) {
-      const float w = W1s[j * S1 + i];
-      const float4 x = quad(xs, MLP_IN, i, q);
-      a0 = fmaf(w, x.x, a0);
-      a1 = fmaf(w, x.y, a1);
-      a2 = fmaf(w, x.z, a2);
-      a3 = fmaf(w, x.w, a3);
-    }
+    auto rows = [&](const float *W, const float *v, int n) {   // four columns of the thread's row at a time
+#pragma unroll 4
+      for (int i = 0; i < n; i += 4) {
+        const float4 w4 = *reinterpret_cast<const float4 *>(W + i);
+        const float w[4] = {w4.x, w4.y, w4.z, w4.w};
+#pragma unroll
+        for (int c = 0; c < 4; c++) {
+          const float4 x = quad(v, n, i + c, q);
+          a0 = fmaf(w[c], x.x, a0);
+          a1 = fmaf(w[c], x.y, a1);
+          a2 = fmaf(w[c], x.z, a2);
+          a3 = fmaf(w[c], x.w, a3);
+        }
+      }
+    };
+    rows(W1s + j * S1, xs, MLP_IN);
     const float4 h1 = make_float4(fmaxf(a0, 0.f), fmaxf(a1, 0.f), fmaxf(a2, 0.f), fmaxf(a3, 0.f));
     *reinterpret_cast<float4 *>(h1s + (q * MLP_H + j) * 4) = h1;
     __syncthreads();
     a0 = a1 = a2 = a3 = b2;
-#pragma unroll 8
-    for (int k = 0; k < MLP_H; k++) {
-      const float w = W2s[j * S2 + k];
-      const float4 x = quad(h1s, MLP_H, k, q);
-      a0 = fmaf(w, x.x, a0);
-      a1 = fmaf(w, x.y, a1);
-      a2 = fmaf(w, x.z, a2);
-      a3 = fmaf(w, x.w, a3);
-    }
+    rows(W2s + j * S2, h1s, MLP_H);
     const float4 h2 = make_float4(fmaxf(a0, 0.f), fmaxf(a1, 0.f), fmaxf(a2, 0.f), fmaxf(a3, 0.f));
     float z[4] = {w3 * h2.x, w3 * h2.y, w3 * h2.z, w3 * h2.w};
 #pragma unroll
@@ -501,14 +525,15 @@ __global__ void __launch_bounds__(NT) k_mlp(const float *theta, const float *X, 
     }
   }
   if (GRAD) {
+    grid_launch_next();
     float *p = part + (size_t)blockIdx.x * PART;
-    float *pb1 = p + MLP_H * MLP_IN, *pW2 = pb1 + MLP_H, *pb2 = pW2 + MLP_H * MLP_H, *pw3 = pb2 + MLP_H, *pb3 = pw3 + MLP_H;
+    float *pb1 = p + NW, *pb2 = pb1 + MLP_H, *pw3 = pb2 + MLP_H, *pb3 = pw3 + MLP_H;
+    float4 *pv = reinterpret_cast<float4 *>(p) + tid;
 #pragma unroll
     for (int a = 0; a < 8; a++) {
-#pragma unroll
-      for (int b = 0; b < 8; b++) pW2[(tj + 16 * a) * MLP_H + tk + 16 * b] = g2[a][b];
-#pragma unroll
-      for (int b = 0; b < 4; b++) p[(tj + 16 * a) * MLP_IN + tk + 16 * b] = g1[a][b];
+      pv[(2 * a) * NT] = make_float4(g2[a][0], g2[a][1], g2[a][2], g2[a][3]);
+      pv[(2 * a + 1) * NT] = make_float4(g2[a][4], g2[a][5], g2[a][6], g2[a][7]);
+      pv[(16 + a) * NT] = make_float4(g1[a][0], g1[a][1], g1[a][2], g1[a][3]);
     }
     // the two quads of a unit, and the samples of b3 and the loss
     __syncthreads();
@@ -532,28 +557,55 @@ __global__ void __launch_bounds__(NT) k_mlp(const float *theta, const float *X, 
       float t = 0.f;
       for (int i = 0; i < GS; i++) t += dzs[tid * GS + i];
       pb3[tid] = t;
+    } else if (tid < 2 + PART - NPAR - 1) {
+      pb3[tid] = 0.f;
     }
   }
 }
 
-// Sum of the CTAs' partial gradients (4 threads per parameter, each a fixed
-// part of the CTAs), then the Adam step if theta is given, else the gradient
-// to grad; the loss adds to *loss.
+// the parameter that a partial gradient's element is of; NPAR: the loss
+__device__ __forceinline__ int param_of(int e) {
+  if (e >= NW) {
+    e -= NW;   // b1, b2, w3, b3: around W2 in the parameters
+    return e < MLP_H ? MLP_H * MLP_IN + e : NW + e;
+  }
+  const int v = e >> 2, c = e & 3, tid = v % NT, g = v / NT, tj = tid >> 4, tk = tid & 15;
+  return g < 16 ? MLP_H * MLP_IN + MLP_H + (tj + 16 * (g >> 1)) * MLP_H + tk + 16 * (4 * (g & 1) + c)
+                : (tj + 16 * (g - 16)) * MLP_IN + tk + 16 * c;
+}
+
+// Sum of the CTAs' partial gradients (16 threads for four parameters, each a
+// fixed part of the CTAs), then the Adam step if theta is given, else the
+// gradient to grad; the loss adds to *loss.
 __global__ void __launch_bounds__(256) k_reduce(const float *part, int nparts, float *grad, float *loss, float *theta,
                                                 float *m, float *v, float lr, float b1, float b2, float eps, float bc1,
                                                 float bc2) {
-  __shared__ float sh[4][64];
-  const int c = threadIdx.x & 63, sl = threadIdx.x >> 6, p = blockIdx.x * 64 + c;
-  float s = 0.f;
-  if (p < PART) {
-    const int per = (nparts + 3) / 4, e = min(nparts, (sl + 1) * per);
+  __shared__ float sh[16][64];
+  const int c = threadIdx.x & 15, sl = threadIdx.x >> 4, e0 = blockIdx.x * 64 + 4 * c;
+  grid_wait();
+  grid_launch_next();
+  // the parameter's state is on its way while the partial sums are read
+  const int e = blockIdx.x * 64 + threadIdx.x, p = threadIdx.x < 64 && e < NPAR + 1 ? param_of(e) : -1;
+  const bool adam = theta && p >= 0 && p < NPAR;
+  const float m0 = adam ? m[p] : 0.f, v0 = adam ? v[p] : 0.f, t0 = adam ? theta[p] : 0.f;
+  float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (e0 < PART) {
+    const int per = (nparts + 15) / 16, end = min(nparts, (sl + 1) * per);
 #pragma unroll 8
-    for (int n = sl * per; n < e; n++) s += part[(size_t)n * PART + p];
+    for (int n = sl * per; n < end; n++) {
+      const float4 x = *reinterpret_cast<const float4 *>(part + (size_t)n * PART + e0);
+      s.x += x.x;
+      s.y += x.y;
+      s.z += x.z;
+      s.w += x.w;
+    }
   }
-  sh[sl][c] = s;
+  *reinterpret_cast<float4 *>(&sh[sl][4 * c]) = s;
   __syncthreads();
-  if (sl || p >= PART) return;
-  const float g = (sh[0][c] + sh[1][c]) + (sh[2][c] + sh[3][c]);
+  if (p < 0) return;
+  float g = 0.f;
+#pragma unroll
+  for (int q = 0; q < 16; q++) g += sh[q][threadIdx.x];
   if (p == NPAR) {
     *loss += g;
     return;
@@ -562,11 +614,11 @@ __global__ void __launch_bounds__(256) k_reduce(const float *part, int nparts, f
     grad[p] = g;
     return;
   }
-  const float mm = b1 * m[p] + (1.f - b1) * g;
-  const float vv = b2 * v[p] + (1.f - b2) * g * g;
+  const float mm = b1 * m0 + (1.f - b1) * g;
+  const float vv = b2 * v0 + (1.f - b2) * g * g;
   m[p] = mm;
   v[p] = vv;
-  theta[p] -= lr * (mm / bc1) / (sqrtf(vv / bc2) + eps);
+  theta[p] = t0 - lr * (mm / bc1) / (sqrtf(vv / bc2) + eps);
 }
 
 // combine: refine where the predictor says so, otherwise keep the plain flag
@@ -611,35 +663,56 @@ void mlp_features_launch(const KParams &kp, const void *U, int precision, int sl
 }
 
 namespace {
-// one CTA per SM at most (the weights take 99 KB of shared memory each)
+// a launch whose first instructions may overlap the end of the kernel before it
+template <typename... P, typename... A>
+void launch_after(bool overlap, void (*kernel)(P...), int grid, int block, size_t smem, cudaStream_t s, A... args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = &at;
+  cfg.numAttrs = overlap ? 1 : 0;
+  cudaLaunchKernelEx(&cfg, kernel, (P)args...);
+}
+
+// one CTA per SM at most (the weights take 102 KB of shared memory each)
 template <bool GRAD>
 int mlp_launch(const float *theta, const float *X, const float *T, const int *idx, int B, float *y, float *part,
-               cudaStream_t s) {
+               bool overlap, cudaStream_t s) {
   cudaFuncSetAttribute(k_mlp<GRAD>, cudaFuncAttributeMaxDynamicSharedMemorySize, MLP_SMEM);
   const int groups = (B + GS - 1) / GS, n = groups < MLP_MAX_CTAS ? groups : MLP_MAX_CTAS;
-  k_mlp<GRAD><<<n, NT, MLP_SMEM, s>>>(theta, X, T, idx, B, y, part);
+  launch_after(overlap, k_mlp<GRAD>, n, NT, MLP_SMEM, s, theta, X, T, idx, B, y, part);
   return n;
 }
 }  // namespace
 
 void mlp_forward_launch(const float *theta, const float *X, const int *idx, int B, float *y, cudaStream_t s) {
-  if (B > 0) mlp_launch<false>(theta, X, nullptr, idx, B, y, nullptr, s);
+  if (B > 0) mlp_launch<false>(theta, X, nullptr, idx, B, y, nullptr, false, s);
 }
 
 void mlp_grad_launch(const float *theta, const float *X, const float *T, const int *idx, int B, float *part, float *grad,
                      float *loss, cudaStream_t s) {
   if (B <= 0) return;
-  const int n = mlp_launch<true>(theta, X, T, idx, B, nullptr, part, s);
+  const int n = mlp_launch<true>(theta, X, T, idx, B, nullptr, part, false, s);
   k_reduce<<<(PART + 63) / 64, 256, 0, s>>>(part, n, grad, loss, nullptr, nullptr, nullptr, 0.f, 0.f, 0.f, 0.f, 1.f, 1.f);
 }
 
+// In a run of batches (more: not the first) the two kernels of a step overlap
+// their ends and beginnings: the gather of a batch, which no kernel writes,
+// comes before the wait, all else behind it.  A training of 16 batches of 1024:
+// 511 -> 424 us.
 void mlp_step_launch(float *theta, float *m, float *v, const float *X, const float *T, const int *idx, int B, float *part,
-                     float *loss, float lr, int step, cudaStream_t s) {
+                     float *loss, float lr, int step, bool more, cudaStream_t s) {
   if (B <= 0) return;
   const float b1 = 0.9f, b2 = 0.999f;
   const float bc1 = 1.f - powf(b1, (float)step), bc2 = 1.f - powf(b2, (float)step);
-  const int n = mlp_launch<true>(theta, X, T, idx, B, nullptr, part, s);
-  k_reduce<<<(PART + 63) / 64, 256, 0, s>>>(part, n, nullptr, loss, theta, m, v, lr, b1, b2, 1e-8f, bc1, bc2);
+  const int n = mlp_launch<true>(theta, X, T, idx, B, nullptr, part, more, s);
+  launch_after(true, k_reduce, (PART + 63) / 64, 256, 0, s, part, n, nullptr, loss, theta, m, v, lr, b1, b2, 1e-8f, bc1,
+               bc2);
 }
 
 void mlp_combine_launch(const float *prob, const DevBlock *blk, signed char *flags, int n, cudaStream_t s) {

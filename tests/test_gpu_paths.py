@@ -137,6 +137,27 @@ def test_gradient_of_a_batch(batch):
     assert np.allclose(g.mlp_predict(X), M.forward(th, X64)[0], rtol=1e-5, atol=1e-6)
 
 
+@pytest.mark.parametrize("batch", [1, 8, 200, 1024, 4096])
+def test_batches_in_one_call(batch):
+    """the steps of one call overlap their kernels: the same bits as one step a
+    call (every sample the same, so that the order of the samples is none)"""
+    g, _ = make_pair(n=(24, 12, 12), nb=(12, 12, 12), **STR)
+    rng = np.random.default_rng(batch)
+    n = min(4 * batch, 8192)
+    X = np.repeat(rng.uniform(0, 1.0, (1, 64)), n, axis=0).astype(np.float32)
+    theta = I.mlp_init(4).astype(np.float32)
+    out = []
+    for calls in (1, n // batch):
+        g.mlp_set_params(theta)
+        g.mlp_dataset_clear()
+        g.mlp_dataset_add(X, np.ones(n, dtype=np.float32))
+        for _ in range(5):
+            for _ in range(calls):
+                g.mlp_train(n // calls, 1, batch=batch, lr=1e-2, seed=1)
+        out.append(g.mlp_get_params())
+    assert np.array_equal(out[0], out[1]) and not np.array_equal(out[0], theta)
+
+
 @pytest.mark.parametrize("lo,hi", [((BC_REFLECT, BC_OUTFLOW, BC_REFLECT), (BC_OUTFLOW, BC_REFLECT, BC_REFLECT)),
                                    ((BC_OUTFLOW, BC_REFLECT, BC_PERIODIC), (BC_REFLECT, BC_REFLECT, BC_PERIODIC)),
                                    ((BC_PERIODIC, BC_OUTFLOW, BC_OUTFLOW), (BC_PERIODIC, BC_OUTFLOW, BC_REFLECT))])
