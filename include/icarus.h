@@ -330,7 +330,8 @@ icarus_status icarus_cell_updates(icarus_ctx *ctx, double *out);
 icarus_status icarus_status_word(icarus_ctx *ctx, uint32_t *word, uint64_t *floor_hits);
 
 /* Stage-kernel tile shape (theta x phi cells per CTA) and radial segment
- * length; 0 = library default.  Used by the autotuner. */
+ * length; 0 = the library's choice, by a cost model of the leaves, the blocks
+ * and the tiles.  Used by the autotuner. */
 icarus_status icarus_set_tile(icarus_ctx *ctx, int tile_theta, int tile_phi, int r_segment);
 
 /* Floor budget.  Density and pressure floors (rho_floor, p_floor) are applied
@@ -422,8 +423,9 @@ icarus_status icarus_alu_peak(int kind, void *stream, double *flops_per_s);
 icarus_status icarus_profile(icarus_ctx *ctx, int enable);
 
 /* Device time (ms) and number of launches per kernel kind accumulated since
- * the previous read, then reset.  Kinds: 0 dt begin, 1 ghost fill from
- * neighbours, 2 physical-boundary ghosts, 3 predictor stage, 4 corrector
+ * the previous read, then reset.  Kinds: 0 dt begin (once per icarus_step
+ * call), 1 ghost fill, prolongation from coarser leaves, 2 ghost fill, physical
+ * boundaries with restriction and copies, 3 predictor stage, 4 corrector
  * stage, 5 reflux, 6 dt finalize, 7 refinement estimator (flagging), 8 regrid
  * data movement, 9 CFL time step of the whole state (after a regrid or a
  * state upload).  Kinds 7-9 are recorded by icarus_flag_refine and

@@ -24,6 +24,20 @@
 // area-weighted face fluxes of block faces that border a different level for
 // the reflux.  The grid is persistent: CTAs stride over (block, tile,
 // r-segment) work items of all levels and all ensemble members.
+//
+// What bounds it.  FP32: latency and the barrier between the phases of a
+// plane, with 53 to 56 % of the issue slots used by 16 warps per SM at 128
+// registers; DRAM is idle (a fifth of its peak).  More CTAs at fewer
+// registers, a single flux buffer with a second barrier, and the staging of
+// U^n in shared memory were slower.  512 x 60 x 180 cells in 64 x 60 x 180
+// blocks: predictor 400 -> 281 us, corrector 489 -> 374 us since cells are
+// stored whole (16-byte copies, one sector per scattered cell), geometry
+// factors are staged per plane and row and no constant is converted per cell.
+// FP64: the FP64 pipe, 80 % busy (19 cycles of an SM for each instruction of a
+// warp), so the arithmetic is arranged for few such instructions: comparisons,
+// minima and signs by integers, reciprocals and roots of three and five
+// instructions, and flux sides added by the multiply-adds that form them; 64 x
+// 60 x 180 cells: both stages 6382 -> 2090 us.
 #include <cstdio>
 
 #include "mhd_device.cuh"
@@ -171,7 +185,8 @@ __global__ void __launch_bounds__(stage_threads(TJ, TK), stage_min_ctas(sizeof(r
   real *dring = s_row + NRF * TJ;
   // for the divergence: r_c^2 per plane; sin, 1 / (sin * two-cell spacing) and
   // 1/sin per row from row -2; 1 / two-cell spacing per column from column -2
-  real *s_rc2 = dring + 4 * DP, *s_fr = s_rc2 + NRP, *s_st = s_fr + NRP, *s_tt = s_st + NJ, *s_ist = s_tt + NJ, *s_ipc2 = s_ist + NJ;
+  real *s_rc2 = dring + 4 * DP, *s_fr = s_rc2 + NRP, *s_st = s_fr + NRP, *s_tt = s_st + NJ, *s_ist = s_tt + NJ,
+       *s_ipc2 = s_ist + NJ;
   real *xring = fend + StageSmem<real>::geo(TJ, TK) + 4 * DP;   // tracer X, 5 planes (if stored)
   const real **s_xsrc = reinterpret_cast<const real **>(xring + 5 * RP + (RP & 1));
   const bool trc = kp.nvs > NVAR;
