@@ -79,11 +79,13 @@ size_t table_count(const icarus_grid_desc *d) {
   return n;
 }
 
-// ghost-fill work items a leaf can need at most: 32-task chunks of the ghost
-// cells of its 26 regions (all of them held by finer leaves)
+// ghost-fill work items a leaf can need at most: RESTRICT_WIDTH cells each of the
+// ghost cells of its 26 regions (all of them held by finer leaves; prolongations
+// need at most as many, PROLONG_WIDTH groups of eight cells each)
 int items_per_block(const icarus_grid_desc *d) {
   const int n0 = d->block[0], n1 = d->block[1], n2 = d->block[2];
-  auto chunks = [](int cells) { return (cells + 31) / 32; };
+  static_assert(RESTRICT_WIDTH <= 8 * PROLONG_WIDTH, "");
+  auto chunks = [](int cells) { return (cells + RESTRICT_WIDTH - 1) / RESTRICT_WIDTH; };
   return 2 * (chunks(NGH * n1 * n2) + chunks(NGH * n0 * n2) + chunks(NGH * n0 * n1)) +
          4 * (chunks(NGH * NGH * n0) + chunks(NGH * NGH * n1) + chunks(NGH * NGH * n2)) + 8 * chunks(NGH * NGH * NGH);
 }
@@ -254,7 +256,7 @@ struct icarus_ctx {
   unsigned int *status = nullptr;
   signed char *flags = nullptr;
   int *all_list = nullptr, *rlist = nullptr, *shell = nullptr;
-  int2 *rent = nullptr;     // (slot, region | finer << 8 | chunk << 9), up to 32 ghost tasks of a region held by coarser / finer leaves
+  int2 *rent = nullptr;     // (slot, region | finer << 8 | chunk << 9): ghost tasks of a region held by coarser / finer leaves
   int *rshell = nullptr;    // per region (start, group-first cells, cells), then the shell cells ordered by region
   int2 *sides = nullptr;
   MoveOp *ops = nullptr;
@@ -559,14 +561,14 @@ icarus_status upload_tree(icarus_ctx *c, DevBlock *blk_dst) {
       }
       if (finer) rl.push_back(slot);
       // the regions held by coarser or finer leaves go to the ghost fill's
-      // work items of up to 32 tasks (2x2x2 groups under a coarser leaf,
-      // cells next to finer ones), face regions first
+      // work items (2x2x2 groups under a coarser leaf, cells next to finer
+      // ones), face regions first
       for (int r = 0; r < 27; r++) {
         if (rs[r] < 2) continue;
         const int dx = r / 9 - 1, dy = (r / 3) % 3 - 1, dz = r % 3 - 1;
         const bool face = (dx != 0) + (dy != 0) + (dz != 0) == 1, fin = rs[r] == 3;
         const int tasks = fin ? c->reg_tab[r][2] : c->reg_tab[r][1];
-        for (int ch = 0; 32 * ch < tasks; ch++)
+        for (int ch = 0; ch * (fin ? RESTRICT_WIDTH : PROLONG_WIDTH) < tasks; ch++)
           items[fin][!face].push_back(make_int2(slot, r | (fin ? 256 : 0) | ch << 9));
         mixed = true;
       }

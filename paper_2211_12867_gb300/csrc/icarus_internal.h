@@ -155,9 +155,10 @@ int stage_ctas(int precision, int tj, int tk, int tracer);   // resident CTAs pe
 // shell's cells from same-level leaves), ghost_prolong, and ghost_physical
 // (the physical edges that come from a ghost cell under a coarser or finer
 // leaf; none with faces_only).  The step's fills leave the ghost cells that
-// same-level leaves hold to their readers (nshell 0).  Items: up to 32 cells
-// (or 2x2x2 groups) of the regions around a leaf; sides: (slot, direction * 2
+// same-level leaves hold to their readers (nshell 0).  Items: up to
+// RESTRICT_WIDTH cells (PROLONG_WIDTH 2x2x2 groups) of a region around a leaf; sides: (slot, direction * 2
 // + side) of the physical faces.
+constexpr int RESTRICT_WIDTH = 32, PROLONG_WIDTH = 8;
 void ghost_first_launch(const KParams &kp, void *U, int precision, const int2 *items, int nitems, const int *rshell,
                         const int2 *sides, int nsides, double tshift_fac, bool faces_only, const int *shell, int nshell,
                         int nleaves, cudaStream_t s);

@@ -186,10 +186,14 @@ __device__ __forceinline__ bool restrict_in_block(const KParams &kp, const real 
 // The ghost fill's work items cover the regions around a leaf (one of the 26,
 // r = 9 (sx + 1) + 3 (sy + 1) + sz + 1) that a coarser leaf holds (one lane
 // per 2 x 2 x 2 group, prolongation) or finer leaves hold (one lane per cell,
-// restriction).  A work item is up to 32 such tasks of one region, taken by
-// one warp: item = (slot, r | finer << 8 | chunk << 9), tasks 32 chunk ..
-// 32 chunk + 31 of the region-ordered shell list (group-first cells first)
-// behind its table of (start, group-first cells, cells) per region.
+// restriction).  A work item is up to WIDTH such tasks of one region: item =
+// (slot, r | finer << 8 | chunk << 9), tasks WIDTH chunk .. WIDTH chunk +
+// WIDTH - 1 of the region-ordered shell list (group-first cells first) behind
+// its table of (start, group-first cells, cells) per region.  Restrictions
+// take a warp each (a face has 2 x 12 x 12 cells), prolongations 8 lanes: an
+// edge has 6 groups and a corner one, and with a warp for each 7 of 32 lanes
+// worked in the corrector's fill.  5981 leaves of 12^3 on three levels: 79 ->
+// 42 us.
 // Same-level halo cells the prolongation's stencil reaches are read from
 // the neighbouring leaf (the step's fills leave those ghost copies unfilled,
 // and the others fill them in the same launch).
@@ -200,8 +204,9 @@ struct Task {
   int q[3];   // padded index in that block
   int G[3];   // global cell
 };
+template <int WIDTH>
 __device__ __forceinline__ bool region_task(const KParams &kp, const int2 e, const int *rshell, Task &t) {
-  const int r = e.y & 255, n = ((e.y >> 9) << 5) + (threadIdx.x & 31);
+  const int r = e.y & 255, n = (e.y >> 9) * WIDTH + (threadIdx.x & (WIDTH - 1));
   if (n >= rshell[3 * r + 1 + ((e.y >> 8) & 1)]) return false;
   const int code = rshell[81 + rshell[3 * r] + n];
   const DevBlock &B = kp.blk[e.x];
@@ -238,10 +243,10 @@ __device__ __forceinline__ bool region_task(const KParams &kp, const int2 e, con
 // itself (blocks are four cells or more).
 template <typename real>
 __global__ void __launch_bounds__(128, sizeof(real) == 4 ? 5 : 3) k_ghost_prolong(const KParams kp, real *U, const int2 *items, int nitems, const int *rshell) {
-  const int w = blockIdx.x * 4 + (threadIdx.x >> 5);
+  const int w = (blockIdx.x * 128 + threadIdx.x) / PROLONG_WIDTH;
   if (w >= nitems) return;
   Task t;
-  if (!region_task(kp, items[w], rshell, t)) return;
+  if (!region_task<PROLONG_WIDTH>(kp, items[w], rshell, t)) return;
   int cb[3], Ic[3];
 #pragma unroll
   for (int d = 0; d < 3; d++) {
@@ -397,10 +402,10 @@ __global__ void __launch_bounds__(128) k_ghost_first(const KParams kp, real *U, 
                                                      int ccopy) {
   int n = blockIdx.x;
   if (n < rblocks) {
-    const int w = n * 4 + (threadIdx.x >> 5);
+    const int w = (n * 128 + threadIdx.x) / RESTRICT_WIDTH;
     if (w >= nitems) return;
     Task t;
-    if (!region_task(kp, items[w], rshell, t)) return;
+    if (!region_task<RESTRICT_WIDTH>(kp, items[w], rshell, t)) return;
     real val[NVAR + 1];
     if (!restrict_in_block<real>(kp, U, t.member, t.L, t.b, t.q, t.G, val)) {
       atomicOr(kp.status, ST_TREE);
@@ -637,7 +642,7 @@ int physical_chunks(const KParams &kp, bool faces_only) {
 void ghost_first_launch(const KParams &kp, void *U, int precision, const int2 *items, int nitems, const int *rshell,
                         const int2 *sides, int nsides, double tfac, bool faces_only, const int *shell, int nshell,
                         int nleaves, cudaStream_t s) {
-  const int nchunk = physical_chunks(kp, faces_only), rblocks = (nitems + 3) / 4;   // one warp per item
+  const int nchunk = physical_chunks(kp, faces_only), rblocks = (nitems * RESTRICT_WIDTH + 127) / 128;
   const int ccopy = (nshell + 127) / 128, grid = rblocks + nsides * nchunk + nleaves * ccopy;
   if (grid <= 0) return;
   if (precision)
@@ -651,7 +656,7 @@ void ghost_first_launch(const KParams &kp, void *U, int precision, const int2 *i
 void ghost_prolong_launch(const KParams &kp, void *U, int precision, const int2 *items, int nitems, const int *rshell,
                           cudaStream_t s) {
   if (nitems <= 0) return;
-  const int grid = (nitems + 3) / 4;
+  const int grid = (nitems * PROLONG_WIDTH + 127) / 128;
   if (precision)
     k_ghost_prolong<float><<<grid, 128, 0, s>>>(kp, (float *)U, items, nitems, rshell);
   else
