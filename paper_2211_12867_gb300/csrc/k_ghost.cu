@@ -431,109 +431,120 @@ __global__ void __launch_bounds__(128) k_ghost_first(const KParams kp, real *U, 
   store(kp, U, to, val);
 }
 
-// reflux of coarse blocks with finer face neighbours; one CTA per block
+// sum over the directions of (|v_d| + c_f,d) / dx_d of a cell.  FP64: with the
+// stage's reciprocals and roots (IEEE divisions and roots cost k_dt_full of 204
+// leaves of 12^3 109 us, now 76)
+__device__ __forceinline__ float speed_sum(const float *u, float gamma, float pfl, float dx0, float dx1, float dx2) {
+  float w[NVAR];
+  cons2prim_speed<float>(u, w, gamma, pfl);
+  return (RT<float>::abs_(w[1]) + fast_speed<float, 0>(w, gamma)) / dx0 +
+         (RT<float>::abs_(w[2]) + fast_speed<float, 1>(w, gamma)) / dx1 +
+         (RT<float>::abs_(w[3]) + fast_speed<float, 2>(w, gamma)) / dx2;
+}
+__device__ __forceinline__ double speed_sum(const double *u, double gamma, double pfl, double dx0, double dx1, double dx2) {
+  const double ir = RT<double>::rcp_(u[0]);
+  double p = pressure_for_speed<double>(u, gamma);
+  if (RT<double>::less_(p, pfl)) p = pfl;
+  const double v[3] = {u[1] * ir, u[2] * ir, u[3] * ir};
+  const double ix[3] = {RT<double>::rcp_(dx0), RT<double>::rcp_(dx1), RT<double>::rcp_(dx2)};
+  return cfl_rate(ir, v, p, u + 5, gamma, ix);
+}
+
+// Reflux of the leaves with a finer face neighbour: one thread per cell of a
+// face (blockIdx.y: chunks of 128 cells of the faces in order).  A cell on
+// several finer faces belongs to the first one's thread, which corrects it
+// face by face and then takes floors and CFL speed as often.  Latency bound
+// (lookups, then 5 x 8 flux loads at once).  A CTA per leaf that went through
+// its faces one after the other, with four lookups a coarse face instead of
+// one, took 24 us between events on a tree of 1914 leaves of 12^3 (FP32) and 29
+// on one of 204 (FP64); now 17 and 24.
 template <typename real>
-__global__ void k_reflux(const KParams kp, real *U, const real *flux, const int *list) {
+__global__ void __launch_bounds__(128) k_reflux(const KParams kp, real *U, const real *flux, const int *list) {
   const int slot = list[blockIdx.x];
-  const DevBlock B = kp.blk[slot];
-  const double dtm = kp.dt_used[B.member];
-  if (!(dtm > 0.0)) return;
-  const real dt = (real)dtm;
-  const int L = B.level;
-  const int nb0 = kp.nb[0], nb1 = kp.nb[1], nb2 = kp.nb[2];
-  const int fc[3] = {nb1 * nb2, nb0 * nb2, nb0 * nb1};
-  const size_t fstride = (size_t)NVAR * 2 * (fc[0] + fc[1] + fc[2]);
-  size_t foff[6];
-  {
-    size_t o = 0;
-    for (int f = 0; f < 6; f++) {
-      foff[f] = o;
-      o += (size_t)NVAR * fc[f / 2];
+  const DevBlock &B = kp.blk[slot];
+  const int fc[3] = {kp.nb[1] * kp.nb[2], kp.nb[0] * kp.nb[2], kp.nb[0] * kp.nb[1]};
+  int f = 0, chunk = blockIdx.y;
+#pragma unroll
+  for (int q = 0; q < 5; q++) {
+    const int n = (fc[q / 2] + 127) / 128;
+    if (f == q && chunk >= n) {
+      chunk -= n;
+      f = q + 1;
     }
   }
+  const double dtm = kp.dt_used[B.member];
+  if (B.nbr[f] != NB_FINER || !(dtm > 0.0)) return;
+  const real dt = (real)dtm;
+  const int L = B.level;
+  const size_t fstride = (size_t)NVAR * 2 * (fc[0] + fc[1] + fc[2]);
   const LevelGeo<real> &G = GeoSel<real>::get(kp.geo, L);
-  for (int f = 0; f < 6; f++) {
-    if (B.nbr[f] != NB_FINER) continue;
-    const int d = f / 2, hi = f % 2;
-    const int d1 = d == 0 ? 1 : 0, d2 = d == 2 ? 1 : 2;
-    for (int t = threadIdx.x; t < fc[d]; t += blockDim.x) {
-      const int t1 = t / kp.nb[d2], t2 = t % kp.nb[d2];
-      int Gc[3];
-      Gc[d1] = B.ix[d1] * kp.nb[d1] + t1;
-      Gc[d2] = B.ix[d2] * kp.nb[d2] + t2;
-      Gc[d] = hi ? (B.ix[d] + 1) * kp.nb[d] : B.ix[d] * kp.nb[d] - 1;  // coarse cell across
+  const real gamma = (real)kp.gamma, pfl = (real)kp.p_floor, rfl = (real)kp.rho_floor;
+  double acc = 0.0;
+  int hits = 0;
+  int q[3];   // the cell inside the leaf
+  const int t = chunk * 128 + threadIdx.x;
+  {
+    const int d = f / 2, d1 = d == 0 ? 1 : 0, d2 = d == 2 ? 1 : 2;
+    q[d] = f % 2 ? kp.nb[d] - 1 : 0;
+    q[d1] = t / kp.nb[d2];
+    q[d2] = t - q[d1] * kp.nb[d2];
+  }
+  unsigned on = 0;   // finer faces the cell lies on
+#pragma unroll
+  for (int e = 0; e < 6; e++)
+    if (B.nbr[e] == NB_FINER && q[e / 2] == (e % 2 ? kp.nb[e / 2] - 1 : 0)) on |= 1u << e;
+  if (t < fc[f / 2] && !(on & ((1u << f) - 1))) {
+    const int I = B.ix[0] * kp.nb[0] + q[0], J = B.ix[1] * kp.nb[1] + q[1];
+    const real V = G.dr3[I + NGH] * G.dcos[J + NGH] * G.dphi;
+    const size_t ci = cell_index(kp, slot, q[0] + NGH, q[1] + NGH, q[2] + NGH);
+    real u[NVAR];
+    ld_cell(U + ci, u);
+    for (unsigned m = on; m; m &= m - 1) {
+      const int e = __ffs(m) - 1, d = e / 2, hi = e & 1, d1 = d == 0 ? 1 : 0, d2 = d == 2 ? 1 : 2;
+      size_t off = 0;   // of the face's fluxes in a slot; low and high face
+      for (int p = 0; p < d; p++) off += (size_t)2 * NVAR * fc[p];
+      const size_t face = (size_t)NVAR * fc[d];
+      // the fine leaf across and its cell next to the coarse cell's corner
+      // (blocks start at even indices: all four fine cells lie in it)
+      int F[3];
+#pragma unroll
+      for (int p = 0; p < 3; p++) F[p] = 2 * (B.ix[p] * kp.nb[p] + q[p]);
+      F[d] += hi ? 2 : -1;
+      bool in;
+#pragma unroll
+      for (int p = 0; p < 3; p++) F[p] = wrap_dim(kp, L + 1, p, F[p], in);
+      const int fsl = lookup(kp, B.member, L + 1, F);
       real fs[NVAR];
 #pragma unroll
       for (int v = 0; v < NVAR; v++) fs[v] = real(0);
-      for (int a = 0; a < 2; a++)
-        for (int c = 0; c < 2; c++) {
-          int F[3];
-          F[d] = hi ? 2 * Gc[d] : 2 * Gc[d] + 1;
-          F[d1] = 2 * Gc[d1] + a;
-          F[d2] = 2 * Gc[d2] + c;
-          bool in;
-          for (int e = 0; e < 3; e++) F[e] = wrap_dim(kp, L + 1, e, F[e], in);
-          const int fsl = lookup(kp, B.member, L + 1, F);
-          if (fsl < 0) {
-            atomicOr(kp.status, ST_TREE);
-            continue;
-          }
-          const DevBlock FB = kp.blk[fsl];
-          const int s1 = F[d1] - FB.ix[d1] * kp.nb[d1], s2 = F[d2] - FB.ix[d2] * kp.nb[d2];
-          const real *src = flux + (size_t)fsl * fstride + foff[2 * d + (hi ? 0 : 1)];
+      if (fsl < 0) {
+        atomicOr(kp.status, ST_TREE);
+      } else {
+        const DevBlock &FB = kp.blk[fsl];
+        const int s1 = F[d1] - FB.ix[d1] * kp.nb[d1], s2 = F[d2] - FB.ix[d2] * kp.nb[d2];
+        const real *src = flux + (size_t)fsl * fstride + off + (hi ? 0 : face) + s1 * kp.nb[d2] + s2;
 #pragma unroll
-          for (int v = 0; v < NVAR; v++) fs[v] += src[(size_t)v * fc[d] + s1 * kp.nb[d2] + s2];
-        }
-      int q[3];
-      q[d] = hi ? NGH + kp.nb[d] - 1 : NGH;
-      q[d1] = NGH + t1;
-      q[d2] = NGH + t2;
-      const int I = B.ix[0] * nb0 + q[0] - NGH, J = B.ix[1] * nb1 + q[1] - NGH;
-      const real V = G.dr3[I + NGH] * G.dcos[J + NGH] * G.dphi;
-      const real *own = flux + (size_t)slot * fstride + foff[f];
-      const real sg = hi ? real(-1) : real(1);
-      const size_t ci = cell_index(kp, slot, q[0], q[1], q[2]);
-      real u[NVAR];
-      ld_cell(U + ci, u);
+        for (int a = 0; a < 2; a++)
 #pragma unroll
-      for (int v = 0; v < NVAR; v++) u[v] += sg * dt / V * (fs[v] - own[(size_t)v * fc[d] + t]);
-      st_cell(U + ci, u);
-    }
-    __syncthreads();
-  }
-  // floors and CFL contribution of every corrected cell
-  const real gamma = (real)kp.gamma, pfl = (real)kp.p_floor, rfl = (real)kp.rho_floor;
-  double acc = 0.0;
-  long long hits = 0;
-  for (int f = 0; f < 6; f++) {
-    if (B.nbr[f] != NB_FINER) continue;
-    const int d = f / 2, hi = f % 2;
-    const int d1 = d == 0 ? 1 : 0, d2 = d == 2 ? 1 : 2;
-    for (int t = threadIdx.x; t < fc[d]; t += blockDim.x) {
-      const int t1 = t / kp.nb[d2], t2 = t % kp.nb[d2];
-      int q[3];
-      q[d] = hi ? NGH + kp.nb[d] - 1 : NGH;
-      q[d1] = NGH + t1;
-      q[d2] = NGH + t2;
-      real u[NVAR];
-      const size_t ci = cell_index(kp, slot, q[0], q[1], q[2]);
-      ld_cell(U + ci, u);
-      hits += apply_floors<real>(u, gamma, pfl, rfl, Isl{(float)kp.isl_pe, (float)kp.isl_beta});
-      st_cell(U + ci, u);
-      real w[NVAR];
-      cons2prim_speed<real>(u, w, gamma, pfl);
-      const int I = B.ix[0] * nb0 + q[0] - NGH + NGH, J = B.ix[1] * nb1 + q[1] - NGH + NGH;
-      real dx0 = G.dr[I], dx1 = G.dth[J], dx2 = G.dphi;
-      if (kp.geometry == 0) {
-        dx1 *= G.rc[I];
-        dx2 *= G.rc[I] * G.sintc[J];
+          for (int c = 0; c < 2; c++)
+#pragma unroll
+            for (int v = 0; v < NVAR; v++) fs[v] += src[(size_t)v * fc[d] + a * kp.nb[d2] + c];
       }
-      const real sp = (RT<real>::abs_(w[1]) + fast_speed<real, 0>(w, gamma)) / dx0 +
-                      (RT<real>::abs_(w[2]) + fast_speed<real, 1>(w, gamma)) / dx1 +
-                      (RT<real>::abs_(w[3]) + fast_speed<real, 2>(w, gamma)) / dx2;
-      acc = fmax(acc, (double)sp);
+      const real *own = flux + (size_t)slot * fstride + off + (hi ? face : 0) + q[d1] * kp.nb[d2] + q[d2];
+      const real sg = hi ? real(-1) : real(1);
+#pragma unroll
+      for (int v = 0; v < NVAR; v++) u[v] += sg * dt / V * (fs[v] - own[(size_t)v * fc[d]]);
     }
-    __syncthreads();
+    real dx0 = G.dr[I + NGH], dx1 = G.dth[J + NGH], dx2 = G.dphi;
+    if (kp.geometry == 0) {
+      dx1 *= G.rc[I + NGH];
+      dx2 *= G.rc[I + NGH] * G.sintc[J + NGH];
+    }
+    for (unsigned m = on; m; m &= m - 1) {
+      hits += apply_floors<real>(u, gamma, pfl, rfl, Isl{(float)kp.isl_pe, (float)kp.isl_beta});
+      acc = fmax(acc, (double)speed_sum(u, gamma, pfl, dx0, dx1, dx2));
+    }
+    st_cell(U + ci, u);
   }
   for (int o = 16; o > 0; o >>= 1) {
     acc = fmax(acc, __shfl_xor_sync(0xffffffffu, acc, o));
@@ -597,19 +608,15 @@ __global__ void k_dt_full(const KParams kp, const real *U) {
   double acc = 0.0;
   for (int c = blockIdx.y * blockDim.x + threadIdx.x; c < kp.icells; c += gridDim.y * blockDim.x) {
     const int k = c % kp.nb[2], j = (c / kp.nb[2]) % kp.nb[1], i = c / (kp.nb[2] * kp.nb[1]);
-    real u[NVAR], w[NVAR];
+    real u[NVAR];
     ld_cell(U + cell_index(kp, slot, i + NGH, j + NGH, k + NGH), u);
-    cons2prim_speed<real>(u, w, gamma, pfl);
     const int I = B.ix[0] * kp.nb[0] + i + NGH, J = B.ix[1] * kp.nb[1] + j + NGH;
     real dx0 = G.dr[I], dx1 = G.dth[J], dx2 = G.dphi;
     if (kp.geometry == 0) {
       dx1 *= G.rc[I];
       dx2 *= G.rc[I] * G.sintc[J];
     }
-    const real sp = (RT<real>::abs_(w[1]) + fast_speed<real, 0>(w, gamma)) / dx0 +
-                    (RT<real>::abs_(w[2]) + fast_speed<real, 1>(w, gamma)) / dx1 +
-                    (RT<real>::abs_(w[3]) + fast_speed<real, 2>(w, gamma)) / dx2;
-    acc = fmax(acc, (double)sp);
+    acc = fmax(acc, (double)speed_sum(u, gamma, pfl, dx0, dx1, dx2));
   }
   for (int o = 16; o > 0; o >>= 1) acc = fmax(acc, __shfl_xor_sync(0xffffffffu, acc, o));
   if ((threadIdx.x & 31) == 0 && acc > 0.0) atomic_max_pos(&kp.inv_max[B.member], acc);
@@ -676,10 +683,13 @@ void ghost_physical_launch(const KParams &kp, void *U, int precision, const int2
 void reflux_launch(const KParams &kp, void *U, const void *flux, int precision, const int *list, int nlist,
                    cudaStream_t s) {
   if (nlist <= 0) return;
+  const int *n = kp.nb;
+  const int chunks = 2 * ((n[1] * n[2] + 127) / 128 + (n[0] * n[2] + 127) / 128 + (n[0] * n[1] + 127) / 128);
+  const dim3 grid(nlist, chunks);
   if (precision)
-    k_reflux<float><<<nlist, 256, 0, s>>>(kp, (float *)U, (const float *)flux, list);
+    k_reflux<float><<<grid, 128, 0, s>>>(kp, (float *)U, (const float *)flux, list);
   else
-    k_reflux<double><<<nlist, 256, 0, s>>>(kp, (double *)U, (const double *)flux, list);
+    k_reflux<double><<<grid, 128, 0, s>>>(kp, (double *)U, (const double *)flux, list);
 }
 
 void dt_begin_launch(const KParams &kp, const double *tstop, cudaStream_t s) {
@@ -693,10 +703,14 @@ void dt_finalize_launch(const KParams &kp, double cfl, const double *tstop, cuda
 
 void dt_full_launch(const KParams &kp, const void *U, int precision, int nleaves, double cfl, cudaStream_t s) {
   if (nleaves > 0) {
+    // cells a CTA: in FP32, where a cell is cheap against a CTA's start and
+    // reduction, 4096 (2481 leaves of 12^3: 39 us; with 1024, 44)
+    const int per = precision ? 4096 : 1024;
+    const dim3 grid(nleaves, (kp.icells + per - 1) / per);
     if (precision)
-      k_dt_full<float><<<dim3(nleaves, (kp.icells + 4095) / 4096), 256, 0, s>>>(kp, (const float *)U);
+      k_dt_full<float><<<grid, 256, 0, s>>>(kp, (const float *)U);
     else
-      k_dt_full<double><<<dim3(nleaves, (kp.icells + 4095) / 4096), 256, 0, s>>>(kp, (const double *)U);
+      k_dt_full<double><<<grid, 256, 0, s>>>(kp, (const double *)U);
   }
   k_dt_from_max<<<(kp.n_members + 127) / 128, 128, 0, s>>>(kp, cfl);
 }
