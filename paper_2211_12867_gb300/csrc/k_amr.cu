@@ -422,68 +422,89 @@ __global__ void k_shock_estimator(const KParams kp, const real *U, int slot0, do
 }
 
 // ---- regrid data movement ----
+// the 2 x 2 x 2 cells of the new leaf (slot dst) at padded cell (p0, p1, p2)
+// from the old parent's coarse cell Ic
 template <typename real>
-__device__ void prolong_child(const KParams &kp, const real *U, int cs, const int *Ic, int ch, real *out) {
-  const DevBlock C = kp.blk[cs];
-  const int Lc = C.level;
+__device__ __forceinline__ void prolong_group(const KParams &kp, const real *U, real *Unew, int cs, const int *Ic, int dst, int p0,
+                              int p1, int p2) {
+  const DevBlock &C = kp.blk[cs];
   const int nv = kp.nvs;   // the MHD variables and, when stored, the CME tracer
   int pc[3];
 #pragma unroll
   for (int d = 0; d < 3; d++) pc[d] = Ic[d] - C.ix[d] * kp.nb[d] + NGH;
   real up[NVAR + 1], s[3][NVAR + 1];
-  auto get = [&](int p0, int p1, int p2, real *u) {
-    ld_cell(U + cell_index(kp, cs, p0, p1, p2), u);
-    if (nv > NVAR) u[TRV] = U[tracer_index(kp, cs, p0, p1, p2)];
+  auto get = [&](int q0, int q1, int q2, real *u) {
+    ld_cell(U + cell_index(kp, cs, q0, q1, q2), u);
+    if (nv > NVAR) u[TRV] = U[tracer_index(kp, cs, q0, q1, q2)];
   };
   get(pc[0], pc[1], pc[2], up);
+  {
+    real um[3][NVAR + 1], uq[3][NVAR + 1];
 #pragma unroll
-  for (int d = 0; d < 3; d++) {
-    real um[NVAR + 1], uq[NVAR + 1];
-    get(pc[0] - (d == 0), pc[1] - (d == 1), pc[2] - (d == 2), um);
-    get(pc[0] + (d == 0), pc[1] + (d == 1), pc[2] + (d == 2), uq);
+    for (int d = 0; d < 3; d++) {
+      get(pc[0] - (d == 0), pc[1] - (d == 1), pc[2] - (d == 2), um[d]);
+      get(pc[0] + (d == 0), pc[1] + (d == 1), pc[2] + (d == 2), uq[d]);
+    }
 #pragma unroll
-    for (int v = 0; v < NVAR + 1; v++)
-      if (v < nv) s[d][v] = mc_slope<real>(um[v], up[v], uq[v]);
-  }
-  const real *d0 = GeoSel<real>::dlt(kp.geo, Lc, 0), *d1 = GeoSel<real>::dlt(kp.geo, Lc, 1),
-             *d2 = GeoSel<real>::dlt(kp.geo, Lc, 2);
-  const real gamma = (real)kp.gamma;
-  bool ok = true;
-  for (int c = 0; c < 8; c++) {
-    const real a = d0[2 * Ic[0] + ((c >> 2) & 1)], b = d1[2 * Ic[1] + ((c >> 1) & 1)], e = d2[2 * Ic[2] + (c & 1)];
-    real u[NVAR + 1];
-#pragma unroll
-    for (int v = 0; v < NVAR + 1; v++)
-      if (v < nv) u[v] = ((up[v] + s[0][v] * a) + s[1][v] * b) + s[2][v] * e;
-    if (!(u[0] > real(0)) || !(pressure_of<real>(u, gamma, Isl{(float)kp.isl_pe, (float)kp.isl_beta}) > real(0))) ok = false;
-    if (c == ch)
+    for (int d = 0; d < 3; d++)
 #pragma unroll
       for (int v = 0; v < NVAR + 1; v++)
-        if (v < nv) out[v] = u[v];
+        if (v < nv) s[d][v] = mc_slope<real>(um[d][v], up[v], uq[d][v]);
   }
-  if (!ok)
-#pragma unroll
-    for (int v = 0; v < NVAR + 1; v++)
-      if (v < nv) out[v] = up[v];
+  prolong_children<real>(kp, up, s, C.level, Ic, [&](int c, const real *u) {
+    const int q0 = p0 + ((c >> 2) & 1), q1 = p1 + ((c >> 1) & 1), q2 = p2 + (c & 1);
+    st_cell(Unew + cell_index(kp, dst, q0, q1, q2), u);
+    if (nv > NVAR) Unew[tracer_index(kp, dst, q0, q1, q2)] = u[TRV];
+  });
 }
 
+// Bound by memory: one thread per 2 x 2 x 2 group of a prolonged leaf, per four
+// cells of a copied one, per cell of a restricted one.  A thread per cell, which
+// for a prolongation computed the eight children of its parent and kept one,
+// took (between events) 120 us for 2481 leaves of 12^3 in FP32 most of whose
+// parents were refined, 84 for 2005 mostly copied ones and 66 for 218 in FP64;
+// now 51, 73 and 55.
 template <typename real>
-__global__ void k_regrid_move(const KParams kpo, const real *Uold, real *Unew, const DevBlock *nblk,
+__global__ void __launch_bounds__(256, sizeof(real) == 4 ? 2 : 1) k_regrid_move(const KParams kpo, const real *Uold, real *Unew, const DevBlock *nblk,
                               const MoveOp *ops) {
-  const MoveOp op = ops[blockIdx.x];
-  const int c = blockIdx.y * blockDim.x + threadIdx.x;
+  const MoveOp &op = ops[blockIdx.x];
+  const int kind = op.kind;
+  if (kind == 0) {   // four cells a thread in flight
+    const int c0 = blockIdx.y * 1024 + threadIdx.x, src = op.src[0], dst = op.dst;
+    real u[4][NVAR + 1];
+    size_t to[4], tt[4];
+#pragma unroll
+    for (int n = 0; n < 4; n++) {
+      const int c = c0 + 256 * n;
+      if (c >= kpo.icells) continue;
+      const int k = c % kpo.nb[2], j = (c / kpo.nb[2]) % kpo.nb[1], i = c / (kpo.nb[2] * kpo.nb[1]);
+      ld_cell(Uold + cell_index(kpo, src, i + NGH, j + NGH, k + NGH), u[n]);
+      to[n] = cell_index(kpo, dst, i + NGH, j + NGH, k + NGH);
+      if (kpo.nvs > NVAR) {
+        u[n][TRV] = Uold[tracer_index(kpo, src, i + NGH, j + NGH, k + NGH)];
+        tt[n] = tracer_index(kpo, dst, i + NGH, j + NGH, k + NGH);
+      }
+    }
+#pragma unroll
+    for (int n = 0; n < 4; n++) {
+      if (c0 + 256 * n >= kpo.icells) continue;
+      st_cell(Unew + to[n], u[n]);
+      if (kpo.nvs > NVAR) Unew[tt[n]] = u[n][TRV];
+    }
+    return;
+  }
+  const int c = blockIdx.y * 256 + threadIdx.x;
   if (c >= kpo.icells) return;
   const int k = c % kpo.nb[2], j = (c / kpo.nb[2]) % kpo.nb[1], i = c / (kpo.nb[2] * kpo.nb[1]);
   const DevBlock N = nblk[op.dst];
   real val[NVAR + 1];
   const int nv = kpo.nvs;
-  if (op.kind == 0) {
-    ld_cell(Uold + cell_index(kpo, op.src[0], i + NGH, j + NGH, k + NGH), val);
-    if (nv > NVAR) val[TRV] = Uold[tracer_index(kpo, op.src[0], i + NGH, j + NGH, k + NGH)];
-  } else if (op.kind == 1) {
-    const int F[3] = {N.ix[0] * kpo.nb[0] + i, N.ix[1] * kpo.nb[1] + j, N.ix[2] * kpo.nb[2] + k};
-    const int Ic[3] = {F[0] >> 1, F[1] >> 1, F[2] >> 1};
-    prolong_child<real>(kpo, Uold, op.src[0], Ic, ((F[0] & 1) << 2) | ((F[1] & 1) << 1) | (F[2] & 1), val);
+  if (kind == 1) {
+    const int g2 = kpo.nb[2] / 2, g1 = kpo.nb[1] / 2, gk = c % g2, gj = (c / g2) % g1, gi = c / (g2 * g1);
+    if (gi >= kpo.nb[0] / 2) return;
+    const int Ic[3] = {N.ix[0] * kpo.nb[0] / 2 + gi, N.ix[1] * kpo.nb[1] / 2 + gj, N.ix[2] * kpo.nb[2] / 2 + gk};
+    prolong_group<real>(kpo, Uold, Unew, op.src[0], Ic, op.dst, 2 * gi + NGH, 2 * gj + NGH, 2 * gk + NGH);
+    return;
   } else {
     const LevelGeo<real> &FG = GeoSel<real>::get(kpo.geo, N.level + 1);
     const int G[3] = {N.ix[0] * kpo.nb[0] + i, N.ix[1] * kpo.nb[1] + j, N.ix[2] * kpo.nb[2] + k};

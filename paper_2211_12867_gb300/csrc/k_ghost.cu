@@ -109,30 +109,11 @@ __device__ __forceinline__ void prolong_into(const KParams &kp, real *U, int cs,
       for (int v = 0; v < NVAR + 1; v++)
         if (v < nv) s[d][v] = mc_slope<real>(um[d][v], up[v], uq[d][v]);
   }
-  const real *d0 = GeoSel<real>::dlt(kp.geo, Lc, 0), *d1 = GeoSel<real>::dlt(kp.geo, Lc, 1),
-             *d2 = GeoSel<real>::dlt(kp.geo, Lc, 2);
-  const real gamma = (real)kp.gamma;
-  const real a0 = d0[2 * Ic[0]], a1 = d0[2 * Ic[0] + 1], b0 = d1[2 * Ic[1]], b1 = d1[2 * Ic[1] + 1],
-             e0 = d2[2 * Ic[2]], e1 = d2[2 * Ic[2] + 1];
-  bool ok = true;
-  for (int c = 0; c < 8; c++) {
-    const real a = (c & 4) ? a1 : a0, b = (c & 2) ? b1 : b0, e = (c & 1) ? e1 : e0;
-    real u[NVAR];
-#pragma unroll
-    for (int v = 0; v < NVAR; v++) u[v] = ((up[v] + s[0][v] * a) + s[1][v] * b) + s[2][v] * e;
-    if (!(u[0] > real(0)) || !(pressure_of<real>(u, gamma, Isl{(float)kp.isl_pe, (float)kp.isl_beta}) > real(0))) ok = false;
-  }
   const size_t wbase = slot_base(kp, slot);
-  const int w0 = pad_cell(kp, p[0], p[1], p[2]);
-  const int P1 = kp.P[1], P2 = kp.P[2];
-  for (int c = 0; c < 8; c++) {
-    const real a = (c & 4) ? a1 : a0, b = (c & 2) ? b1 : b0, e = (c & 1) ? e1 : e0;
-    real u[NVAR + 1];
-#pragma unroll
-    for (int v = 0; v < NVAR + 1; v++)
-      if (v < nv) u[v] = ok ? ((up[v] + s[0][v] * a) + s[1][v] * b) + s[2][v] * e : up[v];
+  const int w0 = pad_cell(kp, p[0], p[1], p[2]), P1 = kp.P[1], P2 = kp.P[2];
+  prolong_children<real>(kp, up, s, Lc, Ic, [&](int c, const real *u) {
     store(kp, U, {wbase, w0 + (((c >> 2) & 1) * P1 + ((c >> 1) & 1)) * P2 + (c & 1)}, u);
-  }
+  });
 }
 
 // slot of the level-L leaf at block coordinates b (>= 0), -1 coarser, -2 refined

@@ -673,6 +673,37 @@ __device__ __forceinline__ int apply_floors(real *u, real gamma, real pfloor, re
   return hits;
 }
 
+// The eight children of coarse cell Ic (global at level Lc) from its value and
+// MC slopes, handed to store(child, variables); if any child's density or
+// pressure is not positive all eight take the parent's value.  A first pass
+// checks, a second one stores (the CME tracer follows the MHD variables).
+template <typename real, typename Store>
+__device__ __forceinline__ void prolong_children(const KParams &kp, const real *up, const real (*s)[NVAR + 1], int Lc,
+                                                 const int *Ic, Store store) {
+  const int nv = kp.nvs;
+  const real *d0 = GeoSel<real>::dlt(kp.geo, Lc, 0), *d1 = GeoSel<real>::dlt(kp.geo, Lc, 1),
+             *d2 = GeoSel<real>::dlt(kp.geo, Lc, 2);
+  const real gamma = (real)kp.gamma;
+  const real a0 = d0[2 * Ic[0]], a1 = d0[2 * Ic[0] + 1], b0 = d1[2 * Ic[1]], b1 = d1[2 * Ic[1] + 1],
+             e0 = d2[2 * Ic[2]], e1 = d2[2 * Ic[2] + 1];
+  bool ok = true;
+  for (int c = 0; c < 8; c++) {
+    const real a = (c & 4) ? a1 : a0, b = (c & 2) ? b1 : b0, e = (c & 1) ? e1 : e0;
+    real u[NVAR];
+#pragma unroll
+    for (int v = 0; v < NVAR; v++) u[v] = ((up[v] + s[0][v] * a) + s[1][v] * b) + s[2][v] * e;
+    if (!(u[0] > real(0)) || !(pressure_of<real>(u, gamma, Isl{(float)kp.isl_pe, (float)kp.isl_beta}) > real(0))) ok = false;
+  }
+  for (int c = 0; c < 8; c++) {
+    const real a = (c & 4) ? a1 : a0, b = (c & 2) ? b1 : b0, e = (c & 1) ? e1 : e0;
+    real u[NVAR + 1];
+#pragma unroll
+    for (int v = 0; v < NVAR + 1; v++)
+      if (v < nv) u[v] = ok ? ((up[v] + s[0][v] * a) + s[1][v] * b) + s[2][v] * e : up[v];
+    store(c, u);
+  }
+}
+
 // atomic max of a non-negative double through its bit pattern
 __device__ __forceinline__ void atomic_max_pos(unsigned long long *addr, double v) {
   atomicMax(addr, (unsigned long long)__double_as_longlong(v));
