@@ -265,6 +265,10 @@ __global__ void __cluster_dims__(EST_CTAS, 1, 1) __launch_bounds__(256, 5)
   extern __shared__ float est_sm[];
   __shared__ int s_any, s_code[EST_CTAS];   // s_code: of the cluster's CTAs, in its first one
   __shared__ volatile int s_refine;
+  // another CTA's shared memory may be written only once that CTA runs: every
+  // thread arrives here and waits ahead of the write
+  cg::cluster_group cl = cg::this_cluster();
+  cl.barrier_arrive();
   const int part = blockIdx.x % EST_CTAS, leaf = blockIdx.x / EST_CTAS, slot = slot0 + leaf;
   const DevBlock &B = kp.blk[slot];
   const int sh = B.level - 1, tid = threadIdx.x;
@@ -330,7 +334,7 @@ __global__ void __cluster_dims__(EST_CTAS, 1, 1) __launch_bounds__(256, 5)
     }
   }
   code = (__syncthreads_or(code & 2) ? 2 : 0) | (__syncthreads_or(code & 1) ? 1 : 0);
-  cg::cluster_group cl = cg::this_cluster();
+  cl.barrier_wait();
   if (tid == 0) *cl.map_shared_rank(&s_code[part], 0) = code;
   cl.sync();
   if (part == 0 && tid == 0) {
