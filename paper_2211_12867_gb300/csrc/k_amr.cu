@@ -195,14 +195,17 @@ __global__ void k_estimator(const KParams kp, const real *U, int slot0, double e
 // before 220.
 constexpr int EST_CTAS = 4;
 
-// Pressure to within one FP32 rounding.  FP64 state: FP64 operations.  FP32
-// state: in pairs of FP32 numbers (exact products and sums by fused
-// multiply-adds, Dekker's and Knuth's error-free transformations), whose error
-// is below 2^-42 e; NaN, which is not decided, where the pressure is below
-// 2^-16 e.
+// Pressure to within one FP32 rounding of est_pressure's.  FP64 state: FP64
+// operations in another order; with a thermal energy of at least 2^-26 e the
+// two, each within 7 2^-53 e, differ by 2^-23 of it at most.  FP32 state: in
+// pairs of FP32 numbers (exact products and sums by fused multiply-adds,
+// Dekker's and Knuth's error-free transformations), whose error is below
+// 2^-42 e.  NaN, which is not decided, where the thermal energy is below
+// 2^-26 e, in FP32 states the pressure below 2^-16 e.
 __device__ __forceinline__ float rounded_pressure(const double *u, double gamma, float) {
   const double ke2 = (u[1] * u[1] + u[2] * u[2] + u[3] * u[3]) * RT<double>::rcp_(u[0]);
-  return (float)((gamma - 1.0) * fma(-0.5, ke2 + (u[5] * u[5] + u[6] * u[6] + u[7] * u[7]), u[4]));
+  const double th = fma(-0.5, ke2 + (u[5] * u[5] + u[6] * u[6] + u[7] * u[7]), u[4]);
+  return RT<double>::less_(0x1p-26 * fabs(u[4]), th) ? (float)((gamma - 1.0) * th) : nanf("");
 }
 __device__ __forceinline__ void pair_add(float a, float &h, float &l) {   // (h, l) += a
   const float s = __fadd_rn(h, a), t = __fsub_rn(s, h);
