@@ -201,7 +201,8 @@ constexpr int EST_CTAS = 4;
 // pairs of FP32 numbers (exact products and sums by fused multiply-adds,
 // Dekker's and Knuth's error-free transformations), whose error is below
 // 2^-42 e.  NaN, which is not decided, where the thermal energy is below
-// 2^-26 e, in FP32 states the pressure below 2^-16 e.
+// 2^-26 e, in FP32 states the pressure below 2^-16 e or the cell out of the
+// range in which no product of the pairs overflows or loses its low part.
 __device__ __forceinline__ float rounded_pressure(const double *u, double gamma, float) {
   const double ke2 = (u[1] * u[1] + u[2] * u[2] + u[3] * u[3]) * RT<double>::rcp_(u[0]);
   const double th = fma(-0.5, ke2 + (u[5] * u[5] + u[6] * u[6] + u[7] * u[7]), u[4]);
@@ -232,14 +233,16 @@ __device__ __forceinline__ float rounded_pressure(const float *u, double, float 
   l *= -0.5f;
   pair_add(u[4], h, l);
   const float p = __fmul_rn(gm1, __fadd_rn(h, l));
-  return p > 1.52587890625e-5f * fabsf(u[4]) ? p : nanf("");
+  const bool in = u[4] > 1e-20f && u[4] < 1e15f && u[0] > 1e-24f && u[0] < 1e15f && u[0] * u[4] > 1e-31f;
+  return in && p > 1.52587890625e-5f * u[4] ? p : nanf("");
 }
 
 // E > e from FP32 values: 1 yes, 0 no, -1 not decided.  Inputs carry a relative
 // error of 2^-22 (see rounded_pressure), each difference and sum one more per
 // operation: |N_f - N| and |S_f - S| stay below 2^-20 (1 + eps) of the sum of the
 // w, for N the norm of the second differences and S that of s.  NaN and
-// infinities are not decided.
+// infinities are not decided, nor are sums of the w so small or large that the
+// squares are not normal numbers to that accuracy.
 __device__ __forceinline__ void loehner32(const float *um, float u0, const float *up, float eps, float *N, float *S,
                                           float *W) {
   float n = 0.f, d = 0.f, t = 0.f;
@@ -254,7 +257,8 @@ __device__ __forceinline__ void loehner32(const float *um, float u0, const float
   }
   *N = sqrtf(n);
   *S = sqrtf(d);
-  *W = t * (1.f + eps);
+  t *= 1.f + eps;
+  *W = t > 1e-15f && t < 1e18f ? t : nanf("");
 }
 __device__ __forceinline__ int decide(float N, float S, float W, float e) {
   const float x = N - e * S, tol = (1.f + e) * 9.5367431640625e-7f * W;

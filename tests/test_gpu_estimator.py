@@ -90,3 +90,20 @@ def test_thresholds_in_cold_streams(p_over_e, precision):
         U[:, 4] = e * (1.0 + p_over_e / 0.5 * (1.0 + 1.5e-3 * rng.random(e.shape)))
         return U
     _check_at_the_thresholds(precision, state)
+
+
+# units in which the squares of densities and pressures leave FP32's normal
+# range at either end
+@pytest.mark.parametrize("precision", [FP64, FP32_MIXED])
+@pytest.mark.parametrize("rough", [1.0, 0.01])
+@pytest.mark.parametrize("unit", [1e-30, 1e-24, 1e-22, 1e-21, 1e-20, 1e-19, 1e-18, 1e-16, 1e-12, 1e12, 1e16, 1e18, 1e19,
+                                  1e20, 1e22])
+def test_thresholds_in_any_unit(unit, rough, precision):
+    def state(shape):
+        rng = np.random.default_rng(6)
+        W = 1.0 + 0.3 * rough * rng.random(shape)
+        U = W.copy()
+        U[:, 1:4] *= W[:, :1]
+        U[:, 4] = 2.0 * W[:, 4] + 0.5 * (U[:, 1:4] ** 2).sum(1) / U[:, 0] + 0.5 * (W[:, 5:8] ** 2).sum(1)
+        return U * np.where(np.arange(8) < 5, unit, math.sqrt(unit))[:, None, None, None]
+    _check_at_the_thresholds(precision, state)
