@@ -2,6 +2,9 @@
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
+#ifdef __CUDACC__
+#include <atomic>
+#endif
 
 #define NVAR 8
 #define TRV 8          // index of the CME tracer rho X in a slot (when stored)
@@ -123,6 +126,23 @@ struct KParams {
   int n_base_cells[3];
   double isl_pe, isl_beta;     // FP64 pressure-island thresholds (FP32 mode)
 };
+
+#ifdef __CUDACC__
+// Dynamic shared memory limit of a kernel on the current device, set once to
+// the most that any launch of it takes: contexts of several threads may launch
+// one kernel with different amounts, and a limit set for each launch would fall
+// below what another thread is about to launch with.
+template <auto KERNEL, size_t BYTES>
+void raise_smem_limit() {
+  static std::atomic<unsigned long long> done{0};   // a bit per device
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return;
+  const unsigned long long bit = dev < 64 ? 1ull << dev : 0ull;
+  if (bit && (done.load() & bit)) return;
+  if (cudaFuncSetAttribute(KERNEL, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BYTES) == cudaSuccess)
+    done.fetch_or(bit);
+}
+#endif
 
 // ---- launch wrappers (defined in the kernel translation units) ----
 struct StageLaunch {

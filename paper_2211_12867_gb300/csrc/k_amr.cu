@@ -729,13 +729,14 @@ void estimator(const KParams &kp, const real *U, int slot0, int nslots, double e
                signed char *flags, cudaStream_t s) {
   // four slabs of a leaf in at most 100 KB each (two CTAs per SM): 12^3 blocks
   // take 8 KB; above, one CTA per leaf without shared planes
+  constexpr size_t most = 100 * 1024;
   const size_t ns = (kp.nb[0] + EST_CTAS - 1) / EST_CTAS, H = (size_t)(kp.nb[1] + 2) * (kp.nb[2] + 2);
   const size_t smem = 2 * sizeof(float) * (ns + 2) * H + ns * kp.nb[1] * kp.nb[2];
-  if (smem > 100 * 1024) {
+  if (smem > most) {
     k_estimator<real><<<nslots, 256, 0, s>>>(kp, U, slot0, e_ref, e_crs, eps, dv, flags);
     return;
   }
-  cudaFuncSetAttribute(k_estimator_slabs<real>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  raise_smem_limit<k_estimator_slabs<real>, most>();
   k_estimator_slabs<real><<<nslots * EST_CTAS, 256, smem, s>>>(kp, U, slot0, e_ref, e_crs, eps, dv, flags);
 }
 }  // namespace

@@ -639,15 +639,16 @@ void features(const KParams &kp, const real *U, int slot0, int nslots, float *ou
   // three planes in at most 100 KB (two CTAs per SM): blocks of up to 36 x 36
   // columns; above, the kernel without shared planes
   const size_t smem = sizeof(double) * (9 * (size_t)(kp.nb[1] + 2) * (kp.nb[2] + 2) + (size_t)kp.nb[1] * kp.nb[2]);
-  if (smem > 100 * 1024) {
+  constexpr size_t most = 100 * 1024;
+  if (smem > most) {
     k_features_large<real><<<nslots, 256, 0, s>>>(kp, U, slot0, out);
     return;
   }
   if constexpr (sizeof(real) == 4) {
-    cudaFuncSetAttribute(k_features_pairs, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    raise_smem_limit<k_features_pairs, most>();
     k_features_pairs<<<nslots, FEAT_NT, smem, s>>>(kp, U, slot0, out);
   } else {
-    cudaFuncSetAttribute(k_features, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    raise_smem_limit<k_features, most>();
     k_features<<<nslots, 256, smem, s>>>(kp, U, slot0, out);
   }
 }
@@ -683,7 +684,7 @@ void launch_after(bool overlap, void (*kernel)(P...), int grid, int block, size_
 template <bool GRAD>
 int mlp_launch(const float *theta, const float *X, const float *T, const int *idx, int B, float *y, float *part,
                bool overlap, cudaStream_t s) {
-  cudaFuncSetAttribute(k_mlp<GRAD>, cudaFuncAttributeMaxDynamicSharedMemorySize, MLP_SMEM);
+  raise_smem_limit<k_mlp<GRAD>, MLP_SMEM>();
   const int groups = (B + GS - 1) / GS, n = groups < MLP_MAX_CTAS ? groups : MLP_MAX_CTAS;
   launch_after(overlap, k_mlp<GRAD>, n, NT, MLP_SMEM, s, theta, X, T, idx, B, y, part);
   return n;

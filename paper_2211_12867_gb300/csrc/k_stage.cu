@@ -834,26 +834,19 @@ __global__ void __launch_bounds__(stage_threads(TJ, TK), stage_min_ctas(sizeof(r
   }
 }
 
-// dynamic shared memory limit of both instances of a tile, raised (never
-// lowered) to what a launch needs
-template <typename real, int TJ, int TK>
-void ensure_smem(size_t smem) {
-  static size_t configured = 0;
-  if (smem > configured) {
-    cudaFuncSetAttribute(k_stage<real, TJ, TK, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    cudaFuncSetAttribute(k_stage<real, TJ, TK, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    configured = smem;
-  }
-}
-
 template <typename real, int TJ, int TK>
 int launch_t(const KParams &kp, const StageLaunch &sl, cudaStream_t s) {
   const size_t smem = StageSmem<real>::bytes(TJ, TK, kp.nvs > NVAR);
-  ensure_smem<real, TJ, TK>(smem);
-  if (sl.stage2)
+  // with the tracer's ring where that fits (227 KB a CTA)
+  constexpr size_t full = StageSmem<real>::bytes(TJ, TK, true);
+  constexpr size_t most = full <= 227 * 1024 ? full : StageSmem<real>::bytes(TJ, TK);
+  if (sl.stage2) {
+    raise_smem_limit<k_stage<real, TJ, TK, true>, most>();
     k_stage<real, TJ, TK, true><<<sl.grid, stage_threads(TJ, TK), smem, s>>>(kp, sl, StageConst<real>(kp));
-  else
+  } else {
+    raise_smem_limit<k_stage<real, TJ, TK, false>, most>();
     k_stage<real, TJ, TK, false><<<sl.grid, stage_threads(TJ, TK), smem, s>>>(kp, sl, StageConst<real>(kp));
+  }
   return cudaPeekAtLastError() == cudaSuccess ? 0 : -1;
 }
 
