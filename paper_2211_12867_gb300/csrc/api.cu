@@ -14,7 +14,10 @@
 #include <new>
 #include <vector>
 
+#include <cuda.h>
+
 #include "../../include/icarus.h"
+#include "host_range.h"
 #include "icarus_internal.h"
 
 namespace {
@@ -1119,17 +1122,38 @@ icarus_status recompute_dt(icarus_ctx *c) {
   return ICARUS_OK;
 }
 
-// Device address of n doubles of pinned host memory, or nullptr (pageable
-// memory, or a range that does not lie in one piece).
-double *mapped_host(double *host, size_t n) {
-  cudaPointerAttributes a{}, b{};
-  if (cudaPointerGetAttributes(&a, host) != cudaSuccess || cudaPointerGetAttributes(&b, host + n - 1) != cudaSuccess) {
+// the page-locked piece that holds host address p, if any
+bool pinned_piece(uintptr_t p, PinnedPiece *q) {
+  using Attribute = CUresult(CUDAAPI *)(void *, CUpointer_attribute, CUdeviceptr);
+  static const Attribute get = [] {
+    void *f = nullptr;
+    cudaDriverEntryPointQueryResult r;
+    if (cudaGetDriverEntryPointByVersion("cuPointerGetAttribute", &f, 12000, cudaEnableDefault, &r) != cudaSuccess ||
+        r != cudaDriverEntryPointSuccess) {
+      cudaGetLastError();
+      f = nullptr;
+    }
+    return reinterpret_cast<Attribute>(f);
+  }();
+  cudaPointerAttributes a{};
+  if (!get || cudaPointerGetAttributes(&a, reinterpret_cast<void *>(p)) != cudaSuccess) {
     cudaGetLastError();
-    return nullptr;
+    return false;
   }
-  if (a.type != cudaMemoryTypeHost || b.type != cudaMemoryTypeHost || !a.devicePointer || !b.devicePointer) return nullptr;
-  double *d = static_cast<double *>(a.devicePointer);
-  return d + (n - 1) == b.devicePointer ? d : nullptr;
+  CUdeviceptr start = 0;
+  if (a.type != cudaMemoryTypeHost ||
+      get(&start, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, (CUdeviceptr)p) != CUDA_SUCCESS ||
+      get(&q->bytes, CU_POINTER_ATTRIBUTE_RANGE_SIZE, (CUdeviceptr)p) != CUDA_SUCCESS)
+    return false;
+  q->start = (uintptr_t)start;
+  q->same_address = reinterpret_cast<uintptr_t>(a.devicePointer) == p;
+  return true;
+}
+
+// Device address of n doubles of page-locked host memory, or nullptr (pageable
+// memory in any part of the range, or another address on the device).
+double *mapped_host(double *host, size_t n) {
+  return pinned_throughout(reinterpret_cast<uintptr_t>(host), n * sizeof(double), pinned_piece) ? host : nullptr;
 }
 
 bool member_ok(icarus_ctx *c, int m) { return c && m >= 0 && m < c->d.n_members; }
