@@ -21,6 +21,8 @@
 // Reflux: a coarse leaf face next to finer leaves takes the sum of the fine
 // area-weighted fluxes of the corrector stage (exact conservation across
 // levels on the stretched spherical grid).
+#include <algorithm>
+
 #include "mhd_device.cuh"
 
 namespace {
@@ -685,9 +687,10 @@ void dt_finalize_launch(const KParams &kp, double cfl, const double *tstop, cuda
 void dt_full_launch(const KParams &kp, const void *U, int precision, int nleaves, double cfl, cudaStream_t s) {
   if (nleaves > 0) {
     // cells a CTA: in FP32, where a cell is cheap against a CTA's start and
-    // reduction, 4096 (2481 leaves of 12^3: 39 us; with 1024, 44)
+    // reduction, 4096 (2481 leaves of 12^3: 39 us; with 1024, 44); more in a
+    // block that would take more CTAs than a grid has rows
     const int per = precision ? 4096 : 1024;
-    const dim3 grid(nleaves, (kp.icells + per - 1) / per);
+    const dim3 grid(nleaves, std::min((kp.icells + per - 1) / per, 65535));
     if (precision)
       k_dt_full<float><<<grid, 256, 0, s>>>(kp, (const float *)U);
     else
