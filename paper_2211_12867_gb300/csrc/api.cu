@@ -1660,22 +1660,41 @@ icarus_status icarus_get_state(icarus_ctx *c, int member, double *host, size_t n
   return ICARUS_OK;
 }
 
+// Padded planes [slot][variable][cell] of nslots leaves, the first nvars
+// variables of each, between host memory and the state's cells, turned on the
+// device in pieces of the staging buffer (a plane fits: blocks are four cells
+// or more, so it is at most eight interiors).
+static icarus_status copy_planes(icarus_ctx *c, int slot0, int nslots, int nvars, unsigned char *host, bool to_host) {
+  const size_t plane = (size_t)c->kp.pcells * c->rsize, units = (size_t)nslots * nvars;
+  const size_t piece = c->lay.staging_doubles * sizeof(double) / plane;
+  for (size_t u0 = 0; u0 < units; u0 += piece) {
+    const size_t n = std::min(piece, units - u0);
+    if (to_host) {
+      planes_launch(c->kp, c->U, c->prec, slot0, nvars, (long long)u0, (long long)n, c->staging, true, c->stream);
+      CK(cudaPeekAtLastError());
+      CK(cudaMemcpyAsync(host + u0 * plane, c->staging, n * plane, cudaMemcpyDeviceToHost, c->stream));
+    } else {
+      CK(cudaMemcpyAsync(c->staging, host + u0 * plane, n * plane, cudaMemcpyHostToDevice, c->stream));
+      planes_launch(c->kp, c->U, c->prec, slot0, nvars, (long long)u0, (long long)n, c->staging, false, c->stream);
+      CK(cudaPeekAtLastError());
+    }
+    CK(cudaStreamSynchronize(c->stream));
+  }
+  return ICARUS_OK;
+}
+
 icarus_status icarus_get_padded(icarus_ctx *c, int member, int leaf, double *host, size_t n) {
   if (!member_ok(c, member) || !host) return ICARUS_ERR_ARG;
   const int nl = (int)c->mem[member].leaves.size();
   if (leaf < 0 || leaf >= nl || n != (size_t)NVAR * c->kp.pcells) return ICARUS_ERR_ARG;
-  const size_t slot = (size_t)c->mem_off[member] + leaf;
   std::vector<unsigned char> raw(n * c->rsize);
-  const size_t stride = (size_t)c->kp.nvs * c->kp.pcells * c->rsize;   // bytes per slot
-  CK(cudaMemcpyAsync(raw.data(), static_cast<const char *>(c->U) + slot * stride, raw.size(),
-                     cudaMemcpyDeviceToHost, c->stream));
-  CK(cudaStreamSynchronize(c->stream));
-  // [cell][8] to the host's [variable][cell]
-  const size_t pc = (size_t)c->kp.pcells;
-  for (size_t q = 0; q < n; q++) {
-    const size_t at = (q % pc) * NVAR + q / pc;
-    host[q] = c->prec ? (double)reinterpret_cast<const float *>(raw.data())[at]
-                      : reinterpret_cast<const double *>(raw.data())[at];
+  const icarus_status st = copy_planes(c, c->mem_off[member] + leaf, 1, NVAR, raw.data(), true);
+  if (st != ICARUS_OK) return st;
+  if (c->prec) {
+    const float *f = reinterpret_cast<const float *>(raw.data());
+    for (size_t q = 0; q < n; q++) host[q] = (double)f[q];
+  } else {
+    memcpy(host, raw.data(), raw.size());
   }
   return ICARUS_OK;
 }
@@ -2232,33 +2251,6 @@ struct CkFile {
 
 size_t slot_bytes(const icarus_ctx *c) { return (size_t)c->kp.nvs * c->kp.pcells * c->rsize; }
 
-// A checkpoint holds a slot's variables one after the other, the device a
-// cell's side by side (the tracer follows them in both): the slots of `raw`
-// are turned from one form into the other in place.
-template <typename real>
-void turn_slots(const icarus_ctx *c, std::vector<unsigned char> &raw, bool to_file) {
-  const size_t pc = (size_t)c->kp.pcells, per = (size_t)c->kp.nvs * pc;
-  const long long ns = (long long)(raw.size() / (per * sizeof(real)));
-#pragma omp parallel
-  {
-    std::vector<real> tmp(NVAR * pc);
-#pragma omp for schedule(static)
-    for (long long s = 0; s < ns; s++) {
-      real *u = reinterpret_cast<real *>(raw.data()) + (size_t)s * per;
-      for (size_t q = 0; q < pc; q++)
-        for (int v = 0; v < NVAR; v++) {
-          const size_t cell = q * NVAR + v, var = v * pc + q;
-          tmp[to_file ? var : cell] = u[to_file ? cell : var];
-        }
-      memcpy(u, tmp.data(), sizeof(real) * NVAR * pc);
-    }
-  }
-}
-void turn_slots(const icarus_ctx *c, std::vector<unsigned char> &raw, bool to_file) {
-  if (c->prec) turn_slots<float>(c, raw, to_file);
-  else turn_slots<double>(c, raw, to_file);
-}
-
 }  // namespace
 
 extern "C" {
@@ -2279,9 +2271,11 @@ icarus_status icarus_save(icarus_ctx *c, const char *path) {
   CK(cudaMemcpyAsync(bmap.data(), c->bmap, sizeof(double) * bmap.size(), cudaMemcpyDeviceToHost, s));
   CK(cudaMemcpyAsync(vbg.data(), c->vbg, sizeof(double) * vbg.size(), cudaMemcpyDeviceToHost, s));
   CK(cudaMemcpyAsync(&hits, c->floor_hits, sizeof(hits), cudaMemcpyDeviceToHost, s));
-  if (!U.empty()) CK(cudaMemcpyAsync(U.data(), c->U, U.size(), cudaMemcpyDeviceToHost, s));
   if (!theta.empty())
     CK(cudaMemcpyAsync(theta.data(), c->mlp_theta, sizeof(float) * theta.size(), cudaMemcpyDeviceToHost, s));
+  // a checkpoint holds a slot's variables one after the other
+  const icarus_status st = copy_planes(c, 0, c->nleaves, c->kp.nvs, U.data(), true);
+  if (st != ICARUS_OK) return st;
   CK(cudaStreamSynchronize(s));
   CkFile F;
   F.f = fopen(path, "wb");
@@ -2310,7 +2304,6 @@ icarus_status icarus_save(icarus_ctx *c, const char *path) {
   F.put(&hits, sizeof(hits));
   const double isl[2] = {c->isl_pe, c->isl_beta};
   F.put(isl, sizeof(isl));
-  turn_slots(c, U, true);
   F.put(U.data(), U.size());
   const int32_t nth = (int32_t)theta.size();
   F.put(&nth, sizeof(nth));
@@ -2379,7 +2372,6 @@ icarus_status icarus_load(icarus_ctx *c, const char *path) {
   std::vector<float> theta(nth);
   F.get(theta.data(), sizeof(float) * nth);
   if (!F.ok) return ICARUS_ERR_ARG;
-  turn_slots(c, U, false);
   // everything read: replace the context's state
   c->mem = std::move(next);
   for (Member &M : c->mem) build_member_map(c, M);
@@ -2400,7 +2392,7 @@ icarus_status icarus_load(icarus_ctx *c, const char *path) {
   CK(cudaMemcpyAsync(c->floor_prev, &hits, sizeof(hits), cudaMemcpyHostToDevice, s));   // the budget counts from here
   CK(cudaMemsetAsync(c->status, 0, sizeof(unsigned int), s));
   c->status_pending = false;
-  if (!U.empty()) CK(cudaMemcpyAsync(c->U, U.data(), U.size(), cudaMemcpyHostToDevice, s));
+  if ((st = copy_planes(c, 0, c->nleaves, c->kp.nvs, U.data(), false)) != ICARUS_OK) return st;
   if (nth) {
     CK(cudaMemcpyAsync(c->mlp_theta, theta.data(), sizeof(float) * nth, cudaMemcpyHostToDevice, s));
     CK(cudaMemsetAsync(c->mlp_m, 0, sizeof(float) * nth, s));

@@ -10,6 +10,9 @@
 // IEEE FP64 evaluation of the same formula on the same stored state.
 #include <cooperative_groups.h>
 
+#include <algorithm>
+#include <type_traits>
+
 #include "mhd_device.cuh"
 
 namespace cg = cooperative_groups;
@@ -77,6 +80,22 @@ __global__ void k_unpack_tracer(const KParams kp, real *U, int slot0, int nslots
     const int s = (int)(e / kp.icells), c = (int)(e - (size_t)s * kp.icells);
     const int k = c % kp.nb[2], j = (c / kp.nb[2]) % kp.nb[1], i = c / (kp.nb[2] * kp.nb[1]);
     U[tracer_index(kp, slot0 + s, i + NGH, j + NGH, k + NGH)] = (real)in[e];
+  }
+}
+
+// Padded planes [slot][variable][cell] (a checkpoint's order) from and to the
+// cells; blockIdx.x is a plane.  Its side of the state is one value in a cell's
+// 32 or 64 bytes; the copy over the link is what takes the time.
+template <typename real, bool OUT>
+__global__ void k_planes(const KParams kp, real *U, int slot0, int nvars, long long unit0, real *buf) {
+  const long long u = unit0 + blockIdx.x;
+  const int slot = slot0 + (int)(u / nvars), v = (int)(u % nvars);
+  real *b = buf + (size_t)blockIdx.x * kp.pcells;
+  real *cells = U + slot_base(kp, slot) + (v < NVAR ? (size_t)v : (size_t)NVAR * kp.pcells);
+  const size_t step = v < NVAR ? NVAR : 1;
+  for (size_t c = (size_t)blockIdx.y * blockDim.x + threadIdx.x; c < (size_t)kp.pcells; c += (size_t)gridDim.y * blockDim.x) {
+    if (OUT) b[c] = cells[step * c];
+    else cells[step * c] = b[c];
   }
 }
 
@@ -712,6 +731,19 @@ void unpack_tracer_launch(const KParams &kp, void *U, int precision, int slot0, 
     k_unpack_tracer<float><<<1024, 256, 0, s>>>(kp, (float *)U, slot0, nslots, in);
   else
     k_unpack_tracer<double><<<1024, 256, 0, s>>>(kp, (double *)U, slot0, nslots, in);
+}
+
+void planes_launch(const KParams &kp, void *U, int precision, int slot0, int nvars, long long unit0, long long nunits,
+                   void *buf, bool out, cudaStream_t s) {
+  if (nunits <= 0) return;
+  const dim3 grid((unsigned)nunits, (unsigned)std::min((kp.pcells + 1023) / 1024, 1024));
+  auto launch = [&](auto *u, auto *b) {
+    using real = std::remove_pointer_t<decltype(u)>;
+    if (out) k_planes<real, true><<<grid, 256, 0, s>>>(kp, u, slot0, nvars, unit0, b);
+    else k_planes<real, false><<<grid, 256, 0, s>>>(kp, u, slot0, nvars, unit0, b);
+  };
+  if (precision) launch((float *)U, (float *)buf);
+  else launch((double *)U, (double *)buf);
 }
 
 void unpack_state_launch(const KParams &kp, void *U, int precision, int slot0, int nslots, const double *in,
