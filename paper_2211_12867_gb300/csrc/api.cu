@@ -852,12 +852,10 @@ void prof_mark(icarus_ctx *c, int kind, int end) {
   cudaEventRecord(c->ev[c->ev_used], c->stream);
   c->ev_used++;
 }
-// The tile shapes a caller may set.  The library's own choice also takes
-// 8 x 12, 8 x 16, 12 x 16 and 16 x 16.
+// The tile shapes a caller may set: what icarus_set_tile accepts and refuses is
+// part of its interface and no matter of what fits (the library's own choice
+// also takes 8 x 12, 8 x 16, 12 x 16, 16 x 16 and the larger ones of FP64).
 bool tile_settable(const icarus_ctx *c, int tj, int tk) {
-#ifdef ALL_TILES
-  return true;
-#endif
   static const int shapes[][2] = {{8, 8}, {12, 12}, {8, 24}, {4, 32}, {6, 36}, {10, 24}, {12, 20}, {8, 32}};
   // FP64 takes the first seven, with the tracer the first four
   const int n = c->prec ? 8 : (c->d.tracer ? 4 : 7);
