@@ -225,7 +225,9 @@ __device__ __forceinline__ void cons2prim(const real *u, real *w, real gamma, re
   w[6] = u[6];
   w[7] = u[7];
 }
-// FP64: the two energies in one chain of products (14 FP64-pipe instructions)
+// FP64: the two energies in one chain of products (14 FP64-pipe instructions),
+// the radial one, the largest in the wind, last: only it then rounds at the size
+// of the sum, which the pressure is the small difference to.
 template <>
 __device__ __forceinline__ void cons2prim<double>(const double *u, double *w, double gamma, double pfloor, Isl) {
   const double ir = RT<double>::rcp_(u[0]);
@@ -233,7 +235,7 @@ __device__ __forceinline__ void cons2prim<double>(const double *u, double *w, do
   w[1] = u[1] * ir;
   w[2] = u[2] * ir;
   w[3] = u[3] * ir;
-  const double t = u[1] * w[1] + u[2] * w[2] + u[3] * w[3] + u[5] * u[5] + u[6] * u[6] + u[7] * u[7];
+  const double t = fma(u[1], w[1], fma(u[2], w[2], fma(u[3], w[3], u[5] * u[5] + u[6] * u[6] + u[7] * u[7])));
   const double p = (gamma - 1.0) * fma(-0.5, t, u[4]);
   w[4] = RT<double>::less_(p, pfloor) ? pfloor : p;
   w[5] = u[5];
@@ -466,36 +468,35 @@ __device__ __forceinline__ double cfl_rate(double ir, const double *v, double p,
          (fabs(v[2]) + fast_speed_of(ir, gp, hgp, hb2, q0 + q1)) * ix[2];
 }
 
-// One side's part of the TVDLF flux, G = F(W) + sc U(W) with sc = +c_max on
-// the left and -c_max on the right (the flux is (G_L + G_R) / 2), added to the
-// other side's G by the same multiply-adds that form it (LAST) or started.
-// Written out per component with w = v_n + sc:
+// Both sides' parts of the TVDLF flux, G_L + G_R with G = F(W) + sc U(W) and sc =
+// +c_max on the left, -c_max on the right (the flux is half of it).  Per
+// component with w = v_n + sc:
 //   mass rho w;  momentum (rho w) v_k - B_n B_k (+ p_T along n);
 //   energy e w + p_T v_n - B_n (v.B);  induction B_k w - B_n v_k (k != n).
-template <int D, bool LAST>
-__device__ __forceinline__ void side_flux(const double *W, double hb2, double igm1, double sc, double *G) {
-  const double vn = W[1 + D], Bn = W[5 + D];
-  const double w = vn + sc;
-  const double v2 = W[1] * W[1] + W[2] * W[2] + W[3] * W[3];
-  const double pt = W[4] + hb2;
-  const double e = fma(W[4], igm1, fma(0.5 * W[0], v2, hb2));
-  const double vB = W[1] * W[5] + W[2] * W[6] + W[3] * W[7];
-  const double m = W[0] * w;
-  auto add = [&](double a, double b, double &g) { g = LAST ? fma(a, b, g) : a * b; };
-  if (LAST) G[0] += m;
-  else G[0] = m;
+// One chain of multiply-adds a component, the terms with w, the large ones in a
+// fast wind, last: only they round at the size of the sum.  Against 80-bit
+// arithmetic over 37 winds with CMEs on 12 x 16 x 32 cells, five steps, the state
+// is off by 2.3e-16 of its norm (correctly rounded reciprocals and roots, sides
+// added at the end: 2.7e-16).
+template <int D>
+__device__ __forceinline__ void sides_flux(const double *L, const double *R, double hbL, double hbR, double igm1,
+                                           double cm, double *G) {
+  const double vL = L[1 + D], vR = R[1 + D], bL = L[5 + D], bR = R[5 + D];
+  const double wL = vL + cm, wR = vR - cm;
+  const double pL = L[4] + hbL, pR = R[4] + hbR;
+  const double qL = fma(L[1], L[1], fma(L[2], L[2], L[3] * L[3])), qR = fma(R[1], R[1], fma(R[2], R[2], R[3] * R[3]));
+  const double eL = fma(L[4], igm1, fma(0.5 * L[0], qL, hbL)), eR = fma(R[4], igm1, fma(0.5 * R[0], qR, hbR));
+  const double dL = L[1] * L[5] + L[2] * L[6] + L[3] * L[7], dR = R[1] * R[5] + R[2] * R[6] + R[3] * R[7];
+  const double mL = L[0] * wL, mR = R[0] * wR;
+  G[0] = fma(R[0], wR, mL);
 #pragma unroll
   for (int k = 0; k < 3; k++) {
-    add(m, W[1 + k], G[1 + k]);
-    G[1 + k] = fma(-Bn, W[5 + k], G[1 + k]);
-    if (k != D) {
-      add(W[5 + k], w, G[5 + k]);
-      G[5 + k] = fma(-Bn, W[1 + k], G[5 + k]);
-    }
+    double g = fma(-bR, R[5 + k], -(bL * L[5 + k]));
+    if (k == D) g += pL + pR;
+    G[1 + k] = fma(mR, R[1 + k], fma(mL, L[1 + k], g));
+    if (k != D) G[5 + k] = fma(R[5 + k], wR, fma(L[5 + k], wL, fma(-bR, R[1 + k], -(bL * L[1 + k]))));
   }
-  G[1 + D] += pt;
-  add(e, w, G[4]);
-  G[4] = fma(-Bn, vB, fma(pt, vn, G[4]));
+  G[4] = fma(eR, wR, fma(eL, wL, fma(pR, vR, fma(pL, vL, fma(-bR, dR, -(bL * dL))))));
 }
 
 // TVDLF flux from reconstructed face states WL | WR (primitive variables),
@@ -521,8 +522,7 @@ __device__ __forceinline__ void tvdlf_states(double *WL, double *WR, const doubl
   const double cl = RT<double>::abs_(WL[1 + D]) + face_speed(WL[0], gamma * WL[4], hg * WL[4], hbL, tL);
   const double cr = RT<double>::abs_(WR[1 + D]) + face_speed(WR[0], gamma * WR[4], hg * WR[4], hbR, tR);
   const double cm = RT<double>::max_(cl, cr);
-  side_flux<D, false>(WL, hbL, igm1, cm, F2);
-  side_flux<D, true>(WR, hbR, igm1, -cm, F2);
+  sides_flux<D>(WL, WR, hbL, hbR, igm1, cm, F2);
   F2[5 + D] = 0.0;
 }
 
