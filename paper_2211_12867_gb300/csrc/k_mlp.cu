@@ -46,7 +46,7 @@ __device__ __forceinline__ void feature_prims(const KParams &kp, const real *U, 
   ld_cell(U + cell_index(kp, slot, i, j, k), u);
   const double r = widen(u[0]), m1 = widen(u[1]), m2 = widen(u[2]), m3 = widen(u[3]);
   const double b1 = widen(u[5]), b2 = widen(u[6]), b3 = widen(u[7]);
-  const double ir = RT<double>::rcp_(r);
+  const double ir = RT<double>::rcp_inf_(r);
   w[0] = r;
   w[1] = m1 * ir;
   w[2] = (kp.gamma - 1.0) * fma(-0.5, (m1 * m1 + m2 * m2 + m3 * m3) * ir + (b1 * b1 + b2 * b2 + b3 * b3), widen(u[4]));
@@ -60,7 +60,7 @@ __device__ __forceinline__ double feature_of(const double *w0, const double (*d)
 #pragma unroll
   for (int q = 0; q < 3; q++) {
     const double s = d[0][q] * d[0][q] + d[1][q] * d[1][q] + d[2][q] * d[2][q];
-    g += RT<double>::sqrt_(s) * RT<double>::rcp_(fabs(w0[q]) + 1e-30);
+    g += RT<double>::sqrt_inf_(s) * RT<double>::rcp_inf_(fabs(w0[q]) + 1e-30);
   }
   return g;   // of doubled differences: the caller divides by 2 and by 3
 }

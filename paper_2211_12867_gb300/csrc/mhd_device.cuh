@@ -20,7 +20,9 @@ template <typename real> struct RT;
 // (Householder's iteration; the error e^3 is below 2^-56).  Over 4 M arguments
 // of 2^-900 .. 2^900 both are within 1 ulp of the correctly rounded functions
 // (the reciprocal differs in 0.03 % of them, the root in 12 %), at 3 and 5
-// FP64-pipe instructions instead of 5 and 8.
+// FP64-pipe instructions instead of 5 and 8.  1/0, 1/inf and sqrt(inf) are NaN
+// (a step of a state with zero density or an infinite value ends as non-physical
+// in IEEE arithmetic as well), the root of zero and of subnormal numbers is zero.
 template <> struct RT<double> {
   static __device__ __forceinline__ double sqrt_(double x) {
     double y;
@@ -43,6 +45,15 @@ template <> struct RT<double> {
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
     const double e = fma(-x, y, 1.0);
     return fma(y, fma(e, e, e), y);
+  }
+  // the same with IEEE's 1/0, 1/inf and sqrt(inf)
+  static __device__ __forceinline__ double sqrt_inf_(double x) {
+    return __double2hiint(x) == 0x7ff00000 ? x : sqrt_(x);
+  }
+  static __device__ __forceinline__ double rcp_inf_(double x) {
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));   // infinite or zero: the result
+    return ((unsigned)__double2hiint(y) & 0x7fffffffu) - 0x00100000u < 0x7fe00000u ? rcp_(x) : y;
   }
   // x > 0; not for NaN
   static __device__ __forceinline__ bool pos_(double x) {
