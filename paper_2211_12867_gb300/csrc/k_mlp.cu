@@ -48,7 +48,11 @@ __device__ __forceinline__ void feature_prims(const KParams &kp, const real *U, 
   const double b1 = widen(u[5]), b2 = widen(u[6]), b3 = widen(u[7]);
   const double ir = RT<double>::rcp_inf_(r);
   w[0] = r;
-  w[1] = m1 * ir;
+  // the quotient with its remainder: equal speeds come out equal whatever the
+  // densities (infinite and zero ones as they are)
+  const double v = m1 * ir;
+  const bool normal = ((unsigned)__double2hiint(v) & 0x7fffffffu) - 0x00100000u < 0x7fe00000u;
+  w[1] = normal ? fma(fma(-v, r, m1), ir, v) : v;
   w[2] = (kp.gamma - 1.0) * fma(-0.5, (m1 * m1 + m2 * m2 + m3 * m3) * ir + (b1 * b1 + b2 * b2 + b3 * b3), widen(u[4]));
 }
 
@@ -219,9 +223,10 @@ __device__ __forceinline__ void pair_prims(const KParams &kp, const float *U, in
   const float2 K = pair_add(pair_mul(M, ir), B);
   const float2 P = pair_add(make_float2(E, 0.f), make_float2(-0.5f * K.x, -0.5f * K.y));
   if (P.x >= 0x1p-12f * E && E > 1e-20f && E < 1e15f && r > 1e-24f && r < 1e15f && r * E > 1e-31f) {
-    const float2 v = pair_mul(make_float2(u[1], 0.f), ir), p = pair_mul(P, gm1);
+    const float2 p = pair_mul(P, gm1);
+    const float v = __fmul_rn(u[1], ir.x);   // and its remainder, as in feature_prims
     w[0] = make_float2(r, 0.f);
-    w[1] = renorm(v.x, v.y);
+    w[1] = renorm(v, __fmul_rn(__fmaf_rn(-v, r, u[1]), ir.x));
     w[2] = renorm(p.x, p.y);
     ratio = fmaxf(ratio, __fdividef(E, P.x));
   } else {
@@ -236,6 +241,17 @@ __device__ __forceinline__ void pair_prims(const KParams &kp, const float *U, in
   }
 }
 
+// A sub-cube whose feature is below FEAT_REL E / p (its differences are within
+// the pairs' last 26 bits) is done again in FP64: the feature's relative
+// error is 2^-46 (E / p) / f at most, 2^-26 where the pairs are kept, a
+// quarter of the final rounding.  Smooth wind has features of 1e-3 and more
+// and E / p of 100 to 300.
+// That is for neighbours of the cell's own size, up to twice it.  Where they are
+// c times it, their errors count c times: a cell whose own term is below FEAT_REL
+// c, in the pressure, whose E / p is 2^12 at most, 2^12 times that, sends its
+// sub-cube to FP64 as well.
+constexpr float FEAT_REL = 0x1p-20f;
+
 // feature_of in pairs, of the cell at P[q stride] (planes before, of and behind
 // it; rows of h2); the differences are taken relative to the cell first, so
 // that their squares stay in range whatever the units
@@ -245,35 +261,40 @@ __device__ __forceinline__ float2 pair_feature(const float2 *Pm, const float2 *P
   for (int q = 0; q < 3; q++) {
     const float2 *C = P + q * stride;
     auto diff = [](float2 a, float2 b) { return pair_add(a, make_float2(-b.x, -b.y)); };
-    const float2 d0 = diff(Pp[q * stride], Pm[q * stride]), d1 = diff(C[h2], C[-h2]), d2 = diff(C[1], C[-1]);
+    const float2 p0 = Pp[q * stride], p1 = C[h2], p2 = C[1];
+    const float2 d0 = diff(p0, Pm[q * stride]), d1 = diff(p1, C[-h2]), d2 = diff(p2, C[-1]);
+    // the others are as large, or d tells
+    auto top = [&] { return fmaxf(fmaxf(fabsf(p0.x), fabsf(p1.x)), fabsf(p2.x)); };
     const float sg = C->x < 0.f ? -1.f : 1.f;
     float2 w = make_float2(sg * C->x, sg * C->y);
     if (w.x < 1e-15f) {   // where the 1e-30 that the magnitude is raised by counts
       w = pair_add(w, make_float2(1e-30f, 0.f));
-      // too small for a pair: nothing if the neighbours are equal, else FP64
+      // too small for a pair: nothing if the neighbours are equal and as small,
+      // else FP64
       if (w.x < 1e-22f) {
-        if (!(d0.x == 0.f && d1.x == 0.f && d2.x == 0.f)) g.x = INFINITY;
+        if (!(d0.x == 0.f && d1.x == 0.f && d2.x == 0.f && top() <= 2.f * w.x)) g.x = INFINITY;
         continue;
       }
     }
     const float2 y = pair_rcp(w);
     const float2 s = pair_norm2(pair_mul(d0, y), pair_mul(d1, y), pair_mul(d2, y));
+    float f = 0.f;
     if (s.x != 0.f) {
       float t;
       asm("rsqrt.approx.f32 %0, %1;" : "=f"(t) : "f"(s.x));
-      const float f = __fmul_rn(s.x, t), e = __fadd_rn(__fmaf_rn(-f, f, s.x), s.y);
+      f = __fmul_rn(s.x, t);
+      const float e = __fadd_rn(__fmaf_rn(-f, f, s.x), s.y);
       g = pair_add(g, make_float2(f, __fmul_rn(0.5f * t, e)));
+    }
+    // neighbours far above the cell that nearly agree (see FEAT_REL; densities
+    // are exact): FP64
+    if (q > 0) {
+      const float c = top() * y.x;
+      if (c > 2.f && !(f >= (q == 2 ? 4096.f * FEAT_REL : FEAT_REL) * c)) g.x = INFINITY;
     }
   }
   return g;
 }
-
-// A sub-cube whose feature is below FEAT_REL E / p (its differences are within
-// the pairs' last 26 bits) is done again in FP64: the feature's relative
-// error is 2^-46 (E / p) / f at most, 2^-26 where the pairs are kept, a
-// quarter of the final rounding.  Smooth wind has features of 1e-3 and more
-// and E / p of 100 to 300.
-constexpr float FEAT_REL = 0x1p-20f;
 
 // k_features for FP32 states.  The halo cells at a plane's corners are not
 // read: a 12 x 12 plane takes the 192 threads once.  A sub-cube's sum and its
