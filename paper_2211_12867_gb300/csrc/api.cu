@@ -1120,7 +1120,8 @@ icarus_status recompute_dt(icarus_ctx *c) {
   return ICARUS_OK;
 }
 
-// the page-locked piece that holds host address p, if any
+// the page-locked piece that holds host address p and that the device may
+// write, if any
 bool pinned_piece(uintptr_t p, PinnedPiece *q) {
   using Attribute = CUresult(CUDAAPI *)(void *, CUpointer_attribute, CUdeviceptr);
   static const Attribute get = [] {
@@ -1139,7 +1140,10 @@ bool pinned_piece(uintptr_t p, PinnedPiece *q) {
     return false;
   }
   CUdeviceptr start = 0;
+  unsigned access = 0;   // memory may be page-locked for reading only
   if (a.type != cudaMemoryTypeHost ||
+      get(&access, CU_POINTER_ATTRIBUTE_ACCESS_FLAGS, (CUdeviceptr)p) != CUDA_SUCCESS ||
+      access != CU_POINTER_ATTRIBUTE_ACCESS_FLAG_READWRITE ||
       get(&start, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, (CUdeviceptr)p) != CUDA_SUCCESS ||
       get(&q->bytes, CU_POINTER_ATTRIBUTE_RANGE_SIZE, (CUdeviceptr)p) != CUDA_SUCCESS)
     return false;
