@@ -210,8 +210,8 @@ __global__ void k_estimator(const KParams kp, const real *U, int slot0, double e
 // without an open gate is done after its gate test.  Five CTAs per SM (48
 // registers, spills on the exact path only): a slab is a chain of short phases,
 // and two CTAs per SM at 108 registers took 201 us for 1914 leaves of 12^3 FP32
-// cells on three levels; now 119 us, one CTA per leaf 367.  808 leaves: 53 us,
-// before 220.
+// cells on three levels; now 124 us, one CTA per leaf 367.  808 leaves: 50 to 62
+// us, before 220.
 constexpr int EST_CTAS = 4;
 
 // Pressure to within one FP32 rounding of est_pressure's.  FP64 state: FP64

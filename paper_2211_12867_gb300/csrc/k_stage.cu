@@ -27,7 +27,7 @@
 //
 // What bounds it.  FP32: latency and the barrier between the phases of a
 // plane, with 53 to 56 % of the issue slots used by 16 warps per SM at 128
-// registers; DRAM is idle (a fifth of its peak).  More CTAs at fewer
+// registers; DRAM is idle (16 % of its peak).  More CTAs at fewer
 // registers, a single flux buffer with a second barrier, and the staging of
 // U^n in shared memory were slower.  512 x 60 x 180 cells in 64 x 60 x 180
 // blocks: predictor 400 -> 281 us, corrector 489 -> 374 us since cells are

@@ -461,6 +461,8 @@ class Icarus:
 
 MLP_PARAMS = 128 * 64 + 128 + 128 * 128 + 128 + 128 + 1
 
+# ghost_neighbour: prolongations; ghost_physical: physical boundaries,
+# restrictions and copies (names kept for the reports that use them)
 PROFILE_KINDS = ["dt_begin", "ghost_neighbour", "ghost_physical", "stage_predictor", "stage_corrector",
                  "reflux", "dt_finalize", "estimator", "regrid_move", "dt_full"]
 STEP_KINDS = 7   # the first seven kinds are the step's launches
