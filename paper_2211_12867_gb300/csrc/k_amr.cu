@@ -41,21 +41,22 @@ __global__ void k_pack(const KParams kp, const real *U, int slot0, int nslots, d
   }
 }
 
-template <typename real>
-__global__ void k_unpack(const KParams kp, real *U, int slot0, int nslots, const double *in, int is_prim) {
+template <typename real, bool PRIM>
+__global__ void __launch_bounds__(256) k_unpack(const KParams kp, real *U, int slot0, int nslots, const double *in) {
   const size_t n = (size_t)nslots * kp.icells;
   for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
-    const int c = (int)(e % kp.icells);
-    const int s = (int)(e / kp.icells);
-    const int k = c % kp.nb[2], j = (c / kp.nb[2]) % kp.nb[1], i = c / (kp.nb[2] * kp.nb[1]);
-    double x[NVAR], u[NVAR];
+    const int s = (int)(e / kp.icells), c = (int)(e - (size_t)s * kp.icells);
+    double u[NVAR];
+    if constexpr (PRIM) {
+      double x[NVAR];
 #pragma unroll
-    for (int v = 0; v < NVAR; v++) x[v] = in[((size_t)s * NVAR + v) * kp.icells + c];
-    if (is_prim)
+      for (int v = 0; v < NVAR; v++) x[v] = in[((size_t)s * NVAR + v) * kp.icells + c];
       prim2cons<double>(x, u, 1.0 / (kp.gamma - 1.0));
-    else
+    } else {
 #pragma unroll
-      for (int v = 0; v < NVAR; v++) u[v] = x[v];
+      for (int v = 0; v < NVAR; v++) u[v] = in[((size_t)s * NVAR + v) * kp.icells + c];
+    }
+    const int k = c % kp.nb[2], j = (c / kp.nb[2]) % kp.nb[1], i = c / (kp.nb[2] * kp.nb[1]);
     real o[NVAR];
 #pragma unroll
     for (int v = 0; v < NVAR; v++) o[v] = (real)u[v];
@@ -749,10 +750,13 @@ void planes_launch(const KParams &kp, void *U, int precision, int slot0, int nva
 void unpack_state_launch(const KParams &kp, void *U, int precision, int slot0, int nslots, const double *in,
                          int is_prim, cudaStream_t s) {
   if (nslots <= 0) return;
-  if (precision)
-    k_unpack<float><<<1024, 256, 0, s>>>(kp, (float *)U, slot0, nslots, in, is_prim);
-  else
-    k_unpack<double><<<1024, 256, 0, s>>>(kp, (double *)U, slot0, nslots, in, is_prim);
+  auto launch = [&](auto *u) {
+    using real = std::remove_pointer_t<decltype(u)>;
+    if (is_prim) k_unpack<real, true><<<1024, 256, 0, s>>>(kp, u, slot0, nslots, in);
+    else k_unpack<real, false><<<1024, 256, 0, s>>>(kp, u, slot0, nslots, in);
+  };
+  if (precision) launch((float *)U);
+  else launch((double *)U);
 }
 
 namespace {
