@@ -1662,26 +1662,16 @@ icarus_status icarus_get_state(icarus_ctx *c, int member, double *host, size_t n
   return ICARUS_OK;
 }
 
-// Padded planes [slot][variable][cell] of nslots leaves, the first nvars
-// variables of each, between host memory and the state's cells, turned on the
-// device in pieces of the staging buffer (a plane fits: blocks are four cells
-// or more, so it is at most eight interiors).
-static icarus_status copy_planes(icarus_ctx *c, int slot0, int nslots, int nvars, unsigned char *host, bool to_host) {
-  const size_t plane = (size_t)c->kp.pcells * c->rsize, units = (size_t)nslots * nvars;
-  const size_t piece = c->lay.staging_doubles * sizeof(double) / plane;
-  for (size_t u0 = 0; u0 < units; u0 += piece) {
-    const size_t n = std::min(piece, units - u0);
-    if (to_host) {
-      planes_launch(c->kp, c->U, c->prec, slot0, nvars, (long long)u0, (long long)n, c->staging, true, c->stream);
-      CK(cudaPeekAtLastError());
-      CK(cudaMemcpyAsync(host + u0 * plane, c->staging, n * plane, cudaMemcpyDeviceToHost, c->stream));
-    } else {
-      CK(cudaMemcpyAsync(c->staging, host + u0 * plane, n * plane, cudaMemcpyHostToDevice, c->stream));
-      planes_launch(c->kp, c->U, c->prec, slot0, nvars, (long long)u0, (long long)n, c->staging, false, c->stream);
-      CK(cudaPeekAtLastError());
-    }
-    CK(cudaStreamSynchronize(c->stream));
-  }
+// Padded planes [slot][variable][cell] of nslots leaves between host memory and
+// the state's cells, turned on the device in the stage buffer, which holds
+// nothing between steps.  bytes: of the planes wanted (those of the last leaf may
+// end early).  The caller synchronises.
+static icarus_status copy_planes(icarus_ctx *c, int slot0, int nslots, unsigned char *host, size_t bytes, bool to_host) {
+  if (bytes == 0) return ICARUS_OK;
+  if (!to_host) CK(cudaMemcpyAsync(c->Us, host, bytes, cudaMemcpyHostToDevice, c->stream));
+  planes_launch(c->kp, c->U, c->prec, slot0, nslots, c->Us, to_host, c->stream);
+  CK(cudaPeekAtLastError());
+  if (to_host) CK(cudaMemcpyAsync(host, c->Us, bytes, cudaMemcpyDeviceToHost, c->stream));
   return ICARUS_OK;
 }
 
@@ -1690,8 +1680,9 @@ icarus_status icarus_get_padded(icarus_ctx *c, int member, int leaf, double *hos
   const int nl = (int)c->mem[member].leaves.size();
   if (leaf < 0 || leaf >= nl || n != (size_t)NVAR * c->kp.pcells) return ICARUS_ERR_ARG;
   std::vector<unsigned char> raw(n * c->rsize);
-  const icarus_status st = copy_planes(c, c->mem_off[member] + leaf, 1, NVAR, raw.data(), true);
+  const icarus_status st = copy_planes(c, c->mem_off[member] + leaf, 1, raw.data(), raw.size(), true);
   if (st != ICARUS_OK) return st;
+  CK(cudaStreamSynchronize(c->stream));
   if (c->prec) {
     const float *f = reinterpret_cast<const float *>(raw.data());
     for (size_t q = 0; q < n; q++) host[q] = (double)f[q];
@@ -2276,7 +2267,7 @@ icarus_status icarus_save(icarus_ctx *c, const char *path) {
   if (!theta.empty())
     CK(cudaMemcpyAsync(theta.data(), c->mlp_theta, sizeof(float) * theta.size(), cudaMemcpyDeviceToHost, s));
   // a checkpoint holds a slot's variables one after the other
-  const icarus_status st = copy_planes(c, 0, c->nleaves, c->kp.nvs, U.data(), true);
+  const icarus_status st = copy_planes(c, 0, c->nleaves, U.data(), U.size(), true);
   if (st != ICARUS_OK) return st;
   CK(cudaStreamSynchronize(s));
   CkFile F;
@@ -2394,7 +2385,7 @@ icarus_status icarus_load(icarus_ctx *c, const char *path) {
   CK(cudaMemcpyAsync(c->floor_prev, &hits, sizeof(hits), cudaMemcpyHostToDevice, s));   // the budget counts from here
   CK(cudaMemsetAsync(c->status, 0, sizeof(unsigned int), s));
   c->status_pending = false;
-  if ((st = copy_planes(c, 0, c->nleaves, c->kp.nvs, U.data(), false)) != ICARUS_OK) return st;
+  if ((st = copy_planes(c, 0, c->nleaves, U.data(), U.size(), false)) != ICARUS_OK) return st;
   if (nth) {
     CK(cudaMemcpyAsync(c->mlp_theta, theta.data(), sizeof(float) * nth, cudaMemcpyHostToDevice, s));
     CK(cudaMemsetAsync(c->mlp_m, 0, sizeof(float) * nth, s));

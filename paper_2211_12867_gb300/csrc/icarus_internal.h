@@ -199,10 +199,10 @@ void pack_tracer_launch(const KParams &kp, const void *U, int precision, int slo
                         cudaStream_t s);
 void unpack_tracer_launch(const KParams &kp, void *U, int precision, int slot0, int nslots, const double *in,
                           cudaStream_t s);
-// padded planes unit0 .. unit0 + nunits - 1, counted [slot from slot0][variable
-// below nvars], out of the state's cells (out) or into them
-void planes_launch(const KParams &kp, void *U, int precision, int slot0, int nvars, long long unit0, long long nunits,
-                   void *buf, bool out, cudaStream_t s);
+// padded planes [slot from slot0][variable][cell], the tracer's among them, out of
+// the state's cells (out) or into them
+void planes_launch(const KParams &kp, void *U, int precision, int slot0, int nslots, void *planes, bool out,
+                   cudaStream_t s);
 void unpack_state_launch(const KParams &kp, void *U, int precision, int slot0, int nslots, const double *in,
                          int is_prim, cudaStream_t s);
 void estimator_launch(const KParams &kp, const void *U, int precision, int slot0, int nslots, double e_ref,

@@ -85,18 +85,25 @@ __global__ void k_unpack_tracer(const KParams kp, real *U, int slot0, int nslots
 }
 
 // Padded planes [slot][variable][cell] (a checkpoint's order) from and to the
-// cells; blockIdx.x is a plane.  Its side of the state is one value in a cell's
-// 32 or 64 bytes; the copy over the link is what takes the time.
+// cells; blockIdx.x is a leaf.  Bound by memory, and the copy over the link that
+// goes with it takes ten times as long.
 template <typename real, bool OUT>
-__global__ void k_planes(const KParams kp, real *U, int slot0, int nvars, long long unit0, real *buf) {
-  const long long u = unit0 + blockIdx.x;
-  const int slot = slot0 + (int)(u / nvars), v = (int)(u % nvars);
-  real *b = buf + (size_t)blockIdx.x * kp.pcells;
-  real *cells = U + slot_base(kp, slot) + (v < NVAR ? (size_t)v : (size_t)NVAR * kp.pcells);
-  const size_t step = v < NVAR ? NVAR : 1;
-  for (size_t c = (size_t)blockIdx.y * blockDim.x + threadIdx.x; c < (size_t)kp.pcells; c += (size_t)gridDim.y * blockDim.x) {
-    if (OUT) b[c] = cells[step * c];
-    else cells[step * c] = b[c];
+__global__ void __launch_bounds__(256) k_planes(const KParams kp, real *U, int slot0, real *planes) {
+  real *cells = U + slot_base(kp, slot0 + blockIdx.x), *p = planes + slot_base(kp, blockIdx.x);
+  const size_t n = kp.pcells;
+  for (size_t c = (size_t)blockIdx.y * blockDim.x + threadIdx.x; c < n; c += (size_t)gridDim.y * blockDim.x) {
+    real u[NVAR];
+    if (OUT) ld_cell(cells + NVAR * c, u);
+#pragma unroll
+    for (int v = 0; v < NVAR; v++) {
+      if (OUT) p[v * n + c] = u[v];
+      else u[v] = p[v * n + c];
+    }
+    if (!OUT) st_cell(cells + NVAR * c, u);
+    if (kp.nvs > NVAR) {   // the tracer's plane is one in both
+      if (OUT) p[NVAR * n + c] = cells[NVAR * n + c];
+      else cells[NVAR * n + c] = p[NVAR * n + c];
+    }
   }
 }
 
@@ -734,17 +741,17 @@ void unpack_tracer_launch(const KParams &kp, void *U, int precision, int slot0, 
     k_unpack_tracer<double><<<1024, 256, 0, s>>>(kp, (double *)U, slot0, nslots, in);
 }
 
-void planes_launch(const KParams &kp, void *U, int precision, int slot0, int nvars, long long unit0, long long nunits,
-                   void *buf, bool out, cudaStream_t s) {
-  if (nunits <= 0) return;
-  const dim3 grid((unsigned)nunits, (unsigned)std::min((kp.pcells + 1023) / 1024, 1024));
-  auto launch = [&](auto *u, auto *b) {
+void planes_launch(const KParams &kp, void *U, int precision, int slot0, int nslots, void *planes, bool out,
+                   cudaStream_t s) {
+  if (nslots <= 0) return;
+  const dim3 grid(nslots, (unsigned)std::min((kp.pcells + 1023) / 1024, 65535));
+  auto launch = [&](auto *u, auto *p) {
     using real = std::remove_pointer_t<decltype(u)>;
-    if (out) k_planes<real, true><<<grid, 256, 0, s>>>(kp, u, slot0, nvars, unit0, b);
-    else k_planes<real, false><<<grid, 256, 0, s>>>(kp, u, slot0, nvars, unit0, b);
+    if (out) k_planes<real, true><<<grid, 256, 0, s>>>(kp, u, slot0, p);
+    else k_planes<real, false><<<grid, 256, 0, s>>>(kp, u, slot0, p);
   };
-  if (precision) launch((float *)U, (float *)buf);
-  else launch((double *)U, (double *)buf);
+  if (precision) launch((float *)U, (float *)planes);
+  else launch((double *)U, (double *)planes);
 }
 
 void unpack_state_launch(const KParams &kp, void *U, int precision, int slot0, int nslots, const double *in,

@@ -16,8 +16,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 STR = dict(x_min=(0.1, math.pi / 6, 0.0), x_max=(2.0, 5 * math.pi / 6, 2 * math.pi), stretch=True)
 
 
-# a block whose plane takes the whole staging buffer of a leaf, ragged ones, and
-# more leaves than one piece holds
+# the smallest block, ragged ones, large ones
 @pytest.mark.parametrize("precision", [FP64, FP32_MIXED])
 @pytest.mark.parametrize("n,nb", [((4, 4, 4), (4, 4, 4)), ((12, 6, 10), (6, 6, 10)), ((128, 60, 180), (64, 60, 60))])
 def test_planes_of_a_checkpoint(n, nb, precision, tmp_path):
